@@ -71,6 +71,8 @@ using namespace dev;
 template <bool DENSE, bool EP_SMEM, bool H>
 __global__ void __launch_bounds__(kSearchWarps * 32, 1)
     k_search(const SearchParams P) {
+  // a screened search: the listed kernel has it, unless the list is too long
+  if (!DENSE && P.n_list && __ldg(P.n_list) <= P.list_cap) return;
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
@@ -217,6 +219,160 @@ __global__ void __launch_bounds__(kSearchWarps * 32, 1)
       }
       out[i] = e;
     }
+  }
+}
+
+// The search of the listed trajectories (k_screen.cu), the same top-K as
+// k_search over the whole range: per warp group the larger screening
+// subsets first, then for the trajectories left the light curve itself
+// (phase 1, the FP64 solve and its bound, phase 2) with the same device
+// functions, so the same bits.  The list holds a few per cent of the grid,
+// its entries scattered over the lines, so cells come through L1 (no band
+// tables) and every sweep takes its trajectories in pairs (the last of an
+// odd number twice: one copy of the sweep's code).
+//
+// A subset whose bounds discard too little to pay for itself (light curves
+// of weak signal) is left out by a warp once it has seen that, but for
+// every sixteenth group, which keeps looking.
+template <bool EPS, bool H>
+__global__ void __launch_bounds__(kSearchWarps * 32, 1)
+    k_search_list(const SearchParams P) {
+  const unsigned n = __ldg(P.n_list);
+  if (n > P.list_cap) return;  // k_search has it
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5;
+  const int K = P.top_k;
+  BlockTopK T;
+  __shared__ int s_cur, s_nk, s_lock, s_next;
+  __shared__ double s_thr;
+  unsigned char *p = smem;
+  T.buf0 = reinterpret_cast<Entry *>(p);
+  T.buf1 = T.buf0 + K;
+  T.wbuf = T.buf1 + K;
+  p += sizeof(Entry) * ((size_t)2 * K + kSearchWarps * 32);
+  T.cur = &s_cur;
+  T.nk = &s_nk;
+  T.lock = &s_lock;
+  T.thr = &s_thr;
+  float4 *sm_ep = reinterpret_cast<float4 *>(p);
+  if (EPS) {  // the light curve and subsets 1 .. n_lv - 1 after it
+    float4 *d = sm_ep;
+    for (int e = threadIdx.x; e < P.n_ep; e += blockDim.x) d[e] = P.ep[e];
+    d += P.n_ep;
+    for (int l = 1; l < P.n_lv; ++l) {
+      for (int e = threadIdx.x; e < P.lv[l].m; e += blockDim.x)
+        d[e] = P.lv[l].ep[e];
+      d += P.lv[l].m;
+    }
+  }
+  if (threadIdx.x == 0) {
+    s_cur = 0;
+    s_nk = 0;
+    s_lock = P.lock0;
+    s_next = 0;
+    s_thr = CUDART_INF;
+  }
+  __syncthreads();
+
+  // entries per group: few enough that every warp of the grid has work
+  const unsigned warps = gridDim.x * kSearchWarps;
+  int tpg = 2;
+  while (tpg < 32 && (unsigned)tpg * warps < n) tpg <<= 1;
+  const unsigned n_groups = (n + tpg - 1) / tpg;
+  unsigned long long n_exact = 0;
+  unsigned tried[kScreenLevels] = {}, killed[kScreenLevels] = {};
+  for (int seen = 0;; ++seen) {
+    unsigned g = 0;
+    if (lane == 0) g = (unsigned)atomicAdd(&s_next, 1);
+    g = __shfl_sync(kFull, g, 0) * gridDim.x + blockIdx.x;
+    if (g >= n_groups) break;
+    const unsigned lo = g * tpg;
+    const int nv = (int)min((unsigned)tpg, n - lo);
+    const unsigned off = P.list[lo + (lane < nv ? lane : 0)];
+    const unsigned my = (unsigned)P.first + off;
+    double xi, xo;
+    TrajC mine = traj_base_of(P, my, xi, xo);
+    const float xin = __double2float_rd(xi), xout = __double2float_ru(xo);
+    double thr = *T.thr;
+    if (P.gthr) thr = fmin(thr, bits_to_chi2(__ldcg(P.gthr)));
+    const float thr_f = __double2float_ru(thr);
+    unsigned act = nv == 32 ? kFull : (1u << nv) - 1u;
+    Acc ms;
+    const float4 *lv_ep = EPS ? sm_ep + P.n_ep : nullptr;
+    for (int l = 1; l <= P.n_lv; ++l) {
+      const bool last = l == P.n_lv;  // the light curve itself
+      const int m = last ? P.n_ep : P.lv[l].m;
+      const float4 *blk = EPS ? (last ? sm_ep : lv_ep)
+                              : (last ? P.ep : P.lv[l].ep);
+      if (!last) {
+        lv_ep += m;
+        const unsigned t = tried[l], k = killed[l];
+        if (t >= 64 && (seen & 15) != 0 &&
+            (float)k * (float)(P.n_ep - m) < (float)t * (float)m)
+          continue;
+      }
+      const Epochs ep = epochs_at(blk, m);
+      mine.e_in = epoch_search_f(ep, m, xin, true);
+      mine.e_out = max(mine.e_in, epoch_search_f(ep, m, xout, false));
+      ms = {0.f, 0.f, 0.f};
+      for (unsigned todo = act; todo;) {
+        const int k = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const int k2 = todo ? __ffs(todo) - 1 : k;
+        todo &= todo - 1;
+        const TrajC ca = shfl_traj(mine, k), cb = shfl_traj(mine, k2);
+        Acc ra, rb;
+        phase1_pair_n<H>(P, ep, m, ca, cb, lane, ra, rb);
+        if (lane == k2) ms = rb;
+        if (lane == k) ms = ra;
+      }
+      if (!last) {
+        const bool stay = (act >> lane & 1u) && screen_lb(P.lv[l], ms) <= thr_f;
+        const unsigned left = __ballot_sync(kFull, stay);
+        tried[l] += __popc(act);
+        killed[l] += __popc(act & ~left);
+        act = left;
+        if (!act) break;
+      }
+    }
+    if (!act) continue;
+    const Epochs ep = epochs_at(EPS ? sm_ep : P.ep, P.n_ep);
+    const Solved sol =
+        solve2(P, (double)ms.a, (double)ms.b, (double)ms.d);
+    bool cand = act >> lane & 1u;
+    if (cand && thr < CUDART_INF) cand = may_reach(P, sol, thr);
+    const float myFs = __double2float_rn(sol.Fs);
+    const float myBc = __double2float_rn(sol.Bc);
+    double my_chi2 = CUDART_INF;
+    unsigned todo = __ballot_sync(kFull, cand);
+    n_exact += __popc(todo);
+    while (todo) {
+      const int k = __ffs(todo) - 1;
+      todo &= todo - 1;
+      const TrajC c = shfl_traj(mine, k);
+      const double chi2 =
+          phase2<H>(P, ep, c, lane, __shfl_sync(kFull, myFs, k),
+                    __shfl_sync(kFull, myBc, k));
+      if (lane == k) my_chi2 = isnan(chi2) ? CUDART_INF : chi2;
+    }
+    const bool keep = my_chi2 <= thr && my_chi2 < CUDART_INF;
+    warp_merge(P, T, K, warp, lane, keep, my_chi2, (long long)my);
+  }
+  if (P.stat_exact && lane == 0 && n_exact) atomicAdd(P.stat_exact, n_exact);
+  __syncthreads();
+  const int nk = s_nk;
+  const Entry *cur = s_cur ? T.buf1 : T.buf0;
+  Entry *out = P.partial + (size_t)blockIdx.x * K;
+  for (int i = threadIdx.x; i < K; i += blockDim.x) {
+    Entry e;
+    if (i < nk) {
+      e = cur[i];
+    } else {
+      e.chi2 = CUDART_INF;  // unique sentinel keys, ascending
+      e.idx = 0x7fff000000000000LL + ((long long)blockIdx.x * K + i);
+    }
+    out[i] = e;
   }
 }
 
@@ -501,6 +657,53 @@ cudaError_t launch_search(const SearchParams &P, bool dense, bool ep_smem,
     launch_search_h<true>(P, dense, ep_smem, grid, smem, st);
   else
     launch_search_h<false>(P, dense, ep_smem, grid, smem, st);
+  return cudaGetLastError();
+}
+
+size_t list_smem_bytes(const SearchParams &P, bool staged) {
+  size_t n = 0;
+  if (staged) {
+    n = (size_t)P.n_ep;
+    for (int l = 1; l < P.n_lv; ++l) n += (size_t)P.lv[l].m;
+  }
+  return search_smem_bytes((int)n, P.top_k);
+}
+
+template <bool E, bool H>
+static int list_occupancy(size_t smem) {
+  if (cudaFuncSetAttribute(k_search_list<E, H>,
+                           cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)smem) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  int b = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+          &b, k_search_list<E, H>, kSearchWarps * 32, smem) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return b;
+}
+
+int list_blocks_per_sm(bool staged, bool h16, size_t smem) {
+  if (staged) return h16 ? list_occupancy<true, true>(smem)
+                         : list_occupancy<true, false>(smem);
+  return h16 ? list_occupancy<false, true>(smem)
+             : list_occupancy<false, false>(smem);
+}
+
+cudaError_t launch_search_list(const SearchParams &P, bool staged, int grid,
+                               size_t smem, cudaStream_t st) {
+  const int threads = kSearchWarps * 32;
+  if (staged && P.quadh)
+    k_search_list<true, true><<<grid, threads, smem, st>>>(P);
+  else if (staged)
+    k_search_list<true, false><<<grid, threads, smem, st>>>(P);
+  else if (P.quadh)
+    k_search_list<false, true><<<grid, threads, smem, st>>>(P);
+  else
+    k_search_list<false, false><<<grid, threads, smem, st>>>(P);
   return cudaGetLastError();
 }
 

@@ -508,6 +508,22 @@ void event_params(const morse_event *ev, SearchParams *P) {
   P->CFF = ev->CFF;
   const double m = (double)((ev->n + 31) / 32);
   P->gamma = (m + 10.0) * ldexp(1.0, -24);
+  P->n_lv = ev->n_sub;
+  for (int l = 0; l < ev->n_sub; ++l) {
+    const morse_subset &u = ev->sub[l];
+    ScreenLv &V = P->lv[l];
+    V.ep = ev->ep + u.off;
+    V.m = u.m;
+    V.S1 = (float)u.S1;
+    V.iS1 = (float)(1.0 / u.S1);
+    V.SF = (float)u.SF;
+    V.sqSFF = nextafterf((float)sqrt(u.SFF), INFINITY);
+    V.CFF = nextafterf((float)(u.SFF - u.SF * u.SF / u.S1), 0.0f);
+    // terms of one sum: the smallest subset is summed by one lane, the
+    // others by 32
+    const double k = l == 0 ? (double)u.m : (double)((u.m + 31) / 32);
+    V.g = (float)(2.0 * (k + 12.0) * ldexp(1.0, -24));
+  }
 }
 
 void grid_params(const morse_grid *g, const Tables &T, SearchParams *P) {
@@ -551,6 +567,9 @@ struct Plan {
   int grid;
   size_t off_tab, off_lmax, off_hdr, off_pub, off_pa, off_pb, off_out, bytes;
   int tab_n;  // band-table entries (0: the search reads the global table)
+  // screened search (k_screen.cu); want = 0: off
+  unsigned want, pilot_cap, list_cap;
+  size_t off_code, off_hist, off_pil, off_ub, off_list;
 };
 
 // What the line-aligned pass needs to read its map cells from shared-memory
@@ -596,6 +615,36 @@ morse_status hdr_init(morse_ctx *ctx, char *base, const Plan &pl,
   P->err = &h->err;
   P->stat_exact = &h->stat_exact;
   return MORSE_OK;
+}
+
+// Pilot trajectories whose bounds seed the pruning threshold.
+double pilot_want(int K, long long count) {
+  return std::max(morse::kPilotMinK * K,
+                  morse::kPilotSqrt * std::sqrt((double)K * (double)count));
+}
+
+// Whether a top-K search of `count` trajectories is screened, and the
+// workspace of it from offset `at` on.
+size_t plan_screen(const morse_event *ev, const morse_grid *g,
+                   long long count, size_t at, Plan *pl) {
+  pl->want = 0;
+  const double want = std::max(pilot_want(pl->K, count), 512.0);
+  const double total =
+      (double)g->n_u0 * g->n_alpha * (double)g->n_t0 * g->n_tE;
+  if (ev->n_sub < 1 || count < 16384 || count > (1LL << 25) ||
+      total >= 2147483648.0 || want * 4.0 > (double)count)
+    return at;
+  pl->want = (unsigned)want;
+  pl->pilot_cap = 2 * pl->want;
+  pl->list_cap = (unsigned)(count / 2);
+  pl->off_hist = align_up(at, 256);  // histogram and list lengths: cleared
+  pl->off_code =
+      align_up(pl->off_hist + sizeof(unsigned) * (morse::kScreenBins + 2), 256);
+  pl->off_pil = align_up(
+      pl->off_code + sizeof(unsigned short) * (size_t)(count + 8), 256);
+  pl->off_ub = pl->off_pil + sizeof(unsigned) * (size_t)pl->pilot_cap;
+  pl->off_list = pl->off_ub + sizeof(float) * (size_t)pl->pilot_cap;
+  return pl->off_list + sizeof(unsigned) * (size_t)pl->list_cap;
 }
 
 // Reset the pruning threshold between the maps of a sweep (it is per map).
@@ -694,6 +743,8 @@ morse_status plan_search(morse_ctx *ctx, const morse_event *ev,
   size_t out_bytes = dense ? sizeof(double) * 3 * (size_t)n_out
                            : sizeof(morse_fit) * (size_t)K * (size_t)n_out;
   pl->bytes = pl->off_out + out_bytes;
+  pl->want = 0;
+  if (!dense) pl->bytes = plan_screen(ev, g, count, pl->bytes, pl);
   return MORSE_OK;
 }
 
@@ -738,11 +789,58 @@ morse_status enqueue_topk(morse_ctx *ctx, const Plan &pl,
   P.tab_n = pl.tab_n;
   P.tab_c = (unsigned)(P.half + 1) - 0x4B400000u;
   int r;
+  int list_grid = 0;
+  bool staged = false;
+  size_t list_smem = 0;
+  if (pl.want > 0) {
+    // the listed search: staged light curve and subsets when they fit
+    for (int s = 1; s >= 0 && list_grid == 0; --s) {
+      staged = s != 0;
+      list_smem = morse::list_smem_bytes(P, staged);
+      if (list_smem + 2048 > ctx->smem_optin) continue;
+      if (morse::list_blocks_per_sm(staged, P.quadh != nullptr, list_smem) >=
+          1)
+        list_grid = pl.grid;
+    }
+  }
+  if (list_grid > 0) {
+    morse::ScreenBufs B;
+    B.code = (unsigned short *)(base + pl.off_code);
+    B.hist = (unsigned *)(base + pl.off_hist);
+    B.n = B.hist + morse::kScreenBins;
+    B.pilot = (unsigned *)(base + pl.off_pil);
+    B.ub = (float *)(base + pl.off_ub);
+    B.list = (unsigned *)(base + pl.off_list);
+    B.pilot_cap = pl.pilot_cap;
+    B.list_cap = pl.list_cap;
+    B.want = pl.want;
+    MORSE_CUDA(ctx, cudaMemsetAsync(
+                        B.hist, 0,
+                        sizeof(unsigned) * (morse::kScreenBins + 2),
+                        ctx->stream));
+    r = t_begin(ctx, KT_SEARCH);
+    MORSE_CUDA(ctx, morse::launch_screen(P, B, ctx->sm_count, ctx->stream));
+    MORSE_CUDA(ctx, morse::launch_screen_pilot_list(P, B, ctx->sm_count,
+                                                    ctx->stream));
+    MORSE_CUDA(ctx, morse::launch_screen_pilot(P, B, ctx->smem_optin,
+                                               ctx->sm_count, ctx->stream));
+    MORSE_CUDA(ctx, morse::launch_screen_list(P, B, ctx->sm_count,
+                                              ctx->stream));
+    P.list = B.list;
+    P.n_list = B.n + 1;
+    P.list_cap = B.list_cap;
+    P.pub_tag = next_pub_tag(ctx);
+    P.pub_nb = list_grid;
+    P.pub_me = -1;
+    P.pub_stride = list_grid;
+    MORSE_CUDA(ctx, morse::launch_search_list(P, staged, list_grid, list_smem,
+                                              ctx->stream));
+    t_end(ctx, r);
+    ctx->launches += 5;
+  }
   // pilot: a strided subset of ~sqrt(K N) trajectories (at least 16 K)
   // seeds the grid-wide pruning threshold
-  const double want =
-      std::max(morse::kPilotMinK * pl.K,
-               morse::kPilotSqrt * std::sqrt((double)pl.K * P.count));
+  const double want = list_grid > 0 ? 0.0 : pilot_want(pl.K, P.count);
   // (no pilot when the sample would be under one trajectory)
   const long long stride = want >= 1.0 ? (long long)(P.count / want) : 0;
   if (P.gthr && stride >= 4) {
@@ -1878,6 +1976,87 @@ void morse_map_free(morse_map *map) {
 }
 
 // ------------------------------------------------------------------ events
+// The screening subsets of a light curve (k_screen.cu), appended to its n
+// slots h: 32 epochs (64 from 640 epochs on), an eighth of it from 1024
+// epochs on and a third from 2048 on.  An epoch's share grows with its
+// information w (F - F_mean)^2, since that is what a wrong trajectory's
+// chi^2 is made of, and a tenth of the shares is even (it pins the
+// baseline): along the cumulated shares, capped at one epoch each, every
+// crossing of a half-integer takes an epoch.  Light curves whose sums are
+// out of the FP32 bounds' range (screen_lb) have no subsets.
+static void screen_subsets(morse_event *ev, std::vector<float4> &h, int64_t n,
+                           double S1, double SF, double SFF) {
+  ev->n_sub = 0;
+  const int sizes[kScreenLevels] = {n < 640 ? 32 : 64,
+                                    n >= 1024 ? (int)(n / 8) : 0,
+                                    n >= 2048 ? (int)(n / 3) : 0};
+  if (n < 128 || n > (1 << 20) || !(S1 > 1e-12 && S1 < 1e15 && SFF > 1e-12 &&
+                                    SFF < 1e15))
+    return;
+  std::vector<double> x((size_t)n);
+  std::vector<int> sel;
+  for (int l = 0; l < kScreenLevels && sizes[l] > 0; ++l) {
+    const int m = sizes[l];
+    const float2 *tw = reinterpret_cast<const float2 *>(h.data());
+    const float *wf = reinterpret_cast<const float *>(tw + n);
+    const float *fc = wf + n;
+    const double mean = SF / S1;
+    double sum = 0.0;
+    for (int64_t i = 0; i < n; ++i) {
+      const double d = (double)fc[i] - mean;
+      sum += x[(size_t)i] = (double)tw[i].y * d * d;
+    }
+    const double even = 0.1 / (double)n;
+    const double per = sum > 0.0 ? 0.9 / sum : 0.0;
+    for (int64_t i = 0; i < n; ++i) x[(size_t)i] = x[(size_t)i] * per + even;
+    // scale so that the shares, capped at 1, add up to m
+    double scale = (double)m / (sum > 0.0 ? 1.0 : 0.1);
+    for (int it = 0; it < 8; ++it) {
+      double capped = 0.0, rest = 0.0;
+      for (int64_t i = 0; i < n; ++i) {
+        const double v = x[(size_t)i] * scale;
+        if (v >= 1.0)
+          capped += 1.0;
+        else
+          rest += v;
+      }
+      if (rest <= 0.0 || capped >= (double)m) break;
+      const double f = ((double)m - capped) / rest;
+      if (f < 1.0001 && f > 0.9999) break;
+      scale *= f;
+    }
+    sel.clear();
+    double acc = 0.5;
+    for (int64_t i = 0; i < n; ++i) {
+      const double next = acc + std::min(1.0, x[(size_t)i] * scale);
+      if (std::floor(next) > std::floor(acc)) sel.push_back((int)i);
+      acc = next;
+    }
+    if (sel.size() < 8 || (l == 0 && sel.size() > 128)) return;
+    morse_subset &u = ev->sub[l];
+    u.m = (int)sel.size();
+    u.off = (int)h.size();
+    u.S1 = u.SF = u.SFF = 0.0;
+    h.resize(h.size() + sel.size());
+    const float2 *stw = reinterpret_cast<const float2 *>(h.data());
+    const float *swf = reinterpret_cast<const float *>(stw + n);
+    const float *sfc = swf + n;
+    float2 *dtw = reinterpret_cast<float2 *>(h.data() + u.off);
+    float *dwf = reinterpret_cast<float *>(dtw + u.m);
+    float *dfc = dwf + u.m;
+    for (int k = 0; k < u.m; ++k) {
+      const int i = sel[(size_t)k];
+      dtw[k] = stw[i];
+      dwf[k] = swf[i];
+      dfc[k] = sfc[i];
+      u.S1 += (double)dtw[k].y;
+      u.SF += (double)dtw[k].y * (double)dfc[k];
+      u.SFF += (double)dtw[k].y * (double)dfc[k] * (double)dfc[k];
+    }
+    ev->n_sub = l + 1;
+  }
+}
+
 morse_status morse_event_create(morse_ctx *ctx, const double *t,
                                 const double *flux, const double *sigma,
                                 int64_t n, double t_ref, morse_event **out) {
@@ -1954,13 +2133,15 @@ morse_status morse_event_create(morse_ctx *ctx, const double *t,
   MORSE_CUDA(ctx, cudaSetDevice(ctx->device));
   morse_event *ev = (morse_event *)calloc(1, sizeof(morse_event));
   if (!ev) return fail(ctx, MORSE_ENOMEM, "event");
-  if (morse::dev_alloc(ctx, (void **)&ev->ep, sizeof(float4) * (size_t)n) !=
+  screen_subsets(ev, h, n, S1, SF, SFF);
+  if (morse::dev_alloc(ctx, (void **)&ev->ep, sizeof(float4) * h.size()) !=
       cudaSuccess) {
     cudaGetLastError();
     free(ev);
     return fail(ctx, MORSE_ENOMEM, "event of %lld epochs", (long long)n);
   }
-  cudaError_t e = cudaMemcpyAsync(ev->ep, h.data(), sizeof(float4) * (size_t)n,
+  cudaError_t e = cudaMemcpyAsync(ev->ep, h.data(),
+                                  sizeof(float4) * h.size(),
                                   cudaMemcpyHostToDevice, ctx->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
   if (e != cudaSuccess) {

@@ -74,13 +74,25 @@ struct morse_map {
   int lookup;               // MORSE_STORE_FP32 or MORSE_STORE_FP16LOG
 };
 
+// Screening subsets of a light curve: at most this many, smallest first.
+constexpr int kScreenLevels = 3;
+
+// One subset of m epochs (time-sorted), stored like the light curve itself
+// at ep + off, with the FP64 sums of its stored values.
+struct morse_subset {
+  int m, off;
+  double S1, SF, SFF;
+};
+
 struct morse_event {
   morse_ctx *ctx;
   int64_t n;
   double t_ref;
   float4 *ep;               // n float4 slots holding, as arrays,
                             // (t - t_ref, w)[n], w (F - F_ref)[n],
-                            // (F - F_ref)[n]
+                            // (F - F_ref)[n]; then the subsets' slots
+  int n_sub;                // subsets (0: the search does not screen)
+  morse_subset sub[kScreenLevels];
   double S1, SF, SFF, Fref; // FP64 sums of the stored FP32 values
   double invS1, CFF;        // 1/S_1, S_FF - S_F^2/S_1
   double t_span;            // max |t - t_ref| over the epochs
@@ -210,6 +222,15 @@ struct Entry {
 // levels of published block quantiles (search_group.cuh: pub_update)
 constexpr int kPubLevels = 3;
 
+// A screening subset as the kernels read it: its epochs and the FP32
+// constants of its lower bound (screen_lb in search_common.cuh).
+struct ScreenLv {
+  const float4 *ep;
+  int m;
+  float S1, iS1, SF, sqSFF, CFF;  // CFF rounded down, sqSFF up
+  float g;                  // relative error bound of the FP32 sums, doubled
+};
+
 struct SearchParams {
   // map: the lookup reads quadh (FP16 log10 quads) when it is set, else
   // quad (FP32 A - 1 quads); both share qpitch and the index folding
@@ -279,7 +300,28 @@ struct SearchParams {
   // lists.
   int tab_n;
   unsigned tab_c;           // half + 1 - 0x4B400000: floor bits -> cell
+  // Screened search (k_screen.cu); n_lv = 0: off.
+  int n_lv;
+  ScreenLv lv[kScreenLevels];
+  const unsigned *list;     // trajectories (offsets from first) to search
+  const unsigned *n_list;   // their number, or more than list_cap if they
+  unsigned list_cap;        // do not fit: then the whole range is searched
 };
+
+// Workspace of a screened search.
+struct ScreenBufs {
+  unsigned short *code;     // [count] lower bound of each trajectory's
+                            // chi^2: the upper half of its FP32 bits
+  unsigned *hist;           // [kScreenBins] trajectories per code >> 3
+  unsigned *n;              // [2] lengths of the two lists
+  unsigned *pilot;          // [pilot_cap] trajectories of the pilot
+  float *ub;                // [pilot_cap] their chi^2 bounds from above
+  unsigned *list;           // [list_cap]
+  unsigned pilot_cap, list_cap;
+  unsigned want;            // pilot trajectories asked for
+};
+constexpr int kScreenBins = 4096;
+constexpr unsigned kScreenCut = 0xFFFFu;  // code of a cut line's trajectory
 
 // ------------------------------------------- host set-up of a search
 // Grid tables in device memory: the lines' tau intervals inside the map,
@@ -369,6 +411,29 @@ inline long long main_groups(long long line, long long first,
   const long long ng = (line + t - 1) / t;
   return ((first + count - 1) / line - first / line + 1) * ng;
 }
+
+// ---------------------------------------------------------------- screen
+// codes and histogram of trajectories first .. first + count - 1
+cudaError_t launch_screen(const SearchParams &P, const ScreenBufs &B,
+                          int sm_count, cudaStream_t st);
+// the pilot's trajectories: the `want` of lowest code
+cudaError_t launch_screen_pilot_list(const SearchParams &P,
+                                     const ScreenBufs &B, int sm_count,
+                                     cudaStream_t st);
+// their upper bounds
+cudaError_t launch_screen_pilot(const SearchParams &P, const ScreenBufs &B,
+                                size_t smem_optin, int sm_count,
+                                cudaStream_t st);
+// *P.gthr <- the pilot's top_k-th bound; the list of trajectories whose
+// code does not exceed it
+cudaError_t launch_screen_list(const SearchParams &P, const ScreenBufs &B,
+                               int sm_count, cudaStream_t st);
+// shared memory of the listed search with staged epochs (0: they do not
+// fit), and its launch
+size_t list_smem_bytes(const SearchParams &P, bool staged);
+int list_blocks_per_sm(bool staged, bool h16, size_t smem);
+cudaError_t launch_search_list(const SearchParams &P, bool staged, int grid,
+                               size_t smem, cudaStream_t st);
 
 size_t search_smem_bytes(int n_ep_smem, int top_k);
 int search_blocks_per_sm(bool dense, bool ep_smem, bool h16, size_t smem);

@@ -74,9 +74,8 @@ __device__ __forceinline__ bool key_less(double ca, long long ia, double cb,
 // (strict) or upwards: no FP32 value lies strictly between x and that
 // rounding, so t > x <=> t > RD(x) and t >= x <=> t >= RU(x) exactly, and
 // the search needs no FP64 compares.
-__device__ __forceinline__ int epoch_search(const Epochs &ep, int n, double x,
-                                            bool strict) {
-  const float xf = strict ? __double2float_rd(x) : __double2float_ru(x);
+__device__ __forceinline__ int epoch_search_f(const Epochs &ep, int n,
+                                              float xf, bool strict) {
   int lo = 0, hi = n;
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
@@ -88,6 +87,11 @@ __device__ __forceinline__ int epoch_search(const Epochs &ep, int n, double x,
       lo = mid + 1;
   }
   return lo;
+}
+__device__ __forceinline__ int epoch_search(const Epochs &ep, int n, double x,
+                                            bool strict) {
+  return epoch_search_f(
+      ep, n, strict ? __double2float_rd(x) : __double2float_ru(x), strict);
 }
 
 // The tau interval (lo, hi) in which the line of (u0, alpha) is inside the
@@ -126,11 +130,14 @@ __device__ __forceinline__ void slab_tau(double L, double u, double c,
 // and tau = (t - t0)/tE the coordinates are v = a t + b.  The track is
 // inside the map (|y1| < L and |y2| < L) for tau in (tau_lo, tau_hi), i.e.
 // for the epochs [e_in, e_out).
-__device__ __forceinline__ TrajC make_traj(const SearchParams &P,
-                                           const Epochs &ep, double u,
+// The constants without the epoch range, and the times (xin, xout) between
+// which the track is inside the map: an epoch at t is inside iff
+// t > RD(xin) and t < RU(xout) (xin = +inf: the line misses the map).
+__device__ __forceinline__ TrajC traj_base(const SearchParams &P, double u,
                                            double c, double s, double t0,
                                            double k, double tE, double tlo,
-                                           double thi) {
+                                           double thi, double &xin,
+                                           double &xout) {
   // u = u0, (c, s) = (cos, sin) alpha, t0 relative to t_ref,
   // k = 1/(tE Delta), (tlo, thi) = the line's tau interval in the map
   const double ax = __dmul_rn(c, k), ay = __dmul_rn(s, k);
@@ -146,13 +153,37 @@ __device__ __forceinline__ TrajC make_traj(const SearchParams &P,
   o.bt = __double2float_rn(-__dmul_rn(t0, kt));
   o.u02 = __double2float_rn(__dmul_rn(u, u));
   if (tlo < thi) {
-    o.e_in = epoch_search(ep, P.n_ep, t0 + tlo * tE, true);
-    o.e_out = epoch_search(ep, P.n_ep, t0 + thi * tE, false);
+    xin = t0 + tlo * tE;
+    xout = t0 + thi * tE;
+  } else {
+    xin = xout = CUDART_INF;
+  }
+  o.e_in = o.e_out = 0;
+  return o;
+}
+
+// the epochs [e_in, e_out) of a light curve that lie inside the map
+__device__ __forceinline__ void traj_range(const Epochs &ep, int n,
+                                           double xin, double xout,
+                                           TrajC &o) {
+  if (xin < CUDART_INF) {
+    o.e_in = epoch_search(ep, n, xin, true);
+    o.e_out = epoch_search(ep, n, xout, false);
     if (o.e_out < o.e_in) o.e_out = o.e_in;
   } else {
-    o.e_in = P.n_ep;
-    o.e_out = P.n_ep;
+    o.e_in = n;
+    o.e_out = n;
   }
+}
+
+__device__ __forceinline__ TrajC make_traj(const SearchParams &P,
+                                           const Epochs &ep, double u,
+                                           double c, double s, double t0,
+                                           double k, double tE, double tlo,
+                                           double thi) {
+  double xin, xout;
+  TrajC o = traj_base(P, u, c, s, t0, k, tE, tlo, thi, xin, xout);
+  traj_range(ep, P.n_ep, xin, xout, o);
   return o;
 }
 
@@ -181,6 +212,33 @@ __device__ __forceinline__ TrajC traj_consts(const SearchParams &P,
   }
   return make_traj(P, ep, P.u0v[iu], P.ca[ia], P.sa[ia], P.t0rel[it0],
                    P.invtEd[itE], tE, sl.x, sl.y);
+}
+
+// the same without the epoch range, from a 32-bit index (screened searches:
+// the whole grid has fewer than 2^31 trajectories)
+__device__ __forceinline__ TrajC traj_base_of(const SearchParams &P,
+                                              unsigned j, double &xin,
+                                              double &xout) {
+  unsigned r = j;
+  const unsigned itE = r % (unsigned)P.n_tE;
+  r /= (unsigned)P.n_tE;
+  const unsigned it0 = r % (unsigned)P.n_t0;
+  r /= (unsigned)P.n_t0;
+  const unsigned iu = r / (unsigned)P.n_alpha;
+  const unsigned ia = r - iu * (unsigned)P.n_alpha;
+  const double2 sl = P.slab[r];
+  double tE = P.tEv[itE], k = P.invtEd[itE], t0 = P.t0rel[it0];
+  if (P.lu) {  // line grid (as traj_consts)
+    if (P.ltE) {
+      tE = P.ltE[iu];
+      k = 1.0 / (tE * P.dlt);
+    }
+    t0 = t0 - P.lsh[iu] * tE;
+    return traj_base(P, P.lu[iu], P.lc[iu], P.ls[iu], t0, k, tE, sl.x, sl.y,
+                     xin, xout);
+  }
+  return traj_base(P, P.u0v[iu], P.ca[ia], P.sa[ia], t0, k, tE, sl.x, sl.y,
+                   xin, xout);
 }
 
 __device__ __forceinline__ TrajC shfl_traj(const TrajC &m, int k) {
@@ -645,12 +703,14 @@ __device__ __forceinline__ Acc phase1(const SearchParams &P, const Epochs &ep,
 // Phase 1 of two trajectories at once: the epoch axis is cut at both
 // trajectories' map entry and exit, and each segment runs the matching
 // inside/outside combination with one epoch load per lane for both.
+// (n_ep epochs: the light curve, or a screening subset of it)
 template <bool H, int TB = 0>
-__device__ __forceinline__ void phase1_pair(const SearchParams &P,
-                                            const Epochs &ep, const TrajC &ca,
-                                            const TrajC &cb, const int lane,
-                                            Acc &ra, Acc &rb,
-                                            const float4 *tab = nullptr) {
+__device__ __forceinline__ void phase1_pair_n(const SearchParams &P,
+                                              const Epochs &ep,
+                                              const int n_ep, const TrajC &ca,
+                                              const TrajC &cb, const int lane,
+                                              Acc &ra, Acc &rb,
+                                              const float4 *tab = nullptr) {
   Acc2 s = {f2(0.f), f2(0.f), f2(0.f)};
   const TrajP cp = pack_traj(ca, cb);
   // cut points, sorted (warp-uniform)
@@ -660,7 +720,7 @@ __device__ __forceinline__ void phase1_pair(const SearchParams &P,
   if (p1 > p3) { t = p1; p1 = p3; p3 = t; }
   if (p2 > p4) { t = p2; p2 = p4; p4 = t; }
   if (p2 > p3) { t = p2; p2 = p3; p3 = t; }
-  const int cut[6] = {0, p1, p2, p3, p4, P.n_ep};
+  const int cut[6] = {0, p1, p2, p3, p4, n_ep};
 #pragma unroll
   for (int i = 0; i < 5; ++i) {
     const int e0 = cut[i], e1 = cut[i + 1];
@@ -679,6 +739,15 @@ __device__ __forceinline__ void phase1_pair(const SearchParams &P,
   const Acc sa = {s.a.x, s.b.x, s.d.x}, sb = {s.a.y, s.b.y, s.d.y};
   ra = acc_reduce(sa);
   rb = acc_reduce(sb);
+}
+
+template <bool H, int TB = 0>
+__device__ __forceinline__ void phase1_pair(const SearchParams &P,
+                                            const Epochs &ep, const TrajC &ca,
+                                            const TrajC &cb, const int lane,
+                                            Acc &ra, Acc &rb,
+                                            const float4 *tab = nullptr) {
+  phase1_pair_n<H, TB>(P, ep, P.n_ep, ca, cb, lane, ra, rb, tab);
 }
 
 // Phase 2: chi^2 = sum w (F - Fs A - Fb)^2, written with centred values as
@@ -822,6 +891,31 @@ __device__ __forceinline__ double chi2_upper(const SearchParams &P, double SA,
                        16.0 * 1.1102230246251565e-16 * absum;
   const double ub = (q + slack) * 1.0001000100010002;
   return ub == ub ? ub : CUDART_INF;  // NaN sums: no bound
+}
+
+// Lower bound of the chi^2 of a trajectory from the sums over a screening
+// subset of the epochs.  For any subset, the smallest chi^2 of the subset
+// over all (Fs, Fb) is at most the subset's share of the full chi^2 at the
+// full fit, so
+//     chi^2 >= C_FF - C_AF^2 / C_AA     (the sums of the subset).
+// In FP32: with the relative error g of the sums (a serial or lane-split
+// sum of the m terms, doubled) and u = 2^-24, T_A <= sqrt(S_1 S_AA) and
+// T_AF <= sqrt(S_AA S_FF) as in solve2,
+//   C_AA >= fl(C_AA) - (3.1 g + 6 u) S_AA      (taken as 4 g S_AA),
+//   |C_AF| <= |fl(C_AF)| + (2 g + 6 u) sqrt(S_AA S_FF)    (taken as 3 g),
+// where g >= 22 u covers the u terms.  The quotient's rounding and the
+// margin may_reach allows the exact sweep's own FP32 rounding (1e-4) are
+// taken off the result.  0 (never discarded) where the bound says nothing:
+// a nearly constant A, sums out of FP32's range, or NaN.
+__device__ __forceinline__ float screen_lb(const ScreenLv &V, const Acc &s) {
+  const float CAA = __fmaf_rn(-__fmul_rn(s.a, s.a), V.iS1, s.b);
+  const float CAF = __fmaf_rn(-__fmul_rn(s.a, V.SF), V.iS1, s.d);
+  const float den = __fmaf_rn(-4.f * V.g, s.b, CAA);
+  const float num = __fmaf_rn(3.f * V.g, __fmul_ru(__fsqrt_ru(s.b), V.sqSFF),
+                              fabsf(CAF));
+  const float ex = __fmul_rn(__fdiv_rn(num, den), num) * 1.00001f;
+  const float lb = (V.CFF * 0.999999f - ex) * 0.9998f;
+  return (s.b > 1e-25f && den > 1e-7f * s.b && lb > 0.f) ? lb : 0.f;
 }
 
 __device__ __forceinline__ double bits_to_chi2(unsigned long long b) {

@@ -1,0 +1,114 @@
+"""The screened trajectory search (k_screen.cu) against the dense ranking.
+
+The dense call evaluates every trajectory; the screened top-K must be its
+smallest K by (chi2, index), bit for bit: at the epoch counts where the
+subsets' sizes change, on light curves whose bounds discard nearly all, some
+or none of the grid (the last searches the whole range), for ranges, cut
+lines, FP16 tables, line grids and several K.
+"""
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def m():
+    import paper_1511_01157_gb300 as lib
+    return lib
+
+
+@pytest.fixture(scope="module")
+def setup(m):
+    ctx = m.Context(0)
+    mp = ctx.build_map(1.1, 3e-3, 2.0, 301, 2100, image_halfwidth=3.0,
+                       deflect="fp32")
+    yield ctx, mp
+    ctx.close()
+
+
+def _event(ctx, n, kind, seed=5):
+    t = synth.epoch_times(n, seed)
+    if kind == "flat":      # no signal: no bound can discard anything
+        f = np.full(n, 2.0)
+    elif kind == "weak":
+        f = 3.0 + 1.0 / np.sqrt(0.5 + (t / 60.0) ** 2)
+    else:                   # high magnification, two bumps
+        f = (0.4 + 1.0 / np.sqrt(2e-4 + (t / 15.0) ** 2) +
+             3.0 * np.exp(-((t - 1.3) / 0.2) ** 2))
+    F, sig = synth.photometry(f, seed, 0.01 if kind == "strong" else 0.0)
+    return ctx.event(t, F, sig)
+
+
+def _grid(m, top_k, a_min=0.0, n_tE=9):
+    return m.Grid.make(12, 20, 11, n_tE, 1e-3, 0.5, -2.0, 2.0, 5.0, 80.0,
+                       True, True, top_k, a_min)
+
+
+def _best(chi2, k, first=0):
+    idx = np.lexsort((np.arange(len(chi2)), chi2))[:k]
+    idx = idx[np.isfinite(chi2[idx])]
+    return idx + first, chi2[idx]
+
+
+@pytest.mark.parametrize("kind", ["strong", "weak", "flat"])
+@pytest.mark.parametrize("n", [127, 128, 639, 640, 1023, 1024, 2047, 2048,
+                               3001])
+def test_screened_equals_dense(m, setup, n, kind):
+    ctx, mp = setup
+    ev = _event(ctx, n, kind)
+    for k in (1, 33):
+        g = _grid(m, k)
+        got = ctx.grid_chi2(ev, mp, g)
+        chi2, fs, fb = ctx.grid_chi2_dense(ev, mp, g)
+        idx, val = _best(chi2, k)
+        assert np.array_equal(got["idx"], idx)
+        assert np.array_equal(got["chi2"], val)
+        assert np.array_equal(got["Fs"], fs[idx])
+        assert np.array_equal(got["Fb"], fb[idx])
+
+
+@pytest.mark.parametrize("kind", ["strong", "flat"])
+def test_screened_forms(m, setup, kind):
+    ctx, mp = setup
+    ev = _event(ctx, 1500, kind)
+    g = _grid(m, 700)
+    chi2, *_ = ctx.grid_chi2_dense(ev, mp, g)
+    idx, val = _best(chi2, 700)
+    got = ctx.grid_chi2(ev, mp, g)
+    assert np.array_equal(got["idx"], idx)
+    assert np.array_equal(got["chi2"], val)
+    # a range that starts and ends inside a line
+    for first, count in ((1, g.size - 2), (1237, 17001)):
+        r = ctx.grid_chi2_range(ev, mp, g, first, count)
+        idx, val = _best(chi2[first:first + count], 700, first)
+        assert np.array_equal(r["idx"], idx)
+        assert np.array_equal(r["chi2"], val)
+    # FP16 table
+    mp.set_lookup(True)
+    h16, *_ = ctx.grid_chi2_dense(ev, mp, g)
+    got = ctx.grid_chi2(ev, mp, g)
+    mp.set_lookup(False)
+    idx, val = _best(h16, 700)
+    assert np.array_equal(got["idx"], idx)
+    assert np.array_equal(got["chi2"], val)
+    # the minimum-magnification cut
+    top = ctx.line_max(mp, g)
+    cut = _grid(m, 700, float(np.median(top)))
+    kept, *_ = ctx.grid_chi2_dense(ev, mp, cut)
+    idx, val = _best(kept, 700)
+    got = ctx.grid_chi2(ev, mp, cut)
+    assert np.array_equal(got["idx"][:len(idx)], idx)
+    assert np.array_equal(got["chi2"][:len(idx)], val)
+    # the same lines as a line grid, an odd number of tE
+    g = _grid(m, 20, n_tE=13)
+    u0 = np.exp(np.linspace(np.log(1e-3), np.log(0.5), 12))
+    lines = np.array([(u, 2 * np.pi * j / 20, 0.0) for u in u0
+                      for j in range(20)])
+    lg = m.Grid.make(len(lines), 1, 11, 13, 1.0, 1.0, -2.0, 2.0, 5.0, 80.0,
+                     False, True, 20)
+    a, b = ctx.grid_chi2_lines(ev, mp, lg, lines), ctx.grid_chi2(ev, mp, g)
+    assert np.array_equal(a["idx"], b["idx"])
+    np.testing.assert_allclose(a["chi2"], b["chi2"], rtol=1e-6)
