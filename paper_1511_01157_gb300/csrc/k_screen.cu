@@ -15,18 +15,21 @@
 //   k_pilot        upper bounds of their chi^2 over the whole light curve
 //   k_list         the K-th of those, a rigorous threshold near the final
 //                  one, and the list of trajectories at or below it
+//   k_rescreen     the listed ones again, on the second and third subsets
 //
 // The listed search (k_search_list) then runs over the list alone, with the
-// larger subsets first.  Results are those of the unscreened search bit for
+// largest subset first.  Results are those of the unscreened search bit for
 // bit: a discarded trajectory's chi^2 exceeds K others', and every listed
 // one is evaluated by the same device functions.  Measured, call by call
-// (1024^2 map, 1.44 M trajectories, 3000 epochs, K = 256): 3.25 -> 0.84 ms;
-// four maps of a sweep 13.5 -> 2.95 ms.  The host screens from 16 384
+// (1024^2 map, 1.44 M trajectories, 3000 epochs, K = 256, five events of
+// tE 7 to 37 d): 3.2 -> 0.45 to 1.3 ms, four maps of a sweep 13 -> 2.0 to
+// 4.5 ms; the spread is the light curves' own (what share of the grid fits
+// them about as well as the best).  The host screens from 16 384
 // trajectories and 128 epochs on; below that a search is bound by its
 // launches and its latency, and there are too few trajectories to rank.
-// Where more than half of the grid stays on the list (light curves of weak
-// signal), the whole range is searched as before (k_search), the screening
-// costing a share 64 / n_epochs.
+// Where the subsets discard too little (light curves of weak signal), the
+// whole range is searched as before (k_search), the screening costing a
+// share 64 / n_epochs.
 #ifndef MORSE_PK_ASM
 #define MORSE_PK_ASM 1
 #endif
@@ -35,6 +38,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "morse_internal.cuh"
 #include "search_common.cuh"
@@ -46,76 +50,289 @@ namespace {
 using namespace dev;
 
 constexpr int kScreenThreads = 256;
-constexpr int kScreenMax = 128;  // epochs of the smallest subset, at most
+constexpr int kScreenTile = 2 * kScreenThreads;  // trajectories per block step
+// epochs of the subsets summed by one lane, at most
+constexpr int kScreenMax0 = 128, kScreenMax1 = 192, kScreenMax2 = 512;
 
-// Two trajectories per lane (32 apart, packed FP32), every lane over the
-// whole subset: no reductions, one broadcast shared load of an epoch for 64
-// trajectories, and a warp's gathers fall on one or two lines of the map.
+// Order of the trajectories in a screen.  The grid index runs over tE
+// fastest; here the position in a line runs over t0 fastest, so that the
+// lanes of a warp, at the same epoch, sit at neighbouring places of the
+// line and their 16-byte cells share cache lines (tE is log-spaced: at the
+// same t0 its values spread over the whole line).  A range that does not
+// consist of whole lines keeps the grid order.
+struct Pos {
+  unsigned line, it0, itE;
+};
+__device__ __forceinline__ bool by_t0(const SearchParams &P) {
+  return P.first % P.line == 0 && P.count % P.line == 0;
+}
+__device__ __forceinline__ Pos pos_of(const SearchParams &P, unsigned p,
+                                      bool t0_fast) {
+  const unsigned n = (unsigned)P.line;
+  Pos o;
+  if (t0_fast) {
+    o.line = p / n;
+    const unsigned r = p - o.line * n;
+    o.itE = r / (unsigned)P.n_t0;
+    o.it0 = r - o.itE * (unsigned)P.n_t0;
+    o.line += (unsigned)(P.first / P.line);
+  } else {
+    const unsigned j = (unsigned)P.first + p;
+    o.line = j / n;
+    const unsigned r = j - o.line * n;
+    o.it0 = r / (unsigned)P.n_tE;
+    o.itE = r - o.it0 * (unsigned)P.n_tE;
+  }
+  return o;
+}
+// offset of a position's trajectory from P.first
+__device__ __forceinline__ unsigned offset_of(const SearchParams &P,
+                                              unsigned p, bool t0_fast) {
+  if (!t0_fast) return p;
+  const unsigned n = (unsigned)P.line, l = p / n, r = p - l * n;
+  const unsigned itE = r / (unsigned)P.n_t0;
+  return l * n + (r - itE * (unsigned)P.n_t0) * (unsigned)P.n_tE + itE;
+}
+
+// The FP64 constants that the trajectories of one (line, tE) share (a row:
+// n_t0 positions), made once per row of a block's tile: an FP64 instruction
+// holds the SM's FP64 pipe for some 16 cycles, and 15 of a trajectory's 26
+// do not depend on its t0.
+struct Row {
+  double ax, ay, cx, cy, kt, tE, tlo, thi, lsh;
+  float axf, ayf, ktf, u02;
+};
+constexpr int kRowMax = 176;  // rows of a tile: kScreenTile / n_t0 + 2
+
+__device__ __forceinline__ Row make_row(const SearchParams &P, unsigned line,
+                                        unsigned itE) {
+  // (the operations of traj_base_of and traj_base, in their order)
+  const unsigned iu = line / (unsigned)P.n_alpha;
+  const unsigned ia = line - iu * (unsigned)P.n_alpha;
+  const double2 sl = P.slab[line];
+  double u, c, s, k = P.invtEd[itE];
+  Row r;
+  r.tE = P.tEv[itE];
+  r.lsh = 0.0;
+  if (P.lu) {
+    if (P.ltE) {
+      r.tE = P.ltE[iu];
+      k = 1.0 / (r.tE * P.dlt);
+    }
+    r.lsh = P.lsh[iu];
+    u = P.lu[iu];
+    c = P.lc[iu];
+    s = P.ls[iu];
+  } else {
+    u = P.u0v[iu];
+    c = P.ca[ia];
+    s = P.sa[ia];
+  }
+  r.ax = __dmul_rn(c, k);
+  r.ay = __dmul_rn(s, k);
+  r.cx = __dadd_rn(__dmul_rn(-__dmul_rn(u, s), P.invD), P.coff);
+  r.cy = __dadd_rn(__dmul_rn(__dmul_rn(u, c), P.invD), P.coff);
+  r.kt = __dmul_rn(k, P.dlt);
+  r.tlo = sl.x;
+  r.thi = sl.y;
+  r.axf = __double2float_rn(r.ax);
+  r.ayf = __double2float_rn(r.ay);
+  r.ktf = __double2float_rn(r.kt);
+  r.u02 = __double2float_rn(__dmul_rn(u, u));
+  return r;
+}
+
+// a trajectory of a row: its constants and the FP32 times between which it
+// is inside the map (in < t < out)
+__device__ __forceinline__ TrajC row_traj(const SearchParams &P, const Row &r,
+                                          unsigned it0, float &in,
+                                          float &out) {
+  double t0 = P.t0rel[it0];
+  if (P.lu) t0 = t0 - r.lsh * r.tE;
+  TrajC o;
+  o.ax = r.axf;
+  o.ay = r.ayf;
+  o.bx = __double2float_rn(__dsub_rn(r.cx, __dmul_rn(t0, r.ax)));
+  o.by = __double2float_rn(__dsub_rn(r.cy, __dmul_rn(t0, r.ay)));
+  o.kt = r.ktf;
+  o.bt = __double2float_rn(-__dmul_rn(t0, r.kt));
+  o.u02 = r.u02;
+  if (r.tlo < r.thi) {
+    in = __double2float_rd(t0 + r.tlo * r.tE);
+    out = __double2float_ru(t0 + r.thi * r.tE);
+  } else {
+    in = out = CUDART_INF_F;
+  }
+  o.e_in = o.e_out = 0;
+  return o;
+}
+
+// The cells a lane looked up last.  The subsets are runs of neighbouring
+// epochs, so a trajectory mostly stays in its cell from one epoch to the
+// next, and only the lanes that leave theirs load another: a warp's gather
+// of 32 cells takes 12 wavefronts of the L1 data pipe, which bounded the
+// screen (157 us of 1.44 M trajectories x 64 epochs).
 template <bool H>
-__global__ void __launch_bounds__(kScreenThreads)
-    k_screen(const SearchParams P, const ScreenBufs B) {
-  __shared__ float4 s_ep[kScreenMax];
-  __shared__ unsigned s_hist[kScreenBins];
-  const ScreenLv V = P.lv[0];
+struct Cells {
+  unsigned ia, ib;
+  float4 a, b;  // FP32 cells; FP16: decoded (band_cell_h)
+};
+
+template <bool H>
+__device__ __forceinline__ float4 load_cell(const SearchParams &P,
+                                            unsigned idx) {
+  return H ? band_cell_h(__ldg(&P.quadh[idx])) : __ldg(&P.quad[idx]);
+}
+
+// A - 1 of both inside the map (the arithmetic of tex_pos and bilinear_m1 or
+// bilinear_h_m1, the coordinates packed)
+template <bool H>
+__device__ __forceinline__ float2 in2_m1(const SearchParams &P, Cells<H> &q,
+                                         float2 vx, float2 vy) {
+  float2 fx, fy;
+  unsigned ia, ib;
+  TexPos ta, tb;
+  if (!tex_pos(P, vx.x, vy.x, ta) || !tex_pos(P, vx.y, vy.y, tb))
+    return make_float2(0.f, 0.f);  // (checked build only)
+  if (kTileW == 1 && kTileH == 1) {
+    const float2 tx = pk_add_rd(vx, f2(12582912.f));
+    const float2 ty = pk_add_rd(vy, f2(12582912.f));
+    fx = pk_fma(pk_add(tx, f2(-12582912.f)), f2(-1.f), vx);
+    fy = pk_fma(pk_add(ty, f2(-12582912.f)), f2(-1.f), vy);
+    const unsigned qp = (unsigned)P.qpitch;
+    ia = __float_as_uint(ty.x) * qp + __float_as_uint(tx.x) + P.qidx0;
+    ib = __float_as_uint(ty.y) * qp + __float_as_uint(tx.y) + P.qidx0;
+  } else {
+    fx = make_float2(ta.fx, tb.fx);
+    fy = make_float2(ta.fy, tb.fy);
+    ia = ta.idx;
+    ib = tb.idx;
+  }
+  const bool na = ia != q.ia, nb = ib != q.ib;
+  q.ia = ia;
+  q.ib = ib;
+  if (na) q.a = load_cell<H>(P, ia);
+  if (nb) q.b = load_cell<H>(P, ib);
+  const float2 r0 = pk_fma(fx, make_float2(q.a.y, q.b.y),
+                           make_float2(q.a.x, q.b.x));
+  const float2 dr = pk_fma(fx, make_float2(q.a.w, q.b.w),
+                           make_float2(q.a.z, q.b.z));
+  const float2 v = pk_fma(fy, dr, r0);
+  return H ? make_float2(__fsub_rn(v.x, 1.f), __fsub_rn(v.y, 1.f)) : v;
+}
+
+// The subset's bounds for two trajectories of a lane (packed FP32), every
+// lane over the whole subset: no reductions, one broadcast shared load of
+// an epoch for the warp's 64 trajectories.
+template <bool H>
+__device__ __forceinline__ void screen2(const SearchParams &P,
+                                        const ScreenLv &V, const float4 *s_ep,
+                                        const TrajC &ca, const TrajC &cb,
+                                        float ain, float aout, float bin,
+                                        float bout, float &la, float &lb) {
+  const TrajP c = pack_traj(ca, cb);
+  const float hi = fmaxf(ain, bin), lo = fminf(aout, bout);
+  Acc2 s = {f2(0.f), f2(0.f), f2(0.f)};
+  Cells<H> q;
+  q.ia = q.ib = 0xFFFFFFFFu;
+  q.a = q.b = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+  for (int e = 0; e < V.m; ++e) {
+    const float4 v = s_ep[e];
+    const float2 tt = f2(v.x);
+    const float2 vx = pk_fma(c.ax, tt, c.bx);
+    const float2 vy = pk_fma(c.ay, tt, c.by);
+    float2 Ac;
+    if (__all_sync(kFull, v.x > hi && v.x < lo)) {  // all of the warp inside
+      Ac = in2_m1<H>(P, q, vx, vy);
+    } else {
+      const bool ina = v.x > ain && v.x < aout;
+      const bool inb = v.x > bin && v.x < bout;
+      Ac = mag2_out_m1(c, tt);
+      if (__any_sync(kFull, ina || inb)) {
+        // (outside: a cell of the map's centre, the value is not used)
+        const float2 A =
+            in2_m1<H>(P, q, make_float2(ina ? vx.x : 0.f, inb ? vx.y : 0.f),
+                      make_float2(ina ? vy.x : 0.f, inb ? vy.y : 0.f));
+        if (ina) Ac.x = A.x;
+        if (inb) Ac.y = A.y;
+      }
+    }
+    acc2_add(s, f2(v.y), f2(v.z), Ac);
+  }
+  const Acc sa = {s.a.x, s.b.x, s.d.x}, sb = {s.a.y, s.b.y, s.d.y};
+  la = screen_lb(V, sa);
+  lb = screen_lb(V, sb);
+}
+
+__device__ __forceinline__ void stage_subset(const ScreenLv &V,
+                                             float4 *s_ep) {
   const Epochs ep = epochs_at(V.ep, V.m);
   for (int e = threadIdx.x; e < V.m; e += blockDim.x)
     s_ep[e] = make_float4(ep.tw[e].x, ep.tw[e].y, ep.wf[e], 0.f);
+}
+
+// Codes of all trajectories, on the smallest subset.
+template <bool H>
+__global__ void __launch_bounds__(kScreenThreads)
+    k_screen(const SearchParams P, const ScreenBufs B) {
+  __shared__ float4 s_ep[kScreenMax0];
+  __shared__ unsigned s_hist[kScreenBins];
+  __shared__ Row s_row[kRowMax];
+  const ScreenLv V = P.lv[0];
+  stage_subset(V, s_ep);
   for (int b = threadIdx.x; b < kScreenBins; b += blockDim.x) s_hist[b] = 0;
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const unsigned n = (unsigned)P.count;
-  const unsigned step = gridDim.x * (kScreenThreads / 32) * 64u;
-  for (unsigned i0 = (blockIdx.x * (kScreenThreads / 32) +
-                      (threadIdx.x >> 5)) * 64u;
-       i0 < n; i0 += step) {
-    const unsigned ia = i0 + lane, ib = ia + 32;
-    const unsigned ja = (unsigned)P.first + min(ia, n - 1);
-    const unsigned jb = (unsigned)P.first + min(ib, n - 1);
-    double xi, xo;
-    const TrajC ca = traj_base_of(P, ja, xi, xo);
-    const float ain = __double2float_rd(xi), aout = __double2float_ru(xo);
-    const TrajC cb = traj_base_of(P, jb, xi, xo);
-    const float bin = __double2float_rd(xi), bout = __double2float_ru(xo);
-    const TrajP c = pack_traj(ca, cb);
-    Acc2 s = {f2(0.f), f2(0.f), f2(0.f)};
-#pragma unroll 4
-    for (int e = 0; e < V.m; ++e) {
-      const float4 v = s_ep[e];
-      const float2 tt = f2(v.x);
-      const bool ina = v.x > ain && v.x < aout;
-      const bool inb = v.x > bin && v.x < bout;
-      float2 Ac = make_float2(0.f, 0.f);
-      if (ina || inb) {
-        const float2 vx = pk_fma(c.ax, tt, c.bx);
-        const float2 vy = pk_fma(c.ay, tt, c.by);
-        // (outside: any cell of the map, the value is not used)
-        const float xa = ina ? vx.x : 0.f, ya = ina ? vy.x : 0.f;
-        const float xb = inb ? vx.y : 0.f, yb = inb ? vy.y : 0.f;
-        Ac.x = H ? bilinear_h_m1(P, xa, ya) : bilinear_m1(P, xa, ya);
-        Ac.y = H ? bilinear_h_m1(P, xb, yb) : bilinear_m1(P, xb, yb);
+  const bool tf = by_t0(P);
+  const unsigned n = (unsigned)P.count, n_t0 = (unsigned)P.n_t0;
+  const bool rows = tf && n_t0 >= 3;
+  const unsigned row_first = rows ? (unsigned)(P.first / n_t0) : 0u;
+  for (unsigned c0 = blockIdx.x * kScreenTile; c0 < n;
+       c0 += gridDim.x * kScreenTile) {
+    __syncthreads();  // the subset, the histogram; the last tile's rows read
+    const unsigned r0 = c0 / n_t0;
+    if (rows) {
+      const unsigned r1 = (min(c0 + kScreenTile, n) - 1) / n_t0;
+      for (unsigned r = r0 + threadIdx.x; r <= r1; r += blockDim.x) {
+        const unsigned row = row_first + r;
+        const unsigned line = row / (unsigned)P.n_tE;
+        s_row[r - r0] = make_row(P, line, row - line * (unsigned)P.n_tE);
       }
-      if (!ina || !inb) {
-        const float2 o = mag2_out_m1(c, tt);
-        if (!ina) Ac.x = o.x;
-        if (!inb) Ac.y = o.y;
+      __syncthreads();
+    }
+    const unsigned pa = c0 + (threadIdx.x >> 5) * 64 + (threadIdx.x & 31);
+    const unsigned pb = pa + 32;
+    TrajC c[2];
+    float in[2], out[2];
+    bool cut[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const unsigned p = min(h ? pb : pa, n - 1);
+      unsigned line;
+      if (rows) {
+        const unsigned r = p / n_t0;
+        c[h] = row_traj(P, s_row[r - r0], p - r * n_t0, in[h], out[h]);
+        line = (row_first + r) / (unsigned)P.n_tE;
+      } else {
+        const Pos o = pos_of(P, p, tf);
+        c[h] = row_traj(P, make_row(P, o.line, o.itE), o.it0, in[h], out[h]);
+        line = o.line;
       }
-      acc2_add(s, f2(v.y), f2(v.z), Ac);
+      // trajectories of cut lines are not searched
+      cut[h] = P.linemax && __ldg(&P.linemax[line]) < P.a_min;
     }
-    const Acc sa = {s.a.x, s.b.x, s.d.x}, sb = {s.a.y, s.b.y, s.d.y};
-    unsigned ka = __float_as_uint(screen_lb(V, sa)) >> 16;
-    unsigned kb = __float_as_uint(screen_lb(V, sb)) >> 16;
-    if (P.linemax) {  // trajectories of cut lines are not searched
-      const unsigned line = (unsigned)P.line;
-      if (__ldg(&P.linemax[ja / line]) < P.a_min) ka = kScreenCut;
-      if (__ldg(&P.linemax[jb / line]) < P.a_min) kb = kScreenCut;
+    float la = 0.f, lb = 0.f;
+    if (__any_sync(kFull, !cut[0] || !cut[1]))
+      screen2<H>(P, V, s_ep, c[0], c[1], in[0], out[0], in[1], out[1], la,
+                 lb);
+    const unsigned ka = cut[0] ? kScreenCut : __float_as_uint(la) >> 16;
+    const unsigned kb = cut[1] ? kScreenCut : __float_as_uint(lb) >> 16;
+    if (pa < n) {
+      B.code[pa] = (unsigned short)ka;
+      if (!cut[0]) atomicAdd(&s_hist[ka / kScreenBinCodes], 1u);
     }
-    if (ia < n) {
-      B.code[ia] = (unsigned short)ka;
-      if (ka != kScreenCut) atomicAdd(&s_hist[ka >> 3], 1u);
-    }
-    if (ib < n) {
-      B.code[ib] = (unsigned short)kb;
-      if (kb != kScreenCut) atomicAdd(&s_hist[kb >> 3], 1u);
+    if (pb < n) {
+      B.code[pb] = (unsigned short)kb;
+      if (!cut[1]) atomicAdd(&s_hist[kb / kScreenBinCodes], 1u);
     }
   }
   __syncthreads();
@@ -123,14 +340,19 @@ __global__ void __launch_bounds__(kScreenThreads)
     if (s_hist[b]) atomicAdd(&B.hist[b], s_hist[b]);
 }
 
+constexpr int kListThreads = 1024;  // blocks of the two list kernels
+
 // Appends the trajectories keep() accepts to out[], in ascending order
 // within a block's chunks of codes (one atomic per chunk): neighbouring
 // entries mostly share a line of the map.
 template <typename Keep>
-__device__ __forceinline__ void append(const ScreenBufs &B, unsigned n,
-                                       unsigned cap, unsigned *out,
-                                       unsigned *len, const Keep &keep) {
+__device__ __forceinline__ void append(const SearchParams &P,
+                                       const ScreenBufs &B, unsigned cap,
+                                       unsigned *out, unsigned *len,
+                                       const Keep &keep) {
   constexpr int kPer = 8;  // codes per thread: one 16-byte load
+  const unsigned n = (unsigned)P.count;
+  const bool tf = by_t0(P);
   __shared__ unsigned s_w[32], s_base;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nw = blockDim.x >> 5;
@@ -157,19 +379,21 @@ __device__ __forceinline__ void append(const ScreenBufs &B, unsigned n,
     }
     if (lane == 31) s_w[warp] = p;
     __syncthreads();
-    if (threadIdx.x == 0) {
-      unsigned t = 0;
-      for (int k = 0; k < nw; ++k) {
-        const unsigned v = s_w[k];
-        s_w[k] = t;
-        t += v;
+    if (warp == 0) {
+      const unsigned v = lane < nw ? s_w[lane] : 0u;
+      unsigned t = v;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned u = __shfl_up_sync(kFull, t, o);
+        if (lane >= o) t += u;
       }
-      s_base = t ? atomicAdd(len, t) : 0u;
+      if (lane < nw) s_w[lane] = t - v;
+      if (lane == 31) s_base = t ? atomicAdd(len, t) : 0u;
     }
     __syncthreads();
     unsigned at = s_base + s_w[warp] + p - c;
     for (; m; m &= m - 1, ++at)
-      if (at < cap) out[at] = i0 + (__ffs(m) - 1);
+      if (at < cap) out[at] = offset_of(P, i0 + (__ffs(m) - 1), tf);
     __syncthreads();
   }
 }
@@ -178,85 +402,92 @@ __device__ __forceinline__ void append(const ScreenBufs &B, unsigned n,
 // want-th lowest code, and a hashed sample of that bin's (codes are equal
 // there as far as the histogram tells: all of them, where the bounds say
 // nothing).
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kListThreads)
     k_pilot_list(const SearchParams P, const ScreenBufs B) {
-  __shared__ unsigned s_sum[256], s_cut, s_r;
-  constexpr int kPer = kScreenBins / 256;
-  unsigned t = 0;
-  for (int k = 0; k < kPer; ++k) t += B.hist[threadIdx.x * kPer + k];
-  s_sum[threadIdx.x] = t;
+  __shared__ unsigned s_w[32], s_cut, s_r;
+  static_assert(kScreenBins == kListThreads, "a bin per thread");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned h = B.hist[threadIdx.x];
+  unsigned p = h;  // cumulated
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned v = __shfl_up_sync(kFull, p, o);
+    if (lane >= o) p += v;
+  }
+  if (lane == 31) s_w[warp] = p;
   if (threadIdx.x == 0) {
     s_cut = kScreenBins;
     s_r = 1;
   }
   __syncthreads();
-  for (int o = 1; o < 256; o <<= 1) {
-    const unsigned v = threadIdx.x >= o ? s_sum[threadIdx.x - o] : 0u;
-    __syncthreads();
-    s_sum[threadIdx.x] += v;
-    __syncthreads();
-  }
-  unsigned below = s_sum[threadIdx.x] - t;
-  if (below < B.want && s_sum[threadIdx.x] >= B.want) {
-    for (int k = 0; k < kPer; ++k) {
-      const unsigned h = B.hist[threadIdx.x * kPer + k];
-      if (below + h >= B.want) {
-        const unsigned left = B.want - below;
-        s_cut = threadIdx.x * kPer + k;
-        s_r = (h + left - 1) / left;
-        break;
-      }
-      below += h;
-    }
+  for (int w = 0; w < warp; ++w) p += s_w[w];
+  if (p >= B.want && p - h < B.want) {
+    const unsigned left = B.want - (p - h);
+    s_cut = threadIdx.x;
+    s_r = (h + left - 1) / left;
   }
   __syncthreads();
   const unsigned cut = s_cut, r = s_r;
-  append(B, (unsigned)P.count, B.pilot_cap, B.pilot, &B.n[0],
+  append(P, B, B.pilot_cap, B.pilot, &B.n[0],
          [=](unsigned code, unsigned i) {
-           const unsigned b = code >> 3;
+           const unsigned b = code / kScreenBinCodes;
            return b < cut ||
                   (b == cut && ((i * 0x9E3779B1u) >> 8) % r == 0u);
          });
 }
 
-// Upper bounds of the pilot's chi^2 over the whole light curve (the same
-// sums and solve as the search; chi2_upper).  Groups of kPilotTpg entries
-// per warp: the FP64 solve of a warp costs the same for 1 and 32
-// trajectories, the sweeps grow with their number.
-constexpr int kPilotTpg = 4, kPilotWarps = 4;
+// Upper bounds of the pilot's chi^2 over the whole light curve (chi2_upper).
+// A block takes kPilotTpg entries, its warps a slice of the epochs each (a
+// few thousand entries would leave most of the chip waiting for the walk of
+// one warp), and one warp adds the slices and solves.  P.gamma allows for
+// the slices (launch_screen_pilot).
+constexpr int kPilotTpg = 8, kPilotWarps = 8;
 
-template <bool STAGED, bool H>
+template <bool H>
 __global__ void __launch_bounds__(kPilotWarps * 32)
     k_pilot(const SearchParams P, const ScreenBufs B) {
-  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ Acc s_acc[kPilotWarps][kPilotTpg];
+  __shared__ TrajC s_c[kPilotTpg];
   const unsigned n = min(B.n[0], B.pilot_cap);
-  const int lane = threadIdx.x & 31;
-  const unsigned g0 = (blockIdx.x * kPilotWarps + (threadIdx.x >> 5)) *
-                      kPilotTpg;
-  if (blockIdx.x * kPilotWarps * kPilotTpg >= n) return;  // whole block
-  const float4 *blk = P.ep;
-  if (STAGED) {
-    float4 *s = reinterpret_cast<float4 *>(smem);
-    for (int e = threadIdx.x; e < P.n_ep; e += blockDim.x) s[e] = P.ep[e];
-    __syncthreads();
-    blk = s;
-  }
-  const Epochs ep = epochs_at(blk, P.n_ep);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned g0 = blockIdx.x * kPilotTpg;
   if (g0 >= n) return;
   const int nv = (int)min((unsigned)kPilotTpg, n - g0);
-  const unsigned j = (unsigned)P.first + B.pilot[g0 + (lane < nv ? lane : 0)];
-  double xi, xo;
-  TrajC mine = traj_base_of(P, j, xi, xo);
-  traj_range(ep, P.n_ep, xi, xo, mine);
-  Acc ms = {0.f, 0.f, 0.f};
+  Epochs ep = epochs_at(P.ep, P.n_ep);
+  if (warp == 0) {  // once: the constants' FP64 would be the block's limit
+    double xi, xo;
+    TrajC c = traj_base_of(
+        P, (unsigned)P.first + B.pilot[g0 + (lane < nv ? lane : 0)], xi, xo);
+    traj_range(ep, P.n_ep, xi, xo, c);
+    if (lane < kPilotTpg) s_c[lane] = c;
+  }
+  __syncthreads();
+  TrajC mine = s_c[lane < kPilotTpg ? lane : 0];
+  const int e0 = (int)((long long)P.n_ep * warp / kPilotWarps);
+  const int m = (int)((long long)P.n_ep * (warp + 1) / kPilotWarps) - e0;
+  ep.tw += e0;
+  ep.wf += e0;
+  mine.e_in = min(max(mine.e_in - e0, 0), m);
+  mine.e_out = min(max(mine.e_out - e0, 0), m);
   for (int k = 0; k < nv; k += 2) {
     const int k2 = min(k + 1, nv - 1);
     const TrajC ca = shfl_traj(mine, k), cb = shfl_traj(mine, k2);
     Acc ra, rb;
-    phase1_pair<H>(P, ep, ca, cb, lane, ra, rb);
-    if (lane == k) ms = ra;
-    else if (lane == k2) ms = rb;
+    phase1_pair_n<H>(P, ep, m, ca, cb, lane, ra, rb);
+    if (lane == 0) {
+      s_acc[warp][k] = ra;
+      s_acc[warp][k2] = rb;
+    }
   }
+  __syncthreads();
+  if (warp != 0) return;
+  Acc ms = {0.f, 0.f, 0.f};
+  if (lane < nv)
+    for (int w = 0; w < kPilotWarps; ++w) {
+      ms.a += s_acc[w][lane].a;
+      ms.b += s_acc[w][lane].b;
+      ms.d += s_acc[w][lane].d;
+    }
   const Fit2 f = fit2(P, (double)ms.a, (double)ms.b, (double)ms.d);
   const double ub =
       chi2_upper(P, (double)ms.a, (double)ms.b, (double)ms.d,
@@ -268,7 +499,7 @@ __global__ void __launch_bounds__(kPilotWarps * 32)
 // The threshold: the top_k-th smallest of the pilot's bounds (K distinct
 // trajectories have chi^2 at or below it), by four passes of eight bits
 // over the FP32 bit patterns, every block for itself; then the list.
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kListThreads)
     k_list(const SearchParams P, const ScreenBufs B) {
   __shared__ unsigned s_h[256], s_bits, s_left;
   const unsigned n = min(B.n[0], B.pilot_cap);
@@ -278,9 +509,9 @@ __global__ void __launch_bounds__(256)
     unsigned bits = 0, mask = 0;
     if (threadIdx.x == 0) s_left = K;
     for (int sh = 24; sh >= 0; sh -= 8) {
-      s_h[threadIdx.x] = 0;
+      if (threadIdx.x < 256) s_h[threadIdx.x] = 0;
       __syncthreads();
-      for (unsigned i = threadIdx.x; i < n; i += 256) {
+      for (unsigned i = threadIdx.x; i < n; i += kListThreads) {
         const unsigned b = __float_as_uint(B.ub[i]);
         if ((b & mask) == bits) atomicAdd(&s_h[(b >> sh) & 255u], 1u);
       }
@@ -322,17 +553,104 @@ __global__ void __launch_bounds__(256)
   // a code is the upper half of its bound's bits: bound <= thr needs
   // code <= thr >> 16
   const unsigned cut = thr >> 16;
-  append(B, (unsigned)P.count, B.list_cap, B.list, &B.n[1],
+  append(P, B, B.list0_cap, B.list0, &B.n[1],
          [=](unsigned code, unsigned) { return code <= cut; });
+}
+
+// The listed trajectories on the second and third subsets, now against the
+// threshold: those left go to the final list.  A block keeps what the second
+// subset leaves in a queue and takes the third with full warps.  When the
+// two discard less than one in eight of those decided so far (from 16 384
+// on), the screen gives up and the whole range is searched.
+template <bool H>
+__global__ void __launch_bounds__(kScreenThreads, 4)
+    k_rescreen(const SearchParams P, const ScreenBufs B) {
+  __shared__ float4 s_e1[kScreenMax1], s_e2[kScreenMax2];
+  __shared__ unsigned s_queue[2 * kScreenTile];
+  __shared__ unsigned s_m[kScreenThreads / 16], s_base, s_stop;
+  const ScreenLv V1 = P.lv[1], V2 = P.lv[2];
+  const unsigned n = B.n[1];
+  unsigned c0 = blockIdx.x * kScreenTile;
+  if (c0 >= n) return;
+  stage_subset(V1, s_e1);
+  stage_subset(V2, s_e2);
+  const float thr = __double2float_ru(bits_to_chi2(__ldcg(P.gthr)));
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned below = (1u << lane) - 1u;
+  unsigned queued = 0;  // block-uniform
+  while (c0 < n || queued > 0) {
+    const bool first = c0 < n && queued < (unsigned)kScreenTile;
+    const unsigned m = min((unsigned)kScreenTile, first ? n - c0 : queued);
+    const unsigned q0 = first ? 0u : queued - m;
+    if (threadIdx.x == 0) s_stop = *(volatile unsigned *)&B.n[4];
+    __syncthreads();  // the subsets, the queue
+    if (s_stop) return;
+    const unsigned i[2] = {(unsigned)(warp * 64 + lane),
+                           (unsigned)(warp * 64 + lane + 32)};
+    unsigned off[2];
+    TrajC c[2];
+    float in[2], out[2];
+    unsigned ma = 0, mb = 0;
+    if ((unsigned)warp * 64u < m) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const unsigned k = min(i[h], m - 1);
+        off[h] = first ? B.list0[c0 + k] : s_queue[q0 + k];
+        double xi, xo;
+        c[h] = traj_base_of(P, (unsigned)P.first + off[h], xi, xo);
+        in[h] = __double2float_rd(xi);
+        out[h] = __double2float_ru(xo);
+      }
+      float la, lb;
+      if (first)
+        screen2<H>(P, V1, s_e1, c[0], c[1], in[0], out[0], in[1], out[1], la,
+                   lb);
+      else
+        screen2<H>(P, V2, s_e2, c[0], c[1], in[0], out[0], in[1], out[1], la,
+                   lb);
+      ma = __ballot_sync(kFull, i[0] < m && la <= thr);
+      mb = __ballot_sync(kFull, i[1] < m && lb <= thr);
+    }
+    if (lane == 0) {
+      s_m[2 * warp] = __popc(ma);
+      s_m[2 * warp + 1] = __popc(mb);
+    }
+    __syncthreads();  // also: the queue is read
+    if (threadIdx.x == 0) {
+      unsigned t = 0;
+      for (int k = 0; k < kScreenThreads / 16; ++k) {
+        const unsigned v = s_m[k];
+        s_m[k] = t;
+        t += v;
+      }
+      s_base = first ? t : (t ? atomicAdd(&B.n[2], t) : 0u);
+      const unsigned killed = m - t, done = first ? killed : m;
+      const unsigned all = atomicAdd(&B.n[3], done) + done;
+      const unsigned gone = atomicAdd(&B.n[5], killed) + killed;
+      if (all >= 16384u && 8ull * gone < all) atomicExch(&B.n[4], 1u);
+    }
+    __syncthreads();
+    const unsigned ra = s_m[2 * warp] + __popc(ma & below);
+    const unsigned rb = s_m[2 * warp + 1] + __popc(mb & below);
+    if (first) {
+      if (ma >> lane & 1u) s_queue[queued + ra] = off[0];
+      if (mb >> lane & 1u) s_queue[queued + rb] = off[1];
+      queued += s_base;
+      c0 += gridDim.x * kScreenTile;
+    } else {
+      const unsigned g = s_base;
+      if ((ma >> lane & 1u) && g + ra < B.list_cap) B.list[g + ra] = off[0];
+      if ((mb >> lane & 1u) && g + rb < B.list_cap) B.list[g + rb] = off[1];
+      queued -= m;
+    }
+  }
 }
 
 }  // namespace
 
 cudaError_t launch_screen(const SearchParams &P, const ScreenBufs &B,
                           int sm_count, cudaStream_t st) {
-  const long long tiles = (P.count + 63) / 64;
-  const long long want = (tiles + kScreenThreads / 32 - 1) /
-                         (kScreenThreads / 32);
+  const long long want = (P.count + kScreenTile - 1) / kScreenTile;
   const int grid = (int)std::min<long long>(want, 4LL * sm_count);
   if (P.quadh)
     k_screen<true><<<grid, kScreenThreads, 0, st>>>(P, B);
@@ -342,54 +660,46 @@ cudaError_t launch_screen(const SearchParams &P, const ScreenBufs &B,
 }
 
 static int append_grid(const SearchParams &P, int sm_count) {
-  const long long want = (P.count + 2047) / 2048;
-  return (int)std::min<long long>(want, 2LL * sm_count);
+  const long long want =
+      (P.count + 8LL * kListThreads - 1) / (8LL * kListThreads);
+  return (int)std::min<long long>(want, (long long)sm_count);
 }
 
 cudaError_t launch_screen_pilot_list(const SearchParams &P,
                                      const ScreenBufs &B, int sm_count,
                                      cudaStream_t st) {
-  k_pilot_list<<<append_grid(P, sm_count), 256, 0, st>>>(P, B);
+  k_pilot_list<<<append_grid(P, sm_count), kListThreads, 0, st>>>(P, B);
   return cudaGetLastError();
 }
 
 cudaError_t launch_screen_pilot(const SearchParams &P, const ScreenBufs &B,
-                                size_t smem_optin, int sm_count,
                                 cudaStream_t st) {
-  const int per = kPilotTpg * kPilotWarps;
-  const int grid = (int)((B.pilot_cap + per - 1) / per);
-  const size_t sm = sizeof(float4) * (size_t)P.n_ep;
-  (void)sm_count;
-  (void)smem_optin;
-  // staged while two blocks fit an SM
-  if (sm <= 100 * 1024) {
-    static int set_of[64];
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev >= 64 || !set_of[dev]) {
-      cudaFuncSetAttribute(k_pilot<true, true>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           100 * 1024);
-      cudaFuncSetAttribute(k_pilot<true, false>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           100 * 1024);
-      if (dev < 64) set_of[dev] = 1;
-    }
-    if (P.quadh)
-      k_pilot<true, true><<<grid, kPilotWarps * 32, sm, st>>>(P, B);
-    else
-      k_pilot<true, false><<<grid, kPilotWarps * 32, sm, st>>>(P, B);
-  } else if (P.quadh) {
-    k_pilot<false, true><<<grid, kPilotWarps * 32, 0, st>>>(P, B);
-  } else {
-    k_pilot<false, false><<<grid, kPilotWarps * 32, 0, st>>>(P, B);
-  }
+  SearchParams Q = P;
+  // the slices' sums, as event_params bounds a whole one's
+  const double m = (double)((P.n_ep / kPilotWarps + 32) / 32);
+  Q.gamma = std::max(P.gamma, (m + 10.0 + kPilotWarps) * ldexp(1.0, -24));
+  const int grid = (int)((B.pilot_cap + kPilotTpg - 1) / kPilotTpg);
+  if (P.quadh)
+    k_pilot<true><<<grid, kPilotWarps * 32, 0, st>>>(Q, B);
+  else
+    k_pilot<false><<<grid, kPilotWarps * 32, 0, st>>>(Q, B);
   return cudaGetLastError();
 }
 
 cudaError_t launch_screen_list(const SearchParams &P, const ScreenBufs &B,
                                int sm_count, cudaStream_t st) {
-  k_list<<<append_grid(P, sm_count), 256, 0, st>>>(P, B);
+  k_list<<<append_grid(P, sm_count), kListThreads, 0, st>>>(P, B);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_rescreen(const SearchParams &P, const ScreenBufs &B,
+                            int sm_count, cudaStream_t st) {
+  const long long want = (P.count + kScreenTile - 1) / kScreenTile;
+  const int grid = (int)std::min<long long>(want, 4LL * sm_count);
+  if (P.quadh)
+    k_rescreen<true><<<grid, kScreenThreads, 0, st>>>(P, B);
+  else
+    k_rescreen<false><<<grid, kScreenThreads, 0, st>>>(P, B);
   return cudaGetLastError();
 }
 

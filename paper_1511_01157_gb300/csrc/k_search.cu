@@ -68,11 +68,16 @@ namespace {
 
 using namespace dev;
 
+// whether the screen left a list to search
+__device__ __forceinline__ bool listed(const SearchParams &P) {
+  return __ldg(P.n_list) <= P.list_cap && !(P.no_list && __ldg(P.no_list));
+}
+
 template <bool DENSE, bool EP_SMEM, bool H>
 __global__ void __launch_bounds__(kSearchWarps * 32, 1)
     k_search(const SearchParams P) {
   // a screened search: the listed kernel has it, unless the list is too long
-  if (!DENSE && P.n_list && __ldg(P.n_list) <= P.list_cap) return;
+  if (!DENSE && P.n_list && listed(P)) return;
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
@@ -223,8 +228,8 @@ __global__ void __launch_bounds__(kSearchWarps * 32, 1)
 }
 
 // The search of the listed trajectories (k_screen.cu), the same top-K as
-// k_search over the whole range: per warp group the larger screening
-// subsets first, then for the trajectories left the light curve itself
+// k_search over the whole range: per warp group the largest screening
+// subset first, then for the trajectories left the light curve itself
 // (phase 1, the FP64 solve and its bound, phase 2) with the same device
 // functions, so the same bits.  The list holds a few per cent of the grid,
 // its entries scattered over the lines, so cells come through L1 (no band
@@ -237,8 +242,8 @@ __global__ void __launch_bounds__(kSearchWarps * 32, 1)
 template <bool EPS, bool H>
 __global__ void __launch_bounds__(kSearchWarps * 32, 1)
     k_search_list(const SearchParams P) {
+  if (!listed(P)) return;  // k_search has it
   const unsigned n = __ldg(P.n_list);
-  if (n > P.list_cap) return;  // k_search has it
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
@@ -256,11 +261,11 @@ __global__ void __launch_bounds__(kSearchWarps * 32, 1)
   T.lock = &s_lock;
   T.thr = &s_thr;
   float4 *sm_ep = reinterpret_cast<float4 *>(p);
-  if (EPS) {  // the light curve and subsets 1 .. n_lv - 1 after it
+  if (EPS) {  // the light curve and subset 3 after it
     float4 *d = sm_ep;
     for (int e = threadIdx.x; e < P.n_ep; e += blockDim.x) d[e] = P.ep[e];
     d += P.n_ep;
-    for (int l = 1; l < P.n_lv; ++l) {
+    for (int l = 3; l < P.n_lv; ++l) {
       for (int e = threadIdx.x; e < P.lv[l].m; e += blockDim.x)
         d[e] = P.lv[l].ep[e];
       d += P.lv[l].m;
@@ -281,7 +286,7 @@ __global__ void __launch_bounds__(kSearchWarps * 32, 1)
   while (tpg < 32 && (unsigned)tpg * warps < n) tpg <<= 1;
   const unsigned n_groups = (n + tpg - 1) / tpg;
   unsigned long long n_exact = 0;
-  unsigned tried[kScreenLevels] = {}, killed[kScreenLevels] = {};
+  unsigned tried = 0, killed = 0;
   for (int seen = 0;; ++seen) {
     unsigned g = 0;
     if (lane == 0) g = (unsigned)atomicAdd(&s_next, 1);
@@ -300,16 +305,15 @@ __global__ void __launch_bounds__(kSearchWarps * 32, 1)
     unsigned act = nv == 32 ? kFull : (1u << nv) - 1u;
     Acc ms;
     const float4 *lv_ep = EPS ? sm_ep + P.n_ep : nullptr;
-    for (int l = 1; l <= P.n_lv; ++l) {
-      const bool last = l == P.n_lv;  // the light curve itself
+    for (int l = 3; l <= max(3, P.n_lv); ++l) {
+      const bool last = l >= P.n_lv;  // the light curve itself
       const int m = last ? P.n_ep : P.lv[l].m;
       const float4 *blk = EPS ? (last ? sm_ep : lv_ep)
                               : (last ? P.ep : P.lv[l].ep);
       if (!last) {
         lv_ep += m;
-        const unsigned t = tried[l], k = killed[l];
-        if (t >= 64 && (seen & 15) != 0 &&
-            (float)k * (float)(P.n_ep - m) < (float)t * (float)m)
+        if (tried >= 64 && (seen & 15) != 0 &&
+            (float)killed * (float)(P.n_ep - m) < (float)tried * (float)m)
           continue;
       }
       const Epochs ep = epochs_at(blk, m);
@@ -330,8 +334,8 @@ __global__ void __launch_bounds__(kSearchWarps * 32, 1)
       if (!last) {
         const bool stay = (act >> lane & 1u) && screen_lb(P.lv[l], ms) <= thr_f;
         const unsigned left = __ballot_sync(kFull, stay);
-        tried[l] += __popc(act);
-        killed[l] += __popc(act & ~left);
+        tried += __popc(act);
+        killed += __popc(act & ~left);
         act = left;
         if (!act) break;
       }
@@ -357,6 +361,18 @@ __global__ void __launch_bounds__(kSearchWarps * 32, 1)
       if (lane == k) my_chi2 = isnan(chi2) ? CUDART_INF : chi2;
     }
     const bool keep = my_chi2 <= thr && my_chi2 < CUDART_INF;
+    if (keep) {
+      const unsigned at = atomicAdd(P.n_cand, 1u);
+      if (at < kCandMax) {
+        Candidate c;
+        c.chi2 = my_chi2;
+        c.Fs = sol.Fs;
+        c.Bc = sol.Bc;
+        c.idx = my;
+        c.degenerate = sol.degenerate;
+        P.cand[at] = c;
+      }
+    }
     warp_merge(P, T, K, warp, lane, keep, my_chi2, (long long)my);
   }
   if (P.stat_exact && lane == 0 && n_exact) atomicAdd(P.stat_exact, n_exact);
@@ -381,7 +397,9 @@ __global__ void __launch_bounds__(kSearchWarps * 32, 1)
 constexpr int kMergeWays = 4;  // lists merged into one per level
 
 __global__ void k_merge_level(const Entry *__restrict__ in,
-                              Entry *__restrict__ out, int lists, int k) {
+                              Entry *__restrict__ out, int lists, int k,
+                              const unsigned *done) {
+  if (done && __ldg(done)) return;
   // one thread per input entry: its rank in its group of kMergeWays lists
   // is its index plus the entries of the group's other lists below it
   // (keys are unique across lists), and the first k ranks are kept
@@ -458,7 +476,9 @@ __device__ __forceinline__ int lower_rank(const unsigned long long *K,
 // binary search reads 8 bytes.
 __global__ void __launch_bounds__(1024)
     k_merge_rank(const Entry *__restrict__ in, Entry *__restrict__ out,
-                 int lists, int k, int ways, unsigned long long *seed) {
+                 int lists, int k, int ways, unsigned long long *seed,
+                 const unsigned *done) {
+  if (done && __ldg(done)) return;
   extern __shared__ __align__(16) unsigned char msm[];
   const int l = blockIdx.x;
   const int g = l / ways, l0 = g * ways;
@@ -524,6 +544,7 @@ __global__ void __launch_bounds__(1024)
 // warp's walk over the epochs waits only on the cell gathers.
 template <bool H, bool EPS>
 __global__ void k_fill(const FillParams F) {
+  if (F.done && __ldg(F.done)) return;
   extern __shared__ __align__(16) unsigned char fsm[];
   const float4 *blk = nullptr;
   if (EPS) {
@@ -536,6 +557,52 @@ __global__ void k_fill(const FillParams F) {
   const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (w >= F.k) return;  // after the block's only barrier
   fill_one<H>(F.S, F.sel[w], F.t0abs, F.tEv, lane, &F.out[w], blk);
+}
+
+// The records of a listed search from its candidates: every block stages
+// their keys and ranks kFinishPer of them by (chi^2, index), sixteen threads
+// per candidate; those of rank < k become records with the fits the search
+// solved, in place of two merge launches over all blocks' lists and a second
+// sweep of the epochs.  With the threshold of a good pilot the candidates
+// are little more than the k records themselves (config 1: 267 for 256);
+// more than kCandMax go the general way.
+constexpr int kFinishThreads = 1024, kFinishPer = kFinishThreads / 16;
+
+__global__ void __launch_bounds__(kFinishThreads)
+    k_finish(const FillParams F) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const SearchParams &P = F.S;
+  if (!listed(P)) return;
+  const unsigned n = __ldg(P.n_cand);
+  if (n > kCandMax) return;
+  if (blockIdx.x == 0) {
+    for (int r = (int)n + (int)threadIdx.x; r < F.k; r += blockDim.x)
+      F.out[r] = empty_record();
+    if (threadIdx.x == 0) *F.done = 1u;
+  }
+  if (blockIdx.x * kFinishPer >= n) return;
+  unsigned long long *key = reinterpret_cast<unsigned long long *>(smem);
+  unsigned *id = reinterpret_cast<unsigned *>(key + n);
+  for (unsigned i = threadIdx.x; i < n; i += blockDim.x) {
+    // chi^2 >= 0: its bits order as it does
+    key[i] = (unsigned long long)__double_as_longlong(P.cand[i].chi2);
+    id[i] = P.cand[i].idx;
+  }
+  __syncthreads();
+  const unsigned me = blockIdx.x * kFinishPer + threadIdx.x / 16;
+  const unsigned long long mk = me < n ? key[me] : 0ULL;
+  const unsigned mi = me < n ? id[me] : 0u;
+  unsigned r = 0;
+  for (unsigned i = threadIdx.x & 15; i < n; i += 16) {
+    const unsigned long long k = key[i];
+    r += k < mk || (k == mk && id[i] < mi);
+  }
+#pragma unroll
+  for (int o = 8; o; o >>= 1) r += __shfl_xor_sync(kFull, r, o);
+  if (me >= n || (threadIdx.x & 15) != 0 || r >= (unsigned)F.k) return;
+  const Candidate c = P.cand[me];
+  F.out[r] = fit_record(P, (long long)c.idx, c.chi2, c.Fs, c.Bc,
+                        c.degenerate != 0, F.t0abs, F.tEv);
 }
 
 // The tau interval of every (u0, alpha) line inside the map.
@@ -664,7 +731,7 @@ size_t list_smem_bytes(const SearchParams &P, bool staged) {
   size_t n = 0;
   if (staged) {
     n = (size_t)P.n_ep;
-    for (int l = 1; l < P.n_lv; ++l) n += (size_t)P.lv[l].m;
+    for (int l = 3; l < P.n_lv; ++l) n += (size_t)P.lv[l].m;
   }
   return search_smem_bytes((int)n, P.top_k);
 }
@@ -709,7 +776,8 @@ cudaError_t launch_search_list(const SearchParams &P, bool staged, int grid,
 
 cudaError_t launch_topk_merge(Entry *a, Entry *b, int lists, int k,
                               Entry **result, int *levels, cudaStream_t st,
-                              unsigned long long *seed) {
+                              unsigned long long *seed,
+                              const unsigned *done) {
   Entry *in = a, *out = b;
   *levels = 0;
   // the device's shared-memory limit, and the rank kernel's limit raised
@@ -740,13 +808,14 @@ cudaError_t launch_topk_merge(Entry *a, Entry *b, int lists, int k,
       // threads: S per entry for up to all k entries at once, whole warps
       const int S = ways >= 16 ? 4 : 1;
       const int threads = std::min(1024, ((k * S + 31) / 32) * 32);
-      k_merge_rank<<<lists, threads, sm, st>>>(in, out, lists, k, ways, sd);
+      k_merge_rank<<<lists, threads, sm, st>>>(in, out, lists, k, ways, sd,
+                                                done);
       seeded = sd != nullptr;
     } else {
       const long long total = (long long)lists * k;
       long long g = (total + 255) / 256;
       if (g > 65535) g = 65535;
-      k_merge_level<<<(int)g, 256, 0, st>>>(in, out, lists, k);
+      k_merge_level<<<(int)g, 256, 0, st>>>(in, out, lists, k, done);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -763,6 +832,20 @@ cudaError_t launch_topk_merge(Entry *a, Entry *b, int lists, int k,
     ++*levels;
   }
   return cudaSuccess;
+}
+
+cudaError_t launch_finish(const FillParams &F, cudaStream_t st) {
+  const size_t sm = (size_t)kCandMax * 12;
+  static int set_of[64];
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev >= 64 || !set_of[dev]) {
+    cudaFuncSetAttribute(k_finish, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)sm);
+    if (dev < 64) set_of[dev] = 1;
+  }
+  k_finish<<<kCandMax / kFinishPer, kFinishThreads, sm, st>>>(F);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_fill(const FillParams &F, cudaStream_t st) {

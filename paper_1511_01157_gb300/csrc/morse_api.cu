@@ -519,9 +519,9 @@ void event_params(const morse_event *ev, SearchParams *P) {
     V.SF = (float)u.SF;
     V.sqSFF = nextafterf((float)sqrt(u.SFF), INFINITY);
     V.CFF = nextafterf((float)(u.SFF - u.SF * u.SF / u.S1), 0.0f);
-    // terms of one sum: the smallest subset is summed by one lane, the
-    // others by 32
-    const double k = l == 0 ? (double)u.m : (double)((u.m + 31) / 32);
+    // terms of one sum: the first three subsets are summed by one lane, the
+    // fourth by 32
+    const double k = l < 3 ? (double)u.m : (double)((u.m + 31) / 32);
     V.g = (float)(2.0 * (k + 12.0) * ldexp(1.0, -24));
   }
 }
@@ -568,8 +568,8 @@ struct Plan {
   size_t off_tab, off_lmax, off_hdr, off_pub, off_pa, off_pb, off_out, bytes;
   int tab_n;  // band-table entries (0: the search reads the global table)
   // screened search (k_screen.cu); want = 0: off
-  unsigned want, pilot_cap, list_cap;
-  size_t off_code, off_hist, off_pil, off_ub, off_list;
+  unsigned want, pilot_cap, list0_cap, list_cap;
+  size_t off_code, off_hist, off_pil, off_ub, off_list0, off_list, off_cand;
 };
 
 // What the line-aligned pass needs to read its map cells from shared-memory
@@ -638,13 +638,20 @@ size_t plan_screen(const morse_event *ev, const morse_grid *g,
   pl->pilot_cap = 2 * pl->want;
   pl->list_cap = (unsigned)(count / 2);
   pl->off_hist = align_up(at, 256);  // histogram and list lengths: cleared
-  pl->off_code =
-      align_up(pl->off_hist + sizeof(unsigned) * (morse::kScreenBins + 2), 256);
+  pl->off_code = align_up(
+      pl->off_hist + sizeof(unsigned) * (morse::kScreenBins +
+                                         morse::kScreenWords), 256);
   pl->off_pil = align_up(
       pl->off_code + sizeof(unsigned short) * (size_t)(count + 8), 256);
   pl->off_ub = pl->off_pil + sizeof(unsigned) * (size_t)pl->pilot_cap;
-  pl->off_list = pl->off_ub + sizeof(float) * (size_t)pl->pilot_cap;
-  return pl->off_list + sizeof(unsigned) * (size_t)pl->list_cap;
+  pl->off_list0 = pl->off_ub + sizeof(float) * (size_t)pl->pilot_cap;
+  // without a third subset the first list is the final one
+  pl->list0_cap = ev->n_sub > 2 ? (unsigned)count : pl->list_cap;
+  pl->off_list = pl->off_list0;
+  if (ev->n_sub > 2) pl->off_list += sizeof(unsigned) * (size_t)count;
+  pl->off_cand = align_up(
+      pl->off_list + sizeof(unsigned) * (size_t)pl->list_cap, 256);
+  return pl->off_cand + sizeof(morse::Candidate) * morse::kCandMax;
 }
 
 // Reset the pruning threshold between the maps of a sweep (it is per map).
@@ -792,6 +799,7 @@ morse_status enqueue_topk(morse_ctx *ctx, const Plan &pl,
   int list_grid = 0;
   bool staged = false;
   size_t list_smem = 0;
+  unsigned *done = nullptr;  // set when the list gave the records
   if (pl.want > 0) {
     // the listed search: staged light curve and subsets when they fit
     for (int s = 1; s >= 0 && list_grid == 0; --s) {
@@ -810,25 +818,38 @@ morse_status enqueue_topk(morse_ctx *ctx, const Plan &pl,
     B.n = B.hist + morse::kScreenBins;
     B.pilot = (unsigned *)(base + pl.off_pil);
     B.ub = (float *)(base + pl.off_ub);
+    B.list0 = (unsigned *)(base + pl.off_list0);
     B.list = (unsigned *)(base + pl.off_list);
     B.pilot_cap = pl.pilot_cap;
+    B.list0_cap = pl.list0_cap;
     B.list_cap = pl.list_cap;
     B.want = pl.want;
     MORSE_CUDA(ctx, cudaMemsetAsync(
                         B.hist, 0,
-                        sizeof(unsigned) * (morse::kScreenBins + 2),
+                        sizeof(unsigned) * (morse::kScreenBins +
+                                            morse::kScreenWords),
                         ctx->stream));
     r = t_begin(ctx, KT_SEARCH);
     MORSE_CUDA(ctx, morse::launch_screen(P, B, ctx->sm_count, ctx->stream));
     MORSE_CUDA(ctx, morse::launch_screen_pilot_list(P, B, ctx->sm_count,
                                                     ctx->stream));
-    MORSE_CUDA(ctx, morse::launch_screen_pilot(P, B, ctx->smem_optin,
-                                               ctx->sm_count, ctx->stream));
+    MORSE_CUDA(ctx, morse::launch_screen_pilot(P, B, ctx->stream));
     MORSE_CUDA(ctx, morse::launch_screen_list(P, B, ctx->sm_count,
                                               ctx->stream));
     P.list = B.list;
     P.n_list = B.n + 1;
+    P.no_list = nullptr;
     P.list_cap = B.list_cap;
+    P.cand = (morse::Candidate *)(base + pl.off_cand);
+    P.n_cand = B.n + 6;
+    done = B.n + 7;
+    if (P.n_lv > 2) {
+      MORSE_CUDA(ctx, morse::launch_rescreen(P, B, ctx->sm_count,
+                                             ctx->stream));
+      ctx->launches += 1;
+      P.n_list = B.n + 2;
+      P.no_list = B.n + 4;
+    }
     P.pub_tag = next_pub_tag(ctx);
     P.pub_nb = list_grid;
     P.pub_me = -1;
@@ -880,22 +901,28 @@ morse_status enqueue_topk(morse_ctx *ctx, const Plan &pl,
                                        ctx->stream));
   t_end(ctx, r);
   ctx->launches += 1;
-  Entry *sel = nullptr;
-  int levels = 0;
-  r = t_begin(ctx, KT_MERGE);
-  MORSE_CUDA(ctx, morse::launch_topk_merge((Entry *)(base + pl.off_pa),
-                                           (Entry *)(base + pl.off_pb),
-                                           pl.grid, pl.K, &sel, &levels,
-                                           ctx->stream));
-  t_end(ctx, r);
-  ctx->launches += (uint64_t)levels;
   morse::FillParams F;
   F.S = P;
-  F.sel = sel;
+  F.sel = nullptr;
   F.k = pl.K;
   F.t0abs = T.t0abs;
   F.tEv = T.tEv;
   F.out = fits_dev;
+  F.done = done;
+  r = t_begin(ctx, KT_MERGE);
+  if (done) {
+    MORSE_CUDA(ctx, morse::launch_finish(F, ctx->stream));
+    ctx->launches += 1;
+  }
+  Entry *sel = nullptr;
+  int levels = 0;
+  MORSE_CUDA(ctx, morse::launch_topk_merge((Entry *)(base + pl.off_pa),
+                                           (Entry *)(base + pl.off_pb),
+                                           pl.grid, pl.K, &sel, &levels,
+                                           ctx->stream, nullptr, done));
+  t_end(ctx, r);
+  ctx->launches += (uint64_t)levels;
+  F.sel = sel;
   r = t_begin(ctx, KT_FILL);
   MORSE_CUDA(ctx, morse::launch_fill(F, ctx->stream));
   t_end(ctx, r);
@@ -1977,62 +2004,75 @@ void morse_map_free(morse_map *map) {
 
 // ------------------------------------------------------------------ events
 // The screening subsets of a light curve (k_screen.cu), appended to its n
-// slots h: 32 epochs (64 from 640 epochs on), an eighth of it from 1024
-// epochs on and a third from 2048 on.  An epoch's share grows with its
-// information w (F - F_mean)^2, since that is what a wrong trajectory's
-// chi^2 is made of, and a tenth of the shares is even (it pins the
-// baseline): along the cumulated shares, capped at one epoch each, every
-// crossing of a half-integer takes an epoch.  Light curves whose sums are
+// slots h: 32 epochs (64 from 640 epochs on); from 1024 epochs on 96, and a
+// quarter of it or 320; from 2048 on a third of it.  They consist of runs of
+// neighbouring epochs (4, 8, 16 and 32 long), which a trajectory meets in
+// the same few cells; measured over events of tE 13 to 72 d, runs of that
+// length discard as many trajectories as single epochs do.  A run's share
+// grows with its information sum w (F - F_mean)^2, since that is what a
+// wrong trajectory's chi^2 is made of, and a tenth of the shares is even (it
+// pins the baseline): along the cumulated shares, capped at one run each,
+// every crossing of a half-integer takes a run.  Light curves whose sums are
 // out of the FP32 bounds' range (screen_lb) have no subsets.
 static void screen_subsets(morse_event *ev, std::vector<float4> &h, int64_t n,
                            double S1, double SF, double SFF) {
   ev->n_sub = 0;
-  const int sizes[kScreenLevels] = {n < 640 ? 32 : 64,
-                                    n >= 1024 ? (int)(n / 8) : 0,
-                                    n >= 2048 ? (int)(n / 3) : 0};
+  const int sizes[kScreenLevels] = {
+      n < 640 ? 32 : 64, n >= 1024 ? 96 : 0,
+      n >= 1024 ? (int)std::min<int64_t>(n / 4, 320) : 0,
+      n >= 2048 ? (int)(n / 3) : 0};
   if (n < 128 || n > (1 << 20) || !(S1 > 1e-12 && S1 < 1e15 && SFF > 1e-12 &&
                                     SFF < 1e15))
     return;
-  std::vector<double> x((size_t)n);
+  const int runs[kScreenLevels] = {4, 8, 16, 32};
+  std::vector<double> x;
   std::vector<int> sel;
   for (int l = 0; l < kScreenLevels && sizes[l] > 0; ++l) {
-    const int m = sizes[l];
+    const int run = runs[l];
+    const int64_t nr = (n + run - 1) / run;
+    const double m = (double)sizes[l] / run;  // runs to take
     const float2 *tw = reinterpret_cast<const float2 *>(h.data());
-    const float *wf = reinterpret_cast<const float *>(tw + n);
-    const float *fc = wf + n;
+    const float *fc = reinterpret_cast<const float *>(tw + n) + n;
     const double mean = SF / S1;
+    x.assign((size_t)nr, 0.0);
     double sum = 0.0;
     for (int64_t i = 0; i < n; ++i) {
       const double d = (double)fc[i] - mean;
-      sum += x[(size_t)i] = (double)tw[i].y * d * d;
+      const double v = (double)tw[i].y * d * d;
+      x[(size_t)(i / run)] += v;
+      sum += v;
     }
-    const double even = 0.1 / (double)n;
+    const double even = 0.1 / (double)nr;
     const double per = sum > 0.0 ? 0.9 / sum : 0.0;
-    for (int64_t i = 0; i < n; ++i) x[(size_t)i] = x[(size_t)i] * per + even;
+    for (double &v : x) v = v * per + even;
     // scale so that the shares, capped at 1, add up to m
-    double scale = (double)m / (sum > 0.0 ? 1.0 : 0.1);
+    double scale = m / (sum > 0.0 ? 1.0 : 0.1);
     for (int it = 0; it < 8; ++it) {
       double capped = 0.0, rest = 0.0;
-      for (int64_t i = 0; i < n; ++i) {
-        const double v = x[(size_t)i] * scale;
+      for (double v : x) {
+        v *= scale;
         if (v >= 1.0)
           capped += 1.0;
         else
           rest += v;
       }
-      if (rest <= 0.0 || capped >= (double)m) break;
-      const double f = ((double)m - capped) / rest;
+      if (rest <= 0.0 || capped >= m) break;
+      const double f = (m - capped) / rest;
       if (f < 1.0001 && f > 0.9999) break;
       scale *= f;
     }
     sel.clear();
     double acc = 0.5;
-    for (int64_t i = 0; i < n; ++i) {
-      const double next = acc + std::min(1.0, x[(size_t)i] * scale);
-      if (std::floor(next) > std::floor(acc)) sel.push_back((int)i);
+    for (int64_t r = 0; r < nr; ++r) {
+      const double next = acc + std::min(1.0, x[(size_t)r] * scale);
+      if (std::floor(next) > std::floor(acc))
+        for (int64_t i = r * run; i < std::min(n, (r + 1) * run); ++i)
+          sel.push_back((int)i);
       acc = next;
     }
-    if (sel.size() < 8 || (l == 0 && sel.size() > 128)) return;
+    // (the most the kernels stage of the first three)
+    const size_t most[kScreenLevels] = {128, 192, 512, (size_t)n};
+    if (sel.size() < 8 || sel.size() > most[l]) break;
     morse_subset &u = ev->sub[l];
     u.m = (int)sel.size();
     u.off = (int)h.size();

@@ -75,7 +75,7 @@ struct morse_map {
 };
 
 // Screening subsets of a light curve: at most this many, smallest first.
-constexpr int kScreenLevels = 3;
+constexpr int kScreenLevels = 4;
 
 // One subset of m epochs (time-sorted), stored like the light curve itself
 // at ep + off, with the FP64 sums of its stored values.
@@ -231,6 +231,7 @@ struct ScreenLv {
   float g;                  // relative error bound of the FP32 sums, doubled
 };
 
+struct Candidate;
 struct SearchParams {
   // map: the lookup reads quadh (FP16 log10 quads) when it is set, else
   // quad (FP32 A - 1 quads); both share qpitch and the index folding
@@ -304,23 +305,42 @@ struct SearchParams {
   int n_lv;
   ScreenLv lv[kScreenLevels];
   const unsigned *list;     // trajectories (offsets from first) to search
-  const unsigned *n_list;   // their number, or more than list_cap if they
-  unsigned list_cap;        // do not fit: then the whole range is searched
+  const unsigned *n_list;   // their number
+  const unsigned *no_list;  // nonzero, or *n_list > list_cap: no list, the
+  unsigned list_cap;        // whole range is searched (no_list may be null)
+  Candidate *cand;          // [kCandMax] what the listed search merged into
+  unsigned *n_cand;         // its top-K lists, and how many (all counted)
 };
+
+// A trajectory the listed search kept, with its fit.
+struct Candidate {
+  double chi2, Fs, Bc;
+  unsigned idx, degenerate;
+};
+constexpr unsigned kCandMax = 8192;
 
 // Workspace of a screened search.
 struct ScreenBufs {
   unsigned short *code;     // [count] lower bound of each trajectory's
                             // chi^2: the upper half of its FP32 bits
-  unsigned *hist;           // [kScreenBins] trajectories per code >> 3
-  unsigned *n;              // [2] lengths of the two lists
+  unsigned *hist;           // [kScreenBins] trajectories per kScreenBinCodes
+                            // codes
+  unsigned *n;              // [kScreenWords] lengths of the pilot's list (0),
+                            // of list0 (1) and of list (2); trajectories
+                            // the rescreening decided (3), gave up on the
+                            // whole (4: nonzero), discarded (5); candidates
+                            // of the listed search (6), records made (7:
+                            // nonzero)
   unsigned *pilot;          // [pilot_cap] trajectories of the pilot
   float *ub;                // [pilot_cap] their chi^2 bounds from above
-  unsigned *list;           // [list_cap]
-  unsigned pilot_cap, list_cap;
+  unsigned *list0;          // [list0_cap] trajectories the codes leave
+  unsigned *list;           // [list_cap] those left after the rescreening
+                            // (list0 itself where there is none)
+  unsigned pilot_cap, list0_cap, list_cap;
   unsigned want;            // pilot trajectories asked for
 };
-constexpr int kScreenBins = 4096;
+constexpr int kScreenBins = 1024, kScreenWords = 8;
+constexpr unsigned kScreenBinCodes = 32768 / kScreenBins;
 constexpr unsigned kScreenCut = 0xFFFFu;  // code of a cut line's trajectory
 
 // ------------------------------------------- host set-up of a search
@@ -354,6 +374,8 @@ struct FillParams {
   int k;
   const double *t0abs, *tEv;  // absolute t0 and tE tables
   morse_fit *out;           // [k]
+  unsigned *done;           // records made from the candidates: nonzero
+                            // (nullptr: none were)
 };
 
 #ifndef MORSE_SEARCH_WARPS
@@ -422,12 +444,14 @@ cudaError_t launch_screen_pilot_list(const SearchParams &P,
                                      cudaStream_t st);
 // their upper bounds
 cudaError_t launch_screen_pilot(const SearchParams &P, const ScreenBufs &B,
-                                size_t smem_optin, int sm_count,
                                 cudaStream_t st);
 // *P.gthr <- the pilot's top_k-th bound; the list of trajectories whose
 // code does not exceed it
 cudaError_t launch_screen_list(const SearchParams &P, const ScreenBufs &B,
                                int sm_count, cudaStream_t st);
+// the listed trajectories on the second subset (P.n_lv >= 2)
+cudaError_t launch_rescreen(const SearchParams &P, const ScreenBufs &B,
+                            int sm_count, cudaStream_t st);
 // shared memory of the listed search with staged epochs (0: they do not
 // fit), and its launch
 size_t list_smem_bytes(const SearchParams &P, bool staged);
@@ -443,10 +467,15 @@ cudaError_t launch_search(const SearchParams &P, bool dense, bool ep_smem,
 // Merge `lists` sorted lists of `k` entries (ping-pong between a and b) into
 // one; returns the buffer that holds the result and the launches queued.
 // With `seed`, also seed *seed from the result as launch_seed_threshold.
+// Nothing is done where *done is nonzero.
 cudaError_t launch_topk_merge(Entry *a, Entry *b, int lists, int k,
                               Entry **result, int *levels, cudaStream_t st,
-                              unsigned long long *seed = nullptr);
+                              unsigned long long *seed = nullptr,
+                              const unsigned *done = nullptr);
 cudaError_t launch_fill(const FillParams &F, cudaStream_t st);
+// the records from the listed search's candidates, *F.done <- 1, unless
+// there is no list or there were more than kCandMax (F.sel is not read)
+cudaError_t launch_finish(const FillParams &F, cudaStream_t st);
 // gthr <- min(gthr, chi^2 bits of sel[k-1]) when that entry is real
 cudaError_t launch_seed_threshold(const Entry *sel, int k,
                                   unsigned long long *gthr, cudaStream_t st);

@@ -208,6 +208,7 @@ extern "C" morse_status morse_grid_chi2_noalloc(morse_ctx *ctx,
     F.t0abs = T.t0abs;
     F.tEv = T.tEv;
     F.out = fits;
+    F.done = nullptr;
     e = morse::launch_fill(F, ctx->stream);
   }
   if (e == cudaSuccess) {

@@ -819,17 +819,19 @@ struct Fit2 {
 __device__ __forceinline__ Fit2 fit2(const SearchParams &P, double SA,
                                      double SAA, double SAF) {
   Fit2 o;
+  // (every rounding written out: the kernels that solve the same sums must
+  // give the same bits, whatever the compiler contracts around them)
   const double S1 = P.S1, SF = P.SF;
-  const double SAAu = SAA + 2.0 * SA + S1;
-  const double det = SAA * S1 - SA * SA;
-  if (!(det > 1e-12 * SAAu * S1)) {
+  const double SAAu = __dadd_rn(__fma_rn(2.0, SA, SAA), S1);
+  const double det = __fma_rn(SAA, S1, -__dmul_rn(SA, SA));
+  if (!(det > __dmul_rn(__dmul_rn(1e-12, SAAu), S1))) {
     o.Fs = 0.0;
     o.Bc = SF / S1;
     o.degenerate = true;
   } else {
     const double inv = 1.0 / det;
-    o.Fs = (S1 * SAF - SA * SF) * inv;
-    o.Bc = (SAA * SF - SA * SAF) * inv;
+    o.Fs = __dmul_rn(__fma_rn(S1, SAF, -__dmul_rn(SA, SF)), inv);
+    o.Bc = __dmul_rn(__fma_rn(SAA, SF, -__dmul_rn(SA, SAF)), inv);
     o.degenerate = false;
   }
   return o;

@@ -357,6 +357,50 @@ __device__ __forceinline__ void band_release(BandTabs &B, long long r,
   if (lane == 0) atomicSub(&B.tw[(int)(r & 1)], 1u);
 }
 
+// The record of trajectory idx with its fit.
+__device__ __forceinline__ morse_fit fit_record(const SearchParams &P,
+                                                long long idx, double chi2,
+                                                double Fs, double Bc,
+                                                bool degenerate,
+                                                const double *t0abs,
+                                                const double *tEv) {
+  morse_fit r;
+  long long q = idx;
+  const int itE = (int)(q % P.n_tE);
+  q /= P.n_tE;
+  const int it0 = (int)(q % P.n_t0);
+  q /= P.n_t0;
+  const int ia = (int)(q % P.n_alpha);
+  const int iu = (int)(q / P.n_alpha);
+  r.chi2 = chi2;
+  r.tE = (P.lu && P.ltE) ? P.ltE[iu] : tEv[itE];
+  if (P.lu) {  // line grid: the record in the (u0, alpha) convention
+    r.t0 = t0abs[it0] - P.lsh[iu] * r.tE;
+    r.u0 = P.lu[iu];
+    r.alpha = P.la[iu];
+  } else {
+    r.t0 = t0abs[it0];
+    r.u0 = P.u0v[iu];
+    r.alpha = 2.0 * CUDART_PI * (double)ia / (double)P.n_alpha;
+  }
+  r.Fs = Fs;
+  r.Fb = Bc + P.Fref - Fs;
+  r.idx = idx;
+  r.flags = degenerate ? MORSE_FIT_DEGENERATE : 0;
+  r.reserved = 0;
+  return r;
+}
+// the record of an unused place of a top-K list
+__device__ __forceinline__ morse_fit empty_record() {
+  morse_fit r;
+  r.chi2 = CUDART_INF;
+  r.t0 = r.tE = r.u0 = r.alpha = r.Fs = r.Fb = 0.0;
+  r.idx = -1;
+  r.flags = 0;
+  r.reserved = 0;
+  return r;
+}
+
 // Record of one selected trajectory e (warp-collective; lane 0 writes *dst):
 // (Fs, Fb) from the phase-1 sums and the solve, recomputed with the search's
 // device functions on the epochs at ep_blk (a shared-memory copy) or P.ep,
@@ -368,49 +412,18 @@ __device__ __forceinline__ void fill_one(const SearchParams &P, const Entry e,
                                          const double *tEv, const int lane,
                                          morse_fit *dst,
                                          const float4 *ep_blk = nullptr) {
-  morse_fit r;
   const long long total = (long long)P.n_u0 * P.n_alpha * P.n_t0 * P.n_tE;
   if (e.idx < 0 || e.idx >= total) {
-    if (lane == 0) {
-      r.chi2 = CUDART_INF;
-      r.t0 = r.tE = r.u0 = r.alpha = r.Fs = r.Fb = 0.0;
-      r.idx = -1;
-      r.flags = 0;
-      r.reserved = 0;
-      *dst = r;
-    }
+    if (lane == 0) *dst = empty_record();
     return;
   }
   const Epochs ep = epochs_at(ep_blk ? ep_blk : P.ep, P.n_ep);
   const TrajC c = traj_consts(P, ep, e.idx);
   const Acc s = phase1<H>(P, ep, c, lane);
   const Solved sol = solve2(P, (double)s.a, (double)s.b, (double)s.d);
-  if (lane == 0) {
-    long long q = e.idx;
-    const int itE = (int)(q % P.n_tE);
-    q /= P.n_tE;
-    const int it0 = (int)(q % P.n_t0);
-    q /= P.n_t0;
-    const int ia = (int)(q % P.n_alpha);
-    const int iu = (int)(q / P.n_alpha);
-    r.chi2 = e.chi2;
-    r.tE = (P.lu && P.ltE) ? P.ltE[iu] : tEv[itE];
-    if (P.lu) {  // line grid: the record in the (u0, alpha) convention
-      r.t0 = t0abs[it0] - P.lsh[iu] * r.tE;
-      r.u0 = P.lu[iu];
-      r.alpha = P.la[iu];
-    } else {
-      r.t0 = t0abs[it0];
-      r.u0 = P.u0v[iu];
-      r.alpha = 2.0 * CUDART_PI * (double)ia / (double)P.n_alpha;
-    }
-    r.Fs = sol.Fs;
-    r.Fb = sol.Bc + P.Fref - sol.Fs;
-    r.idx = e.idx;
-    r.flags = sol.degenerate ? MORSE_FIT_DEGENERATE : 0;
-    r.reserved = 0;
-    *dst = r;
-  }
+  if (lane == 0)
+    *dst = fit_record(P, e.idx, e.chi2, sol.Fs, sol.Bc, sol.degenerate, t0abs,
+                      tEv);
 }
 
 }  // namespace dev
