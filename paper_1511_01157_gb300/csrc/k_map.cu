@@ -227,12 +227,171 @@ __device__ __forceinline__ void shoot_f32(const RayParams &P, uint32_t *win,
   }
 }
 
-// FP32: two blocks per SM (at most 64 registers: the packed sub-block loop
-// keeps its twelve column pairs in registers).
-template <bool FP64>
-__global__ void __launch_bounds__(kRayThreads, FP64 ? 1 : 2)
+// The FP64 deflection's counts at FP32 cost.  A ray's bin is its FP64
+// coordinate rounded down, and FP32 finds the same bin unless the coordinate
+// lies within FP32's error of a bin edge; those rays (about 1 in 500) are
+// queued and take deflect64, so the counts are the FP64 definition's.
+//
+// Error in bins, u = 2^-24.  A tile's columns and rows are made in FP64
+// (once per tile: an FP64 instruction holds the SM's FP64 pipe for some 16
+// cycles, and the plain form takes 70 of them per ray) and rounded once:
+// x' = (x + L)/Delta, d1, d2 and x2 carry u each.  Then r1, r2 carry 4 u,
+// their product 9 u, its approximate reciprocal 11 u, a_k = -e_k'/r_k 20 u,
+// a term T_k = a_k d_k 22 u; the two sums round at most S = |T1| + |T2| and
+// B + S, B = (X + L)/Delta the bound of x'.  So |v - v_exact| <= u (2 B + 24
+// S), and for the second coordinate the same with S = |a1 + a2| |x2| (a1 and
+// a2 have one sign), taken as 4 and 26; the FP64 form's own rounding is
+// 2^-29 of that.  Anything not provably inside a bin -- NaN and infinity on
+// a lens, |v| >= 2^22 where floor bits fail and the error exceeds 1/2 --
+// compares false and goes to deflect64.
+//
+// 4000^2 rays on 512^2 texels: 2.16 -> 0.048 ms.
+struct RayTile {
+  float x1s[kRayTileX], d1[kRayTileX], d2[kRayTileX];
+  float x2[kRayWarps * kRaySubRowsMax], x2s[kRayWarps * kRaySubRowsMax];
+  unsigned n_q;
+  unsigned q[kRayQueue];  // column | row << 16 of the rays for deflect64
+};
+
+__device__ __forceinline__ void ray_tile(const RayParams &P, RayTile &T,
+                                         long long i0, long long j0, int th,
+                                         int tid) {
+  const double iD = 1.0 / P.dlt;
+  if (tid < kRayTileX) {
+    const double x1 = __dadd_rn(
+        -P.X, __dmul_rn(__dadd_rn((double)(i0 + tid), 0.5), P.h));
+    T.x1s[tid] = __double2float_rn((x1 + P.L) * iD);
+    T.d1[tid] = __double2float_rn(x1 - P.xa);
+    T.d2[tid] = __double2float_rn(x1 - P.xb);
+  } else if (tid - kRayTileX < th) {
+    const int b = tid - kRayTileX;
+    const double x2 = __dadd_rn(
+        -P.X, __dmul_rn(__dadd_rn((double)(j0 + b), 0.5), P.h));
+    T.x2[b] = __double2float_rn(x2);
+    T.x2s[b] = __double2float_rn((x2 + P.L) * iD);
+  }
+  if (tid == 0) T.n_q = 0;
+}
+
+// Bins one ray by the FP64 deflection; returns deflect64's status.  (Not
+// inlined: its registers would cost the FP32 loop its second block per SM.)
+__device__ __noinline__ int bin64(const RayParams &P, uint32_t *win, int wx0,
+                                  int wy0, long long i, long long j) {
+  const double x2 =
+      __dadd_rn(-P.X, __dmul_rn(__dadd_rn((double)j, 0.5), P.h));
+  int ix = 0, iy = 0;
+  const int st = deflect64(P, i, x2, __dmul_rn(x2, x2), &ix, &iy);
+  if (st == 0) {
+    const unsigned lx = (unsigned)(ix - wx0), ly = (unsigned)(iy - wy0);
+    if (lx < (unsigned)kRayWin && ly < (unsigned)kRayWin)
+      atomicAdd(&win[ly * kRayWin + lx], 1u);
+    else
+      atomicAdd(&P.counts[(size_t)iy * P.npix + ix], 1u);
+  }
+  return st;
+}
+
+template <bool FULL>
+__device__ __forceinline__ void shoot_f64(const RayParams &P, uint32_t *win,
+                                          RayTile &T, int wx0, int wy0,
+                                          long long i0, long long j0, int c0,
+                                          int b0, int na, int nb,
+                                          unsigned &n_off, unsigned &n_lost) {
+  constexpr int NP = kSubX / 2;
+  float2 x1s[NP], d1[NP], d2[NP];
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {
+    x1s[p] = *reinterpret_cast<const float2 *>(&T.x1s[c0 + 2 * p]);
+    d1[p] = *reinterpret_cast<const float2 *>(&T.d1[c0 + 2 * p]);
+    d2[p] = *reinterpret_cast<const float2 *>(&T.d2[c0 + 2 * p]);
+  }
+  const float2 ne1 = f2r(-P.e1f * P.invdf), ne2 = f2r(-P.e2f * P.invdf);
+  const float2 M = f2r(12582912.f), E0 = f2r(P.err0);
+  const unsigned W = (unsigned)min(kRayWin, P.npix);
+  const unsigned cx = 0x4B400000u + (unsigned)wx0;
+  const unsigned cy = 0x4B400000u + (unsigned)wy0;
+#pragma unroll 1
+  for (int b = 0; b < nb; ++b) {
+    const float x2 = T.x2[b0 + b];
+    const float2 x2p = f2r(x2), x2sq = f2r(x2 * x2);
+    const float2 x2s = f2r(T.x2s[b0 + b]);
+    const float2 k2 = f2r(-kRayErr * fabsf(x2));
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      if (!FULL && 2 * p >= na) break;
+      const float2 r1 = __ffma2_rn(d1[p], d1[p], x2sq);
+      const float2 r2 = __ffma2_rn(d2[p], d2[p], x2sq);
+      const float2 rr = __fmul2_rn(r1, r2);
+      const float2 inv = make_float2(rcp_approx(rr.x), rcp_approx(rr.y));
+      const float2 a1 = __fmul2_rn(ne1, __fmul2_rn(r2, inv));  // -e1' / r1
+      const float2 a2 = __fmul2_rn(ne2, __fmul2_rn(r1, inv));  // -e2' / r2
+      const float2 a12 = __fadd2_rn(a1, a2);
+      const float2 t1 = __fmul2_rn(a1, d1[p]), t2 = __fmul2_rn(a2, d2[p]);
+      const float2 v1 = __fadd2_rn(__fadd2_rn(t1, t2), x1s[p]);
+      const float2 v2 = __ffma2_rn(a12, x2p, x2s);
+      const float2 tx = __fadd2_rd(v1, M);
+      const float2 ty = __fadd2_rd(v2, M);
+      // distances of the fractions from 1/2, and the error bounds
+      const float2 h = f2r(-0.5f);
+      const float2 g1 = __fadd2_rn(
+          h, __ffma2_rn(__fadd2_rn(tx, f2r(-12582912.f)), f2r(-1.f), v1));
+      const float2 g2 = __fadd2_rn(
+          h, __ffma2_rn(__fadd2_rn(ty, f2r(-12582912.f)), f2r(-1.f), v2));
+      const float2 q1 =
+          __ffma2_rn(make_float2(fabsf(t1.x) + fabsf(t2.x),
+                                 fabsf(t1.y) + fabsf(t2.y)),
+                     f2r(kRayErr), E0);
+      const float2 q2 = __ffma2_rn(a12, k2, E0);
+      const bool s0 = fabsf(g1.x) + q1.x < 0.5f && fabsf(g2.x) + q2.x < 0.5f;
+      const bool s1 = fabsf(g1.y) + q1.y < 0.5f && fabsf(g2.y) + q2.y < 0.5f;
+      const bool two = FULL || 2 * p + 1 < na;
+      if (s0 && s1 && two) {
+        // as shoot_f32: a ray known to a bin is not lost
+        const unsigned lx0 = (unsigned)__float_as_int(tx.x) - cx;
+        const unsigned ly0 = (unsigned)__float_as_int(ty.x) - cy;
+        const unsigned lx1 = (unsigned)__float_as_int(tx.y) - cx;
+        const unsigned ly1 = (unsigned)__float_as_int(ty.y) - cy;
+        if (max(max(lx0, ly0), max(lx1, ly1)) < W) {
+          atomicAdd(&win[ly0 * kRayWin + lx0], 1u);
+          atomicAdd(&win[ly1 * kRayWin + lx1], 1u);
+          continue;
+        }
+        bin_ray(P, win, cx, cy, W, tx.x, ty.x, false, n_off, n_lost);
+        bin_ray(P, win, cx, cy, W, tx.y, ty.y, false, n_off, n_lost);
+        continue;
+      }
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        if (k == 1 && !two) break;
+        if (k ? s1 : s0) {
+          bin_ray(P, win, cx, cy, W, k ? tx.y : tx.x, k ? ty.y : ty.x, false,
+                  n_off, n_lost);
+        } else {
+          const unsigned at = atomicAdd(&T.n_q, 1u);
+          const unsigned c = (unsigned)(c0 + 2 * p + k);
+          const unsigned r = (unsigned)(b0 + b);
+          if (at < (unsigned)kRayQueue)
+            T.q[at] = c | r << 16;
+          else {
+            const int st = bin64(P, win, wx0, wy0, i0 + c, j0 + r);
+            n_off += st == 1;
+            n_lost += st == 2;
+          }
+        }
+      }
+    }
+  }
+}
+
+// Two blocks per SM (at most 64 registers: the packed sub-block loop keeps
+// its twelve column pairs in registers); the plain FP64 form one.
+// MODE: kRayF32, kRayF64 (every ray by deflect64) or kRayF64Filtered.
+template <int MODE>
+__global__ void __launch_bounds__(kRayThreads, MODE == kRayF64 ? 1 : 2)
     k_rayshoot(const RayParams P) {
   extern __shared__ __align__(16) uint32_t win[];  // kRayWin^2 bins
+  constexpr bool FP64 = MODE == kRayF64;
+  RayTile &T = *reinterpret_cast<RayTile *>(win + kRayWin * kRayWin);
   __shared__ int s_wx, s_wy, s_tile;
   const int tid = threadIdx.x;
   uint4 *win4 = reinterpret_cast<uint4 *>(win);
@@ -281,6 +440,7 @@ __global__ void __launch_bounds__(kRayThreads, FP64 ? 1 : 2)
         s_wy = min(max(wy, 0), wmax);
       }
     }
+    if (MODE == kRayF64Filtered) ray_tile(P, T, i0, j0, (int)tile_h, tid);
     __syncthreads();
     const int wx0 = s_wx, wy0 = s_wy;
     const long long ib = i0 + sx * kSubX;
@@ -288,7 +448,25 @@ __global__ void __launch_bounds__(kRayThreads, FP64 ? 1 : 2)
     // rays of the sub-block row inside the grid, and the first one's x1
     const int na = (int)max(0LL, min((long long)kSubX, P.nray - ib));
     const float x1b = fmaf((float)ib, P.hf, P.x0f);
-    if (!FP64) {
+    if (MODE == kRayF64Filtered) {
+      const int b0 = sy * P.sub_rows;
+      const int nb =
+          (int)max(0LL, min((long long)P.sub_rows, P.nray - jb));
+      if (na == kSubX)
+        shoot_f64<true>(P, win, T, wx0, wy0, i0, j0, sx * kSubX, b0, na, nb,
+                        n_off, n_lost);
+      else if (na > 0)
+        shoot_f64<false>(P, win, T, wx0, wy0, i0, j0, sx * kSubX, b0, na, nb,
+                         n_off, n_lost);
+      __syncthreads();
+      const int nq = (int)min(T.n_q, (unsigned)kRayQueue);
+      for (int k = tid; k < nq; k += kRayThreads) {
+        const int st = bin64(P, win, wx0, wy0, i0 + (T.q[k] & 0xFFFFu),
+                             j0 + (T.q[k] >> 16));
+        n_off += st == 1;
+        n_lost += st == 2;
+      }
+    } else if (!FP64) {
       if (na == kSubX)
         shoot_f32<true>(P, win, wx0, wy0, jb, na, x1b, n_off, n_lost);
       else if (na > 0)
@@ -296,27 +474,11 @@ __global__ void __launch_bounds__(kRayThreads, FP64 ? 1 : 2)
     } else {
 #pragma unroll 1
       for (int b = 0; b < P.sub_rows; ++b) {
-        const long long j = jb + b;
-        if (j >= P.nray) break;
-        const double x2d = __dadd_rn(-P.X, __dmul_rn(__dadd_rn((double)j, 0.5), P.h));
-        const double x2sqd = __dmul_rn(x2d, x2d);
-#pragma unroll
-        for (int a = 0; a < kSubX; ++a) {
-          if (a < na) {
-            int ix = 0, iy = 0;
-            const int st = deflect64(P, ib + a, x2d, x2sqd, &ix, &iy);
-            if (st == 0) {
-              unsigned lx = (unsigned)(ix - wx0), ly = (unsigned)(iy - wy0);
-              if (lx < (unsigned)kRayWin && ly < (unsigned)kRayWin)
-                atomicAdd(&win[ly * kRayWin + lx], 1u);
-              else
-                atomicAdd(&P.counts[(size_t)iy * P.npix + ix], 1u);
-            } else if (st == 1) {
-              ++n_off;
-            } else {
-              ++n_lost;
-            }
-          }
+        if (jb + b >= P.nray) break;
+        for (int a = 0; a < na; ++a) {
+          const int st = bin64(P, win, wx0, wy0, ib + a, jb + b);
+          n_off += st == 1;
+          n_lost += st == 2;
         }
       }
     }
@@ -372,24 +534,42 @@ __device__ __forceinline__ float4 quad_of(float a00, float a10, float a01,
   return make_float4(m00, d0, __fsub_rn(m01, m00), __fsub_rn(d1, d0));
 }
 
-// counts -> A, one FP64 product per texel (the cells are then built from A
-// by k_quads_from_A: one product per texel instead of four per cell, the
-// FP64 pipe being the limiter of a fused form)
+// counts -> A: RN32 of the FP64 product n f.  With f = fh + fl in FP32 and n
+// below 2^24 the product is p + low, p = RN(n fh), low = (n fh - p) + n fl;
+// where p + low rounds to the same FP32 value for low - e and low + e, e
+// above every error left (2^-44 p), that value is the product's, else
+// the FP64 product is taken.  (Three FP64-pipe instructions per texel
+// bounded the kernel: 4096^2 texels 94 -> 34 us, their 134 MB take 20.)
+__device__ __forceinline__ float texel_of(uint32_t n, double f, float fh,
+                                          float fl) {
+  if (n < (1u << 24)) {
+    const float nf = (float)n;
+    const float p = __fmul_rn(nf, fh);
+    const float low = __fmaf_rn(nf, fl, __fmaf_rn(nf, fh, -p));
+    const float e = p * 5.684341886080802e-14f;
+    const float a = __fadd_rn(p, __fsub_rn(low, e));
+    if (a == __fadd_rn(p, __fadd_rn(low, e)) && (p > 1e-20f || n == 0))
+      return a;
+  }
+  return __double2float_rn(__dmul_rn((double)n, f));
+}
+
+// (the cells are then built from A by k_quads_from_A: one product per texel
+// instead of four per cell)
 __global__ void k_counts_to_A(const uint32_t *__restrict__ counts, int npix,
-                              double f, float *__restrict__ A) {
+                              double f, float fh, float fl,
+                              float *__restrict__ A) {
   const size_t n = (size_t)npix * npix;
   for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n;
        k += (size_t)gridDim.x * blockDim.x)
-    A[k] = __double2float_rn(__dmul_rn((double)counts[k], f));
+    A[k] = texel_of(counts[k], f, fh, fl);
 }
 
 __global__ void k_quads_from_A(const float *__restrict__ A, int npix,
                                float4 *__restrict__ quad, int qpitch) {
-  const int side = npix + 1;
-  const size_t n = (size_t)side * side;
-  for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n;
-       k += (size_t)gridDim.x * blockDim.x) {
-    const int c = (int)(k % side), r = (int)(k / side);
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c > npix) return;
+  for (int r = blockIdx.y; r <= npix; r += gridDim.y) {
     const int x0 = clampi(c - 1, npix), x1 = clampi(c, npix);
     const int y0 = clampi(r - 1, npix), y1 = clampi(r, npix);
     quad[cell_index(c, r, qpitch)] = quad_of(
@@ -399,28 +579,42 @@ __global__ void k_quads_from_A(const float *__restrict__ A, int npix,
 }
 
 // FP16 storage code of one FP32 value: log10 in FP64, rounded once to
-// binary16 (round to nearest even)
-__device__ __forceinline__ uint16_t half_code(float a, double a_floor) {
-  const double v = (double)a;
-  return __half_as_ushort(__double2half(log10(v > a_floor ? v : a_floor)));
+// binary16 (round to nearest even).  log10f is within 2 ulp (CUDA's stated
+// bound, 2^-22 of its value); where the values 2^-21 below and above it round
+// to one code, that is the FP64 logarithm's code too (rounding is monotone),
+// else (about 1 texel in 500) the FP64 logarithm is taken.  The FP64 form
+// of every texel took 1.06 ms for 4096^2 texels, this 0.046.
+__device__ __forceinline__ uint16_t half_code64(double v) {
+  return __half_as_ushort(__double2half(log10(v)));
+}
+__device__ __forceinline__ uint16_t half_code(float a, double a_floor,
+                                              float floor_rd) {
+  // a > a_floor: an FP32 value exceeds it iff it exceeds it rounded down
+  if (!(a > floor_rd)) return half_code64(a_floor);
+  const float y = log10f(a);
+  const float e = fabsf(y) * 4.76837158203125e-7f;
+  const unsigned short lo = __half_as_ushort(__float2half_rn(y - e));
+  const unsigned short hi = __half_as_ushort(__float2half_rn(y + e));
+  // (|y| below 1e-4: close to 1, or subnormal codes)
+  if (lo == hi && fabsf(y) > 1e-4f) return lo;
+  return half_code64((double)a);
 }
 
 __global__ void k_half_codes(const float *__restrict__ A, size_t n,
                              double a_floor, uint16_t *__restrict__ codes) {
+  const float fl = __double2float_rd(a_floor);
   for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n;
        k += (size_t)gridDim.x * blockDim.x)
-    codes[k] = half_code(A[k], a_floor);
+    codes[k] = half_code(A[k], a_floor, fl);
 }
 
 // (x00, x10) in .x and (x01, x11) in .y, low half first; same cells and
 // edge repetition as the FP32 quads, codes undifferenced
 __global__ void k_half_quads(const uint16_t *__restrict__ codes, int npix,
                              uint2 *__restrict__ quadh, int qpitch) {
-  const int side = npix + 1;
-  const size_t n = (size_t)side * side;
-  for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n;
-       k += (size_t)gridDim.x * blockDim.x) {
-    const int c = (int)(k % side), r = (int)(k / side);
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c > npix) return;
+  for (int r = blockIdx.y; r <= npix; r += gridDim.y) {
     const int x0 = clampi(c - 1, npix), x1 = clampi(c, npix);
     const int y0 = clampi(r - 1, npix), y1 = clampi(r, npix);
     const unsigned c00 = codes[(size_t)y0 * npix + x0];
@@ -434,38 +628,49 @@ __global__ void k_half_quads(const uint16_t *__restrict__ codes, int npix,
 
 }  // namespace
 
-static size_t ray_smem() { return sizeof(uint32_t) * kRayWin * kRayWin; }
+static size_t ray_smem(int mode) {
+  return sizeof(uint32_t) * kRayWin * kRayWin +
+         (mode == kRayF64Filtered ? sizeof(RayTile) : 0);
+}
 
-int rayshoot_blocks_per_sm() {
+template <int MODE>
+static int ray_occupancy() {
   static int cached = -1;
   if (cached > 0) return cached;
-  cudaFuncSetAttribute(k_rayshoot<true>,
+  cudaFuncSetAttribute(k_rayshoot<MODE>,
                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)ray_smem());
-  cudaFuncSetAttribute(k_rayshoot<false>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)ray_smem());
+                       (int)ray_smem(MODE));
   int b = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-          &b, k_rayshoot<false>, kRayThreads, ray_smem()) != cudaSuccess ||
+          &b, k_rayshoot<MODE>, kRayThreads, ray_smem(MODE)) != cudaSuccess ||
       b < 1)
     b = 1;
   cached = b;
   return b;
 }
 
-cudaError_t launch_rayshoot(const RayParams &P, bool fp64, int grid,
+int rayshoot_blocks_per_sm(int mode) {
+  return mode == kRayF32   ? ray_occupancy<kRayF32>()
+         : mode == kRayF64 ? ray_occupancy<kRayF64>()
+                           : ray_occupancy<kRayF64Filtered>();
+}
+
+cudaError_t launch_rayshoot(const RayParams &P, int mode, int grid,
                             cudaStream_t st) {
-  rayshoot_blocks_per_sm();  // sets the shared-memory attribute once
-  if (fp64)
-    k_rayshoot<true><<<grid, kRayThreads, ray_smem(), st>>>(P);
+  rayshoot_blocks_per_sm(mode);  // sets the shared-memory attribute once
+  const size_t sm = ray_smem(mode);
+  if (mode == kRayF32)
+    k_rayshoot<kRayF32><<<grid, kRayThreads, sm, st>>>(P);
+  else if (mode == kRayF64)
+    k_rayshoot<kRayF64><<<grid, kRayThreads, sm, st>>>(P);
   else
-    k_rayshoot<false><<<grid, kRayThreads, ray_smem(), st>>>(P);
+    k_rayshoot<kRayF64Filtered><<<grid, kRayThreads, sm, st>>>(P);
   return cudaGetLastError();
 }
 
-static size_t quad_cells(int npix) {
-  return (size_t)(npix + 1) * (size_t)(npix + 1);
+// a block column per 256 cells of a row (no division of a flat index)
+static dim3 cells_grid(int npix) {
+  return dim3((unsigned)(npix / 256 + 1), (unsigned)(npix + 1));
 }
 
 static int elementwise_grid(size_t n) {
@@ -478,18 +683,19 @@ static int elementwise_grid(size_t n) {
 cudaError_t launch_counts_to_map(const uint32_t *counts, int npix, double f,
                                  float *A, float4 *quad, int qpitch,
                                  cudaStream_t st) {
+  const float fh = (float)f, fl = (float)(f - (double)fh);
   k_counts_to_A<<<elementwise_grid((size_t)npix * npix), 256, 0, st>>>(
-      counts, npix, f, A);
+      counts, npix, f, fh, fl, A);
   cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_quads_from_A<<<elementwise_grid(quad_cells(npix)), 256, 0, st>>>(
+  if (e != cudaSuccess || !quad) return e;
+  k_quads_from_A<<<cells_grid(npix), 256, 0, st>>>(
       A, npix, quad, qpitch);
   return cudaGetLastError();
 }
 
 cudaError_t launch_quads_from_A(const float *A, int npix, float4 *quad,
                                 int qpitch, cudaStream_t st) {
-  k_quads_from_A<<<elementwise_grid(quad_cells(npix)), 256, 0, st>>>(
+  k_quads_from_A<<<cells_grid(npix), 256, 0, st>>>(
       A, npix, quad, qpitch);
   return cudaGetLastError();
 }
@@ -501,7 +707,7 @@ cudaError_t launch_half_from_A(const float *A, int npix, double a_floor,
   k_half_codes<<<elementwise_grid(n), 256, 0, st>>>(A, n, a_floor, codes);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_half_quads<<<elementwise_grid(quad_cells(npix)), 256, 0, st>>>(
+  k_half_quads<<<cells_grid(npix), 256, 0, st>>>(
       codes, npix, quadh, qpitch);
   return cudaGetLastError();
 }

@@ -163,6 +163,8 @@ struct BuildSpec {
   bool fp64;
   bool fp16;  // also write the FP16 log10 table and search through it
   bool poly;  // the lens polynomial per texel instead of ray shooting
+  bool half_only;  // a sweep's map searched through its FP16 table: the
+                   // FP32 cells (16 bytes per texel) are not read, not made
 };
 
 morse_status check_build(morse_ctx *ctx, double s, double q, double extent,
@@ -203,6 +205,7 @@ morse_status check_build(morse_ctx *ctx, double s, double q, double extent,
   b->npix = npix;
   b->nray = rays_per_axis;
   b->fp64 = deflect == MORSE_DEFLECT_FP64;
+  b->half_only = false;
   return MORSE_OK;
 }
 
@@ -339,8 +342,20 @@ morse_status enqueue_build(morse_ctx *ctx, morse_map *m, const BuildSpec &b) {
   // last round with few tiles leaves SMs idle, so pick the sub-block rows r
   // (tile height 16 r) that minimise rounds x (tile rays + a per-tile cost
   // of about 2000 rays: window placement, flush, barriers).
+  // FP64 counts by FP32 rays while the bound of their error holds: squared
+  // distances whose product stays inside FP32's range (1e30), and an error
+  // far below a bin (0.02 of one from the coordinates alone)
+  int mode = b.fp64 ? morse::kRayF64 : morse::kRayF32;
+  if (b.fp64) {
+    const double far = b.X + std::fabs(P.xa) + std::fabs(P.xb);
+    const double e0 = 4.0 * ldexp(1.0, -24) * (b.X + b.L) / P.dlt;
+    if (far < 2e7 && e0 < 0.02 && P.dlt > 1e-12 && P.dlt < 1e12) {
+      mode = morse::kRayF64Filtered;
+      P.err0 = nextafterf((float)e0, 1.0f);
+    }
+  }
   const long long blocks =
-      (long long)morse::rayshoot_blocks_per_sm() * ctx->sm_count;
+      (long long)morse::rayshoot_blocks_per_sm(mode) * ctx->sm_count;
   {
     double best = 0.0;
     P.sub_rows = morse::kRaySubRowsMax;
@@ -370,14 +385,15 @@ morse_status enqueue_build(morse_ctx *ctx, morse_map *m, const BuildSpec &b) {
   long long tiles = (long long)P.tiles_x * P.tiles_y;
   int grid = (int)std::min<long long>(tiles, blocks);
   int r = t_begin(ctx, KT_RAY);
-  MORSE_CUDA(ctx, morse::launch_rayshoot(P, b.fp64, grid, ctx->stream));
+  MORSE_CUDA(ctx, morse::launch_rayshoot(P, mode, grid, ctx->stream));
   t_end(ctx, r);
   ctx->launches += 1;
   const double f = (P.h * P.h) / (P.dlt * P.dlt);
   r = t_begin(ctx, KT_MAP);
-  MORSE_CUDA(ctx, morse::launch_counts_to_map(m->counts, b.npix, f, m->A,
-                                              m->quad, m->qpitch,
-                                              ctx->stream));
+  MORSE_CUDA(ctx, morse::launch_counts_to_map(
+                      m->counts, b.npix, f, m->A,
+                      b.half_only ? nullptr : m->quad, m->qpitch,
+                      ctx->stream));
   // FP16 floor: half a ray, 0.5 h^2 / Delta^2
   m->a_floor = 0.5 * f;
   m->half_valid = false;
@@ -387,7 +403,7 @@ morse_status enqueue_build(morse_ctx *ctx, morse_map *m, const BuildSpec &b) {
     m->lookup = MORSE_STORE_FP16LOG;
   }
   t_end(ctx, r);
-  ctx->launches += 2;  // counts -> A, A -> cells
+  ctx->launches += b.half_only ? 1 : 2;  // counts -> A, A -> cells
   return MORSE_OK;
 }
 
@@ -968,6 +984,7 @@ morse_status sweep_impl(morse_ctx *ctx, const morse_event *ev,
     mb->L = extent;
   }
   const bool h16 = n_maps > 0 && specs[0].fp16;
+  for (BuildSpec &b : specs) b.half_only = h16;
   for (int b = 0; b < (two ? 2 : 1); ++b)
     if (h16 && !map_ensure_half(*bufs[b]))
       return fail(ctx, MORSE_ENOMEM, "FP16 table of %d^2 texels", npix);

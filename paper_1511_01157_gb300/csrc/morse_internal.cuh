@@ -115,6 +115,7 @@ struct RayParams {
   float x0f, hf;            // first ray centre, ray spacing
   float invdf, offf;        // v = y / Delta + L / Delta
   float npixf;
+  float err0;               // kRayF64Filtered: 4 u (X + L)/Delta, rounded up
   int npix;
   int64_t nray;
   int tiles_x, tiles_y;
@@ -133,7 +134,12 @@ constexpr int kRaySubRowsMax = 16;  // tile height at most 256 rays (512:
 constexpr int kRayWin = 128;      // shared-memory window side (bins)
 constexpr int kRayThreads = 512;  // threads per ray-shooting block
 
-cudaError_t launch_rayshoot(const RayParams &P, bool fp64, int grid,
+// Ray-shooting forms: FP32; FP64, every ray; FP64 counts by FP32 rays, the
+// FP64 deflection only for those near a bin edge (k_map.cu)
+enum { kRayF32 = 0, kRayF64 = 1, kRayF64Filtered = 2 };
+constexpr int kRayQueue = 4096;  // rays per tile queued for deflect64
+constexpr float kRayErr = 26.f / 16777216.f;  // 26 u
+cudaError_t launch_rayshoot(const RayParams &P, int mode, int grid,
                             cudaStream_t st);
 // Cell tables: (npix + 1)^2 bilinear cells, stored either row-major with a
 // row pitch of quad_pitch cells (MORSE_TILE_W = 1), or in tiles of
@@ -189,6 +195,7 @@ inline unsigned quad_idx0(int npix) {
          (unsigned)(quad_pitch(npix) + 1);
 }
 
+// (quad null: the texels alone)
 cudaError_t launch_counts_to_map(const uint32_t *counts, int npix, double f,
                                  float *A, float4 *quad, int qpitch,
                                  cudaStream_t st);
@@ -198,7 +205,7 @@ cudaError_t launch_quads_from_A(const float *A, int npix, float4 *quad,
 cudaError_t launch_half_from_A(const float *A, int npix, double a_floor,
                                uint16_t *codes, uint2 *quadh, int qpitch,
                                cudaStream_t st);
-int rayshoot_blocks_per_sm();
+int rayshoot_blocks_per_sm(int mode);
 // finite-source map: A convolved with the (2R+1)^2 weights W (rows dy),
 // rowhw[dy + R] = largest |dx| of a nonzero weight in row dy (-1: none)
 size_t fs_smem_bytes(int R);
