@@ -52,7 +52,7 @@ using namespace dev;
 constexpr int kScreenThreads = 256;
 constexpr int kScreenTile = 2 * kScreenThreads;  // trajectories per block step
 // epochs of the subsets summed by one lane, at most
-constexpr int kScreenMax0 = 128, kScreenMax1 = 192, kScreenMax2 = 512;
+constexpr int kScreenMax0 = 128, kScreenMax1 = 192, kScreenMax2 = 1024;
 
 // Order of the trajectories in a screen.  The grid index runs over tE
 // fastest; here the position in a line runs over t0 fastest, so that the
@@ -274,8 +274,8 @@ __device__ __forceinline__ void stage_subset(const ScreenLv &V,
 
 // Codes of all trajectories, on the smallest subset.
 template <bool H>
-__global__ void __launch_bounds__(kScreenThreads)
-    k_screen(const SearchParams P, const ScreenBufs B) {
+__device__ __forceinline__ void screen_all(const SearchParams &P,
+                                           const ScreenBufs &B) {
   __shared__ float4 s_ep[kScreenMax0];
   __shared__ unsigned s_hist[kScreenBins];
   __shared__ Row s_row[kRowMax];
@@ -402,8 +402,8 @@ __device__ __forceinline__ void append(const SearchParams &P,
 // want-th lowest code, and a hashed sample of that bin's (codes are equal
 // there as far as the histogram tells: all of them, where the bounds say
 // nothing).
-__global__ void __launch_bounds__(kListThreads)
-    k_pilot_list(const SearchParams P, const ScreenBufs B) {
+__device__ __forceinline__ void make_pilot_list(const SearchParams &P,
+                                                const ScreenBufs &B) {
   __shared__ unsigned s_w[32], s_cut, s_r;
   static_assert(kScreenBins == kListThreads, "a bin per thread");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -439,13 +439,12 @@ __global__ void __launch_bounds__(kListThreads)
 // Upper bounds of the pilot's chi^2 over the whole light curve (chi2_upper).
 // A block takes kPilotTpg entries, its warps a slice of the epochs each (a
 // few thousand entries would leave most of the chip waiting for the walk of
-// one warp), and one warp adds the slices and solves.  P.gamma allows for
-// the slices (launch_screen_pilot).
+// one warp), and one warp adds the slices and solves.
 constexpr int kPilotTpg = 8, kPilotWarps = 8;
 
 template <bool H>
-__global__ void __launch_bounds__(kPilotWarps * 32)
-    k_pilot(const SearchParams P, const ScreenBufs B) {
+__device__ __forceinline__ void pilot_bounds(const SearchParams &P,
+                                             const ScreenBufs &B) {
   __shared__ Acc s_acc[kPilotWarps][kPilotTpg];
   __shared__ TrajC s_c[kPilotTpg];
   const unsigned n = min(B.n[0], B.pilot_cap);
@@ -489,18 +488,23 @@ __global__ void __launch_bounds__(kPilotWarps * 32)
       ms.d += s_acc[w][lane].d;
     }
   const Fit2 f = fit2(P, (double)ms.a, (double)ms.b, (double)ms.d);
+  // the relative error of the slices' sums, as event_params bounds a whole
+  // one's: the terms of a lane, the butterfly and the slices
+  const float terms =
+      (float)(P.n_ep / kPilotWarps / 32 + 2 + 10 + kPilotWarps);
+  const double gamma = fmax(P.gamma, (double)(terms * 5.9604645e-8f));
   const double ub =
       chi2_upper(P, (double)ms.a, (double)ms.b, (double)ms.d,
                  (double)__double2float_rn(f.Fs),
-                 (double)__double2float_rn(f.Bc));
+                 (double)__double2float_rn(f.Bc), gamma);
   if (lane < nv) B.ub[g0 + lane] = fmaxf(__double2float_ru(ub), 0.f);
 }
 
 // The threshold: the top_k-th smallest of the pilot's bounds (K distinct
 // trajectories have chi^2 at or below it), by four passes of eight bits
 // over the FP32 bit patterns, every block for itself; then the list.
-__global__ void __launch_bounds__(kListThreads)
-    k_list(const SearchParams P, const ScreenBufs B) {
+__device__ __forceinline__ void make_list(const SearchParams &P,
+                                          const ScreenBufs &B) {
   __shared__ unsigned s_h[256], s_bits, s_left;
   const unsigned n = min(B.n[0], B.pilot_cap);
   const unsigned K = (unsigned)P.top_k;
@@ -563,8 +567,9 @@ __global__ void __launch_bounds__(kListThreads)
 // two discard less than one in eight of those decided so far (from 16 384
 // on), the screen gives up and the whole range is searched.
 template <bool H>
-__global__ void __launch_bounds__(kScreenThreads, 4)
-    k_rescreen(const SearchParams P, const ScreenBufs B) {
+__device__ __forceinline__ void rescreen_listed(const SearchParams &P,
+                                                const ScreenBufs &B) {
+  if (P.n_lv < 3) return;  // (of a batch: the list is final)
   __shared__ float4 s_e1[kScreenMax1], s_e2[kScreenMax2];
   __shared__ unsigned s_queue[2 * kScreenTile];
   __shared__ unsigned s_m[kScreenThreads / 16], s_base, s_stop;
@@ -646,6 +651,36 @@ __global__ void __launch_bounds__(kScreenThreads, 4)
   }
 }
 
+// The kernels: one search, its parameters by value, or a batch of them
+// (blockIdx.y), each block with its search's parameters in shared memory.
+__device__ __forceinline__ void load_task(const ScreenTask *t, ScreenTask &s) {
+  const uint4 *src = reinterpret_cast<const uint4 *>(t);
+  uint4 *dst = reinterpret_cast<uint4 *>(&s);
+  for (int i = threadIdx.x; i < (int)(sizeof(ScreenTask) / 16);
+       i += blockDim.x)
+    dst[i] = __ldg(src + i);
+  __syncthreads();
+}
+#define MORSE_SCREEN_KERNELS(NAME, BODY, THREADS, MIN)                       \
+  template <bool H>                                                          \
+  __global__ void __launch_bounds__(THREADS, MIN)                            \
+      NAME(const SearchParams P, const ScreenBufs B) {                       \
+    BODY(P, B);                                                              \
+  }                                                                          \
+  template <bool H>                                                          \
+  __global__ void __launch_bounds__(THREADS, MIN)                            \
+      NAME##_batch(const ScreenTask *t) {                                    \
+    __shared__ ScreenTask s;                                                 \
+    load_task(t + blockIdx.y, s);                                            \
+    BODY(s.F.S, s.B);                                                        \
+  }
+MORSE_SCREEN_KERNELS(k_screen, screen_all<H>, kScreenThreads, 4)
+MORSE_SCREEN_KERNELS(k_pilot_list, make_pilot_list, kListThreads, 1)
+MORSE_SCREEN_KERNELS(k_pilot, pilot_bounds<H>, kPilotWarps * 32, 4)
+MORSE_SCREEN_KERNELS(k_list, make_list, kListThreads, 1)
+MORSE_SCREEN_KERNELS(k_rescreen, rescreen_listed<H>, kScreenThreads, 4)
+#undef MORSE_SCREEN_KERNELS
+
 }  // namespace
 
 cudaError_t launch_screen(const SearchParams &P, const ScreenBufs &B,
@@ -668,27 +703,23 @@ static int append_grid(const SearchParams &P, int sm_count) {
 cudaError_t launch_screen_pilot_list(const SearchParams &P,
                                      const ScreenBufs &B, int sm_count,
                                      cudaStream_t st) {
-  k_pilot_list<<<append_grid(P, sm_count), kListThreads, 0, st>>>(P, B);
+  k_pilot_list<false><<<append_grid(P, sm_count), kListThreads, 0, st>>>(P, B);
   return cudaGetLastError();
 }
 
 cudaError_t launch_screen_pilot(const SearchParams &P, const ScreenBufs &B,
                                 cudaStream_t st) {
-  SearchParams Q = P;
-  // the slices' sums, as event_params bounds a whole one's
-  const double m = (double)((P.n_ep / kPilotWarps + 32) / 32);
-  Q.gamma = std::max(P.gamma, (m + 10.0 + kPilotWarps) * ldexp(1.0, -24));
   const int grid = (int)((B.pilot_cap + kPilotTpg - 1) / kPilotTpg);
   if (P.quadh)
-    k_pilot<true><<<grid, kPilotWarps * 32, 0, st>>>(Q, B);
+    k_pilot<true><<<grid, kPilotWarps * 32, 0, st>>>(P, B);
   else
-    k_pilot<false><<<grid, kPilotWarps * 32, 0, st>>>(Q, B);
+    k_pilot<false><<<grid, kPilotWarps * 32, 0, st>>>(P, B);
   return cudaGetLastError();
 }
 
 cudaError_t launch_screen_list(const SearchParams &P, const ScreenBufs &B,
                                int sm_count, cudaStream_t st) {
-  k_list<<<append_grid(P, sm_count), kListThreads, 0, st>>>(P, B);
+  k_list<false><<<append_grid(P, sm_count), kListThreads, 0, st>>>(P, B);
   return cudaGetLastError();
 }
 
@@ -701,6 +732,34 @@ cudaError_t launch_rescreen(const SearchParams &P, const ScreenBufs &B,
   else
     k_rescreen<false><<<grid, kScreenThreads, 0, st>>>(P, B);
   return cudaGetLastError();
+}
+
+template <bool H>
+static cudaError_t screen_batch(const ScreenTask *t, int n,
+                                const SearchParams &P0, const ScreenBufs &B0,
+                                bool rescreen, cudaStream_t st) {
+  const unsigned tiles =
+      (unsigned)((P0.count + kScreenTile - 1) / kScreenTile);
+  const unsigned chunks =
+      (unsigned)((P0.count + 8LL * kListThreads - 1) / (8LL * kListThreads));
+  const unsigned y = (unsigned)n;
+  const unsigned pilot = (B0.pilot_cap + kPilotTpg - 1) / kPilotTpg;
+  // a few tiles per block amortise the subset's staging and the histogram
+  k_screen_batch<H><<<dim3((tiles + 3) / 4, y), kScreenThreads, 0, st>>>(t);
+  k_pilot_list_batch<false><<<dim3(chunks, y), kListThreads, 0, st>>>(t);
+  k_pilot_batch<H><<<dim3(pilot, y), kPilotWarps * 32, 0, st>>>(t);
+  k_list_batch<false><<<dim3(chunks, y), kListThreads, 0, st>>>(t);
+  if (rescreen)
+    k_rescreen_batch<H><<<dim3((tiles + 7) / 8, y), kScreenThreads, 0, st>>>(
+        t);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_screen_batch(const ScreenTask *t, int n,
+                                const SearchParams &P0, const ScreenBufs &B0,
+                                bool rescreen, cudaStream_t st) {
+  return P0.quadh ? screen_batch<true>(t, n, P0, B0, rescreen, st)
+                  : screen_batch<false>(t, n, P0, B0, rescreen, st);
 }
 
 }  // namespace morse

@@ -240,8 +240,7 @@ __global__ void __launch_bounds__(kSearchWarps * 32, 1)
 // of weak signal) is left out by a warp once it has seen that, but for
 // every sixteenth group, which keeps looking.
 template <bool EPS, bool H>
-__global__ void __launch_bounds__(kSearchWarps * 32, 1)
-    k_search_list(const SearchParams P) {
+__device__ __forceinline__ void search_listed(const SearchParams &P) {
   if (!listed(P)) return;  // k_search has it
   const unsigned n = __ldg(P.n_list);
   extern __shared__ __align__(16) unsigned char smem[];
@@ -376,6 +375,7 @@ __global__ void __launch_bounds__(kSearchWarps * 32, 1)
     warp_merge(P, T, K, warp, lane, keep, my_chi2, (long long)my);
   }
   if (P.stat_exact && lane == 0 && n_exact) atomicAdd(P.stat_exact, n_exact);
+  if (!P.partial) return;
   __syncthreads();
   const int nk = s_nk;
   const Entry *cur = s_cur ? T.buf1 : T.buf0;
@@ -390,6 +390,24 @@ __global__ void __launch_bounds__(kSearchWarps * 32, 1)
     }
     out[i] = e;
   }
+}
+
+template <bool EPS, bool H>
+__global__ void __launch_bounds__(kSearchWarps * 32, 1)
+    k_search_list(const SearchParams P) {
+  search_listed<EPS, H>(P);
+}
+// the searches of a batch (blockIdx.y)
+template <bool H>
+__global__ void __launch_bounds__(kSearchWarps * 32, 1)
+    k_search_list_batch(const ScreenTask *t) {
+  __shared__ alignas(16) SearchParams s_P;
+  const int *src = reinterpret_cast<const int *>(&t[blockIdx.y].F.S);
+  for (int i = threadIdx.x; i < (int)(sizeof(SearchParams) / 4);
+       i += blockDim.x)
+    reinterpret_cast<int *>(&s_P)[i] = __ldg(src + i);
+  __syncthreads();
+  search_listed<false, H>(s_P);
 }
 
 // One level of the merge tree: lists 4p .. 4p + 3 -> list p, keeping the
@@ -566,11 +584,15 @@ __global__ void k_fill(const FillParams F) {
 // sweep of the epochs.  With the threshold of a good pilot the candidates
 // are little more than the k records themselves (config 1: 267 for 256);
 // more than kCandMax go the general way.
+// Blocks per search of a batch's listed search: a long light curve of weak
+// signal can leave one search with most of the batch's work (12 blocks: 9.1
+// ms with half the SMs idle in its tail).
+constexpr int kListBatchBlocks = 76;
+
 constexpr int kFinishThreads = 1024, kFinishPer = kFinishThreads / 16;
 
-__global__ void __launch_bounds__(kFinishThreads)
-    k_finish(const FillParams F) {
-  extern __shared__ __align__(16) unsigned char smem[];
+__device__ __forceinline__ void finish(const FillParams &F,
+                                       unsigned char *smem) {
   const SearchParams &P = F.S;
   if (!listed(P)) return;
   const unsigned n = __ldg(P.n_cand);
@@ -589,20 +611,40 @@ __global__ void __launch_bounds__(kFinishThreads)
     id[i] = P.cand[i].idx;
   }
   __syncthreads();
-  const unsigned me = blockIdx.x * kFinishPer + threadIdx.x / 16;
-  const unsigned long long mk = me < n ? key[me] : 0ULL;
-  const unsigned mi = me < n ? id[me] : 0u;
-  unsigned r = 0;
-  for (unsigned i = threadIdx.x & 15; i < n; i += 16) {
-    const unsigned long long k = key[i];
-    r += k < mk || (k == mk && id[i] < mi);
-  }
+  for (unsigned c0 = blockIdx.x * kFinishPer; c0 < n;
+       c0 += gridDim.x * kFinishPer) {
+    const unsigned me = c0 + threadIdx.x / 16;
+    const unsigned long long mk = me < n ? key[me] : 0ULL;
+    const unsigned mi = me < n ? id[me] : 0u;
+    unsigned r = 0;
+    for (unsigned i = threadIdx.x & 15; i < n; i += 16) {
+      const unsigned long long k = key[i];
+      r += k < mk || (k == mk && id[i] < mi);
+    }
 #pragma unroll
-  for (int o = 8; o; o >>= 1) r += __shfl_xor_sync(kFull, r, o);
-  if (me >= n || (threadIdx.x & 15) != 0 || r >= (unsigned)F.k) return;
-  const Candidate c = P.cand[me];
-  F.out[r] = fit_record(P, (long long)c.idx, c.chi2, c.Fs, c.Bc,
-                        c.degenerate != 0, F.t0abs, F.tEv);
+    for (int o = 8; o; o >>= 1) r += __shfl_xor_sync(kFull, r, o);
+    if (me < n && (threadIdx.x & 15) == 0 && r < (unsigned)F.k) {
+      const Candidate c = P.cand[me];
+      F.out[r] = fit_record(P, (long long)c.idx, c.chi2, c.Fs, c.Bc,
+                            c.degenerate != 0, F.t0abs, F.tEv);
+    }
+  }
+}
+__global__ void __launch_bounds__(kFinishThreads)
+    k_finish(const FillParams F) {
+  extern __shared__ __align__(16) unsigned char fin[];
+  finish(F, fin);
+}
+__global__ void __launch_bounds__(kFinishThreads)
+    k_finish_batch(const ScreenTask *t) {
+  extern __shared__ __align__(16) unsigned char fin[];
+  __shared__ alignas(16) FillParams s_F;
+  const int *src = reinterpret_cast<const int *>(&t[blockIdx.y].F);
+  for (int i = threadIdx.x; i < (int)(sizeof(FillParams) / 4);
+       i += blockDim.x)
+    reinterpret_cast<int *>(&s_F)[i] = __ldg(src + i);
+  __syncthreads();
+  finish(s_F, fin);
 }
 
 // The tau interval of every (u0, alpha) line inside the map.
@@ -834,7 +876,7 @@ cudaError_t launch_topk_merge(Entry *a, Entry *b, int lists, int k,
   return cudaSuccess;
 }
 
-cudaError_t launch_finish(const FillParams &F, cudaStream_t st) {
+static size_t finish_smem() {
   const size_t sm = (size_t)kCandMax * 12;
   static int set_of[64];
   int dev = 0;
@@ -842,9 +884,33 @@ cudaError_t launch_finish(const FillParams &F, cudaStream_t st) {
   if (dev >= 64 || !set_of[dev]) {
     cudaFuncSetAttribute(k_finish, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)sm);
+    cudaFuncSetAttribute(k_finish_batch,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (dev < 64) set_of[dev] = 1;
   }
-  k_finish<<<kCandMax / kFinishPer, kFinishThreads, sm, st>>>(F);
+  return sm;
+}
+
+cudaError_t launch_finish(const FillParams &F, cudaStream_t st) {
+  k_finish<<<kCandMax / kFinishPer, kFinishThreads, finish_smem(), st>>>(F);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_list_batch(const ScreenTask *t, int n,
+                              const SearchParams &P0, cudaStream_t st) {
+  const size_t sm = search_smem_bytes(0, P0.top_k);
+  cudaError_t e = cudaFuncSetAttribute(
+      P0.quadh ? (const void *)k_search_list_batch<true>
+               : (const void *)k_search_list_batch<false>,
+      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  const dim3 grid(kListBatchBlocks, (unsigned)n);
+  if (P0.quadh)
+    k_search_list_batch<true><<<grid, kSearchWarps * 32, sm, st>>>(t);
+  else
+    k_search_list_batch<false><<<grid, kSearchWarps * 32, sm, st>>>(t);
+  const size_t fs = finish_smem();
+  k_finish_batch<<<dim3(2, (unsigned)n), kFinishThreads, fs, st>>>(t);
   return cudaGetLastError();
 }
 

@@ -652,7 +652,9 @@ size_t plan_screen(const morse_event *ev, const morse_grid *g,
     return at;
   pl->want = (unsigned)want;
   pl->pilot_cap = 2 * pl->want;
-  pl->list_cap = (unsigned)(count / 2);
+  // (the rescreening's own rule: a list that leaves out less than one in
+  // eight is not worth having)
+  pl->list_cap = (unsigned)(count - count / 8);
   pl->off_hist = align_up(at, 256);  // histogram and list lengths: cleared
   pl->off_code = align_up(
       pl->off_hist + sizeof(unsigned) * (morse::kScreenBins +
@@ -668,6 +670,34 @@ size_t plan_screen(const morse_event *ev, const morse_grid *g,
   pl->off_cand = align_up(
       pl->off_list + sizeof(unsigned) * (size_t)pl->list_cap, 256);
   return pl->off_cand + sizeof(morse::Candidate) * morse::kCandMax;
+}
+
+// The buffers of a screened search planned at offsets of base (histogram and
+// counters at words), and the search parameters that name them.
+void screen_bufs(const Plan &pl, char *base, char *words,
+                 morse::ScreenBufs *B, morse::SearchParams *P) {
+  B->code = (unsigned short *)(base + pl.off_code);
+  B->hist = (unsigned *)words;
+  B->n = B->hist + morse::kScreenBins;
+  B->pilot = (unsigned *)(base + pl.off_pil);
+  B->ub = (float *)(base + pl.off_ub);
+  B->list0 = (unsigned *)(base + pl.off_list0);
+  B->list = (unsigned *)(base + pl.off_list);
+  B->pilot_cap = pl.pilot_cap;
+  B->list0_cap = pl.list0_cap;
+  B->list_cap = pl.list_cap;
+  B->want = pl.want;
+  const bool two = P->n_lv > 2;  // a rescreened list
+  if (!two) {  // list0 is the final list
+    B->list0 = B->list;
+    B->list0_cap = B->list_cap;
+  }
+  P->list = B->list;
+  P->n_list = B->n + (two ? 2 : 1);
+  P->no_list = two ? B->n + 4 : nullptr;
+  P->list_cap = B->list_cap;
+  P->cand = (morse::Candidate *)(base + pl.off_cand);
+  P->n_cand = B->n + 6;
 }
 
 // Reset the pruning threshold between the maps of a sweep (it is per map).
@@ -829,17 +859,7 @@ morse_status enqueue_topk(morse_ctx *ctx, const Plan &pl,
   }
   if (list_grid > 0) {
     morse::ScreenBufs B;
-    B.code = (unsigned short *)(base + pl.off_code);
-    B.hist = (unsigned *)(base + pl.off_hist);
-    B.n = B.hist + morse::kScreenBins;
-    B.pilot = (unsigned *)(base + pl.off_pil);
-    B.ub = (float *)(base + pl.off_ub);
-    B.list0 = (unsigned *)(base + pl.off_list0);
-    B.list = (unsigned *)(base + pl.off_list);
-    B.pilot_cap = pl.pilot_cap;
-    B.list0_cap = pl.list0_cap;
-    B.list_cap = pl.list_cap;
-    B.want = pl.want;
+    screen_bufs(pl, base, base + pl.off_hist, &B, &P);
     MORSE_CUDA(ctx, cudaMemsetAsync(
                         B.hist, 0,
                         sizeof(unsigned) * (morse::kScreenBins +
@@ -852,19 +872,11 @@ morse_status enqueue_topk(morse_ctx *ctx, const Plan &pl,
     MORSE_CUDA(ctx, morse::launch_screen_pilot(P, B, ctx->stream));
     MORSE_CUDA(ctx, morse::launch_screen_list(P, B, ctx->sm_count,
                                               ctx->stream));
-    P.list = B.list;
-    P.n_list = B.n + 1;
-    P.no_list = nullptr;
-    P.list_cap = B.list_cap;
-    P.cand = (morse::Candidate *)(base + pl.off_cand);
-    P.n_cand = B.n + 6;
     done = B.n + 7;
     if (P.n_lv > 2) {
       MORSE_CUDA(ctx, morse::launch_rescreen(P, B, ctx->sm_count,
                                              ctx->stream));
       ctx->launches += 1;
-      P.n_list = B.n + 2;
-      P.no_list = B.n + 4;
     }
     P.pub_tag = next_pub_tag(ctx);
     P.pub_nb = list_grid;
@@ -1107,6 +1119,11 @@ struct BatchHost {
   int ep_cap = 0;
   int main_global = 0;  // the main pass's units of unstaged light curves,
                         // first in `main` (a launch of their own)
+  // screened searches (k_screen.cu), one per pair in processing order, in
+  // chunks of `chunk` that share scratch memory; empty: not screened
+  std::vector<morse::ScreenTask> tasks;
+  Plan scr;             // sizes and offsets of one search's scratch
+  int chunk = 0;
 };
 
 // Units of one pass over `pairs` pairs: groups [0, groups(p)) of each pair
@@ -1168,7 +1185,12 @@ struct BatchLayout {
   size_t off_tab, off_ev, off_ptr, off_up, off_um, off_lp, off_lm, off_gthr,
       off_hdr, off_pub, off_pa, off_pb, off_res, off_fit, bytes;
   size_t lists;  // top-K lists of the larger pass
+  size_t off_task, off_done, off_hist, off_scr;
 };
+// bytes of a screened search's histogram and counters in a batch
+const size_t kScreenWordBytes =
+    align_up(sizeof(unsigned) * (morse::kScreenBins + morse::kScreenWords),
+             256);
 
 struct BatchHdr {
   unsigned counter[3];  // pilot, main (unstaged units), main (staged)
@@ -1191,7 +1213,9 @@ BatchLayout batch_layout(const BatchHost &H, int pairs, int K) {
   L.off_um = take(sizeof(morse::BatchUnit) * H.main.size());
   L.off_lp = take(sizeof(int) * H.pilot_list0.size());
   L.off_lm = take(sizeof(int) * H.main_list0.size());
+  L.off_task = take(sizeof(morse::ScreenTask) * H.tasks.size());
   L.off_gthr = take(sizeof(unsigned long long) * (size_t)pairs);
+  L.off_done = take(sizeof(unsigned) * (size_t)pairs);
   L.off_hdr = take(sizeof(BatchHdr));
   const size_t lists = (size_t)std::max(
       H.pilot_list0.empty() ? 0 : H.pilot_list0.back(), H.main_list0.back());
@@ -1201,6 +1225,8 @@ BatchLayout batch_layout(const BatchHost &H, int pairs, int K) {
   L.off_pb = take(sizeof(Entry) * lists * (size_t)K);
   L.off_res = take(sizeof(Entry) * (size_t)pairs * K);
   L.off_fit = take(sizeof(morse_fit) * (size_t)pairs * K);
+  L.off_hist = take(kScreenWordBytes * (size_t)H.chunk);
+  L.off_scr = take(H.scr.bytes * (size_t)H.chunk);
   L.bytes = o;
   return L;
 }
@@ -1211,7 +1237,7 @@ morse_status batch_prepare(morse_ctx *ctx, const morse_event *const *evs,
                            int n_ev, const morse_map *const *maps, int n_maps,
                            const morse_grid *g,
                            const std::vector<morse_batch_shape> &shape_ev,
-                           bool with_pilot, BatchHost &H) {
+                           bool screen, BatchHost &H) {
   const int K = g->top_k;
   const long long N = grid_size(g);
   const long long line = (long long)g->n_t0 * g->n_tE;
@@ -1263,6 +1289,36 @@ morse_status batch_prepare(morse_ctx *ctx, const morse_event *const *evs,
   std::vector<morse_batch_shape> shape_pair((size_t)pairs);
   for (int p = 0; p < pairs; ++p)
     shape_pair[(size_t)p] = shape_fit[(size_t)(p / n_maps)];
+  // screened when every light curve has subsets and the grid is large enough
+  H.tasks.clear();
+  H.chunk = 0;
+  memset(&H.scr, 0, sizeof(H.scr));
+  H.scr.K = K;
+  const morse_event *most = evs[0];  // with the most subsets
+  for (int e = 0; e < n_ev; ++e) {
+    if (evs[e]->n_sub < 1) screen = false;
+    if (evs[e]->n_sub > most->n_sub) most = evs[e];
+  }
+  if (screen) {
+    H.scr.bytes = align_up(plan_screen(most, g, N, 0, &H.scr), 256);
+    if (H.scr.want > 0) {
+      // as many pairs at a time as 512 MB of scratch hold
+      H.chunk = (int)std::max<size_t>(
+          1, std::min<size_t>({(size_t)pairs, (512u << 20) / H.scr.bytes,
+                               (size_t)1024}));
+      H.tasks.resize((size_t)pairs);
+      for (int k = 0; k < pairs; ++k) {  // the rest: batch_tasks
+        morse::ScreenTask &t = H.tasks[(size_t)k];
+        memset(&t, 0, sizeof(t));
+        const int p = order[(size_t)k];
+        map_params(maps[p % n_maps], &t.F.S);
+        event_params(evs[p / n_maps], &t.F.S);
+        t.F.k = p;  // (until batch_tasks)
+      }
+    } else {
+      memset(&H.scr, 0, sizeof(H.scr));
+    }
+  }
   // pilot: a strided sample of ~sqrt(K N) trajectories per pair
   const double want = std::max(morse::kBatchPilotMinK * K,
                                morse::kBatchPilotSqrt * std::sqrt((double)K * N));
@@ -1271,7 +1327,7 @@ morse_status batch_prepare(morse_ctx *ctx, const morse_event *const *evs,
   H.pilot_list0.clear();
   H.pilot_count = 0;
   H.pilot_stride = 0;
-  if (with_pilot && stride >= 4) {
+  if (H.tasks.empty() && stride >= 4) {
     H.pilot_stride = stride;
     H.pilot_count = (N + stride - 1) / stride;
     std::vector<morse_batch_shape> sp = shape_pair;
@@ -1307,6 +1363,48 @@ morse_status batch_prepare(morse_ctx *ctx, const morse_event *const *evs,
 }
 
 // Upload a prepared batch; returns the kernel parameters of its passes.
+// The device addresses of the screened searches' parameters (tab: the grid
+// tables, laid out as batch_upload does).
+void batch_tasks(BatchHost &H, const BatchLayout &L, char *base,
+                 const morse_grid *g, double *tab) {
+  double *u0 = tab + (size_t)2 * g->n_u0 * g->n_alpha;
+  Tables T;
+  T.slab = (double2 *)tab;
+  T.u0v = u0;
+  T.ca = u0 + g->n_u0;
+  T.sa = T.ca + g->n_alpha;
+  T.invtEd = T.sa + g->n_alpha;
+  T.t0abs = T.invtEd + g->n_tE;
+  T.tEv = T.t0abs + g->n_t0;
+  double *rel = T.tEv + g->n_tE;
+  BatchHdr *hd = (BatchHdr *)(base + L.off_hdr);
+  const int n_maps = (int)H.tab.size();
+  for (size_t k = 0; k < H.tasks.size(); ++k) {
+    morse::ScreenTask &t = H.tasks[k];
+    const int p = t.F.k;
+    T.t0rel = rel + (size_t)(p / n_maps) * g->n_t0;
+    morse::SearchParams &P = t.F.S;
+    grid_params(g, T, &P);
+    P.first = 0;
+    P.count = grid_size(g);
+    P.stride = 1;
+    morse::set_groups(&P);
+    P.gthr = (unsigned long long *)(base + L.off_gthr) + p;
+    P.err = &hd->err;
+    P.stat_exact = &hd->stat_exact;
+    const size_t slot = k % (size_t)H.chunk;
+    char *scr = base + L.off_scr + H.scr.bytes * slot;
+    screen_bufs(H.scr, scr, base + L.off_hist + kScreenWordBytes * slot,
+                &t.B, &P);
+    t.F.sel = nullptr;
+    t.F.k = H.scr.K;
+    t.F.t0abs = T.t0abs;
+    t.F.tEv = T.tEv;
+    t.F.out = (morse_fit *)(base + L.off_fit) + (size_t)p * H.scr.K;
+    t.F.done = (unsigned *)(base + L.off_done) + p;
+  }
+}
+
 morse_status batch_upload(morse_ctx *ctx, BatchHost &H, const BatchLayout &L,
                           char *base, const morse_grid *g,
                           const morse_map *map0, int n_ev,
@@ -1321,6 +1419,10 @@ morse_status batch_upload(morse_ctx *ctx, BatchHost &H, const BatchLayout &L,
     H.ev[(size_t)e].t0rel = tab + o_rel + (size_t)e * g->n_t0;
   // one staging buffer, one copy, one wait (the host vectors are pageable)
   std::vector<char> h(L.off_gthr);
+  batch_tasks(H, L, base, g, tab);
+  if (!H.tasks.empty())
+    memcpy(h.data() + L.off_task, H.tasks.data(),
+           sizeof(morse::ScreenTask) * H.tasks.size());
   memcpy(h.data() + L.off_tab, H.tables.data(),
          sizeof(double) * H.tables.size());
   memcpy(h.data() + L.off_ev, H.ev.data(),
@@ -1368,6 +1470,7 @@ morse_status batch_upload(morse_ctx *ctx, BatchHost &H, const BatchLayout &L,
   B.n_maps = (int)H.tab.size();
   B.gthr = (unsigned long long *)(base + L.off_gthr);
   B.partial = (Entry *)(base + L.off_pa);
+  B.done = H.tasks.empty() ? nullptr : (const unsigned *)(base + L.off_done);
   B.ep_cap = H.ep_cap;
   // published list quantiles: rows of the larger pass's list count, cleared
   // by every call (a graph replay reuses the tags); tags 1 and 2
@@ -1406,7 +1509,7 @@ morse_status batch_enqueue(morse_ctx *ctx, const BatchLayout &L, char *base,
                            const morse::BatchParams &Bm, bool h16, int pairs,
                            const double *t0abs, const double *tEv,
                            int grid, size_t smem, int main_global,
-                           int grid_g, size_t smem_g) {
+                           int grid_g, size_t smem_g, const BatchHost &H) {
   const int K = Bm.S.top_k;
   MORSE_CUDA(ctx, cudaMemsetAsync(base + L.off_gthr, 0xFF,
                                   sizeof(unsigned long long) * pairs,
@@ -1420,6 +1523,30 @@ morse_status batch_enqueue(morse_ctx *ctx, const BatchLayout &L, char *base,
   Entry *pa = (Entry *)(base + L.off_pa), *pb = (Entry *)(base + L.off_pb);
   Entry *res = (Entry *)(base + L.off_res);
   int r;
+  if (!H.tasks.empty()) {
+    // the screened searches, a chunk of pairs at a time; pairs that end
+    // without records (Bm.done) are searched whole below
+    MORSE_CUDA(ctx, cudaMemsetAsync(base + L.off_done, 0,
+                                    sizeof(unsigned) * pairs, ctx->stream));
+    r = t_begin(ctx, KT_SEARCH);
+    for (int k = 0; k < pairs; k += H.chunk) {
+      const int n = std::min(H.chunk, pairs - k);
+      const morse::ScreenTask *t =
+          (const morse::ScreenTask *)(base + L.off_task) + k;
+      const morse::ScreenTask &t0 = H.tasks[(size_t)k];
+      bool rescreen = false;
+      for (int j = k; j < k + n; ++j)
+        rescreen |= H.tasks[(size_t)j].F.S.n_lv > 2;
+      MORSE_CUDA(ctx, cudaMemsetAsync(base + L.off_hist, 0,
+                                      kScreenWordBytes * (size_t)n,
+                                      ctx->stream));
+      MORSE_CUDA(ctx, morse::launch_screen_batch(t, n, t0.F.S, t0.B, rescreen,
+                                                 ctx->stream));
+      MORSE_CUDA(ctx, morse::launch_list_batch(t, n, t0.F.S, ctx->stream));
+      ctx->launches += rescreen ? 7 : 6;
+    }
+    t_end(ctx, r);
+  }
   if (Bp.n_units > 0) {
     r = t_begin(ctx, KT_SEARCH);
     MORSE_CUDA(ctx, morse::launch_batch(
@@ -1457,7 +1584,7 @@ morse_status batch_enqueue(morse_ctx *ctx, const BatchLayout &L, char *base,
   MORSE_CUDA(ctx, morse::launch_batch_merge(pa, pb,
                                             (const int *)(base + L.off_lm),
                                             pairs, K, res, nullptr,
-                                            ctx->stream));
+                                            ctx->stream, Bm.done));
   t_end(ctx, r);
   ctx->launches += 1;
   r = t_begin(ctx, KT_FILL);
@@ -1528,7 +1655,7 @@ morse_status batch_tune(morse_ctx *ctx, const morse_event *ev,
   for (size_t c = 0; c < cands.size() && st == MORSE_OK; ++c) {
     std::vector<morse_batch_shape> sh(1, cands[c]);
     BatchHost H;
-    st = batch_prepare(ctx, evs, 1, maps, 1, g, sh, true, H);
+    st = batch_prepare(ctx, evs, 1, maps, 1, g, sh, false, H);
     if (st != MORSE_OK) break;
     // time an evenly spaced sample of the pair's units, about
     // kTuneTrajs trajectories
@@ -2022,7 +2149,8 @@ void morse_map_free(morse_map *map) {
 // ------------------------------------------------------------------ events
 // The screening subsets of a light curve (k_screen.cu), appended to its n
 // slots h: 32 epochs (64 from 640 epochs on); from 1024 epochs on 96, and a
-// quarter of it or 320; from 2048 on a third of it.  They consist of runs of
+// quarter of it but no more than 320, or a sixteenth up to 1008; from 2048 on
+// a third of it.  They consist of runs of
 // neighbouring epochs (4, 8, 16 and 32 long), which a trajectory meets in
 // the same few cells; measured over events of tE 13 to 72 d, runs of that
 // length discard as many trajectories as single epochs do.  A run's share
@@ -2036,7 +2164,10 @@ static void screen_subsets(morse_event *ev, std::vector<float4> &h, int64_t n,
   ev->n_sub = 0;
   const int sizes[kScreenLevels] = {
       n < 640 ? 32 : 64, n >= 1024 ? 96 : 0,
-      n >= 1024 ? (int)std::min<int64_t>(n / 4, 320) : 0,
+      n >= 1024 ? (int)std::min<int64_t>(
+                      n / 4, std::min<int64_t>(
+                                 1008, std::max<int64_t>(320, n / 16)))
+                : 0,
       n >= 2048 ? (int)(n / 3) : 0};
   if (n < 128 || n > (1 << 20) || !(S1 > 1e-12 && S1 < 1e15 && SFF > 1e-12 &&
                                     SFF < 1e15))
@@ -2088,7 +2219,7 @@ static void screen_subsets(morse_event *ev, std::vector<float4> &h, int64_t n,
       acc = next;
     }
     // (the most the kernels stage of the first three)
-    const size_t most[kScreenLevels] = {128, 192, 512, (size_t)n};
+    const size_t most[kScreenLevels] = {128, 192, 1024, (size_t)n};
     if (sel.size() < 8 || sel.size() > most[l]) break;
     morse_subset &u = ev->sub[l];
     u.m = (int)sel.size();
@@ -2770,7 +2901,7 @@ morse_status morse_grid_chi2_batch(morse_ctx *ctx,
                                          cudaStreamCaptureModeThreadLocal));
   morse_status st = batch_enqueue(ctx, L, base, Bp, Bm, h16, pairs, t0abs,
                                   tEv, bps * ctx->sm_count, smem, H.main_global,
-                                  bps_g * ctx->sm_count, smem_g);
+                                  bps_g * ctx->sm_count, smem_g, H);
   cudaGraph_t graph = nullptr;
   cudaError_t ce = cudaStreamEndCapture(ctx->stream, &graph);
   if (st != MORSE_OK || ce != cudaSuccess) {

@@ -282,7 +282,8 @@ struct SearchParams {
   double a_min;             // the cut (with linemax)
   int top_k;
   // outputs
-  Entry *partial;           // [gridDim.x][top_k] (top-K mode)
+  Entry *partial;           // [gridDim.x][top_k] (top-K mode; null in a
+                            // batch's listed search: the lists are not kept)
   double *dchi2, *dFs, *dFb;  // [count] (dense mode)
   // optional device words (nullptr: unused)
   unsigned long long *gthr; // grid-wide pruning threshold (chi^2 bits),
@@ -375,16 +376,6 @@ void ctx_params(const morse_ctx *ctx, SearchParams *P);
 // failure of morse_inject_fault (cudaErrorMemoryAllocation, nothing made)
 cudaError_t dev_alloc(morse_ctx *ctx, void **p, size_t bytes);
 
-struct FillParams {
-  SearchParams S;
-  const Entry *sel;         // [k] selected (chi2, idx)
-  int k;
-  const double *t0abs, *tEv;  // absolute t0 and tE tables
-  morse_fit *out;           // [k]
-  unsigned *done;           // records made from the candidates: nonzero
-                            // (nullptr: none were)
-};
-
 #ifndef MORSE_SEARCH_WARPS
 #define MORSE_SEARCH_WARPS 16
 #endif
@@ -441,7 +432,29 @@ inline long long main_groups(long long line, long long first,
   return ((first + count - 1) / line - first / line + 1) * ng;
 }
 
+struct FillParams {
+  SearchParams S;
+  const Entry *sel;         // [k] selected (chi2, idx)
+  int k;
+  const double *t0abs, *tEv;  // absolute t0 and tE tables
+  morse_fit *out;           // [k]
+  unsigned *done;           // records made from the candidates: nonzero
+                            // (nullptr: none were)
+};
+
 // ---------------------------------------------------------------- screen
+// One screened search of a batch: the kernels of a batch take an array of
+// them in device memory, one per blockIdx.y.
+struct alignas(16) ScreenTask {
+  FillParams F;             // F.S: its search parameters
+  ScreenBufs B;
+};
+// every step of n screened searches of one signature (P0, B0: any of them)
+cudaError_t launch_screen_batch(const ScreenTask *t, int n,
+                                const SearchParams &P0, const ScreenBufs &B0,
+                                bool rescreen, cudaStream_t st);
+cudaError_t launch_list_batch(const ScreenTask *t, int n,
+                              const SearchParams &P0, cudaStream_t st);
 // codes and histogram of trajectories first .. first + count - 1
 cudaError_t launch_screen(const SearchParams &P, const ScreenBufs &B,
                           int sm_count, cudaStream_t st);
@@ -566,6 +579,8 @@ struct BatchParams {
   int n_lists;
   Entry *partial;           // [lists][top_k]
   int ep_cap;               // staged-epoch capacity of shared memory
+  const unsigned *done;     // [pairs] nonzero: the pair's screened search made
+                            // its records (nullptr: nothing was screened)
 };
 
 size_t batch_smem_bytes(int ep_cap, int top_k);
@@ -578,7 +593,8 @@ cudaError_t launch_batch(const BatchParams &B, bool h16, int grid,
 // result[p]; with gthr set, also lower gthr[p] to the merged K-th chi^2
 cudaError_t launch_batch_merge(Entry *a, Entry *b, const int *list0,
                                int pairs, int k, Entry *result,
-                               unsigned long long *gthr, cudaStream_t st);
+                               unsigned long long *gthr, cudaStream_t st,
+                               const unsigned *done = nullptr);
 // records of result[pairs][k] into out[pairs][k]
 cudaError_t launch_batch_fill(const BatchParams &B, bool h16,
                               const Entry *result, int pairs,

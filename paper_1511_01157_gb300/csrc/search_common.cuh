@@ -880,8 +880,8 @@ __device__ __forceinline__ bool may_reach(const SearchParams &P,
 // of the sweep (the margin may_reach allows it).
 __device__ __forceinline__ double chi2_upper(const SearchParams &P, double SA,
                                             double SAA, double SAF, double a,
-                                            double b) {
-  const double g = 2.0 * P.gamma;
+                                            double b, double gamma) {
+  const double g = 2.0 * gamma;
   const double TA = (double)__fsqrt_ru(__double2float_ru(P.S1 * SAA));
   const double TAF = (double)__fsqrt_ru(__double2float_ru(SAA * P.SFF));
   const double q = P.SFF - 2.0 * a * SAF - 2.0 * b * P.SF + a * a * SAA +

@@ -232,7 +232,8 @@ __device__ __forceinline__ void search_group(const SearchParams &P,
     // pilot: the bound from the sums, no sweep
     if (cand_me)
       my_chi2 = chi2_upper(P, (double)mine_s.a, (double)mine_s.b,
-                           (double)mine_s.d, (double)myFs, (double)myBc);
+                           (double)mine_s.d, (double)myFs, (double)myBc,
+                           P.gamma);
     cand_me = false;
   }
   unsigned todo = __ballot_sync(kFull, cand_me);

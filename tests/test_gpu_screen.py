@@ -112,3 +112,24 @@ def test_screened_forms(m, setup, kind):
     a, b = ctx.grid_chi2_lines(ev, mp, lg, lines), ctx.grid_chi2(ev, mp, g)
     assert np.array_equal(a["idx"], b["idx"])
     np.testing.assert_allclose(a["chi2"], b["chi2"], rtol=1e-6)
+
+
+def test_screened_batch_equals_single_searches(m, setup):
+    """Light curves with one, three and four subsets, of strong and of no
+    signal (pairs that fall back to the whole range), in one batch."""
+    ctx, mp = setup
+    other = ctx.build_map(0.7, 2e-2, 2.0, 301, 2100, image_halfwidth=3.0,
+                          deflect="fp32")
+    evs = [_event(ctx, n, kind) for n, kind in
+           ((130, "strong"), (700, "weak"), (1500, "strong"),
+            (1500, "flat"), (3000, "strong"), (3000, "flat"))]
+    g = _grid(m, 40)
+    for h16 in (False, True):
+        mp.set_lookup(h16)
+        other.set_lookup(h16)
+        got = ctx.grid_chi2_batch(evs, [mp, other], g)
+        for i, ev in enumerate(evs):
+            for j, x in enumerate((mp, other)):
+                assert np.array_equal(got[i, j], ctx.grid_chi2(ev, x, g))
+    mp.set_lookup(False)
+    other.free()
