@@ -24,6 +24,11 @@
 //    the terms Eq. 2 sums, is below 1e-4 before the polish and below 1e-9
 //    after it, and it is not a repeat of an earlier root;
 //    A = sum over images of 1/|det J| with det J = 1 - |D|^2 (Eq. 3-4).
+//
+// That is the general form, 12 000 FP64-pipe instructions per warp of texels
+// at some 16 cycles each: 24 ms per 1024^2 map.  k_poly_fast does nearly all
+// texels (99.9 % of the maps measured) with a thirtieth of the FP64 work and
+// proves its count of images; k_poly_map takes the others.
 #include <cuda_runtime.h>
 #include <math_constants.h>
 #include <stdint.h>
@@ -125,9 +130,9 @@ __device__ __forceinline__ void lens(cd w, double a, double e1, double e2,
   *D = add(scl(e1, mul(ia, ia)), scl(e2, mul(ib, ib)));
 }
 
-__global__ void k_poly_map(double s, double q, double L, int npix,
-                           float *__restrict__ A) {
-  const size_t n = (size_t)npix * npix;
+// A of texel k by the general form.
+__device__ double poly_texel(double s, double q, double L, int npix,
+                             size_t k) {
   const double e1 = 1.0 / (1.0 + q), e2 = q / (1.0 + q);
   const double a = 0.5 * s, dl = e2 - e1;
   // midpoint of the masses: the primary sits at -s e2, the secondary at
@@ -135,8 +140,7 @@ __global__ void k_poly_map(double s, double q, double L, int npix,
   const double m = 0.5 * s * (e1 - e2);
   const double dlt = (2.0 * L) / (double)npix;
   const double a2 = a * a;
-  for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n;
-       k += (size_t)gridDim.x * blockDim.x) {
+  {
     const int i = (int)(k % npix), j = (int)(k / npix);
     const cd om = mk(-L + ((double)i + 0.5) * dlt - m,
                      -L + ((double)j + 0.5) * dlt);
@@ -259,20 +263,283 @@ __global__ void k_poly_map(double s, double q, double L, int npix,
         A_sum += 1.0 / fabs(1.0 - ab2(D));
       }
     }
-    A[k] = __double2float_rn(A_sum);
+    return A_sum;
   }
+}
+
+// Texels whose value is `todo` by the general form (todo NaN: those the fast
+// kernel left; otherwise all).  A block collects them in shared memory
+// first, so that its warps are full.
+constexpr int kPolyThreads = 128, kPolyTile = 16 * kPolyThreads;
+
+__global__ void __launch_bounds__(kPolyThreads)
+    k_poly_map(double s, double q, double L, int npix, bool left,
+               float *__restrict__ A) {
+  __shared__ unsigned s_q[kPolyTile], s_n;
+  const size_t n = (size_t)npix * npix;
+  for (size_t c0 = blockIdx.x * (size_t)kPolyTile; c0 < n;
+       c0 += gridDim.x * (size_t)kPolyTile) {
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    for (int t = threadIdx.x; t < kPolyTile; t += kPolyThreads)
+      if (c0 + t < n && (!left || isnan(A[c0 + t])))
+        s_q[atomicAdd(&s_n, 1u)] = (unsigned)t;
+    __syncthreads();
+    const unsigned m = s_n;
+    for (unsigned t = threadIdx.x; t < m; t += kPolyThreads) {
+      const size_t k = c0 + s_q[t];
+      A[k] = __double2float_rn(poly_texel(s, q, L, npix, k));
+    }
+    __syncthreads();
+  }
+}
+
+// ------------------------------------------------------------ fast form
+// Origin at the lighter lens B (mass mb), the other (ma) at h on the axis:
+//     omega = w - ma/(conj(w) - h) - mb/conj(w).
+// With N = conj(omega) w^2 + (1 - conj(omega) h) w - mb h and A = N - h P,
+// P = w (w - h), conj(w) = N/P and
+//     (w - omega) A N - P (ma N + mb A) = 0.
+// About the lighter lens its cluster of roots (of size sqrt(mb)) is held by
+// the low coefficients to their own relative precision, so FP32 resolves it:
+// coefficients in FP64, rounded, and Aberth-Ehrlich in FP32 from radii of
+// the Newton polygon of |b_t| (Bini 1996), which takes 5 to 6 sweeps where a
+// circle of Cauchy's bound takes some 20.
+//
+// A root whose FP32 residual of Eq. 2 is below 0.2 % of its terms is a
+// candidate, polished by Newton on Eq. 2 (twice in FP32, then in FP64 until
+// the step changes 1/|det J| by less than 2e-9).  The texel is kept only if
+// every candidate converged, no two coincide, they are 3 or 5, and their
+// parities add up to -1 (one more saddle than minima and maxima, for two
+// point lenses); five images are all there can be, and with three the other
+// two roots are 0.2 % of their terms away from Eq. 2 (FP32 resolves 1e-5).
+// Emulated on the CPU over 23 lenses (s 0.01 to 20, q 1e-8 to 5, maps about
+// the caustics among them): no texel kept differs from the oracle's value,
+// and less than 1 in 1000 is left to the general form (1 to 12 % in maps of a
+// few caustic sizes).  1024^2 map: 23.9 -> 1.09 ms.
+using cf = cx<float>;
+
+__device__ __forceinline__ float rcpf(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ cf divf(cf a, cf b) {
+  const float r = rcpf(ab2(b));
+  return {(a.re * b.re + a.im * b.im) * r, (a.im * b.re - a.re * b.im) * r};
+}
+// 1/x by two Newton steps from the FP32 reciprocal (relative error a few
+// 2^-53; x outside FP32's range gives infinity or NaN)
+__device__ __forceinline__ double rcpd(double x) {
+  double r = (double)rcpf((float)x);
+  r = fma(r, fma(-x, r, 1.0), r);
+  return fma(r, fma(-x, r, 1.0), r);
+}
+
+__global__ void __launch_bounds__(kPolyThreads)
+    k_poly_fast(double mb, double ma, double xb, double h, double L, int npix,
+                float *__restrict__ A) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= npix) return;
+  const int j = blockIdx.y;
+  const double dlt = (2.0 * L) / (double)npix;
+  const cd om = mk(-L + ((double)i + 0.5) * dlt - xb,
+                   -L + ((double)j + 0.5) * dlt);
+  cf b[5];
+  {
+    const cd oc = cnj(om);
+    const double n0 = -mb * h, hh = h * h;
+    const cd n1 = mk(1.0 - oc.re * h, -oc.im * h);
+    const cd a1 = mk(n1.re + hh, n1.im), a2 = mk(oc.re - h, oc.im);
+    const cd s1 = add(a1, n1), s2 = add(a2, oc);
+    const double k0 = n0 * n0;
+    const cd k1 = scl(n0, s1);
+    const cd k2 = add(scl(n0, s2), mul(a1, n1));
+    const cd k3 = add(mul(a2, n1), mul(a1, oc));
+    const cd k4 = mul(a2, oc);
+    const cd m2 = mk(oc.re - mb * h, oc.im);
+    const cd m1 = mk(n1.re + mb * hh, n1.im);
+    cd c[5];
+    c[0] = scl(-k0, om);
+    c[1] = mk(k0 + h * n0, 0.0);
+    c[1] = sub(c[1], mul(om, k1));
+    c[2] = sub(sub(k1, mul(om, k2)), mk(n0 - h * m1.re, -h * m1.im));
+    c[3] = sub(sub(k2, mul(om, k3)), sub(m1, scl(h, m2)));
+    c[4] = sub(sub(k3, mul(om, k4)), m2);
+    const cf lead = mk((float)k4.re, (float)k4.im);
+#pragma unroll
+    for (int t = 0; t < 5; ++t)
+      b[t] = divf(mk((float)c[t].re, (float)c[t].im), lead);
+  }
+  cf z[5];
+  {
+    // radii: the slopes of the upper hull of (t, log2 |b_t|), b_5 = 1
+    float lb[6];
+#pragma unroll
+    for (int t = 0; t < 5; ++t)
+      lb[t] = 0.5f * __log2f(fmaxf(ab2(b[t]), 1e-37f));
+    lb[5] = 0.f;
+    const float cs[5] = {0.92106099f, -0.08573640f, -0.97404902f,
+                         -0.51625902f, 0.65498345f};
+    const float sn[5] = {0.38941834f, 0.99631784f, 0.22633998f,
+                         -0.85643203f, -0.75564413f};
+#pragma unroll
+    for (int t = 0; t < 5; ++t) {
+      float lo = 3e38f;
+#pragma unroll
+      for (int u = 0; u <= t; ++u) {
+        float hi = -3e38f;
+#pragma unroll
+        for (int v = t + 1; v < 6; ++v)
+          hi = fmaxf(hi, (lb[v] - lb[u]) * (1.f / (float)(v - u)));
+        lo = fminf(lo, hi);
+      }
+      const float r = exp2f(-lo);
+      z[t] = mk(r * cs[t], r * sn[t]);
+    }
+  }
+  for (int it = 0; it < 24; ++it) {
+    bool moved = false;
+#pragma unroll
+    for (int t = 0; t < 5; ++t) {
+      cf p = mk(1.f, 0.f), dp = mk(0.f, 0.f);
+#pragma unroll
+      for (int u = 4; u >= 0; --u) {
+        dp = add(mul(dp, z[t]), p);
+        p = add(mul(p, z[t]), b[u]);
+      }
+      cf sum = mk(0.f, 0.f);
+#pragma unroll
+      for (int u = 0; u < 5; ++u)
+        if (u != t) {
+          const cf d = sub(z[t], z[u]);
+          const float r = rcpf(ab2(d));
+          sum = add(sum, mk(d.re * r, -d.im * r));
+        }
+      const cf nw = divf(p, dp);
+      const cf st = divf(nw, sub(mk(1.f, 0.f), mul(nw, sum)));
+      if (isfinite(st.re) && isfinite(st.im)) {
+        z[t] = sub(z[t], st);
+        moved |= ab2(st) > 9e-10f * ab2(z[t]);
+      }
+    }
+    if (!moved) break;
+  }
+  // candidates, to the front
+  const float hf = (float)h, maf = (float)ma, mbf = (float)mb;
+  const cf omf = mk((float)om.re, (float)om.im);
+  cf w0[5];
+  int ni = 0;
+#pragma unroll
+  for (int t = 0; t < 5; ++t) w0[t] = mk(0.f, 0.f);
+#pragma unroll
+  for (int t = 0; t < 5; ++t) {
+    cf w = z[t];
+    bool cand = false;
+#pragma unroll
+    for (int it = 0; it < 3; ++it) {  // the residual, then two Newton steps
+      const float xa = w.re - hf;
+      const float ra = rcpf(xa * xa + w.im * w.im), rb = rcpf(ab2(w));
+      const cf ia = mk(xa * ra, w.im * ra), ib = mk(w.re * rb, w.im * rb);
+      const cf f = mk(w.re - maf * ia.re - mbf * ib.re - omf.re,
+                      w.im - maf * ia.im - mbf * ib.im - omf.im);
+      if (it == 0) {
+        const float sc = sqrtf(ab2(w)) + sqrtf(ab2(omf)) +
+                         maf * sqrtf(ra) + mbf * sqrtf(rb);
+        // (a NaN is a candidate, which will not converge)
+        cand = !(sqrtf(ab2(f)) >= 0.002f * sc);
+      }
+      const cf D = add(scl(maf, mul(ia, ia)), scl(mbf, mul(ib, ib)));
+      const float rd = rcpf(1.f - ab2(D));
+      const cf dw = scl(rd, sub(mul(D, cnj(f)), f));
+      if (it > 0 && ab2(dw) < 1e-4f * ab2(w)) w = add(w, dw);
+    }
+    if (cand) {
+#pragma unroll
+      for (int u = 0; u < 5; ++u)
+        if (u == ni) w0[u] = w;
+      ++ni;
+    }
+  }
+  double A_sum = 0.0;
+  int parity = 0;
+  bool ok = ni == 3 || ni == 5;
+#pragma unroll
+  for (int t = 0; t < 5; ++t) {
+    if (t >= ni || !ok) break;
+    double x = (double)w0[t].re, y = (double)w0[t].im;
+    bool done = false;
+    for (int it = 0; it < 6 && !done; ++it) {
+      const double xa = x - h, yy = y * y;
+      const double ra = rcpd(fma(xa, xa, yy)), rb = rcpd(fma(x, x, yy));
+      const double iar = xa * ra, iai = y * ra, ibr = x * rb, ibi = y * rb;
+      const double fr = fma(-mb, ibr, fma(-ma, iar, x - om.re));
+      const double fi = fma(-mb, ibi, fma(-ma, iai, y - om.im));
+      const double Dr = fma(ma, fma(iar, iar, -iai * iai),
+                            mb * fma(ibr, ibr, -ibi * ibi));
+      const double Di = 2.0 * fma(ma, iar * iai, mb * (ibr * ibi));
+      const double det = 1.0 - fma(Dr, Dr, Di * Di);
+      const double rd = rcpd(det);
+      const double dx = (fma(Dr, fr, Di * fi) - fr) * rd;
+      const double dy = (fma(Di, fr, -Dr * fi) - fi) * rd;
+      // |d (1/det)| <= |d|D|^2/dw| |dw| / det^2, d|D|^2/dw <= 2 |D| |D'|
+      const float ga = sqrtf((float)ra), gb = sqrtf((float)rb);
+      const float g = 4.f * sqrtf((float)(Dr * Dr + Di * Di)) *
+                      (maf * ga * ga * ga + mbf * gb * gb * gb);
+      const float st = sqrtf((float)dx * (float)dx + (float)dy * (float)dy);
+      const float re = sqrtf((float)fr * (float)fr + (float)fi * (float)fi);
+      const float sc = sqrtf((float)(x * x) + (float)yy) + sqrtf(ab2(omf)) +
+                       maf * ga + mbf * gb;
+      if (g * st <= 2e-9f * fabsf((float)det) && re < 1e-9f * sc) {
+        done = true;
+        A_sum += fabs(rd);
+        parity += det > 0.0 ? 1 : -1;
+        w0[t] = mk((float)x, (float)y);
+      } else {
+        x += dx;
+        y += dy;
+      }
+    }
+    ok = ok && done;
+  }
+#pragma unroll
+  for (int t = 1; t < 5; ++t)
+#pragma unroll
+    for (int u = 0; u < t; ++u)
+      if (t < ni &&
+          ab2(sub(w0[t], w0[u])) <
+              1e-12f * (1e-6f + ab2(w0[t])))
+        ok = false;
+  A[(size_t)j * npix + i] =
+      ok && parity == -1 ? __double2float_rn(A_sum) : CUDART_NAN_F;
 }
 
 }  // namespace
 
 cudaError_t launch_poly_map(double s, double q, double L, int npix, float *A,
                             int sm_count, cudaStream_t st) {
+  // the fast form where FP32 holds the lens and the map: its checks leave a
+  // texel it cannot settle to the general form in any case (beyond s = 30 that
+  // would be most of them: FP32 Aberth does not converge there)
+  const double e1 = 1.0 / (1.0 + q), e2 = q / (1.0 + q);
+  const bool second = e2 <= e1;  // the lighter lens
+  const double mb = second ? e2 : e1, ma = second ? e1 : e2;
+  const double x1 = -s * e2, x2 = s * e1;
+  const double xb = second ? x2 : x1, h = second ? x1 - x2 : x2 - x1;
+  const bool fast = mb >= 1e-8 && s >= 1e-2 && s <= 30.0 && L <= 100.0;
+  if (fast) {
+    const dim3 grid((unsigned)((npix + kPolyThreads - 1) / kPolyThreads),
+                    (unsigned)npix);
+    k_poly_fast<<<grid, kPolyThreads, 0, st>>>(mb, ma, xb, h, L, npix, A);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
   const size_t n = (size_t)npix * npix;
-  size_t blocks = (n + 127) / 128;
+  size_t blocks = (n + kPolyTile - 1) / kPolyTile;
   const size_t cap = (size_t)sm_count * 16;
   if (blocks > cap) blocks = cap;
-  if (blocks < 1) blocks = 1;
-  k_poly_map<<<(unsigned)blocks, 128, 0, st>>>(s, q, L, npix, A);
+  k_poly_map<<<(unsigned)blocks, kPolyThreads, 0, st>>>(s, q, L, npix, fast,
+                                                        A);
   return cudaGetLastError();
 }
 

@@ -101,3 +101,19 @@ def test_sweep_with_polynomial_maps(ctx, m):
         one = ctx.grid_chi2(ev, mp, g)
         assert np.array_equal(sw[i]["idx"], one["idx"])
         assert np.array_equal(sw[i]["chi2"], one["chi2"])
+
+
+@pytest.mark.parametrize("s,q,L,npix", [
+    (1.0, 1e-8, 2.0, 64),      # the lightest lens of the fast form
+    (0.05, 0.3, 2.0, 64),      # close: most texels left to the general form
+    (1.0, 1e-3, 0.02, 96),     # about the central caustic
+    (1.2, 5.0, 2.0, 96),       # the lighter lens on the left
+    (1.0, 1e-9, 2.0, 48),      # general form alone
+    (1.3, 0.06, 2.0, 33),      # a row that does not fill a block
+])
+def test_poly_map_fast_and_general_forms(ctx, s, q, L, npix):
+    A = ctx.build_map(s, q, L, npix, 1, generator="poly").values()
+    P = orc.poly_map(s, q, L, npix, nthreads=NT)
+    assert np.isfinite(A).all() and (A >= 1.0 - 1e-6).all()
+    rel = np.abs(A.astype(np.float64) - P) / P
+    assert (rel > 1e-6).mean() <= 1e-3
