@@ -2039,44 +2039,22 @@ morse_status morse_map_finite_source(morse_ctx *ctx, const morse_map *src,
   const int R = (int)ceil(rpx + 0.5);
   const int side = 2 * R + 1;
   MORSE_CUDA(ctx, cudaSetDevice(ctx->device));
-  // the profile integrated over each texel on 8 x 8 midpoint points, on the
-  // device; normalised and rounded to FP32 here
-  std::vector<double> w((size_t)side * side, 0.0);
-  {
-    void *ws0 = nullptr;
-    MORSE_TRY(ws_reserve(ctx, sizeof(double) * w.size(), &ws0));
-    MORSE_CUDA(ctx, morse::launch_fs_weights(rpx, gamma, R, (double *)ws0,
-                                             ctx->stream));
-    ctx->launches += 1;
-    MORSE_CUDA(ctx, cudaMemcpyAsync(w.data(), ws0, sizeof(double) * w.size(),
-                                    cudaMemcpyDeviceToHost, ctx->stream));
-    MORSE_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-  }
-  double tot = 0.0;
-  for (double v : w) tot += v;
-  if (!(tot > 0.0)) {  // sub-texel source: the centre texel alone
-    std::fill(w.begin(), w.end(), 0.0);
-    w[(size_t)R * side + R] = 1.0;
-    tot = 1.0;
-  }
-  std::vector<float> wf(w.size());
-  std::vector<int> hw((size_t)side, -1);
-  for (int dy = 0; dy < side; ++dy)
-    for (int dx = 0; dx < side; ++dx) {
-      const double v = w[(size_t)dy * side + dx] / tot;
-      wf[(size_t)dy * side + dx] = (float)v;
-      if (v != 0.0) hw[(size_t)dy] = std::max(hw[(size_t)dy], std::abs(dx - R));
-    }
+  // the profile integrated over each texel on 8 x 8 midpoint points,
+  // normalised and rounded to FP32, all on the device
   call_begin(ctx);
-  const size_t wbytes = align_up(sizeof(float) * wf.size(), 256);
+  const size_t n_w = (size_t)side * side;
+  const size_t off_wf = align_up(sizeof(double) * n_w, 256);
+  const size_t off_rows = align_up(off_wf + sizeof(float) * n_w, 256);
+  const size_t off_hw = align_up(off_rows + sizeof(double) * side, 256);
   void *ws = nullptr;
-  MORSE_TRY(ws_reserve(ctx, wbytes + sizeof(int) * hw.size(), &ws));
-  float *dW = (float *)ws;
-  int *dhw = (int *)((char *)ws + wbytes);
-  MORSE_CUDA(ctx, cudaMemcpyAsync(dW, wf.data(), sizeof(float) * wf.size(),
-                                  cudaMemcpyHostToDevice, ctx->stream));
-  MORSE_CUDA(ctx, cudaMemcpyAsync(dhw, hw.data(), sizeof(int) * hw.size(),
-                                  cudaMemcpyHostToDevice, ctx->stream));
+  MORSE_TRY(ws_reserve(ctx, off_hw + sizeof(int) * (size_t)side, &ws));
+  float *dW = (float *)((char *)ws + off_wf);
+  int *dhw = (int *)((char *)ws + off_hw);
+  MORSE_CUDA(ctx, morse::launch_fs_weights(
+                      rpx, gamma, R, (double *)ws,
+                      (double *)((char *)ws + off_rows), dW, dhw,
+                      ctx->stream));
+  ctx->launches += 3;
   morse_map *m = map_alloc(ctx, npix, false);
   if (!m) return fail(ctx, MORSE_ENOMEM, "map of %d^2 texels", npix);
   m->L = src->L;

@@ -80,3 +80,23 @@ def test_finite_source_rejects_bad_arguments(ctx, m, base_map):
         with pytest.raises(m.MorseError) as e:
             mp.finite_source(rho, gamma)
         assert e.value.status == m.EINVAL
+
+
+# both sides of every change of kernel: unfolded below 64 texels, two groups
+# of threads up to 140, four with four or eight staged values a thread, and
+# unfolded again; maps narrower than a tile and ragged
+@pytest.mark.parametrize("rho_px,npix", [(62.4, 70), (63.4, 70),
+                                         (139.4, 33), (140.4, 65),
+                                         (311.0, 20), (313.0, 20),
+                                         (650.0, 17), (700.0, 17)])
+def test_folded_convolution_matches_oracle(ctx, rho_px, npix):
+    rng = np.random.default_rng(int(rho_px))
+    A = np.exp(rng.normal(0.0, 1.0, (npix, npix))).astype(np.float32)
+    L = 2.0
+    mp = ctx.map_from_host(A, L)
+    fs = mp.finite_source(rho_px * 2 * L / npix, 0.53)
+    got = fs.values().astype(np.float64)
+    ref = orc.fs_convolve(A, L, orc.fs_weights(rho_px, 0.53), nthreads=NT)
+    assert np.max(np.abs(got - ref) / ref) <= 2e-6
+    fs.free()
+    mp.free()
