@@ -30,6 +30,13 @@
 // Where the subsets discard too little (light curves of weak signal), the
 // whole range is searched as before (k_search), the screening costing a
 // share 64 / n_epochs.
+//
+// Grids of up to kSmallGrid trajectories are too few to rank by subsets and
+// bound by latency: k_bounds takes upper and lower bounds of all of them over
+// the whole light curve, spread over every SM (in k_search they are the FP64
+// solves and the ordered merges of 16 warps on a few SMs), and k_list and the
+// listed search follow.  3600 trajectories x 201 epochs, a call: 208 -> 111
+// us.
 #ifndef MORSE_PK_ASM
 #define MORSE_PK_ASM 1
 #endif
@@ -352,7 +359,7 @@ __device__ __forceinline__ void append(const SearchParams &P,
                                        const Keep &keep) {
   constexpr int kPer = 8;  // codes per thread: one 16-byte load
   const unsigned n = (unsigned)P.count;
-  const bool tf = by_t0(P);
+  const bool tf = B.pilot && by_t0(P);  // (small grids: the grid order)
   __shared__ unsigned s_w[32], s_base;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nw = blockDim.x >> 5;
@@ -442,12 +449,14 @@ __device__ __forceinline__ void make_pilot_list(const SearchParams &P,
 // one warp), and one warp adds the slices and solves.
 constexpr int kPilotTpg = 8, kPilotWarps = 8;
 
-template <bool H>
+// ALL: the entries are the trajectories themselves (small grids), and their
+// lower bounds (solve2's) are coded too.
+template <bool H, bool ALL>
 __device__ __forceinline__ void pilot_bounds(const SearchParams &P,
                                              const ScreenBufs &B) {
   __shared__ Acc s_acc[kPilotWarps][kPilotTpg];
   __shared__ TrajC s_c[kPilotTpg];
-  const unsigned n = min(B.n[0], B.pilot_cap);
+  const unsigned n = ALL ? (unsigned)P.count : min(B.n[0], B.pilot_cap);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned g0 = blockIdx.x * kPilotTpg;
   if (g0 >= n) return;
@@ -455,8 +464,9 @@ __device__ __forceinline__ void pilot_bounds(const SearchParams &P,
   Epochs ep = epochs_at(P.ep, P.n_ep);
   if (warp == 0) {  // once: the constants' FP64 would be the block's limit
     double xi, xo;
-    TrajC c = traj_base_of(
-        P, (unsigned)P.first + B.pilot[g0 + (lane < nv ? lane : 0)], xi, xo);
+    const unsigned k = g0 + (lane < nv ? lane : 0);
+    TrajC c = traj_base_of(P, (unsigned)P.first + (ALL ? k : B.pilot[k]), xi,
+                           xo);
     traj_range(ep, P.n_ep, xi, xo, c);
     if (lane < kPilotTpg) s_c[lane] = c;
   }
@@ -497,7 +507,26 @@ __device__ __forceinline__ void pilot_bounds(const SearchParams &P,
       chi2_upper(P, (double)ms.a, (double)ms.b, (double)ms.d,
                  (double)__double2float_rn(f.Fs),
                  (double)__double2float_rn(f.Bc), gamma);
-  if (lane < nv) B.ub[g0 + lane] = fmaxf(__double2float_ru(ub), 0.f);
+  float up = fmaxf(__double2float_ru(ub), 0.f);
+  if (ALL) {
+    SearchParams Q = P;
+    Q.gamma = gamma;
+    const Solved o =
+        solve2(Q, (double)ms.a, (double)ms.b, (double)ms.d);
+    // may_reach's bound and margin, rounded down
+    const double lb =
+        o.bden > 0.0 ? (P.CFF - o.bnum / o.bden) * (1.0 - 1.01e-4) : 0.0;
+    unsigned code = __float_as_uint(lb > 0.0 ? __double2float_rd(lb) : 0.f)
+                    >> 16;
+    if (P.linemax && lane < nv &&
+        __ldg(&P.linemax[((unsigned)P.first + g0 + lane) /
+                         (unsigned)P.line]) < P.a_min) {
+      code = kScreenCut;  // not searched, and no bound for the others
+      up = CUDART_INF_F;
+    }
+    if (lane < nv) B.code[g0 + lane] = (unsigned short)code;
+  }
+  if (lane < nv) B.ub[g0 + lane] = up;
 }
 
 // The threshold: the top_k-th smallest of the pilot's bounds (K distinct
@@ -506,7 +535,8 @@ __device__ __forceinline__ void pilot_bounds(const SearchParams &P,
 __device__ __forceinline__ void make_list(const SearchParams &P,
                                           const ScreenBufs &B) {
   __shared__ unsigned s_h[256], s_bits, s_left;
-  const unsigned n = min(B.n[0], B.pilot_cap);
+  const unsigned n =
+      B.pilot ? min(B.n[0], B.pilot_cap) : (unsigned)P.count;
   const unsigned K = (unsigned)P.top_k;
   unsigned thr = 0x7F800000u;  // +inf
   if (n >= K) {
@@ -676,10 +706,18 @@ __device__ __forceinline__ void load_task(const ScreenTask *t, ScreenTask &s) {
   }
 MORSE_SCREEN_KERNELS(k_screen, screen_all<H>, kScreenThreads, 4)
 MORSE_SCREEN_KERNELS(k_pilot_list, make_pilot_list, kListThreads, 1)
-MORSE_SCREEN_KERNELS(k_pilot, pilot_bounds<H>, kPilotWarps * 32, 4)
+#define MORSE_PILOT(P, B) pilot_bounds<H, false>(P, B)
+MORSE_SCREEN_KERNELS(k_pilot, MORSE_PILOT, kPilotWarps * 32, 4)
+#undef MORSE_PILOT
 MORSE_SCREEN_KERNELS(k_list, make_list, kListThreads, 1)
 MORSE_SCREEN_KERNELS(k_rescreen, rescreen_listed<H>, kScreenThreads, 4)
 #undef MORSE_SCREEN_KERNELS
+
+template <bool H>
+__global__ void __launch_bounds__(kPilotWarps * 32, 4)
+    k_bounds(const SearchParams P, const ScreenBufs B) {
+  pilot_bounds<H, true>(P, B);
+}
 
 }  // namespace
 
@@ -714,6 +752,16 @@ cudaError_t launch_screen_pilot(const SearchParams &P, const ScreenBufs &B,
     k_pilot<true><<<grid, kPilotWarps * 32, 0, st>>>(P, B);
   else
     k_pilot<false><<<grid, kPilotWarps * 32, 0, st>>>(P, B);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_bounds(const SearchParams &P, const ScreenBufs &B,
+                          cudaStream_t st) {
+  const int grid = (int)((P.count + kPilotTpg - 1) / kPilotTpg);
+  if (P.quadh)
+    k_bounds<true><<<grid, kPilotWarps * 32, 0, st>>>(P, B);
+  else
+    k_bounds<false><<<grid, kPilotWarps * 32, 0, st>>>(P, B);
   return cudaGetLastError();
 }
 

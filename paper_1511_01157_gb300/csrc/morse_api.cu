@@ -583,7 +583,9 @@ struct Plan {
   int grid;
   size_t off_tab, off_lmax, off_hdr, off_pub, off_pa, off_pb, off_out, bytes;
   int tab_n;  // band-table entries (0: the search reads the global table)
-  // screened search (k_screen.cu); want = 0: off
+  // screened search (k_screen.cu); want = 0: off; small: of a small grid,
+  // every trajectory a pilot
+  bool small;
   unsigned want, pilot_cap, list0_cap, list_cap;
   size_t off_code, off_hist, off_pil, off_ub, off_list0, off_list, off_cand;
 };
@@ -642,11 +644,27 @@ double pilot_want(int K, long long count) {
 // Whether a top-K search of `count` trajectories is screened, and the
 // workspace of it from offset `at` on.
 size_t plan_screen(const morse_event *ev, const morse_grid *g,
-                   long long count, size_t at, Plan *pl) {
+                   long long count, bool small_ok, size_t at, Plan *pl) {
   pl->want = 0;
+  pl->small = false;
   const double want = std::max(pilot_want(pl->K, count), 512.0);
   const double total =
       (double)g->n_u0 * g->n_alpha * (double)g->n_t0 * g->n_tE;
+  if (small_ok && count <= morse::kSmallGrid && total < 2147483648.0) {
+    pl->small = true;
+    pl->want = pl->pilot_cap = pl->list0_cap = pl->list_cap = (unsigned)count;
+    pl->off_hist = align_up(at, 256);
+    pl->off_code = align_up(
+        pl->off_hist + sizeof(unsigned) * (morse::kScreenBins +
+                                           morse::kScreenWords), 256);
+    pl->off_pil = pl->off_ub = align_up(
+        pl->off_code + sizeof(unsigned short) * (size_t)(count + 8), 256);
+    pl->off_list0 = pl->off_list = align_up(
+        pl->off_ub + sizeof(float) * (size_t)count, 256);
+    pl->off_cand = align_up(
+        pl->off_list + sizeof(unsigned) * (size_t)count, 256);
+    return pl->off_cand + sizeof(morse::Candidate) * morse::kCandMax;
+  }
   if (ev->n_sub < 1 || count < 16384 || count > (1LL << 25) ||
       total >= 2147483648.0 || want * 4.0 > (double)count)
     return at;
@@ -687,6 +705,10 @@ void screen_bufs(const Plan &pl, char *base, char *words,
   B->list0_cap = pl.list0_cap;
   B->list_cap = pl.list_cap;
   B->want = pl.want;
+  if (pl.small) {
+    B->pilot = nullptr;
+    P->n_lv = 0;  // no subsets
+  }
   const bool two = P->n_lv > 2;  // a rescreened list
   if (!two) {  // list0 is the final list
     B->list0 = B->list;
@@ -797,7 +819,8 @@ morse_status plan_search(morse_ctx *ctx, const morse_event *ev,
                            : sizeof(morse_fit) * (size_t)K * (size_t)n_out;
   pl->bytes = pl->off_out + out_bytes;
   pl->want = 0;
-  if (!dense) pl->bytes = plan_screen(ev, g, count, pl->bytes, pl);
+  pl->small = false;
+  if (!dense) pl->bytes = plan_screen(ev, g, count, true, pl->bytes, pl);
   return MORSE_OK;
 }
 
@@ -866,10 +889,15 @@ morse_status enqueue_topk(morse_ctx *ctx, const Plan &pl,
                                             morse::kScreenWords),
                         ctx->stream));
     r = t_begin(ctx, KT_SEARCH);
-    MORSE_CUDA(ctx, morse::launch_screen(P, B, ctx->sm_count, ctx->stream));
-    MORSE_CUDA(ctx, morse::launch_screen_pilot_list(P, B, ctx->sm_count,
-                                                    ctx->stream));
-    MORSE_CUDA(ctx, morse::launch_screen_pilot(P, B, ctx->stream));
+    if (pl.small) {
+      MORSE_CUDA(ctx, morse::launch_bounds(P, B, ctx->stream));
+    } else {
+      MORSE_CUDA(ctx, morse::launch_screen(P, B, ctx->sm_count, ctx->stream));
+      MORSE_CUDA(ctx, morse::launch_screen_pilot_list(P, B, ctx->sm_count,
+                                                      ctx->stream));
+      MORSE_CUDA(ctx, morse::launch_screen_pilot(P, B, ctx->stream));
+      ctx->launches += 2;
+    }
     MORSE_CUDA(ctx, morse::launch_screen_list(P, B, ctx->sm_count,
                                               ctx->stream));
     done = B.n + 7;
@@ -885,7 +913,23 @@ morse_status enqueue_topk(morse_ctx *ctx, const Plan &pl,
     MORSE_CUDA(ctx, morse::launch_search_list(P, staged, list_grid, list_smem,
                                               ctx->stream));
     t_end(ctx, r);
-    ctx->launches += 5;
+    ctx->launches += 3;
+  }
+  if (list_grid > 0 && pl.small) {
+    // always a list, and never more candidates than fit
+    morse::FillParams F;
+    F.S = P;
+    F.sel = nullptr;
+    F.k = pl.K;
+    F.t0abs = T.t0abs;
+    F.tEv = T.tEv;
+    F.out = fits_dev;
+    F.done = done;
+    r = t_begin(ctx, KT_FILL);
+    MORSE_CUDA(ctx, morse::launch_finish(F, ctx->stream));
+    t_end(ctx, r);
+    ctx->launches += 1;
+    return MORSE_OK;
   }
   // pilot: a strided subset of ~sqrt(K N) trajectories (at least 16 K)
   // seeds the grid-wide pruning threshold
@@ -1300,7 +1344,7 @@ morse_status batch_prepare(morse_ctx *ctx, const morse_event *const *evs,
     if (evs[e]->n_sub > most->n_sub) most = evs[e];
   }
   if (screen) {
-    H.scr.bytes = align_up(plan_screen(most, g, N, 0, &H.scr), 256);
+    H.scr.bytes = align_up(plan_screen(most, g, N, false, 0, &H.scr), 256);
     if (H.scr.want > 0) {
       // as many pairs at a time as 512 MB of scratch hold
       H.chunk = (int)std::max<size_t>(

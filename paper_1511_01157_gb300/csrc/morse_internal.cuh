@@ -341,7 +341,8 @@ struct ScreenBufs {
                             // whole (4: nonzero), discarded (5); candidates
                             // of the listed search (6), records made (7:
                             // nonzero)
-  unsigned *pilot;          // [pilot_cap] trajectories of the pilot
+  unsigned *pilot;          // [pilot_cap] trajectories of the pilot (null:
+                            // all of a small grid, ub[count])
   float *ub;                // [pilot_cap] their chi^2 bounds from above
   unsigned *list0;          // [list0_cap] trajectories the codes leave
   unsigned *list;           // [list_cap] those left after the rescreening
@@ -464,6 +465,10 @@ cudaError_t launch_screen(const SearchParams &P, const ScreenBufs &B,
 cudaError_t launch_screen_pilot_list(const SearchParams &P,
                                      const ScreenBufs &B, int sm_count,
                                      cudaStream_t st);
+// both bounds of every trajectory of a small grid (P.count <= kSmallGrid)
+constexpr long long kSmallGrid = kCandMax;
+cudaError_t launch_bounds(const SearchParams &P, const ScreenBufs &B,
+                          cudaStream_t st);
 // their upper bounds
 cudaError_t launch_screen_pilot(const SearchParams &P, const ScreenBufs &B,
                                 cudaStream_t st);

@@ -133,3 +133,33 @@ def test_screened_batch_equals_single_searches(m, setup):
                 assert np.array_equal(got[i, j], ctx.grid_chi2(ev, x, g))
     mp.set_lookup(False)
     other.free()
+
+
+@pytest.mark.parametrize("n", [3, 33, 257, 3001])
+@pytest.mark.parametrize("dims", [(1, 1, 1, 1), (3, 7, 2, 3),
+                                  (8, 16, 8, 8), (9, 16, 8, 8)])
+def test_small_grid_equals_dense(m, setup, dims, n):
+    """Up to 8192 trajectories every one is bounded over the whole light
+    curve; just above, the unscreened search."""
+    ctx, mp = setup
+    g = m.Grid.make(*dims, 1e-3, 0.5, -2.0, 2.0, 5.0, 80.0, True, True, 37)
+    for kind in ("strong", "flat"):
+        ev = _event(ctx, n, kind)
+        got = ctx.grid_chi2(ev, mp, g)
+        chi2, fs, fb = ctx.grid_chi2_dense(ev, mp, g)
+        idx, val = _best(chi2, 37)
+        k = len(idx)
+        assert np.array_equal(got["idx"][:k], idx)
+        assert np.array_equal(got["chi2"][:k], val)
+        assert np.array_equal(got["Fs"][:k], fs[idx])
+        assert np.all(got["idx"][k:] == -1)
+    if g.size > 100:
+        cut = m.Grid.make(*dims, 1e-3, 0.5, -2.0, 2.0, 5.0, 80.0, True, True,
+                          37, float(np.median(ctx.line_max(mp, g))))
+        kept, *_ = ctx.grid_chi2_dense(ev, mp, cut)
+        idx, val = _best(kept, 37)
+        got = ctx.grid_chi2(ev, mp, cut)
+        assert np.array_equal(got["idx"][:len(idx)], idx)
+        r = ctx.grid_chi2_range(ev, mp, g, 5, 91)
+        idx, val = _best(chi2[5:96], 37, 5)
+        assert np.array_equal(r["idx"], idx)
