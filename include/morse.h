@@ -29,7 +29,9 @@
  *  - Errors: every call returns a morse_status; morse_last_error() gives a
  *    message for the context's most recent failure.  No call aborts, traps
  *    or throws.  Invalid arguments return MORSE_EINVAL before any GPU work.
- *  - Memory: handles own their device memory; input arrays are copied and
+ *  - Memory: handles own their device memory (freed map and event memory
+ *    stays with the context, at most 256 MB of it, for its next handles,
+ *    until morse_destroy); input arrays are copied and
  *    stay owned by the caller; output arrays are caller-allocated HOST
  *    memory unless the name ends in _dev.  Calls are synchronous on the
  *    context's stream unless noted.

@@ -210,6 +210,9 @@ morse_status check_build(morse_ctx *ctx, double s, double q, double extent,
 }
 
 // ---------------------------------------------------------------- maps
+// to the context's pool, after the stream's work so far
+void pool_free(morse_ctx *ctx, void *p) { cudaFreeAsync(p, ctx->stream); }
+
 morse_map *map_alloc(morse_ctx *ctx, int npix, bool counts) {
   morse_map *m = (morse_map *)calloc(1, sizeof(morse_map));
   if (!m) return nullptr;
@@ -218,22 +221,22 @@ morse_map *map_alloc(morse_ctx *ctx, int npix, bool counts) {
   size_t n = (size_t)npix * npix;
   m->qpitch = morse::quad_pitch(npix);
   bool ok =
-      morse::dev_alloc(ctx, (void **)&m->A, n * sizeof(float)) ==
+      morse::pool_alloc(ctx, (void **)&m->A, n * sizeof(float)) ==
           cudaSuccess &&
-      morse::dev_alloc(ctx, (void **)&m->quad,
+      morse::pool_alloc(ctx, (void **)&m->quad,
                        morse::quad_count(npix) * sizeof(float4)) ==
           cudaSuccess &&
-      morse::dev_alloc(ctx, (void **)&m->tot,
+      morse::pool_alloc(ctx, (void **)&m->tot,
                        4 * sizeof(unsigned long long)) == cudaSuccess;
   if (ok && counts)
-    ok = morse::dev_alloc(ctx, (void **)&m->counts,
+    ok = morse::pool_alloc(ctx, (void **)&m->counts,
                           n * sizeof(uint32_t)) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
-    if (m->A) cudaFree(m->A);
-    if (m->quad) cudaFree(m->quad);
-    if (m->tot) cudaFree(m->tot);
-    if (m->counts) cudaFree(m->counts);
+    if (m->A) pool_free(ctx, m->A);
+    if (m->quad) pool_free(ctx, m->quad);
+    if (m->tot) pool_free(ctx, m->tot);
+    if (m->counts) pool_free(ctx, m->counts);
     free(m);
     return nullptr;
   }
@@ -245,13 +248,13 @@ morse_map *map_alloc(morse_ctx *ctx, int npix, bool counts) {
 bool map_ensure_half(morse_map *m) {
   if (m->quadh) return true;
   size_t n = (size_t)m->npix * m->npix;
-  if (morse::dev_alloc(m->ctx, (void **)&m->hcodes, n * sizeof(uint16_t)) !=
+  if (morse::pool_alloc(m->ctx, (void **)&m->hcodes, n * sizeof(uint16_t)) !=
           cudaSuccess ||
-      morse::dev_alloc(m->ctx, (void **)&m->quadh,
+      morse::pool_alloc(m->ctx, (void **)&m->quadh,
                        morse::quad_count(m->npix) * sizeof(uint2)) !=
           cudaSuccess) {
     cudaGetLastError();
-    if (m->hcodes) cudaFree(m->hcodes);
+    if (m->hcodes) pool_free(m->ctx, m->hcodes);
     m->hcodes = nullptr;
     m->quadh = nullptr;
     return false;
@@ -273,12 +276,9 @@ morse_status enqueue_half(morse_ctx *ctx, morse_map *m) {
 
 void map_release(morse_map *m) {
   if (!m) return;
-  if (m->hcodes) cudaFree(m->hcodes);
-  if (m->quadh) cudaFree(m->quadh);
-  if (m->A) cudaFree(m->A);
-  if (m->quad) cudaFree(m->quad);
-  if (m->tot) cudaFree(m->tot);
-  if (m->counts) cudaFree(m->counts);
+  for (void *p : {(void *)m->hcodes, (void *)m->quadh, (void *)m->A,
+                  (void *)m->quad, (void *)m->tot, (void *)m->counts})
+    if (p) pool_free(m->ctx, p);
   free(m);
 }
 
@@ -479,6 +479,20 @@ void tables_at(const morse_grid *g, void *dev, Tables *T) {
   T->invtEd = T->t0rel + g->n_t0;
   T->t0abs = T->invtEd + g->n_tE;
   T->tEv = T->t0abs + g->n_t0;
+}
+
+cudaError_t pool_alloc(morse_ctx *ctx, void **p, size_t bytes) {
+  *p = nullptr;
+  if (ctx->fault_alloc > 0 && --ctx->fault_alloc == 0)
+    return cudaErrorMemoryAllocation;  // injected: nothing allocated
+  cudaError_t e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, ctx->stream);
+  if (e == cudaErrorMemoryAllocation) {  // once more without what is kept
+    cudaGetLastError();
+    cudaStreamSynchronize(ctx->stream);
+    cudaMemPoolTrimTo(ctx->pool, 0);
+    e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, ctx->stream);
+  }
+  return e;
 }
 
 cudaError_t dev_alloc(morse_ctx *ctx, void **p, size_t bytes) {
@@ -1818,6 +1832,9 @@ const char *morse_version(void) {
 const char *morse_version(void) { return "morse-gb300 0.1 sm_103a"; }
 #endif
 
+// freed map and event memory a context keeps for its next ones
+static const unsigned long long kPoolKeep = 256ULL << 20;
+
 morse_status morse_create(morse_ctx **out, int device, void *cuda_stream) {
   if (!out) return MORSE_EINVAL;
   *out = nullptr;
@@ -1861,6 +1878,30 @@ morse_status morse_create(morse_ctx **out, int device, void *cuda_stream) {
     }
     c->own_stream = true;
   }
+  // Maps and events come from a pool of the context: cudaMalloc and cudaFree
+  // of a map's tables (25 MB at 1024^2) cost more than building it.  The
+  // pool keeps at most kPoolKeep bytes of freed memory, in the stream's
+  // order, and is destroyed with the context.
+  {
+    cudaMemPoolProps pp;
+    memset(&pp, 0, sizeof(pp));
+    pp.allocType = cudaMemAllocationTypePinned;
+    pp.location.type = cudaMemLocationTypeDevice;
+    pp.location.id = device;
+    unsigned long long keep = kPoolKeep;
+    cudaError_t e = cudaMemPoolCreate(&c->pool, &pp);
+    if (e == cudaSuccess) {
+      e = cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold,
+                                  &keep);
+      if (e != cudaSuccess) cudaMemPoolDestroy(c->pool);
+    }
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      if (c->own_stream) cudaStreamDestroy(c->stream);
+      delete c;
+      return MORSE_ECUDA;
+    }
+  }
   *out = c;
   return MORSE_OK;
 }
@@ -1879,6 +1920,8 @@ void morse_destroy(morse_ctx *ctx) {
   if (ctx->batch_exec) cudaGraphExecDestroy(ctx->batch_exec);
   if (ctx->ws) cudaFree(ctx->ws);
   for (cudaEvent_t e : ctx->evpool) cudaEventDestroy(e);
+  cudaStreamSynchronize(ctx->stream);
+  cudaMemPoolDestroy(ctx->pool);  // (its memory once every handle is freed)
   if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
   delete ctx;
 }
@@ -2164,7 +2207,6 @@ morse_status morse_map_half(const morse_map *map, uint16_t *host_codes,
 
 void morse_map_free(morse_map *map) {
   if (!map) return;
-  cudaStreamSynchronize(map->ctx->stream);
   map_release(map);
 }
 
@@ -2344,7 +2386,7 @@ morse_status morse_event_create(morse_ctx *ctx, const double *t,
   morse_event *ev = (morse_event *)calloc(1, sizeof(morse_event));
   if (!ev) return fail(ctx, MORSE_ENOMEM, "event");
   screen_subsets(ev, h, n, S1, SF, SFF);
-  if (morse::dev_alloc(ctx, (void **)&ev->ep, sizeof(float4) * h.size()) !=
+  if (morse::pool_alloc(ctx, (void **)&ev->ep, sizeof(float4) * h.size()) !=
       cudaSuccess) {
     cudaGetLastError();
     free(ev);
@@ -2356,7 +2398,7 @@ morse_status morse_event_create(morse_ctx *ctx, const double *t,
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
   if (e != cudaSuccess) {
     cudaStreamSynchronize(ctx->stream);
-    cudaFree(ev->ep);
+    pool_free(ctx, ev->ep);
     free(ev);
     return cuda_fail(ctx, e, "event upload");
   }
@@ -2376,8 +2418,7 @@ morse_status morse_event_create(morse_ctx *ctx, const double *t,
 
 void morse_event_free(morse_event *ev) {
   if (!ev) return;
-  cudaStreamSynchronize(ev->ctx->stream);
-  if (ev->ep) cudaFree(ev->ep);
+  if (ev->ep) pool_free(ev->ctx, ev->ep);
   free(ev);
 }
 

@@ -22,6 +22,8 @@ struct morse_ctx {
   int sm_count;
   size_t smem_optin;        // max dynamic shared memory per block
   char err[512];
+  cudaMemPool_t pool;       // memory of maps and events, in the stream's
+                            // order
   void *ws;                 // device workspace (grow-only)
   size_t ws_bytes;
   // per-call kernel timing: event pairs recorded around each launch, summed
@@ -375,6 +377,9 @@ void map_params(const morse_map *map, SearchParams *P);
 void event_params(const morse_event *ev, SearchParams *P);
 void grid_params(const morse_grid *g, const Tables &T, SearchParams *P);
 void ctx_params(const morse_ctx *ctx, SearchParams *P);
+// device allocation from the context's pool on its stream, or the injected
+// failure
+cudaError_t pool_alloc(morse_ctx *ctx, void **p, size_t bytes);
 // device allocation through the context: cudaMalloc, or the injected
 // failure of morse_inject_fault (cudaErrorMemoryAllocation, nothing made)
 cudaError_t dev_alloc(morse_ctx *ctx, void **p, size_t bytes);
