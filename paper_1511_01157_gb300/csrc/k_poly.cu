@@ -309,8 +309,8 @@ __global__ void __launch_bounds__(kPolyThreads)
 // A root whose FP32 residual of Eq. 2 is below 0.2 % of its terms is a
 // candidate, polished by Newton on Eq. 2 (twice in FP32, then in FP64 until
 // the step changes 1/|det J| by less than 2e-9).  The texel is kept only if
-// every candidate converged, no two coincide, they are 3 or 5, and their
-// parities add up to -1 (one more saddle than minima and maxima, for two
+// every candidate became an image of its own or is shown to be none
+// (spurious), they are 3 or 5, and their parities add up to -1 (one more saddle than minima and maxima, for two
 // point lenses); five images are all there can be, and with three the other
 // two roots are 0.2 % of their terms away from Eq. 2 (FP32 resolves 1e-5).
 // Emulated on the CPU over 23 lenses (s 0.01 to 20, q 1e-8 to 5, maps about
@@ -336,6 +336,63 @@ __device__ __forceinline__ double rcpd(double x) {
   return fma(r, fma(-x, r, 1.0), r);
 }
 
+// coefficients of the quintic, c[5] the leading one
+__device__ __forceinline__ void quintic(double mb, double h, cd om,
+                                        cd (&c)[6]) {
+  const cd oc = cnj(om);
+  const double n0 = -mb * h, hh = h * h;
+  const cd n1 = mk(1.0 - oc.re * h, -oc.im * h);
+  const cd a1 = mk(n1.re + hh, n1.im), a2 = mk(oc.re - h, oc.im);
+  const cd s1 = add(a1, n1), s2 = add(a2, oc);
+  const double k0 = n0 * n0;
+  const cd k1 = scl(n0, s1);
+  const cd k2 = add(scl(n0, s2), mul(a1, n1));
+  const cd k3 = add(mul(a2, n1), mul(a1, oc));
+  const cd k4 = mul(a2, oc);
+  const cd m2 = mk(oc.re - mb * h, oc.im);
+  const cd m1 = mk(n1.re + mb * hh, n1.im);
+  c[0] = scl(-k0, om);
+  c[1] = mk(k0 + h * n0, 0.0);
+  c[1] = sub(c[1], mul(om, k1));
+  c[2] = sub(sub(k1, mul(om, k2)), mk(n0 - h * m1.re, -h * m1.im));
+  c[3] = sub(sub(k2, mul(om, k3)), sub(m1, scl(h, m2)));
+  c[4] = sub(sub(k3, mul(om, k4)), m2);
+  c[5] = k4;
+}
+
+// Whether the root of the quintic near z is no image for certain: polished
+// in FP64 as a root of the quintic, it leaves Eq. 2 by more than 1e-6 of its
+// terms.  (Near a caustic's outside the two roots about to become images
+// are candidates too: a few texels per map, whose general form would keep
+// one warp busy for half a millisecond.)
+__device__ __noinline__ bool spurious(double mb, double ma, double h, cd om,
+                                      cf z) {
+  cd c[6];
+  quintic(mb, h, om, c);
+  cd w = mk((double)z.re, (double)z.im);
+  bool done = false;
+  for (int it = 0; it < 8 && !done; ++it) {
+    cd p = c[5], dp = mk(0.0, 0.0);
+    for (int u = 4; u >= 0; --u) {
+      dp = add(mul(dp, w), p);
+      p = add(mul(p, w), c[u]);
+    }
+    const double r = 1.0 / ab2(dp);
+    const cd st = mk((p.re * dp.re + p.im * dp.im) * r,
+                     (p.im * dp.re - p.re * dp.im) * r);
+    w = sub(w, st);
+    done = ab2(st) < 1e-22 * ab2(w);
+  }
+  if (!done) return false;
+  const double xa = w.re - h;
+  const double ra = 1.0 / (xa * xa + w.im * w.im), rb = 1.0 / ab2(w);
+  const double fr = w.re - ma * xa * ra - mb * w.re * rb - om.re;
+  const double fi = w.im - ma * w.im * ra - mb * w.im * rb - om.im;
+  const double sc = sqrt(ab2(w)) + sqrt(ab2(om)) + ma * sqrt(ra) +
+                    mb * sqrt(rb);
+  return fr * fr + fi * fi > 1e-12 * sc * sc;
+}
+
 __global__ void __launch_bounds__(kPolyThreads)
     k_poly_fast(double mb, double ma, double xb, double h, double L, int npix,
                 float *__restrict__ A) {
@@ -347,26 +404,9 @@ __global__ void __launch_bounds__(kPolyThreads)
                    -L + ((double)j + 0.5) * dlt);
   cf b[5];
   {
-    const cd oc = cnj(om);
-    const double n0 = -mb * h, hh = h * h;
-    const cd n1 = mk(1.0 - oc.re * h, -oc.im * h);
-    const cd a1 = mk(n1.re + hh, n1.im), a2 = mk(oc.re - h, oc.im);
-    const cd s1 = add(a1, n1), s2 = add(a2, oc);
-    const double k0 = n0 * n0;
-    const cd k1 = scl(n0, s1);
-    const cd k2 = add(scl(n0, s2), mul(a1, n1));
-    const cd k3 = add(mul(a2, n1), mul(a1, oc));
-    const cd k4 = mul(a2, oc);
-    const cd m2 = mk(oc.re - mb * h, oc.im);
-    const cd m1 = mk(n1.re + mb * hh, n1.im);
-    cd c[5];
-    c[0] = scl(-k0, om);
-    c[1] = mk(k0 + h * n0, 0.0);
-    c[1] = sub(c[1], mul(om, k1));
-    c[2] = sub(sub(k1, mul(om, k2)), mk(n0 - h * m1.re, -h * m1.im));
-    c[3] = sub(sub(k2, mul(om, k3)), sub(m1, scl(h, m2)));
-    c[4] = sub(sub(k3, mul(om, k4)), m2);
-    const cf lead = mk((float)k4.re, (float)k4.im);
+    cd c[6];
+    quintic(mb, h, om, c);
+    const cf lead = mk((float)c[5].re, (float)c[5].im);
 #pragma unroll
     for (int t = 0; t < 5; ++t)
       b[t] = divf(mk((float)c[t].re, (float)c[t].im), lead);
@@ -428,10 +468,10 @@ __global__ void __launch_bounds__(kPolyThreads)
   // candidates, to the front
   const float hf = (float)h, maf = (float)ma, mbf = (float)mb;
   const cf omf = mk((float)om.re, (float)om.im);
-  cf w0[5];
+  cf w0[5], z0[5];  // their polished and their own places
   int ni = 0;
 #pragma unroll
-  for (int t = 0; t < 5; ++t) w0[t] = mk(0.f, 0.f);
+  for (int t = 0; t < 5; ++t) w0[t] = z0[t] = mk(0.f, 0.f);
 #pragma unroll
   for (int t = 0; t < 5; ++t) {
     cf w = z[t];
@@ -457,13 +497,16 @@ __global__ void __launch_bounds__(kPolyThreads)
     if (cand) {
 #pragma unroll
       for (int u = 0; u < 5; ++u)
-        if (u == ni) w0[u] = w;
+        if (u == ni) {
+          w0[u] = w;
+          z0[u] = z[t];
+        }
       ++ni;
     }
   }
   double A_sum = 0.0;
-  int parity = 0;
-  bool ok = ni == 3 || ni == 5;
+  int parity = 0, images = 0;
+  bool ok = ni >= 3;
 #pragma unroll
   for (int t = 0; t < 5; ++t) {
     if (t >= ni || !ok) break;
@@ -492,26 +535,29 @@ __global__ void __launch_bounds__(kPolyThreads)
                        maf * ga + mbf * gb;
       if (g * st <= 2e-9f * fabsf((float)det) && re < 1e-9f * sc) {
         done = true;
+        w0[t] = mk((float)x, (float)y);
+#pragma unroll
+        for (int u = 0; u < t; ++u)  // (w0 of no image: NaN)
+          if (ab2(sub(w0[t], w0[u])) < 1e-12f * (1e-6f + ab2(w0[t])))
+            done = false;
+        if (!done) break;
+        ++images;
         A_sum += fabs(rd);
         parity += det > 0.0 ? 1 : -1;
-        w0[t] = mk((float)x, (float)y);
       } else {
         x += dx;
         y += dy;
       }
     }
-    ok = ok && done;
+    if (!done) {
+      w0[t] = mk(CUDART_NAN_F, CUDART_NAN_F);
+      ok = spurious(mb, ma, h, om, z0[t]);
+    }
   }
-#pragma unroll
-  for (int t = 1; t < 5; ++t)
-#pragma unroll
-    for (int u = 0; u < t; ++u)
-      if (t < ni &&
-          ab2(sub(w0[t], w0[u])) <
-              1e-12f * (1e-6f + ab2(w0[t])))
-        ok = false;
   A[(size_t)j * npix + i] =
-      ok && parity == -1 ? __double2float_rn(A_sum) : CUDART_NAN_F;
+      ok && (images == 3 || images == 5) && parity == -1
+          ? __double2float_rn(A_sum)
+          : CUDART_NAN_F;
 }
 
 }  // namespace
