@@ -397,9 +397,13 @@ __global__ void __launch_bounds__(kSearchWarps * 32, 1)
     k_search_list(const SearchParams P) {
   search_listed<EPS, H>(P);
 }
-// the searches of a batch (blockIdx.y)
+// The searches of a batch (blockIdx.y).  Two blocks per SM, some registers
+// spilled: the light curves come through L1 here and the walks wait for L2
+// (one block per SM: 10.2, 21.7, 7.9 and 19.3 ms a batch of 48 pairs, two:
+// 9.6, 20.7, 7.2 and 17.4; with the staged light curve of a single search
+// two are the slower, 0.69 -> 0.76 ms).
 template <bool H>
-__global__ void __launch_bounds__(kSearchWarps * 32, 1)
+__global__ void __launch_bounds__(kSearchWarps * 32, 2)
     k_search_list_batch(const ScreenTask *t) {
   __shared__ alignas(16) SearchParams s_P;
   const int *src = reinterpret_cast<const int *>(&t[blockIdx.y].F.S);
