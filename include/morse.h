@@ -554,7 +554,7 @@ enum { MORSE_REFINE_LM = 0 };
  * Levenberg-Marquardt on chi^2(theta): each iteration evaluates chi^2, its
  * gradient and the Gauss-Newton matrix sum w Fs^2 dA/dtheta dA/dtheta^T,
  * accepts the point if chi^2 fell, and steps by (H + lam diag H)^-1 g.
- * One iteration is captured as a CUDA graph and replayed iters times.
+ * All iterations of all starts run in one kernel launch.
  * out[n] (host) receives the best point of each, its chi^2, Fs, Fb, the
  * start's idx and MORSE_FIT_REFINED.  chi^2 never increases from the start.
  * method: MORSE_REFINE_LM.  Errors: EINVAL, EUNSUPPORTED, ENOMEM, ECUDA. */
@@ -564,7 +564,7 @@ morse_status morse_refine(morse_ctx *ctx, const morse_event *ev,
 
 /* morse_refine of starts on several maps in one call: start i is refined
  * on maps[map_of[i]] (0 <= map_of[i] < n_maps), every start in the same
- * batched launches and the same CUDA graph, so that the grid minima of a
+ * one launch, so that the grid minima of a
  * whole (s, q) sweep (config 2: the K best over all maps) refine together
  * with every map they need resident on the device.  The maps must share
  * npix and extent; each start's result is the one morse_refine gives on its

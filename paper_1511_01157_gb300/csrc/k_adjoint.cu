@@ -17,11 +17,10 @@
 //     dA/dt0 = -Gp / tE,   dA/dtE = -tau Gp / tE,
 //     dA/du0 = Gn,         dA/dalpha = tau Gn - u0 Gp.
 // One warp per trajectory; FP32 per lane, FP64 across lanes.
-// Inside-map epoch loops unrolled four times: the sweeps wait on texel
-// gathers from L2, and four independent gathers per warp are in flight.
-#ifndef MORSE_UNROLL
-#define MORSE_UNROLL 4
-#endif
+// Inside-map epoch loops unrolled: the sweeps wait on texel gathers from L2,
+// and four or eight independent gathers per lane are in flight.
+#include <algorithm>
+
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
@@ -59,6 +58,8 @@ using namespace dev;
 // matrix likewise from the nine sums w tau^m g_a g_b (m = 0, 1, 2).
 constexpr int kAdjWarps = 16;          // warps (trajectories) per block
 constexpr int kAdjEpSmemMax = 6144;    // epochs staged in shared memory
+
+constexpr int kRefineDoubles = 39;     // RefineState, th_cur to H_best
 
 struct AdjTraj {
   TrajC c;
@@ -147,16 +148,134 @@ __device__ __forceinline__ float warp_sum_f32(float x) {
   return x;
 }
 
+// constants of theta = (t0, tE, u0, alpha), t0 absolute
+__device__ __forceinline__ AdjTraj adj_traj(const SearchParams &P,
+                                            const Epochs &ep,
+                                            const double *th, double t_ref,
+                                            const float4 *quad) {
+  const double t0 = th[0], tE = th[1];
+  const double u0 = th[2], al = th[3];
+  double sn, cs;
+  sincos(al, &sn, &cs);
+  const double tEc = (tE > 1e-6) ? tE : 1e-6;  // the host rejects tE <= 0
+  double tlo, thi;
+  slab_tau(P.L, u0, cs, sn, tlo, thi);
+  AdjTraj T;
+  T.c = make_traj(P, ep, u0, cs, sn, t0 - t_ref, 1.0 / (tEc * P.dlt), tEc,
+                  tlo, thi);
+  T.cs = (float)cs;
+  T.sn = (float)sn;
+  T.u0 = (float)u0;
+  T.dD = P.dltf;
+  T.kt = 1.0 / tEc;
+  T.u0d = u0;
+  T.csd = cs;
+  T.snd = sn;
+  T.quad = quad;
+  return T;
+}
+
+// sweep 2 of one warp: residuals, chi^2 and the gradient (and Gauss-Newton)
+// sums, across lanes (chi^2 in FP64, as the search's phase 2; the rest FP32)
+template <bool WITH_H, int UN>
+__device__ __forceinline__ double adj_sweep(const SearchParams &Q,
+                                            const Epochs &ep,
+                                            const AdjTraj &T, float fFs,
+                                            float fBc, int lane,
+                                            AdjSums &a) {
+  a.x1 = a.y1 = a.x2 = a.y2 = 0.f;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) a.h[k] = 0.f;
+  float chi = 0.f;
+#pragma unroll 2
+  for (int e = lane_start(0, lane); e < T.c.e_in; e += 32) {
+    const float2 v = ep.tw[e];
+    float tau, gx, gy;
+    const float Ac = out_point(T, v.x, tau, gx, gy);
+    adj_add<WITH_H>(a, chi, v.y, ep.fc[e], Ac, tau, gx, gy, fFs, fBc);
+  }
+#pragma unroll UN
+  for (int e = lane_start(T.c.e_in, lane); e < T.c.e_out; e += 32) {
+    const float2 v = ep.tw[e];
+    float tau, gx, gy;
+    const float Ac = in_point(Q, T, v.x, tau, gx, gy);
+    adj_add<WITH_H>(a, chi, v.y, ep.fc[e], Ac, tau, gx, gy, fFs, fBc);
+  }
+#pragma unroll 2
+  for (int e = lane_start(T.c.e_out, lane); e < Q.n_ep; e += 32) {
+    const float2 v = ep.tw[e];
+    float tau, gx, gy;
+    const float Ac = out_point(T, v.x, tau, gx, gy);
+    adj_add<WITH_H>(a, chi, v.y, ep.fc[e], Ac, tau, gx, gy, fFs, fBc);
+  }
+  double x = (double)chi;
+#pragma unroll
+  for (int o = 16; o; o >>= 1) x = __dadd_rn(x, __shfl_xor_sync(kFull, x, o));
+  a.x1 = warp_sum_f32(a.x1);
+  a.y1 = warp_sum_f32(a.y1);
+  a.x2 = warp_sum_f32(a.x2);
+  a.y2 = warp_sum_f32(a.y2);
+  if (WITH_H) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) a.h[k] = warp_sum_f32(a.h[k]);
+  }
+  return x;
+}
+
+// chi^2, gradient (4) and Gauss-Newton matrix (10, upper triangle,
+// row-major) of one trajectory from its sums; outputs may be null
+template <bool WITH_H>
+__device__ __forceinline__ void adj_assemble(const SearchParams &P,
+                                             const AdjTraj &Tj,
+                                             const AdjSums &a, double fs,
+                                             double x2, double *chi2,
+                                             double *grad, double *h) {
+  const double c = Tj.csd, s = Tj.snd, u0 = Tj.u0d, kt = Tj.kt;
+  const double iD = P.invD;
+  const double P1 = (c * a.x1 + s * a.y1) * iD;
+  const double N1 = (c * a.y1 - s * a.x1) * iD;
+  const double P2 = (c * a.x2 + s * a.y2) * iD;
+  const double N2 = (c * a.y2 - s * a.x2) * iD;
+  if (chi2) *chi2 = isnan(x2) ? CUDART_INF : x2;
+  if (grad) {
+    const double m2 = -2.0 * fs;
+    grad[0] = m2 * (-kt * P1);
+    grad[1] = m2 * (-kt * P2);
+    grad[2] = m2 * N1;
+    grad[3] = m2 * (N2 - u0 * P1);
+  }
+  if (WITH_H && h) {
+    const double d2 = iD * iD, f2 = fs * fs;
+    double spp[3], spn[3], snn[3];
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      const double xx = a.h[3 * m], xy = a.h[3 * m + 1], yy = a.h[3 * m + 2];
+      spp[m] = (c * c * xx + 2.0 * c * s * xy + s * s * yy) * d2;
+      snn[m] = (s * s * xx - 2.0 * c * s * xy + c * c * yy) * d2;
+      spn[m] = (c * s * (yy - xx) + (c * c - s * s) * xy) * d2;
+    }
+    h[0] = f2 * kt * kt * spp[0];
+    h[1] = f2 * kt * kt * spp[1];
+    h[2] = f2 * -kt * spn[0];
+    h[3] = f2 * -kt * (spn[1] - u0 * spp[0]);
+    h[4] = f2 * kt * kt * spp[2];
+    h[5] = f2 * -kt * spn[1];
+    h[6] = f2 * -kt * (spn[2] - u0 * spp[1]);
+    h[7] = f2 * snn[0];
+    h[8] = f2 * (snn[1] - u0 * spn[0]);
+    h[9] = f2 * (snn[2] - 2.0 * u0 * spn[1] + u0 * u0 * spp[0]);
+  }
+}
+
 // theta_i = (t0, tE, u0, alpha) with absolute t0, on the map P.quad or,
 // when tq is set, on the map tq[i] (maps of one geometry).  Outputs (any
-// may be null): chi2[i], grad[4 i + k], H[10 i + m] (upper triangle,
-// row-major), Fs[i], Fb[i], flags[i].
-template <bool WITH_H, bool EP_SMEM>
-__global__ void __launch_bounds__(kAdjWarps * 32, 2)
+// may be null): chi2[i], grad[4 i + k], Fs[i], Fb[i], flags[i].
+// MINB: blocks per SM, UN: inside-map epochs in flight per lane (adj_split).
+template <bool EP_SMEM, int MINB, int UN>
+__global__ void __launch_bounds__(kAdjWarps * 32, MINB)
     k_theta(const SearchParams P, const double *__restrict__ theta,
             const float4 *const *__restrict__ tq, int n, double t_ref,
-            double *chi2, double *grad, double *H, double *Fs, double *Fb,
-            int *flags) {
+            double *chi2, double *grad, double *Fs, double *Fb, int *flags) {
   extern __shared__ __align__(16) float4 s_ep[];
   __shared__ AdjTraj s_tr[kAdjWarps];
   __shared__ Acc s_acc[kAdjWarps];
@@ -174,26 +293,8 @@ __global__ void __launch_bounds__(kAdjWarps * 32, 2)
   // the shared one is still being written)
   if (warp == 0 && lane < kAdjWarps && i0 + lane < n) {
     const int j = i0 + lane;
-    const double t0 = theta[4 * j + 0], tE = theta[4 * j + 1];
-    const double u0 = theta[4 * j + 2], al = theta[4 * j + 3];
-    double sn, cs;
-    sincos(al, &sn, &cs);
-    const double tEc = (tE > 1e-6) ? tE : 1e-6;  // the host rejects tE <= 0
-    double tlo, thi;
-    slab_tau(P.L, u0, cs, sn, tlo, thi);
-    AdjTraj T;
-    T.c = make_traj(P, epochs_at(P.ep, P.n_ep), u0, cs, sn, t0 - t_ref,
-                    1.0 / (tEc * P.dlt), tEc, tlo, thi);
-    T.cs = (float)cs;
-    T.sn = (float)sn;
-    T.u0 = (float)u0;
-    T.dD = P.dltf;
-    T.kt = 1.0 / tEc;
-    T.u0d = u0;
-    T.csd = cs;
-    T.snd = sn;
-    T.quad = tq ? tq[j] : P.quad;
-    s_tr[lane] = T;
+    s_tr[lane] = adj_traj(P, epochs_at(P.ep, P.n_ep), theta + 4 * j, t_ref,
+                          tq ? tq[j] : P.quad);
   }
   __syncthreads();
   const Epochs ep = epochs_at(EP_SMEM ? s_ep : P.ep, P.n_ep);
@@ -204,7 +305,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32, 2)
   Q.quad = live ? T.quad : P.quad;
   // sweep 1: the normal-equation sums (the search's phase 1)
   if (live) {
-    const Acc a = phase1<false>(Q, ep, T.c, lane);
+    const Acc a = phase1<false, 0, UN>(Q, ep, T.c, lane);
     if (lane == 0) s_acc[warp] = a;
   }
   __syncthreads();
@@ -221,43 +322,8 @@ __global__ void __launch_bounds__(kAdjWarps * 32, 2)
     const float fFs = __double2float_rn(s_Fs[warp]);
     const float fBc = __double2float_rn(s_Bc[warp]);
     AdjSums a;
-    a.x1 = a.y1 = a.x2 = a.y2 = 0.f;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) a.h[k] = 0.f;
-    float chi = 0.f;
-#pragma unroll 2
-    for (int e = lane_start(0, lane); e < T.c.e_in; e += 32) {
-      const float2 v = ep.tw[e];
-      float tau, gx, gy;
-      const float Ac = out_point(T, v.x, tau, gx, gy);
-      adj_add<WITH_H>(a, chi, v.y, ep.fc[e], Ac, tau, gx, gy, fFs, fBc);
-    }
-#pragma unroll kUnroll
-    for (int e = lane_start(T.c.e_in, lane); e < T.c.e_out; e += 32) {
-      const float2 v = ep.tw[e];
-      float tau, gx, gy;
-      const float Ac = in_point(Q, T, v.x, tau, gx, gy);
-      adj_add<WITH_H>(a, chi, v.y, ep.fc[e], Ac, tau, gx, gy, fFs, fBc);
-    }
-#pragma unroll 2
-    for (int e = lane_start(T.c.e_out, lane); e < P.n_ep; e += 32) {
-      const float2 v = ep.tw[e];
-      float tau, gx, gy;
-      const float Ac = out_point(T, v.x, tau, gx, gy);
-      adj_add<WITH_H>(a, chi, v.y, ep.fc[e], Ac, tau, gx, gy, fFs, fBc);
-    }
-    // chi^2 across lanes in FP64 (as the search's phase 2), the rest FP32
-    double x = (double)chi;
-#pragma unroll
-    for (int o = 16; o; o >>= 1) x = __dadd_rn(x, __shfl_xor_sync(kFull, x, o));
-    a.x1 = warp_sum_f32(a.x1);
-    a.y1 = warp_sum_f32(a.y1);
-    a.x2 = warp_sum_f32(a.x2);
-    a.y2 = warp_sum_f32(a.y2);
-    if (WITH_H) {
-#pragma unroll
-      for (int k = 0; k < 9; ++k) a.h[k] = warp_sum_f32(a.h[k]);
-    }
+    const double x =
+        adj_sweep<false, UN>(Q, ep, T, fFs, fBc, lane, a);
     if (lane == 0) {
       s_chi[warp] = x;
       s_sum[warp] = a;
@@ -267,45 +333,10 @@ __global__ void __launch_bounds__(kAdjWarps * 32, 2)
   // assembly of the outputs, one lane per trajectory
   if (warp == 0 && lane < kAdjWarps && i0 + lane < n) {
     const int j = i0 + lane;
-    const AdjTraj &Tj = s_tr[lane];
-    const AdjSums &a = s_sum[lane];
-    const double c = Tj.csd, s = Tj.snd, u0 = Tj.u0d, kt = Tj.kt;
-    const double iD = P.invD, fs = s_Fs[lane];
-    const double P1 = (c * a.x1 + s * a.y1) * iD;
-    const double N1 = (c * a.y1 - s * a.x1) * iD;
-    const double P2 = (c * a.x2 + s * a.y2) * iD;
-    const double N2 = (c * a.y2 - s * a.x2) * iD;
-    const double x2 = s_chi[lane];
-    if (chi2) chi2[j] = isnan(x2) ? CUDART_INF : x2;
-    if (grad) {
-      const double m2 = -2.0 * fs;
-      grad[4 * j + 0] = m2 * (-kt * P1);
-      grad[4 * j + 1] = m2 * (-kt * P2);
-      grad[4 * j + 2] = m2 * N1;
-      grad[4 * j + 3] = m2 * (N2 - u0 * P1);
-    }
-    if (WITH_H && H) {
-      const double d2 = iD * iD, f2 = fs * fs;
-      double spp[3], spn[3], snn[3];
-#pragma unroll
-      for (int m = 0; m < 3; ++m) {
-        const double xx = a.h[3 * m], xy = a.h[3 * m + 1], yy = a.h[3 * m + 2];
-        spp[m] = (c * c * xx + 2.0 * c * s * xy + s * s * yy) * d2;
-        snn[m] = (s * s * xx - 2.0 * c * s * xy + c * c * yy) * d2;
-        spn[m] = (c * s * (yy - xx) + (c * c - s * s) * xy) * d2;
-      }
-      double *h = H + 10 * (size_t)j;
-      h[0] = f2 * kt * kt * spp[0];
-      h[1] = f2 * kt * kt * spp[1];
-      h[2] = f2 * -kt * spn[0];
-      h[3] = f2 * -kt * (spn[1] - u0 * spp[0]);
-      h[4] = f2 * kt * kt * spp[2];
-      h[5] = f2 * -kt * spn[1];
-      h[6] = f2 * -kt * (spn[2] - u0 * spp[1]);
-      h[7] = f2 * snn[0];
-      h[8] = f2 * (snn[1] - u0 * spn[0]);
-      h[9] = f2 * (snn[2] - 2.0 * u0 * spn[1] + u0 * u0 * spp[0]);
-    }
+    const double fs = s_Fs[lane];
+    adj_assemble<false>(P, s_tr[lane], s_sum[lane], fs, s_chi[lane],
+                        chi2 ? chi2 + j : nullptr,
+                        grad ? grad + 4 * (size_t)j : nullptr, nullptr);
     if (Fs) Fs[j] = fs;
     if (Fb) Fb[j] = s_Bc[lane] + P.Fref - fs;
     if (flags) flags[j] = s_deg[lane] ? MORSE_FIT_DEGENERATE : 0;
@@ -350,13 +381,22 @@ __device__ bool lm_solve(const double *h, double lam, const double *b,
   return true;
 }
 
-// One Levenberg-Marquardt step per trajectory (one thread each).  The
+__device__ __forceinline__ bool same_traj(const TrajC &a, const TrajC &b) {
+  return __float_as_int(a.ax) == __float_as_int(b.ax) &&
+         __float_as_int(a.bx) == __float_as_int(b.bx) &&
+         __float_as_int(a.ay) == __float_as_int(b.ay) &&
+         __float_as_int(a.by) == __float_as_int(b.by) &&
+         __float_as_int(a.kt) == __float_as_int(b.kt) &&
+         __float_as_int(a.bt) == __float_as_int(b.bt) &&
+         __float_as_int(a.u02) == __float_as_int(b.u02) &&
+         a.e_in == b.e_in && a.e_out == b.e_out;
+}
+
+// One Levenberg-Marquardt step of trajectory i (one thread).  The
 // evaluation at theta_cur is accepted if it lowered chi^2 (damping / 3) or
 // rejected (damping x 4, back to theta_best); then the next point is
 // theta_best - (H + lam diag H)^-1 g at the best point.
-__global__ void k_lm_step(RefineState S, int n) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+__device__ __forceinline__ void lm_step(const RefineState &S, int i) {
   double lam = S.lam[i];
   const double c = S.chi2_cur[i];
   if (c < S.chi2_best[i]) {
@@ -386,6 +426,130 @@ __global__ void k_lm_step(RefineState S, int n) {
   const double tE = S.th_cur[4 * i + 1];
   const double tEb = S.th_best[4 * i + 1];
   if (!(tE > 0.05 * tEb)) S.th_cur[4 * i + 1] = 0.5 * tEb;
+}
+
+// All iterations of the refinement of kAdjWarps trajectories in one launch:
+// their states stay in shared memory, the light curve is staged once.
+//
+// A point whose track constants (the FP32 set that both sweeps use) are
+// those of the best point has the best point's chi^2 bit for bit and is
+// rejected whatever its gradient: its sweeps are not taken.  With the
+// damping at its ceiling such a step repeats for ever, and a block whose
+// trajectories all do so ends.
+//
+// With one launch per evaluation and one per step an iteration of 2047
+// trajectories of 3000 epochs took 59 us, here 40 (81k cycles):
+// the two sweeps 46k, of which 33k are the L1 gather rate, and 34k the chain
+// of FP64 set-up, fit, assembly and step that one warp runs for all 16; with
+// one trajectory per SM 29 us, 27k and 34k.  Two blocks of 8 warps or four of
+// 4 per SM were the same or slower: their FP64 chains share the SM's pipe.
+template <bool EP_SMEM, int MINB, int UN>
+__global__ void __launch_bounds__(kAdjWarps * 32, MINB)
+    k_refine(const SearchParams P, RefineState S,
+             const float4 *const *__restrict__ tq, int n, int iters,
+             double t_ref) {
+  extern __shared__ __align__(16) float4 s_ep[];
+  __shared__ AdjTraj s_tr[kAdjWarps];
+  __shared__ TrajC s_best[kAdjWarps];
+  __shared__ Acc s_acc[kAdjWarps];
+  __shared__ double s_Fs[kAdjWarps], s_Bc[kAdjWarps];
+  __shared__ AdjSums s_sum[kAdjWarps];
+  __shared__ double s_chi[kAdjWarps];
+  __shared__ double s_state[kAdjWarps * kRefineDoubles];
+  __shared__ int s_eval[kAdjWarps], s_more;
+  const int lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5;
+  const int warps = blockDim.x >> 5;
+  const int i0 = blockIdx.x * warps;
+  const bool live = i0 + warp < n;
+  const bool mine = warp == 0 && lane < warps && i0 + lane < n;
+  if (EP_SMEM)
+    for (int e = threadIdx.x; e < P.n_ep; e += blockDim.x) s_ep[e] = P.ep[e];
+  // the block's states (each read and written by one lane of warp 0 only)
+  RefineState B;
+  B.th_cur = s_state;
+  B.th_best = B.th_cur + 4 * kAdjWarps;
+  B.chi2_cur = B.th_best + 4 * kAdjWarps;
+  B.chi2_best = B.chi2_cur + kAdjWarps;
+  B.lam = B.chi2_best + kAdjWarps;
+  B.g_cur = B.lam + kAdjWarps;
+  B.g_best = B.g_cur + 4 * kAdjWarps;
+  B.H_cur = B.g_best + 4 * kAdjWarps;
+  B.H_best = B.H_cur + 10 * kAdjWarps;
+  const float4 *quad = P.quad;
+  if (mine) {
+    const int j = i0 + lane;
+    for (int k = 0; k < 4; ++k) {
+      B.th_cur[4 * lane + k] = S.th_cur[4 * j + k];
+      B.th_best[4 * lane + k] = S.th_best[4 * j + k];
+      B.g_best[4 * lane + k] = 0.0;
+    }
+    for (int k = 0; k < 10; ++k) B.H_best[10 * lane + k] = 0.0;
+    B.chi2_best[lane] = S.chi2_best[j];
+    B.lam[lane] = S.lam[j];
+    if (tq) quad = tq[j];
+  }
+  __syncthreads();
+  const Epochs ep = epochs_at(EP_SMEM ? s_ep : P.ep, P.n_ep);
+  for (int it = 0; it < iters; ++it) {
+    if (mine) {
+      const AdjTraj T = adj_traj(P, ep, B.th_cur + 4 * lane, t_ref, quad);
+      s_tr[lane] = T;
+      s_eval[lane] = !(B.chi2_best[lane] < CUDART_INF) ||
+                     !same_traj(T.c, s_best[lane]);
+    }
+    __syncthreads();
+    const bool eval = live && s_eval[warp];
+    AdjTraj T;
+    SearchParams Q = P;  // this warp's map
+    if (eval) {
+      T = s_tr[warp];
+      Q.quad = T.quad;
+      const Acc a = phase1<false, 0, UN>(Q, ep, T.c, lane);
+      if (lane == 0) s_acc[warp] = a;
+    }
+    __syncthreads();
+    if (mine && s_eval[lane]) {
+      const Acc a = s_acc[lane];
+      const Fit2 f = fit2(P, (double)a.a, (double)a.b, (double)a.d);
+      s_Fs[lane] = f.Fs;
+      s_Bc[lane] = f.Bc;
+    }
+    __syncthreads();
+    if (eval) {
+      AdjSums a;
+      const double x =
+          adj_sweep<true, UN>(Q, ep, T, __double2float_rn(s_Fs[warp]),
+                              __double2float_rn(s_Bc[warp]), lane, a);
+      if (lane == 0) {
+        s_chi[warp] = x;
+        s_sum[warp] = a;
+      }
+    }
+    __syncthreads();
+    if (warp == 0) {
+      bool more = false;
+      if (mine) {
+        const bool better = s_eval[lane] && s_chi[lane] < B.chi2_best[lane];
+        if (s_eval[lane])
+          adj_assemble<true>(P, s_tr[lane], s_sum[lane], s_Fs[lane],
+                             s_chi[lane], B.chi2_cur + lane,
+                             B.g_cur + 4 * lane, B.H_cur + 10 * lane);
+        else
+          B.chi2_cur[lane] = B.chi2_best[lane];
+        more = s_eval[lane] || B.lam[lane] < 1e12;
+        if (more) lm_step(B, lane);
+        if (better) s_best[lane] = s_tr[lane].c;
+      }
+      more = __any_sync(kFull, more);
+      if (lane == 0) s_more = more;
+    }
+    __syncthreads();
+    if (!s_more) break;
+  }
+  if (mine)
+    for (int k = 0; k < 4; ++k)
+      S.th_best[4 * (i0 + lane) + k] = B.th_best[4 * lane + k];
 }
 
 __global__ void k_lm_init(RefineState S, const morse_fit *starts, int n,
@@ -423,54 +587,87 @@ __global__ void k_lm_finish(RefineState S, const morse_fit *starts, int n,
 
 }  // namespace
 
-template <bool WITH_H>
-static cudaError_t launch_theta_h(const SearchParams &P, const double *theta,
-                                  const float4 *const *tq, int n,
-                                  double t_ref, double *chi2, double *grad,
-                                  double *H, double *Fs, double *Fb,
-                                  int *flags, cudaStream_t st) {
-  const int threads = kAdjWarps * 32;
+// The form of the evaluation kernels for a number of blocks.  Up to one per
+// SM a thread may take 128 registers, for eight texel gathers in flight per
+// lane; above, two blocks per SM and four gathers.
+// 2047 trajectories of 3000 epochs: 42 -> 36 us an evaluation; with more
+// blocks than SMs a second wave would cost more (refinement of 4096: 3.2 ms
+// against twice 2.0).
+template <typename... A>
+static void run_theta(const SearchParams &P, int n, int sm_count,
+                      cudaStream_t st, A... args) {
   const int blocks = (n + kAdjWarps - 1) / kAdjWarps;
-  if (P.n_ep <= kAdjEpSmemMax)
-    k_theta<WITH_H, true><<<blocks, threads, sizeof(float4) * P.n_ep, st>>>(
-        P, theta, tq, n, t_ref, chi2, grad, H, Fs, Fb, flags);
-  else
-    k_theta<WITH_H, false><<<blocks, threads, 0, st>>>(
-        P, theta, tq, n, t_ref, chi2, grad, H, Fs, Fb, flags);
-  return cudaGetLastError();
+  const int threads = kAdjWarps * 32;
+  const bool few = blocks <= sm_count;
+  const size_t sh = sizeof(float4) * P.n_ep;
+  if (P.n_ep <= kAdjEpSmemMax) {
+    if (few)
+      k_theta<true, 1, 8><<<blocks, threads, sh, st>>>(P, args...);
+    else
+      k_theta<true, 2, 4><<<blocks, threads, sh, st>>>(P, args...);
+  } else {
+    if (few)
+      k_theta<false, 1, 8><<<blocks, threads, 0, st>>>(P, args...);
+    else
+      k_theta<false, 2, 4><<<blocks, threads, 0, st>>>(P, args...);
+  }
+}
+
+template <typename K>
+static cudaError_t ep_smem(K kernel) {
+  return cudaFuncSetAttribute(kernel,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)(sizeof(float4) * kAdjEpSmemMax));
 }
 
 cudaError_t adjoint_setup() {
-  const int bytes = (int)(sizeof(float4) * kAdjEpSmemMax);
-  cudaError_t e = cudaFuncSetAttribute(
-      k_theta<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_theta<false, true>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             bytes);
+  cudaError_t e = ep_smem(k_theta<true, 1, 8>);
+  if (e == cudaSuccess) e = ep_smem(k_theta<true, 2, 4>);
+  if (e == cudaSuccess) e = ep_smem(k_refine<true, 1, 8>);
+  if (e == cudaSuccess) e = ep_smem(k_refine<true, 2, 4>);
   return e;
 }
 
 cudaError_t launch_theta(const SearchParams &P, const double *theta, int n,
-                         double t_ref, double *chi2, double *grad, double *H,
-                         double *Fs, double *Fb, int *flags, cudaStream_t st,
-                         const float4 *const *tq) {
+                         double t_ref, double *chi2, double *grad, double *Fs,
+                         double *Fb, int *flags, int sm_count,
+                         cudaStream_t st, const float4 *const *tq) {
   if (n <= 0) return cudaSuccess;
-  if (H)
-    return launch_theta_h<true>(P, theta, tq, n, t_ref, chi2, grad, H, Fs,
-                                Fb, flags, st);
-  return launch_theta_h<false>(P, theta, tq, n, t_ref, chi2, grad, nullptr,
-                               Fs, Fb, flags, st);
+  run_theta(P, n, sm_count, st, theta, tq, n, t_ref, chi2, grad, Fs, Fb, flags);
+  return cudaGetLastError();
+}
+
+// Blocks of as many warps as spread the trajectories over the SMs, at most
+// kAdjWarps.
+cudaError_t launch_refine(const SearchParams &P, const RefineState &S, int n,
+                          int iters, double t_ref, int sm_count,
+                          cudaStream_t st, const float4 *const *tq) {
+  if (n <= 0 || iters <= 0) return cudaSuccess;
+  const int warps = std::min(kAdjWarps, (n + sm_count - 1) / sm_count);
+  const int blocks = (n + warps - 1) / warps, threads = 32 * warps;
+  const bool few = blocks <= sm_count;
+  const size_t sh = sizeof(float4) * P.n_ep;
+  if (P.n_ep <= kAdjEpSmemMax) {
+    if (few)
+      k_refine<true, 1, 8><<<blocks, threads, sh, st>>>(P, S, tq, n, iters,
+                                                         t_ref);
+    else
+      k_refine<true, 2, 4><<<blocks, threads, sh, st>>>(P, S, tq, n, iters,
+                                                         t_ref);
+  } else {
+    if (few)
+      k_refine<false, 1, 8><<<blocks, threads, 0, st>>>(P, S, tq, n, iters,
+                                                         t_ref);
+    else
+      k_refine<false, 2, 4><<<blocks, threads, 0, st>>>(P, S, tq, n, iters,
+                                                         t_ref);
+  }
+  return cudaGetLastError();
 }
 
 cudaError_t launch_lm_init(const RefineState &S, const morse_fit *starts,
                            int n, double lam0, cudaStream_t st) {
   k_lm_init<<<(n + 127) / 128, 128, 0, st>>>(S, starts, n, lam0);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_lm_step(const RefineState &S, int n, cudaStream_t st) {
-  k_lm_step<<<(n + 127) / 128, 128, 0, st>>>(S, n);
   return cudaGetLastError();
 }
 

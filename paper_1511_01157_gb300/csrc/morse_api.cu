@@ -2673,7 +2673,7 @@ morse_status morse_chi2_grad_dev(morse_ctx *ctx, const morse_event *ev,
   event_params(ev, &P);
   MORSE_CUDA(ctx, morse::launch_theta(P, theta, (int)n, ev->t_ref, chi2,
                                       grad, nullptr, nullptr, nullptr,
-                                      nullptr, ctx->stream));
+                                      ctx->sm_count, ctx->stream));
   ctx->launches += 1;
   return MORSE_OK;
 }
@@ -2705,7 +2705,7 @@ morse_status morse_chi2_grad(morse_ctx *ctx, const morse_event *ev,
   event_params(ev, &P);
   int r = t_begin(ctx, KT_ADJ);
   MORSE_CUDA(ctx, morse::launch_theta(P, d_th, (int)n, ev->t_ref, d_c, d_g,
-                                      nullptr, d_fs, d_fb, nullptr,
+                                      d_fs, d_fb, nullptr, ctx->sm_count,
                                       ctx->stream));
   t_end(ctx, r);
   ctx->launches += 1;
@@ -2748,9 +2748,9 @@ static morse_status refine_impl(morse_ctx *ctx, const morse_event *ev,
   MORSE_CUDA(ctx, cudaSetDevice(ctx->device));
   call_begin(ctx);
   const size_t nn = (size_t)n;
-  // workspace: 36 doubles + 1 int per trajectory, starts, records, and the
+  // workspace: 13 doubles + 1 int per trajectory, starts, records, and the
   // trajectories' map tables
-  const size_t dbl = nn * 36, bytes = sizeof(double) * dbl + sizeof(int) * nn +
+  const size_t dbl = nn * 13, bytes = sizeof(double) * dbl + sizeof(int) * nn +
                                       2 * sizeof(morse_fit) * nn +
                                       sizeof(void *) * nn + 4096;
   void *ws = nullptr;
@@ -2762,11 +2762,8 @@ static morse_status refine_impl(morse_ctx *ctx, const morse_event *ev,
   S.chi2_cur = S.th_best + 4 * nn;
   S.chi2_best = S.chi2_cur + nn;
   S.lam = S.chi2_best + nn;
-  S.g_cur = S.lam + nn;
-  S.g_best = S.g_cur + 4 * nn;
-  S.H_cur = S.g_best + 4 * nn;
-  S.H_best = S.H_cur + 10 * nn;
-  S.Fs = S.H_best + 10 * nn;
+  S.g_cur = S.g_best = S.H_cur = S.H_best = nullptr;  // in shared memory
+  S.Fs = S.lam + nn;
   S.Fb = S.Fs + nn;
   S.flags = (int *)(S.Fb + nn);
   morse_fit *d_starts = (morse_fit *)align_up(
@@ -2790,43 +2787,17 @@ static morse_status refine_impl(morse_ctx *ctx, const morse_event *ev,
   MORSE_CUDA(ctx, morse::launch_lm_init(S, d_starts, n, 1e-3, ctx->stream));
   ctx->launches += 1;
   if (iters > 0) {
-    // one iteration (evaluate at theta_cur, then step) as a CUDA graph
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
-    MORSE_CUDA(ctx, cudaStreamBeginCapture(ctx->stream,
-                                           cudaStreamCaptureModeThreadLocal));
-    cudaError_t e1 = morse::launch_theta(P, S.th_cur, n, ev->t_ref,
-                                         S.chi2_cur, S.g_cur, S.H_cur,
-                                         nullptr, nullptr, nullptr,
-                                         ctx->stream, d_tq);
-    cudaError_t e2 = morse::launch_lm_step(S, n, ctx->stream);
-    cudaError_t e3 = cudaStreamEndCapture(ctx->stream, &graph);
-    if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess) {
-      if (graph) cudaGraphDestroy(graph);
-      return cuda_fail(ctx, e1 != cudaSuccess ? e1 : (e2 != cudaSuccess ? e2 : e3),
-                       "refine graph capture");
-    }
-    cudaError_t e4 = cudaGraphInstantiate(&exec, graph, 0);
-    cudaGraphDestroy(graph);
-    if (e4 != cudaSuccess) return cuda_fail(ctx, e4, "refine graph");
     int r = t_begin(ctx, KT_LM);
-    for (int it = 0; it < iters; ++it) {
-      cudaError_t e = cudaGraphLaunch(exec, ctx->stream);
-      if (e != cudaSuccess) {
-        cudaGraphExecDestroy(exec);
-        return cuda_fail(ctx, e, "refine graph launch");
-      }
-    }
+    MORSE_CUDA(ctx, morse::launch_refine(P, S, n, iters, ev->t_ref,
+                                         ctx->sm_count, ctx->stream, d_tq));
     t_end(ctx, r);
-    ctx->launches += 2 * (uint64_t)iters;
-    MORSE_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    cudaGraphExecDestroy(exec);
+    ctx->launches += 1;
   }
   // evaluate at the best point (the start if no iteration improved on it)
   int r = t_begin(ctx, KT_ADJ);
   MORSE_CUDA(ctx, morse::launch_theta(P, S.th_best, n, ev->t_ref, S.chi2_cur,
-                                      nullptr, nullptr, S.Fs, S.Fb, S.flags,
-                                      ctx->stream, d_tq));
+                                      nullptr, S.Fs, S.Fb, S.flags,
+                                      ctx->sm_count, ctx->stream, d_tq));
   t_end(ctx, r);
   MORSE_CUDA(ctx, morse::launch_lm_finish(S, d_starts, n, d_out, ctx->stream));
   ctx->launches += 2;

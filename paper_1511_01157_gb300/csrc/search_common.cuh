@@ -508,11 +508,13 @@ __device__ __forceinline__ float mag_out_m1(const TrajC &c, float t) {
   return __fsub_rn(pspl_u2(__fmaf_rn(tau, tau, c.u02)), 1.f);
 }
 
-template <bool H, bool IN, int TB = 0>
+// (UN: inside-map epochs in flight per lane; the order of the sums is the
+// same for all)
+template <bool H, bool IN, int TB = 0, int UN = H ? kUnrollH : kUnroll>
 __device__ __forceinline__ void seg1(const SearchParams &P, const Epochs &ep,
                                      const TrajC &c, int lane, int e0, int e1,
                                      Acc &s, const float4 *tab = nullptr) {
-#pragma unroll (IN ? (H ? kUnrollH : kUnroll) : 2)
+#pragma unroll (IN ? UN : 2)
   for (int e = lane_start(e0, lane); e < e1; e += 32) {
     const float2 v = ep.tw[e];
     const float wf = ep.wf[e];
@@ -689,13 +691,13 @@ __device__ __forceinline__ Acc acc_reduce(Acc s) {
 // Phase 1: FP32 sums of S_A = sum w (A-1), S_AA = sum w (A-1)^2 and
 // S_AF = sum w (F-Fref)(A-1) over the epochs before, inside and after the
 // map, reduced across the warp.
-template <bool H, int TB = 0>
+template <bool H, int TB = 0, int UN = H ? kUnrollH : kUnroll>
 __device__ __forceinline__ Acc phase1(const SearchParams &P, const Epochs &ep,
                                       const TrajC &c, const int lane,
                                       const float4 *tab = nullptr) {
   Acc s = {0.f, 0.f, 0.f};
   seg1<H, false>(P, ep, c, lane, 0, c.e_in, s);
-  seg1<H, true, TB>(P, ep, c, lane, c.e_in, c.e_out, s, tab);
+  seg1<H, true, TB, UN>(P, ep, c, lane, c.e_in, c.e_out, s, tab);
   seg1<H, false>(P, ep, c, lane, c.e_out, P.n_ep, s);
   return acc_reduce(s);
 }

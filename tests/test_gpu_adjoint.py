@@ -315,3 +315,34 @@ def test_gradient_rejects_bad_theta(ctx, m, setup):
         with pytest.raises(m.MorseError) as e:
             ctx.chi2_grad(ev, mp, np.array([bad]))
         assert e.value.status == m.EINVAL
+
+
+@pytest.mark.parametrize("n,n_ep", [(1, 64), (17, 64), (153, 6200),
+                                    (153, 6144), (2433, 64)])
+def test_refine_does_not_depend_on_the_split(ctx, m, setup, n, n_ep):
+    """One launch refines every start: blocks of 1 to 16 warps, one or two
+    per SM, the light curve staged or not.  A start's record is the same to
+    the last bit alone and among n, its chi^2 is the one that the gradient
+    entry point gives there, and a start at which no sweep can be accepted
+    any more (the block ends early) keeps its record over more iterations."""
+    c, mp = setup[0], setup[5]
+    t = synth.epoch_times(n_ep, 11, c["t0"])
+    F, sig = synth.photometry(1.0 + 1.0 / np.sqrt(
+        c["u0"] ** 2 + ((t - c["t0"]) / c["tE"]) ** 2), 11)
+    ev = ctx.event(t, F, sig)
+    rng = np.random.default_rng(n + n_ep)
+    st = np.zeros(n, dtype=m.FIT_DTYPE)
+    st["t0"] = c["t0"] + rng.uniform(-1.0, 1.0, n)
+    st["tE"] = c["tE"] * np.exp(rng.uniform(-0.3, 0.3, n))
+    st["u0"] = c["u0"] * np.exp(rng.uniform(-0.5, 0.5, n))
+    st["alpha"] = c["alpha"] + rng.uniform(-0.2, 0.2, n)
+    st["idx"] = np.arange(n)
+    out = ctx.refine(ev, mp, st, iters=60)
+    for i in sorted({0, n // 2, n - 1}):
+        one = ctx.refine(ev, mp, st[i:i + 1], iters=60)
+        assert one.tobytes() == out[i:i + 1].tobytes()
+    th = np.stack([out["t0"], out["tE"], out["u0"], out["alpha"]], axis=1)
+    assert np.array_equal(ctx.chi2_grad(ev, mp, th)[0], out["chi2"])
+    assert np.all(out["chi2"] <= ctx.refine(ev, mp, st, iters=0)["chi2"])
+    late = ctx.refine(ev, mp, out, iters=2000)
+    assert np.array_equal(ctx.refine(ev, mp, out, iters=4000), late)
