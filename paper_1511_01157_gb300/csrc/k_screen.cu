@@ -58,7 +58,7 @@ using namespace dev;
 
 constexpr int kScreenThreads = 256;
 constexpr int kScreenTile = 2 * kScreenThreads;  // trajectories per block step
-// epochs of the subsets summed by one lane, at most
+// epochs of the subsets, at most
 constexpr int kScreenMax0 = 128, kScreenMax1 = 192, kScreenMax2 = 1024;
 
 // Order of the trajectories in a screen.  The grid index runs over tE
@@ -230,21 +230,33 @@ __device__ __forceinline__ float2 in2_m1(const SearchParams &P, Cells<H> &q,
 
 // The subset's bounds for two trajectories of a lane (packed FP32), every
 // lane over the whole subset: no reductions, one broadcast shared load of
-// an epoch for the warp's 64 trajectories.
+// an epoch for the warp's 64 trajectories.  Or, with lg > 0, 2^lg neighbouring
+// lanes have the same two trajectories, each an equal piece of the subset
+// (split_len; the last past its end: pad_subset), and the sums are
+// added across them (the bound's error covers any order).
+constexpr int kSplitMax = 2;   // 4 lanes a trajectory at most
+constexpr int kSplitPad = 8;   // epochs past the subset: 2 x lanes - 1, or less
+__device__ __forceinline__ int split_len(int m, int lg) {
+  // odd: the lanes' pieces start in different banks
+  return lg ? ((m + (1 << lg) - 1) >> lg) | 1 : m;
+}
 template <bool H>
 __device__ __forceinline__ void screen2(const SearchParams &P,
                                         const ScreenLv &V, const float4 *s_ep,
                                         const TrajC &ca, const TrajC &cb,
                                         float ain, float aout, float bin,
-                                        float bout, float &la, float &lb) {
+                                        float bout, float &la, float &lb,
+                                        int lg = 0) {
   const TrajP c = pack_traj(ca, cb);
   const float hi = fmaxf(ain, bin), lo = fminf(aout, bout);
   Acc2 s = {f2(0.f), f2(0.f), f2(0.f)};
   Cells<H> q;
   q.ia = q.ib = 0xFFFFFFFFu;
   q.a = q.b = make_float4(0.f, 0.f, 0.f, 0.f);
+  const int len = split_len(V.m, lg);
+  s_ep += ((int)threadIdx.x & ((1 << lg) - 1)) * len;
 #pragma unroll 4
-  for (int e = 0; e < V.m; ++e) {
+  for (int e = 0; e < len; ++e) {
     const float4 v = s_ep[e];
     const float2 tt = f2(v.x);
     const float2 vx = pk_fma(c.ax, tt, c.bx);
@@ -267,6 +279,14 @@ __device__ __forceinline__ void screen2(const SearchParams &P,
     }
     acc2_add(s, f2(v.y), f2(v.z), Ac);
   }
+  for (int o = 1; o < 1 << lg; o <<= 1) {
+    s.a = pk_add(s.a, make_float2(__shfl_xor_sync(kFull, s.a.x, o),
+                                  __shfl_xor_sync(kFull, s.a.y, o)));
+    s.b = pk_add(s.b, make_float2(__shfl_xor_sync(kFull, s.b.x, o),
+                                  __shfl_xor_sync(kFull, s.b.y, o)));
+    s.d = pk_add(s.d, make_float2(__shfl_xor_sync(kFull, s.d.x, o),
+                                  __shfl_xor_sync(kFull, s.d.y, o)));
+  }
   const Acc sa = {s.a.x, s.b.x, s.d.x}, sb = {s.a.y, s.b.y, s.d.y};
   la = screen_lb(V, sa);
   lb = screen_lb(V, sb);
@@ -277,6 +297,12 @@ __device__ __forceinline__ void stage_subset(const ScreenLv &V,
   const Epochs ep = epochs_at(V.ep, V.m);
   for (int e = threadIdx.x; e < V.m; e += blockDim.x)
     s_ep[e] = make_float4(ep.tw[e].x, ep.tw[e].y, ep.wf[e], 0.f);
+}
+// epochs without weight after the subset's (for the lanes of split_len)
+__device__ __forceinline__ void pad_subset(const ScreenLv &V, float4 *s_ep) {
+  const float t = epochs_at(V.ep, V.m).tw[V.m - 1].x;
+  for (int e = threadIdx.x; e < kSplitPad; e += blockDim.x)
+    s_ep[V.m + e] = make_float4(t, 0.f, 0.f, 0.f);
 }
 
 // Codes of all trajectories, on the smallest subset.
@@ -596,37 +622,56 @@ __device__ __forceinline__ void make_list(const SearchParams &P,
 // subset leaves in a queue and takes the third with full warps.  When the
 // two discard less than one in eight of those decided so far (from 16 384
 // on), the screen gives up and the whole range is searched.
+//
+// A short list leaves SMs without a tile, and a lane's walk over the subset
+// is a chain of cell loads: the lanes of a tile then take fewer trajectories,
+// 2 or 4 lanes each, while every tile still has a block of its own.  Not in a
+// batch, whose other pairs fill the SMs.  Peak-aligned searches (345 600
+// trajectories) 621, 616, 615, 690 -> 591, 556, 548, 634 us, a grid of 1.44 M
+// whose list is short 452 -> 393, the others within 1.5 %; with 8 lanes the
+// same, and the final list's order (tile by tile) gets worse for its search.
 template <bool H>
 __device__ __forceinline__ void rescreen_listed(const SearchParams &P,
                                                 const ScreenBufs &B) {
   if (P.n_lv < 3) return;  // (of a batch: the list is final)
-  __shared__ float4 s_e1[kScreenMax1], s_e2[kScreenMax2];
+  __shared__ float4 s_e1[kScreenMax1 + kSplitPad],
+      s_e2[kScreenMax2 + kSplitPad];
   __shared__ unsigned s_queue[2 * kScreenTile];
   __shared__ unsigned s_m[kScreenThreads / 16], s_base, s_stop;
   const ScreenLv V1 = P.lv[1], V2 = P.lv[2];
   const unsigned n = B.n[1];
-  unsigned c0 = blockIdx.x * kScreenTile;
+  int lg = 0;
+  if (gridDim.y == 1)
+    while (lg < kSplitMax && ((unsigned long long)n << (lg + 1)) <=
+                                 (unsigned long long)gridDim.x * kScreenTile)
+      ++lg;
+  const unsigned tile = (unsigned)kScreenTile >> lg;
+  unsigned c0 = blockIdx.x * tile;
   if (c0 >= n) return;
   stage_subset(V1, s_e1);
   stage_subset(V2, s_e2);
+  pad_subset(V1, s_e1);
+  pad_subset(V2, s_e2);
   const float thr = __double2float_ru(bits_to_chi2(__ldcg(P.gthr)));
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned below = (1u << lane) - 1u;
   unsigned queued = 0;  // block-uniform
   while (c0 < n || queued > 0) {
-    const bool first = c0 < n && queued < (unsigned)kScreenTile;
-    const unsigned m = min((unsigned)kScreenTile, first ? n - c0 : queued);
+    const bool first = c0 < n && queued < tile;
+    const unsigned m = min(tile, first ? n - c0 : queued);
     const unsigned q0 = first ? 0u : queued - m;
     if (threadIdx.x == 0) s_stop = *(volatile unsigned *)&B.n[4];
     __syncthreads();  // the subsets, the queue
     if (s_stop) return;
-    const unsigned i[2] = {(unsigned)(warp * 64 + lane),
-                           (unsigned)(warp * 64 + lane + 32)};
+    const unsigned w0 = ((unsigned)warp * 64u) >> lg;
+    const unsigned i[2] = {w0 + ((unsigned)lane >> lg),
+                           w0 + ((unsigned)(lane + 32) >> lg)};
+    const bool lead = (lane & ((1 << lg) - 1)) == 0;  // of a trajectory
     unsigned off[2];
     TrajC c[2];
     float in[2], out[2];
     unsigned ma = 0, mb = 0;
-    if ((unsigned)warp * 64u < m) {
+    if (w0 < m) {
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const unsigned k = min(i[h], m - 1);
@@ -638,13 +683,13 @@ __device__ __forceinline__ void rescreen_listed(const SearchParams &P,
       }
       float la, lb;
       if (first)
-        screen2<H>(P, V1, s_e1, c[0], c[1], in[0], out[0], in[1], out[1], la,
-                   lb);
+        screen2<H>(P, V1, s_e1, c[0], c[1], in[0], out[0], in[1],
+                   out[1], la, lb, lg);
       else
-        screen2<H>(P, V2, s_e2, c[0], c[1], in[0], out[0], in[1], out[1], la,
-                   lb);
-      ma = __ballot_sync(kFull, i[0] < m && la <= thr);
-      mb = __ballot_sync(kFull, i[1] < m && lb <= thr);
+        screen2<H>(P, V2, s_e2, c[0], c[1], in[0], out[0], in[1],
+                   out[1], la, lb, lg);
+      ma = __ballot_sync(kFull, lead && i[0] < m && la <= thr);
+      mb = __ballot_sync(kFull, lead && i[1] < m && lb <= thr);
     }
     if (lane == 0) {
       s_m[2 * warp] = __popc(ma);
@@ -671,7 +716,7 @@ __device__ __forceinline__ void rescreen_listed(const SearchParams &P,
       if (ma >> lane & 1u) s_queue[queued + ra] = off[0];
       if (mb >> lane & 1u) s_queue[queued + rb] = off[1];
       queued += s_base;
-      c0 += gridDim.x * kScreenTile;
+      c0 += gridDim.x * tile;
     } else {
       const unsigned g = s_base;
       if ((ma >> lane & 1u) && g + ra < B.list_cap) B.list[g + ra] = off[0];
@@ -773,7 +818,8 @@ cudaError_t launch_screen_list(const SearchParams &P, const ScreenBufs &B,
 
 cudaError_t launch_rescreen(const SearchParams &P, const ScreenBufs &B,
                             int sm_count, cudaStream_t st) {
-  const long long want = (P.count + kScreenTile - 1) / kScreenTile;
+  const int tile = kScreenTile >> kSplitMax;
+  const long long want = (P.count + tile - 1) / tile;
   const int grid = (int)std::min<long long>(want, 4LL * sm_count);
   if (P.quadh)
     k_rescreen<true><<<grid, kScreenThreads, 0, st>>>(P, B);

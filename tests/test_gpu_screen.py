@@ -163,3 +163,25 @@ def test_small_grid_equals_dense(m, setup, dims, n):
         r = ctx.grid_chi2_range(ev, mp, g, 5, 91)
         idx, val = _best(chi2[5:96], 37, 5)
         assert np.array_equal(r["idx"], idx)
+
+
+@pytest.mark.parametrize("kind", ["strong", "weak"])
+@pytest.mark.parametrize("n", [1024, 1027, 3001])
+def test_listed_bounds_on_one_to_four_lanes(m, setup, n, kind):
+    """409 600 trajectories: K from 1 to 4096 makes the list of the second
+    bound from a few tiles, its trajectories on four lanes each, to more
+    than there are blocks, on one."""
+    ctx, mp = setup
+    ev = _event(ctx, n, kind)
+    dims = (40, 40, 16, 16, 1e-3, 0.5, -2.0, 2.0, 5.0, 80.0, True, True)
+    chi2, *_ = ctx.grid_chi2_dense(ev, mp, m.Grid.make(*dims, 1))
+    for h16 in (False, True):
+        mp.set_lookup(h16)
+        if h16:
+            chi2, *_ = ctx.grid_chi2_dense(ev, mp, m.Grid.make(*dims, 1))
+        for k in (1, 64, 1024, 4096):
+            got = ctx.grid_chi2(ev, mp, m.Grid.make(*dims, k))
+            idx, val = _best(chi2, k)
+            assert np.array_equal(got["idx"][:len(idx)], idx)
+            assert np.array_equal(got["chi2"][:len(idx)], val)
+    mp.set_lookup(False)
