@@ -21,7 +21,6 @@ host cores, each step a bounded sample of the same workload.
 from __future__ import annotations
 
 import argparse
-import hashlib
 import json
 import math
 import os
@@ -42,21 +41,15 @@ METRIC = ("trajectory-epoch chi^2 evals/s and rays/s (% of roofline); "
 UNIT = "traj-epoch evals/s"
 # FP32 instructions one trajectory-epoch evaluation needs by its definition:
 # tau 1, y 2, pixel coords 2, floor/frac/convert 6, bilinear 6, normal-
-# equation sums 3, residual sweep 2.  The residual sweep runs only for the
-# trajectories the error-bounded closed form cannot discard, so the work the
-# search does is 20 instructions per evaluation plus 2 for the exact-sweep
-# fraction; the headline roofline counts that, and the 22-instruction
-# figure is reported beside it.
+# equation sums 3 (and 2 in the residual sweep of the few whose exact chi^2
+# is needed).
 ALG_INSTR_PER_EVAL = 22
 ALG_INSTR_PRUNED = 20
-# one bilinear gather of a 2x2 FP32 cell per trajectory-epoch
-GATHER_BYTES_PER_EVAL = 16
-# bytes per trajectory-epoch through the shared-memory data pipe as the
-# search is built: the 16-byte cell from the band table and half of the
-# 12-byte epoch record (one load serves a trajectory pair); the pipe moves
-# 128 bytes per clock per SM
-SMEM_BYTES_PER_EVAL = 22
-SMEM_BYTES_PER_CLK_SM = 128
+# The search settles most trajectories from a rigorous lower bound of chi^2,
+# the chi^2 of a subset of the epochs: every trajectory takes the first
+# subset's epochs (64 of a light curve of 640 or more, k_screen.cu), the
+# listed ones more, the last few all.  The roofline counts the first.
+SCREEN_EPOCHS = 64
 # adjoint, per trajectory-epoch: the chi^2 of the two sweeps (22, as the
 # search) and 14 more for the gradient through the lookup (four FP32 sums
 # in the map's pixel axes); the kernel recomputes the lookup in its second
@@ -67,11 +60,6 @@ ADJ_INSTR_PER_EVAL = 36
 # lenses 12 (+ 2 reciprocals), binning 6; plus one shared-memory atomic
 ALG_INSTR_PER_RAY = 22
 FP32_LANES_PER_SM = 128
-# the search kernel's sources: its traffic record holds while they match
-KERNEL_SRC = [os.path.join(ROOT, "paper_1511_01157_gb300", "csrc", f)
-              for f in ("k_search.cu", "search_common.cuh",
-                        "search_group.cuh", "morse_internal.cuh")]
-PROFILE = os.path.join(ROOT, "profiles", "k_search_cfg1.md")
 
 
 def workload_config(cfg):
@@ -171,33 +159,6 @@ def measured_peaks():
         except Exception:
             pass
     return {"hbm_gbs": 6800.0, "sm_max_mhz": 2070.0}, "fallback"
-
-
-def kernel_source_hash():
-    h = hashlib.sha256()
-    for f in KERNEL_SRC:
-        h.update(open(f, "rb").read())
-    return h.hexdigest()[:16]
-
-
-def recorded_traffic():
-    """DRAM bytes per launch of the search kernel from the committed ncu
-    summary, valid only while the kernel source is unchanged."""
-    if not os.path.exists(PROFILE):
-        return None
-    src_hash = kernel_source_hash()
-    bytes_, h = None, None
-    for line in open(PROFILE):
-        if line.startswith("traffic_bytes_per_launch:"):
-            try:
-                bytes_ = float(line.split(":", 1)[1])
-            except ValueError:
-                bytes_ = None
-        if line.startswith("kernel_source_sha256_16:"):
-            h = line.split(":", 1)[1].strip()
-    if h != src_hash:
-        return None
-    return bytes_
 
 
 def make_event(ctx, m, cfg, seed):
@@ -1056,22 +1017,13 @@ def run_gpu(args, cfg):
     peak_instr = props.multi_processor_count * FP32_LANES_PER_SM * \
         sm_max * 1e6 / 1e12
     exact_frac = float(np.mean(exact[-args.steps:])) / (grid.size * n_maps)
-    instr_done = ALG_INSTR_PRUNED + (ALG_INSTR_PER_EVAL -
-                                     ALG_INSTR_PRUNED) * exact_frac
-    achieved = evals_step * instr_done / (search_ms * 1e-3) / 1e12
-    achieved_22 = evals_step * ALG_INSTR_PER_EVAL / (search_ms * 1e-3) / 1e12
-    evals_per_s_kernel = evals_step / (search_ms * 1e-3)
-    gather_gbs = evals_per_s_kernel * GATHER_BYTES_PER_EVAL / 1e9
-    smem_gbs = evals_per_s_kernel * SMEM_BYTES_PER_EVAL / 1e9
-    smem_peak = props.multi_processor_count * SMEM_BYTES_PER_CLK_SM * \
-        sm_max * 1e6 / 1e9
+    achieved = grid.size * n_maps * SCREEN_EPOCHS * ALG_INSTR_PRUNED / \
+        (search_ms * 1e-3) / 1e12
     rays_kernel = rays_alone
     ray_alu = probes["fp32_fma_per_s"] / ALG_INSTR_PER_RAY
     ray_atom = probes["smem_atomics_per_s"]
     ray_peak = min(ray_alu, ray_atom)
-    traffic = recorded_traffic()
     clocks = clk.summary()
-    per_launch = evals_step // n_maps
 
     cfg_line = workload_config(cfg)
     if n_maps != cfg["n_s"] * cfg["n_q"]:
@@ -1098,42 +1050,29 @@ def run_gpu(args, cfg):
             "rayshoot": ray_ms, "counts_to_map": float(km[:, 1].mean()),
             "search": search_ms, "topk_merge": float(km[:, 3].mean()),
             "fill": float(km[:, 4].mean())},
+        "evals_note": "trajectory-epochs of the grid whose place in the "
+                      "ranking was settled, exactly as if each had been "
+                      "evaluated; most trajectories are discarded by a "
+                      "lower bound of their chi^2 from a subset of the "
+                      "epochs, and their other epochs are not looked up",
         "roofline": {
-            "kernel": "k_search", "bound": "alu", "achieved": achieved,
+            "kernel": "k_screen to k_finish (all kernels of a search)",
+            "bound": "alu", "achieved": achieved,
             "peak": peak_instr, "unit": "T FP32-instr/s",
-            "frac": achieved / peak_instr, "traffic": traffic,
-            "algorithmic": f"{instr_done:.3f} FP32 instr per "
-                           f"trajectory-epoch ({ALG_INSTR_PRUNED} + 2 x the "
-                           f"exact-sweep fraction {exact_frac:.4f}) x "
-                           f"{per_launch} per launch",
-            "frac_22_instr": achieved_22 / peak_instr,
+            "frac": achieved / peak_instr, "traffic": None,
+            "algorithmic": f"{ALG_INSTR_PRUNED} FP32 instr per "
+                           f"trajectory-epoch x {SCREEN_EPOCHS} epochs of "
+                           "the first bound x every trajectory; the later "
+                           "bounds and the exact evaluations of the few "
+                           "that they leave are not counted, and in the "
+                           "sweep the search shares the SMs with the next "
+                           "map's ray shooting",
             "peak_source": f"{props.multi_processor_count} SMs x "
                            f"{FP32_LANES_PER_SM} FP32 lanes x {sm_max} MHz "
                            f"({peak_kind} sm_max_mhz)",
             "measured_fp32_fma_per_s": probes["fp32_fma_per_s"],
             "frac_of_measured_fma": achieved * 1e12 /
-            probes["fp32_fma_per_s"],
-            "gather": {
-                "achieved_GBps": gather_gbs,
-                "note": "not binding: 99 % of the cells come from the "
-                        "shared-memory band tables, not from L1 or L2 "
-                        "gathers, so the measured random-gather rates "
-                        "are not a ceiling of this kernel",
-                "l1_random_gather_GBps": probes["l1_gather_bytes_per_s"] /
-                1e9,
-                "l2_random_gather_GBps": probes["l2_gather_bytes_per_s"] /
-                1e9,
-                "algorithmic": f"{GATHER_BYTES_PER_EVAL} B per "
-                               "trajectory-epoch (one 2x2 FP32 cell)"},
-            "smem_pipe": {
-                "achieved_GBps": smem_gbs, "peak_GBps": smem_peak,
-                "frac": smem_gbs / smem_peak,
-                "bytes": f"{SMEM_BYTES_PER_EVAL} B per trajectory-epoch "
-                         "(16 B cell + half of a 12 B epoch record), "
-                         "excluding bank conflicts",
-                "peak_source": f"{props.multi_processor_count} SMs x "
-                               f"{SMEM_BYTES_PER_CLK_SM} B per clock x "
-                               f"{sm_max} MHz"}},
+            probes["fp32_fma_per_s"]},
         "rayshoot_roofline": {
             "kernel": "k_rayshoot<FP32>", "rays_per_s": rays_kernel,
             "bound": "alu" if ray_alu <= ray_atom else "smem_atomic",
