@@ -310,9 +310,14 @@ __global__ void __launch_bounds__(kPolyThreads)
 // candidate, polished by Newton on Eq. 2 (twice in FP32, then in FP64 until
 // the step changes 1/|det J| by less than 2e-9).  The texel is kept only if
 // every candidate became an image of its own or is shown to be none
-// (spurious), they are 3 or 5, and their parities add up to -1 (one more saddle than minima and maxima, for two
-// point lenses); five images are all there can be, and with three the other
-// two roots are 0.2 % of their terms away from Eq. 2 (FP32 resolves 1e-5).
+// (spurious), they are 3 or 5, and their parities add up to -1 (one more
+// saddle than minima and maxima, for two point lenses).  Two point lenses
+// have 3 or 5 images, so five are all, and three are all once a single root
+// of the quintic is known to be no image: a spurious candidate, or one of the
+// other roots, by a bound that needs no converged root (no_image) or else
+// polished in FP64 (spurious).  (Without that proof, a root that the sweeps
+// had not brought to its place passed for no image: 51 of 1e8 texels about
+// the caustics of lenses of s = 2.5 to 28 lost a pair of images.)
 // Emulated on the CPU over 23 lenses (s 0.01 to 20, q 1e-8 to 5, maps about
 // the caustics among them): no texel kept differs from the oracle's value,
 // and less than 1 in 1000 is left to the general form (1 to 12 % in maps of a
@@ -393,6 +398,34 @@ __device__ __noinline__ bool spurious(double mb, double ma, double h, cd om,
   return fr * fr + fi * fi > 1e-12 * sc * sc;
 }
 
+// Whether a disc about z holds a root of the monic quintic b and no image, by
+// FP32 arithmetic alone: z may be far from converged.  f: |residual of Eq. 2|
+// at z, ra and rb: 1/|z - h|^2 and 1/|z|^2.
+//  * 5 |p/p'| about any point is the radius of a disc with a root.  Horner's
+//    rounding and that of the coefficients are below 40 u sum |b_t| |z|^t.
+//  * Within rho of z the residual changes by less than
+//    rho (1 + 2 ma / |z - h|^2 + 2 mb / |z|^2) when 2 rho is below both
+//    distances.  f's own rounding is some 1e-5 of its terms, f above 0.2 %.
+__device__ __forceinline__ bool no_image(const cf (&b)[5], cf z, float f,
+                                         float ra, float rb, float ma,
+                                         float mb) {
+  cf p = mk(1.f, 0.f), dp = mk(0.f, 0.f);
+  float s = 1.f, ds = 0.f;  // the same of the absolute values
+  const float az = sqrtf(ab2(z));
+#pragma unroll
+  for (int u = 4; u >= 0; --u) {
+    dp = add(mul(dp, z), p);
+    p = add(mul(p, z), b[u]);
+    ds = ds * az + s;
+    s = s * az + sqrtf(ab2(b[u]));
+  }
+  const float e = 40.f / 16777216.f;
+  const float rho = 5.f * (sqrtf(ab2(p)) + e * s) /
+                    (sqrtf(ab2(dp)) - e * ds);
+  return rho > 0.f && 4.f * rho * rho * fmaxf(ra, rb) < 1.f &&
+         2.f * rho * (1.f + 2.f * (ma * ra + mb * rb)) < f;
+}
+
 __global__ void __launch_bounds__(kPolyThreads)
     k_poly_fast(double mb, double ma, double xb, double h, double L, int npix,
                 float *__restrict__ A) {
@@ -470,6 +503,8 @@ __global__ void __launch_bounds__(kPolyThreads)
   const cf omf = mk((float)om.re, (float)om.im);
   cf w0[5], z0[5];  // their polished and their own places
   int ni = 0;
+  cf zn = mk(0.f, 0.f);  // the other root that leaves Eq. 2 the furthest
+  float fn = 0.f, fn_sc = 0.f, ra_n = 0.f, rb_n = 0.f;
 #pragma unroll
   for (int t = 0; t < 5; ++t) w0[t] = z0[t] = mk(0.f, 0.f);
 #pragma unroll
@@ -487,7 +522,15 @@ __global__ void __launch_bounds__(kPolyThreads)
         const float sc = sqrtf(ab2(w)) + sqrtf(ab2(omf)) +
                          maf * sqrtf(ra) + mbf * sqrtf(rb);
         // (a NaN is a candidate, which will not converge)
-        cand = !(sqrtf(ab2(f)) >= 0.002f * sc);
+        const float af = sqrtf(ab2(f));
+        cand = !(af >= 0.002f * sc);
+        if (!cand && af > fn_sc * sc) {
+          zn = w;
+          fn = af;
+          fn_sc = af / sc;
+          ra_n = ra;
+          rb_n = rb;
+        }
       }
       const cf D = add(scl(maf, mul(ia, ia)), scl(mbf, mul(ib, ib)));
       const float rd = rcpf(1.f - ab2(D));
@@ -554,6 +597,11 @@ __global__ void __launch_bounds__(kPolyThreads)
       ok = spurious(mb, ma, h, om, z0[t]);
     }
   }
+  // three images are all there are when one root is known not to be one: a
+  // candidate shown spurious, or another root
+  if (images == 3 && ni == 3)
+    ok = ok && (no_image(b, zn, fn, ra_n, rb_n, maf, mbf) ||
+                spurious(mb, ma, h, om, zn));
   A[(size_t)j * npix + i] =
       ok && (images == 3 || images == 5) && parity == -1
           ? __double2float_rn(A_sum)

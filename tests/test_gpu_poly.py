@@ -117,3 +117,38 @@ def test_poly_map_fast_and_general_forms(ctx, s, q, L, npix):
     assert np.isfinite(A).all() and (A >= 1.0 - 1e-6).all()
     rel = np.abs(A.astype(np.float64) - P) / P
     assert (rel > 1e-6).mean() <= 1e-3
+
+
+# A next to a fold goes as the square root of the distance to it, so an error
+# of a few ulps of the texel's place (4e-16 at |y| < 2) moves A by some
+# 2e-14 A^2 of itself where the caustic's scale is 1e-2
+def _near_caustic(ctx, s, q, L, npix, cols, rows):
+    A = ctx.build_map(s, q, L, npix, 1, generator="poly").values()
+    d = 2 * L / npix
+    got = A[rows[0]:rows[1], cols[0]:cols[1]].astype(np.float64)
+    P = np.array([[orc.mag_point(s, q, -L + (i + 0.5) * d, -L + (j + 0.5) * d)
+                   for i in range(*cols)] for j in range(*rows)])
+    assert np.isfinite(A).all()
+    assert (np.abs(got - P) <= (1e-6 + 2e-14 * P ** 2) * P).all()
+
+
+@pytest.mark.parametrize("s,q,L,col,row", [
+    # FP32 iterations that do not converge, or meet away from the roots: a
+    # pair of images must not be lost with them
+    (5.782718165466182, 0.04254807934035008, 2.0082425727177124, 1813, 2048),
+    (8.05, 0.235, 1.924, 447, 2048),
+    (4.13, 0.867, 2.296, 482, 2047),
+    (3.9046490442410478, 0.33909214800333815, 2.15438373784511, 1206, 2047),
+])
+def test_poly_map_keeps_every_image_pair(ctx, s, q, L, col, row):
+    _near_caustic(ctx, s, q, L, 4096, (col - 3, col + 4), (row - 3, row + 4))
+
+
+@pytest.mark.parametrize("s,q,L", [(4.0, 0.5, 1.6), (8.0, 0.3, 2.2),
+                                   (20.0, 0.1, 2.0)])
+def test_poly_map_about_a_wide_lens_caustic(ctx, s, q, L):
+    """Every texel about the heavier lens' caustic, inside and outside."""
+    e2 = q / (1 + q)
+    col = int((-s * e2 + e2 / s + L) / (2 * L / 4096))
+    assert 40 <= col < 4096 - 40
+    _near_caustic(ctx, s, q, L, 4096, (col - 40, col + 40), (2028, 2068))
