@@ -33,6 +33,8 @@
 #include <math_constants.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "morse_internal.cuh"
 
 namespace morse {
@@ -267,22 +269,35 @@ __device__ double poly_texel(double s, double q, double L, int npix,
   }
 }
 
-// Texels whose value is `todo` by the general form (todo NaN: those the fast
-// kernel left; otherwise all).  A block collects them in shared memory
-// first, so that its warps are full.
+// The general form of every texel, or (LEFT) of those the fast form left, NaN:
+// a block collects them from a tile of texels in shared memory first, so that
+// its warps are full.
+//
+// A texel takes a warp half a millisecond or more whether its other lanes
+// have one too, so what counts is that the texels spread over the SMs: a
+// thread takes one at a time, and the tiles of a small map are small
+// (launch_poly_map).  Every map in tiles of 16 texels per thread took 35 ms
+// at 64^2 and 31 at 256^2, so 2.4 and 6.8 (q = 1e-9).
 constexpr int kPolyThreads = 128, kPolyTile = 16 * kPolyThreads;
 
+template <bool LEFT>
 __global__ void __launch_bounds__(kPolyThreads)
-    k_poly_map(double s, double q, double L, int npix, bool left,
+    k_poly_map(double s, double q, double L, int npix, int tile,
                float *__restrict__ A) {
-  __shared__ unsigned s_q[kPolyTile], s_n;
   const size_t n = (size_t)npix * npix;
-  for (size_t c0 = blockIdx.x * (size_t)kPolyTile; c0 < n;
-       c0 += gridDim.x * (size_t)kPolyTile) {
+  if (!LEFT) {
+    for (size_t k = blockIdx.x * (size_t)kPolyThreads + threadIdx.x; k < n;
+         k += gridDim.x * (size_t)kPolyThreads)
+      A[k] = __double2float_rn(poly_texel(s, q, L, npix, k));
+    return;
+  }
+  __shared__ unsigned s_q[kPolyTile], s_n;
+  for (size_t c0 = blockIdx.x * (size_t)tile; c0 < n;
+       c0 += gridDim.x * (size_t)tile) {
     if (threadIdx.x == 0) s_n = 0;
     __syncthreads();
-    for (int t = threadIdx.x; t < kPolyTile; t += kPolyThreads)
-      if (c0 + t < n && (!left || isnan(A[c0 + t])))
+    for (int t = threadIdx.x; t < tile; t += kPolyThreads)
+      if (c0 + t < n && isnan(A[c0 + t]))
         s_q[atomicAdd(&s_n, 1u)] = (unsigned)t;
     __syncthreads();
     const unsigned m = s_n;
@@ -628,12 +643,23 @@ cudaError_t launch_poly_map(double s, double q, double L, int npix, float *A,
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
+  // one texel per thread; or tiles two to an SM, of one to 16 texels per
+  // thread (larger ones only where there are tiles enough: fuller warps)
   const size_t n = (size_t)npix * npix;
-  size_t blocks = (n + kPolyTile - 1) / kPolyTile;
-  const size_t cap = (size_t)sm_count * 16;
-  if (blocks > cap) blocks = cap;
-  k_poly_map<<<(unsigned)blocks, kPolyThreads, 0, st>>>(s, q, L, npix, fast,
-                                                        A);
+  size_t tile = kPolyThreads;
+  if (fast) {
+    tile = (n / (2 * (size_t)sm_count) + kPolyThreads) / kPolyThreads *
+           kPolyThreads;
+    tile = std::min<size_t>(tile, kPolyTile);
+  }
+  const size_t blocks =
+      std::min((n + tile - 1) / tile, (size_t)sm_count * 16);
+  if (fast)
+    k_poly_map<true><<<(unsigned)blocks, kPolyThreads, 0, st>>>(
+        s, q, L, npix, (int)tile, A);
+  else
+    k_poly_map<false><<<(unsigned)blocks, kPolyThreads, 0, st>>>(
+        s, q, L, npix, (int)tile, A);
   return cudaGetLastError();
 }
 

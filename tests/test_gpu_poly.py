@@ -152,3 +152,28 @@ def test_poly_map_about_a_wide_lens_caustic(ctx, s, q, L):
     col = int((-s * e2 + e2 / s + L) / (2 * L / 4096))
     assert 40 <= col < 4096 - 40
     _near_caustic(ctx, s, q, L, 4096, (col - 40, col + 40), (2028, 2068))
+
+
+def test_poly_map_general_form_spreads_small_maps(ctx):
+    """A 64^2 map by the general form alone has a sixteenth of the texels of
+    a 256^2 one; it must not take as long (half as long would already mean
+    that most of the chip waits)."""
+    ms = {}
+    for npix in (64, 256):
+        t = []
+        for _ in range(4):
+            ctx.build_map(1.0, 1e-9, 2.0, npix, 1, generator="poly").free()
+            t.append(ctx.kernel_ms(0))
+        ms[npix] = min(t)
+    assert ms[64] < 0.5 * ms[256]
+
+
+@pytest.mark.parametrize("npix", [2, 11, 12, 197, 198])
+def test_poly_map_tiles(ctx, npix):
+    """Maps of less and more than a block's tile of texels, of tiles of one
+    and of two texels per thread, and the general form alone."""
+    for s, q in ((0.05, 0.3), (1.0, 1e-9)):
+        A = ctx.build_map(s, q, 2.0, npix, 1, generator="poly").values()
+        P = orc.poly_map(s, q, 2.0, npix, nthreads=NT)
+        rel = np.abs(A.astype(np.float64) - P) / P
+        assert (rel > 1e-6).mean() <= 1e-3
