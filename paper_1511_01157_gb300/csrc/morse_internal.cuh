@@ -94,6 +94,7 @@ struct morse_event {
                             // (t - t_ref, w)[n], w (F - F_ref)[n],
                             // (F - F_ref)[n]; then the subsets' slots
   int n_sub;                // subsets (0: the search does not screen)
+  bool weak;                // the subsets' bounds would discard too little
   morse_subset sub[kScreenLevels];
   double S1, SF, SFF, Fref; // FP64 sums of the stored FP32 values
   double invS1, CFF;        // 1/S_1, S_FF - S_F^2/S_1

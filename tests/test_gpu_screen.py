@@ -185,3 +185,62 @@ def test_listed_bounds_on_one_to_four_lanes(m, setup, n, kind):
             assert np.array_equal(got["idx"][:len(idx)], idx)
             assert np.array_equal(got["chi2"][:len(idx)], val)
     mp.set_lookup(False)
+
+
+def _curve(ctx, n, kind):
+    t = synth.epoch_times(n, 9)
+    f = {"flat": np.full(n, 2.0),
+         "faint": 2.0 + 0.03 / np.sqrt(1.0 + (t / 20.0) ** 2),
+         # no trajectory fits it: screened, and the lists come out too long
+         "wave": 2.0 + 0.5 * np.sin(2 * np.pi * t / 7.0),
+         "strong": 0.4 + 1.0 / np.sqrt(2e-4 + (t / 15.0) ** 2)}[kind]
+    F, sig = synth.photometry(f, 9)
+    return ctx.event(t, F, sig)
+
+
+@pytest.mark.parametrize("n", [300, 1500, 3001])
+def test_light_curves_the_bounds_cannot_use(m, setup, n):
+    """Without a signal that the subsets can discard by, the search is the
+    unscreened one (that of a light curve too short for subsets), not the
+    screen and then all of it again."""
+    ctx, mp = setup
+    # (one subset: on large grids only)
+    big = n < 1024
+    g = m.Grid.make(40, 40, 25 if big else 5, 15 if big else 5, 1e-3, 0.5,
+                    -2.0, 2.0, 5.0, 80.0, True, True, 33)
+
+    def launches(ev):
+        ctx.grid_chi2(ev, mp, g)
+        a = ctx.launch_count()
+        ctx.grid_chi2(ev, mp, g)
+        return ctx.launch_count() - a
+
+    plain = launches(_curve(ctx, 100, "strong"))
+    assert launches(_curve(ctx, n, "strong")) > plain
+    assert launches(_curve(ctx, n, "wave")) > plain
+    for kind in ("flat", "faint"):
+        assert launches(_curve(ctx, n, kind)) == plain
+    for kind in ("wave", "faint"):
+        ev = _curve(ctx, n, kind)
+        for k in (1, 33):
+            chi2, *_ = ctx.grid_chi2_dense(ev, mp, _grid(m, k))
+            idx, val = _best(chi2, k)
+            got = ctx.grid_chi2(ev, mp, _grid(m, k))
+            assert np.array_equal(got["idx"], idx)
+            assert np.array_equal(got["chi2"], val)
+
+
+def test_batch_of_weak_and_strong_light_curves(m, setup):
+    ctx, mp = setup
+    other = ctx.build_map(0.7, 2e-2, 2.0, 301, 2100, image_halfwidth=3.0,
+                          deflect="fp32")
+    g = _grid(m, 40)
+    for kinds in (("strong", "flat", "wave", "faint", "strong", "flat"),
+                  ("flat", "faint", "flat"), ("flat", "strong", "wave")):
+        evs = [_curve(ctx, n, kind) for n, kind in
+               zip((130, 700, 1500, 900, 3000, 5000), kinds)]
+        got = ctx.grid_chi2_batch(evs, [mp, other], g)
+        for i, ev in enumerate(evs):
+            for j, x in enumerate((mp, other)):
+                assert np.array_equal(got[i, j], ctx.grid_chi2(ev, x, g))
+    other.free()
