@@ -671,9 +671,7 @@ size_t plan_screen(const morse_event *ev, const morse_grid *g,
     pl->small = true;
     pl->want = pl->pilot_cap = pl->list0_cap = pl->list_cap = (unsigned)count;
     pl->off_hist = align_up(at, 256);
-    pl->off_code = align_up(
-        pl->off_hist + sizeof(unsigned) * (morse::kScreenBins +
-                                           morse::kScreenWords), 256);
+    pl->off_code = align_up(pl->off_hist + morse::kScreenHeadBytes, 256);
     pl->off_pil = pl->off_ub = align_up(
         pl->off_code + sizeof(unsigned short) * (size_t)(count + 8), 256);
     pl->off_list0 = pl->off_list = align_up(
@@ -692,9 +690,7 @@ size_t plan_screen(const morse_event *ev, const morse_grid *g,
   // eight is not worth having)
   pl->list_cap = (unsigned)(count - count / 8);
   pl->off_hist = align_up(at, 256);  // histogram and list lengths: cleared
-  pl->off_code = align_up(
-      pl->off_hist + sizeof(unsigned) * (morse::kScreenBins +
-                                         morse::kScreenWords), 256);
+  pl->off_code = align_up(pl->off_hist + morse::kScreenHeadBytes, 256);
   pl->off_pil = align_up(
       pl->off_code + sizeof(unsigned short) * (size_t)(count + 8), 256);
   pl->off_ub = pl->off_pil + sizeof(unsigned) * (size_t)pl->pilot_cap;
@@ -715,6 +711,7 @@ void screen_bufs(const Plan &pl, char *base, char *words,
   B->code = (unsigned short *)(base + pl.off_code);
   B->hist = (unsigned *)words;
   B->n = B->hist + morse::kScreenBins;
+  B->smp = (float *)(B->n + morse::kScreenWords);
   B->pilot = (unsigned *)(base + pl.off_pil);
   B->ub = (float *)(base + pl.off_ub);
   B->list0 = (unsigned *)(base + pl.off_list0);
@@ -1249,10 +1246,8 @@ struct BatchLayout {
   size_t lists;  // top-K lists of the larger pass
   size_t off_task, off_done, off_hist, off_scr;
 };
-// bytes of a screened search's histogram and counters in a batch
-const size_t kScreenWordBytes =
-    align_up(sizeof(unsigned) * (morse::kScreenBins + morse::kScreenWords),
-             256);
+// bytes of a screened search's histogram, counters and sample in a batch
+const size_t kScreenWordBytes = align_up(morse::kScreenHeadBytes, 256);
 
 struct BatchHdr {
   unsigned counter[3];  // pilot, main (unstaged units), main (staged)

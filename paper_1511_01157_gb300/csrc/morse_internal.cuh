@@ -344,6 +344,7 @@ struct ScreenBufs {
                             // whole (4: nonzero), discarded (5); candidates
                             // of the listed search (6), records made (7:
                             // nonzero)
+  float *smp;               // [kScreenSample] third-subset bounds of a sample
   unsigned *pilot;          // [pilot_cap] trajectories of the pilot (null:
                             // all of a small grid, ub[count])
   float *ub;                // [pilot_cap] their chi^2 bounds from above
@@ -353,7 +354,10 @@ struct ScreenBufs {
   unsigned pilot_cap, list0_cap, list_cap;
   unsigned want;            // pilot trajectories asked for
 };
-constexpr int kScreenBins = 1024, kScreenWords = 8;
+constexpr int kScreenBins = 1024, kScreenWords = 8, kScreenSample = 512;
+// bytes of hist, n and smp, which lie one after the other
+constexpr size_t kScreenHeadBytes =
+    4 * (size_t)(kScreenBins + kScreenWords + kScreenSample);
 constexpr unsigned kScreenBinCodes = 32768 / kScreenBins;
 constexpr unsigned kScreenCut = 0xFFFFu;  // code of a cut line's trajectory
 

@@ -244,3 +244,26 @@ def test_batch_of_weak_and_strong_light_curves(m, setup):
             for j, x in enumerate((mp, other)):
                 assert np.array_equal(got[i, j], ctx.grid_chi2(ev, x, g))
     other.free()
+
+
+def test_no_list_where_a_sample_says_it_would_be_long(m, setup):
+    """307 200 trajectories that all miss the light curve: the screen must end
+    before the second and third subsets of the whole grid (half as much again
+    as the search of a flat light curve, which is not screened)."""
+    ctx, mp = setup
+    g = m.Grid.make(40, 40, 16, 12, 1e-3, 0.5, -2.0, 2.0, 5.0, 80.0, True,
+                    True, 16)
+    ms = {}
+    for kind in ("flat", "wave"):
+        ev = _curve(ctx, 1100, kind)
+        got = [ctx.grid_chi2(ev, mp, g) for _ in range(2)][-1]
+        t = []
+        for _ in range(7):
+            ctx.grid_chi2(ev, mp, g)
+            t.append(ctx.kernel_ms(2))
+        ms[kind] = min(t)
+        chi2, *_ = ctx.grid_chi2_dense(ev, mp, g)
+        idx, val = _best(chi2, 16)
+        assert np.array_equal(got["idx"], idx)
+        assert np.array_equal(got["chi2"], val)
+    assert ms["wave"] < 1.35 * ms["flat"]
