@@ -443,39 +443,43 @@ __device__ __forceinline__ void lm_step(const RefineState &S, int i) {
 // of FP64 set-up, fit, assembly and step that one warp runs for all 16; with
 // one trajectory per SM 29 us, 27k and 34k.  Two blocks of 8 warps or four of
 // 4 per SM were the same or slower: their FP64 chains share the SM's pipe.
-template <bool EP_SMEM, int MINB, int UN>
+//
+// The chain costs the same for 32 trajectories, its lanes, as for 16: where
+// there are more than one wave of blocks and the sweeps are short, a warp
+// takes TPW = 2 trajectories (launch_refine).
+template <bool EP_SMEM, int MINB, int UN, int TPW>
 __global__ void __launch_bounds__(kAdjWarps * 32, MINB)
     k_refine(const SearchParams P, RefineState S,
              const float4 *const *__restrict__ tq, int n, int iters,
              double t_ref) {
   extern __shared__ __align__(16) float4 s_ep[];
-  __shared__ AdjTraj s_tr[kAdjWarps];
-  __shared__ TrajC s_best[kAdjWarps];
-  __shared__ Acc s_acc[kAdjWarps];
-  __shared__ double s_Fs[kAdjWarps], s_Bc[kAdjWarps];
-  __shared__ AdjSums s_sum[kAdjWarps];
-  __shared__ double s_chi[kAdjWarps];
-  __shared__ double s_state[kAdjWarps * kRefineDoubles];
-  __shared__ int s_eval[kAdjWarps], s_more;
+  constexpr int kTr = kAdjWarps * TPW;  // trajectories of a block, at most
+  __shared__ AdjTraj s_tr[kTr];
+  __shared__ TrajC s_best[kTr];
+  __shared__ Acc s_acc[kTr];
+  __shared__ double s_Fs[kTr], s_Bc[kTr];
+  __shared__ AdjSums s_sum[kTr];
+  __shared__ double s_chi[kTr];
+  __shared__ double s_state[kTr * kRefineDoubles];
+  __shared__ int s_eval[kTr], s_more;
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   const int warps = blockDim.x >> 5;
-  const int i0 = blockIdx.x * warps;
-  const bool live = i0 + warp < n;
-  const bool mine = warp == 0 && lane < warps && i0 + lane < n;
+  const int i0 = blockIdx.x * warps * TPW;
+  const bool mine = warp == 0 && lane < warps * TPW && i0 + lane < n;
   if (EP_SMEM)
     for (int e = threadIdx.x; e < P.n_ep; e += blockDim.x) s_ep[e] = P.ep[e];
   // the block's states (each read and written by one lane of warp 0 only)
   RefineState B;
   B.th_cur = s_state;
-  B.th_best = B.th_cur + 4 * kAdjWarps;
-  B.chi2_cur = B.th_best + 4 * kAdjWarps;
-  B.chi2_best = B.chi2_cur + kAdjWarps;
-  B.lam = B.chi2_best + kAdjWarps;
-  B.g_cur = B.lam + kAdjWarps;
-  B.g_best = B.g_cur + 4 * kAdjWarps;
-  B.H_cur = B.g_best + 4 * kAdjWarps;
-  B.H_best = B.H_cur + 10 * kAdjWarps;
+  B.th_best = B.th_cur + 4 * kTr;
+  B.chi2_cur = B.th_best + 4 * kTr;
+  B.chi2_best = B.chi2_cur + kTr;
+  B.lam = B.chi2_best + kTr;
+  B.g_cur = B.lam + kTr;
+  B.g_best = B.g_cur + 4 * kTr;
+  B.H_cur = B.g_best + 4 * kTr;
+  B.H_best = B.H_cur + 10 * kTr;
   const float4 *quad = P.quad;
   if (mine) {
     const int j = i0 + lane;
@@ -499,14 +503,17 @@ __global__ void __launch_bounds__(kAdjWarps * 32, MINB)
                      !same_traj(T.c, s_best[lane]);
     }
     __syncthreads();
-    const bool eval = live && s_eval[warp];
     AdjTraj T;
-    SearchParams Q = P;  // this warp's map
-    if (eval) {
-      T = s_tr[warp];
+    SearchParams Q = P;  // the trajectory's map
+    bool eval = false;
+#pragma unroll 1
+    for (int k = warp; k < warps * TPW; k += warps) {
+      eval = i0 + k < n && s_eval[k];
+      if (!eval) continue;
+      T = s_tr[k];
       Q.quad = T.quad;
       const Acc a = phase1<false, 0, UN>(Q, ep, T.c, lane);
-      if (lane == 0) s_acc[warp] = a;
+      if (lane == 0) s_acc[k] = a;
     }
     __syncthreads();
     if (mine && s_eval[lane]) {
@@ -516,14 +523,21 @@ __global__ void __launch_bounds__(kAdjWarps * 32, MINB)
       s_Bc[lane] = f.Bc;
     }
     __syncthreads();
-    if (eval) {
+#pragma unroll 1
+    for (int k = warp; k < warps * TPW; k += warps) {
+      if (TPW > 1) {
+        eval = i0 + k < n && s_eval[k];
+        if (eval) T = s_tr[k];
+        Q.quad = T.quad;
+      }
+      if (!eval) continue;
       AdjSums a;
       const double x =
-          adj_sweep<true, UN>(Q, ep, T, __double2float_rn(s_Fs[warp]),
-                              __double2float_rn(s_Bc[warp]), lane, a);
+          adj_sweep<true, UN>(Q, ep, T, __double2float_rn(s_Fs[k]),
+                              __double2float_rn(s_Bc[k]), lane, a);
       if (lane == 0) {
-        s_chi[warp] = x;
-        s_sum[warp] = a;
+        s_chi[k] = x;
+        s_sum[k] = a;
       }
     }
     __syncthreads();
@@ -623,8 +637,9 @@ static cudaError_t ep_smem(K kernel) {
 cudaError_t adjoint_setup() {
   cudaError_t e = ep_smem(k_theta<true, 1, 8>);
   if (e == cudaSuccess) e = ep_smem(k_theta<true, 2, 4>);
-  if (e == cudaSuccess) e = ep_smem(k_refine<true, 1, 8>);
-  if (e == cudaSuccess) e = ep_smem(k_refine<true, 2, 4>);
+  if (e == cudaSuccess) e = ep_smem(k_refine<true, 1, 8, 1>);
+  if (e == cudaSuccess) e = ep_smem(k_refine<true, 2, 4, 1>);
+  if (e == cudaSuccess) e = ep_smem(k_refine<true, 2, 4, 2>);
   return e;
 }
 
@@ -638,7 +653,14 @@ cudaError_t launch_theta(const SearchParams &P, const double *theta, int n,
 }
 
 // Blocks of as many warps as spread the trajectories over the SMs, at most
-// kAdjWarps.
+// kAdjWarps; two trajectories to a warp for light curves of up to
+// kRefinePairEpMax epochs where one to a warp would take more than two blocks
+// per SM.  20 iterations of 4865, 9728, 9800 and 20 000 starts: 64 epochs 856,
+// 961, 1329, 2264 -> 544, 624, 1065, 1640 us, 1500 epochs 1308, 1722, 2301,
+// 3906 -> 1134, 1379, 2255, 3525; 2000 epochs 1443, 1954, 2590, 4440 against
+// 1333, 1624, 2645, 4152 and 4000 epochs 2006, 2958, 3833, 6612 against 2106,
+// 2644, 4216, 6631: the last block's sweeps are twice as long.
+constexpr int kRefinePairEpMax = 1536;
 cudaError_t launch_refine(const SearchParams &P, const RefineState &S, int n,
                           int iters, double t_ref, int sm_count,
                           cudaStream_t st, const float4 *const *tq) {
@@ -647,21 +669,21 @@ cudaError_t launch_refine(const SearchParams &P, const RefineState &S, int n,
   const int blocks = (n + warps - 1) / warps, threads = 32 * warps;
   const bool few = blocks <= sm_count;
   const size_t sh = sizeof(float4) * P.n_ep;
-  if (P.n_ep <= kAdjEpSmemMax) {
-    if (few)
-      k_refine<true, 1, 8><<<blocks, threads, sh, st>>>(P, S, tq, n, iters,
-                                                         t_ref);
-    else
-      k_refine<true, 2, 4><<<blocks, threads, sh, st>>>(P, S, tq, n, iters,
-                                                         t_ref);
-  } else {
-    if (few)
-      k_refine<false, 1, 8><<<blocks, threads, 0, st>>>(P, S, tq, n, iters,
-                                                         t_ref);
-    else
-      k_refine<false, 2, 4><<<blocks, threads, 0, st>>>(P, S, tq, n, iters,
-                                                         t_ref);
-  }
+  if (P.n_ep <= kRefinePairEpMax && blocks > 2 * sm_count)
+    k_refine<true, 2, 4, 2><<<(blocks + 1) / 2, threads, sh, st>>>(
+        P, S, tq, n, iters, t_ref);
+  else if (P.n_ep <= kAdjEpSmemMax && few)
+    k_refine<true, 1, 8, 1><<<blocks, threads, sh, st>>>(P, S, tq, n, iters,
+                                                          t_ref);
+  else if (P.n_ep <= kAdjEpSmemMax)
+    k_refine<true, 2, 4, 1><<<blocks, threads, sh, st>>>(P, S, tq, n, iters,
+                                                          t_ref);
+  else if (few)
+    k_refine<false, 1, 8, 1><<<blocks, threads, 0, st>>>(P, S, tq, n, iters,
+                                                          t_ref);
+  else
+    k_refine<false, 2, 4, 1><<<blocks, threads, 0, st>>>(P, S, tq, n, iters,
+                                                          t_ref);
   return cudaGetLastError();
 }
 

@@ -346,3 +346,53 @@ def test_refine_does_not_depend_on_the_split(ctx, m, setup, n, n_ep):
     assert np.all(out["chi2"] <= ctx.refine(ev, mp, st, iters=0)["chi2"])
     late = ctx.refine(ev, mp, out, iters=2000)
     assert np.array_equal(ctx.refine(ev, mp, out, iters=4000), late)
+
+
+@pytest.mark.parametrize("n,n_ep", [(4864, 64), (4865, 64), (4881, 1536),
+                                    (4865, 1537)])
+def test_refine_of_many_starts(ctx, m, setup, n, n_ep):
+    """More starts than one wave of blocks: two to a warp for short light
+    curves, the last warp with one or none.  Every record is that of a call
+    with fewer starts, to the last bit."""
+    c, mp = setup[0], setup[5]
+    t = synth.epoch_times(n_ep, 12, c["t0"])
+    F, sig = synth.photometry(1.0 + 1.0 / np.sqrt(
+        c["u0"] ** 2 + ((t - c["t0"]) / c["tE"]) ** 2), 12)
+    ev = ctx.event(t, F, sig)
+    rng = np.random.default_rng(n + n_ep)
+    st = np.zeros(n, dtype=m.FIT_DTYPE)
+    st["t0"] = c["t0"] + rng.uniform(-1.0, 1.0, n)
+    st["tE"] = c["tE"] * np.exp(rng.uniform(-0.3, 0.3, n))
+    st["u0"] = c["u0"] * np.exp(rng.uniform(-0.5, 0.5, n))
+    st["alpha"] = c["alpha"] + rng.uniform(-0.2, 0.2, n)
+    st["idx"] = np.arange(n)
+    out = ctx.refine(ev, mp, st, iters=30)
+    parts = [ctx.refine(ev, mp, st[i:i + 2400], iters=30)
+             for i in range(0, n, 2400)]
+    assert out.tobytes() == np.concatenate(parts).tobytes()
+
+
+def test_refine_of_many_starts_of_a_short_light_curve_is_quick(ctx, m, setup):
+    """One start more than two blocks per SM hold does not cost a second wave
+    of blocks (as long again)."""
+    c, mp = setup[0], setup[5]
+    t = synth.epoch_times(64, 12, c["t0"])
+    F, sig = synth.photometry(1.0 + 1.0 / np.sqrt(
+        c["u0"] ** 2 + ((t - c["t0"]) / c["tE"]) ** 2), 12)
+    ev = ctx.event(t, F, sig)
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    ms = []
+    for n in (32 * sms, 32 * sms + 1):
+        rng = np.random.default_rng(3)
+        st = np.zeros(n, dtype=m.FIT_DTYPE)
+        st["t0"] = c["t0"] + rng.uniform(-1.0, 1.0, n)
+        st["tE"] = c["tE"] * np.exp(rng.uniform(-0.3, 0.3, n))
+        st["u0"] = c["u0"] * np.exp(rng.uniform(-0.5, 0.5, n))
+        st["alpha"] = c["alpha"] + rng.uniform(-0.2, 0.2, n)
+        w = []
+        for _ in range(6):
+            ctx.refine(ev, mp, st, iters=30)
+            w.append(ctx.kernel_ms(6))
+        ms.append(min(w))
+    assert ms[1] < 1.4 * ms[0]
