@@ -2244,18 +2244,18 @@ void morse_map_free(morse_map *map) {
 //     0.88 to 1.24, below 1.2: 1.0 to 1.36.
 constexpr double kScreenGainOne = 1.2, kScreenGainThree = 1.9;
 
-// s^2, from at most 1024 pairs of neighbouring epochs
+// s^2, from at most 256 pairs of neighbouring epochs (to 12 %)
 static double noise_variance(const float2 *tw, const float *fc, int64_t n) {
-  const int64_t pairs = std::min<int64_t>(n - 1, 1024);
-  std::vector<double> d((size_t)pairs);
+  double d[256];
+  const int64_t pairs = std::min<int64_t>(n - 1, 256);
   for (int64_t k = 0; k < pairs; ++k) {
     const int64_t i = k * (n - 1) / pairs;
     const double wa = tw[i].y, wb = tw[i + 1].y;
     const double df = (double)fc[i + 1] - (double)fc[i];
-    d[(size_t)k] = df * df * (wa / (wa + wb)) * wb;
+    d[k] = df * df * (wa / (wa + wb)) * wb;
   }
-  std::nth_element(d.begin(), d.begin() + pairs / 2, d.end());
-  return d[(size_t)(pairs / 2)] / 0.4549;  // the median of chi^2_1
+  std::nth_element(d, d + pairs / 2, d + pairs);
+  return d[pairs / 2] / 0.4549;  // the median of chi^2_1
 }
 
 static void screen_subsets(morse_event *ev, std::vector<float4> &h, int64_t n,
@@ -2278,23 +2278,37 @@ static void screen_subsets(morse_event *ev, std::vector<float4> &h, int64_t n,
       (deciding ? kScreenGainThree : kScreenGainOne) * (double)n *
       noise_variance(reinterpret_cast<const float2 *>(h.data()),
                      reinterpret_cast<const float *>(h.data()) + 3 * n, n);
-  std::vector<double> x;
-  std::vector<int> sel;
+  // information of the runs of 4 epochs, in one pass; a level's runs are
+  // pairs of the last one's
+  std::vector<double> info((size_t)(n + 3) / 4, 0.0), x;
+  double sum = 0.0;
+  {
+    const float2 *tw = reinterpret_cast<const float2 *>(h.data());
+    const float *fc = reinterpret_cast<const float *>(tw + n) + n;
+    const double mean = SF / S1;
+    for (size_t r = 0; r < info.size(); ++r) {
+      double v = 0.0;
+      for (int64_t i = 4 * (int64_t)r; i < std::min(n, 4 * (int64_t)r + 4);
+           ++i) {
+        const double d = (double)fc[i] - mean;
+        v += (double)tw[i].y * d * d;
+      }
+      info[r] = v;
+      sum += v;
+    }
+  }
+  std::vector<int> sel;  // the runs taken
   for (int l = 0; l < kScreenLevels && sizes[l] > 0; ++l) {
     const int run = runs[l];
     const int64_t nr = (n + run - 1) / run;
     const double m = (double)sizes[l] / run;  // runs to take
-    const float2 *tw = reinterpret_cast<const float2 *>(h.data());
-    const float *fc = reinterpret_cast<const float *>(tw + n) + n;
-    const double mean = SF / S1;
-    x.assign((size_t)nr, 0.0);
-    double sum = 0.0;
-    for (int64_t i = 0; i < n; ++i) {
-      const double d = (double)fc[i] - mean;
-      const double v = (double)tw[i].y * d * d;
-      x[(size_t)(i / run)] += v;
-      sum += v;
+    if (l > 0) {
+      const size_t last = info.size();
+      for (size_t r = 0; r < (size_t)nr; ++r)
+        info[r] = info[2 * r] + (2 * r + 1 < last ? info[2 * r + 1] : 0.0);
+      info.resize((size_t)nr);
     }
+    x = info;
     const double even = 0.1 / (double)nr;
     const double per = sum > 0.0 ? 0.9 / sum : 0.0;
     for (double &v : x) v = v * per + even;
@@ -2315,39 +2329,49 @@ static void screen_subsets(morse_event *ev, std::vector<float4> &h, int64_t n,
       scale *= f;
     }
     sel.clear();
+    size_t taken = 0;
     double acc = 0.5;
     for (int64_t r = 0; r < nr; ++r) {
       const double next = acc + std::min(1.0, x[(size_t)r] * scale);
-      if (std::floor(next) > std::floor(acc))
-        for (int64_t i = r * run; i < std::min(n, (r + 1) * run); ++i)
-          sel.push_back((int)i);
+      if (std::floor(next) > std::floor(acc)) {
+        sel.push_back((int)r);
+        taken += (size_t)(std::min(n, (r + 1) * run) - r * run);
+      }
       acc = next;
     }
     // (the most the kernels stage of the first three)
     const size_t most[kScreenLevels] = {128, 192, 1024, (size_t)n};
-    if (sel.size() < 8 || sel.size() > most[l]) break;
+    if (taken < 8 || taken > most[l]) break;
     morse_subset &u = ev->sub[l];
-    u.m = (int)sel.size();
+    u.m = (int)taken;
     u.off = (int)h.size();
     u.S1 = u.SF = u.SFF = 0.0;
-    h.resize(h.size() + sel.size());
+    h.resize(h.size() + taken);
     const float2 *stw = reinterpret_cast<const float2 *>(h.data());
     const float *swf = reinterpret_cast<const float *>(stw + n);
     const float *sfc = swf + n;
     float2 *dtw = reinterpret_cast<float2 *>(h.data() + u.off);
     float *dwf = reinterpret_cast<float *>(dtw + u.m);
     float *dfc = dwf + u.m;
-    for (int k = 0; k < u.m; ++k) {
-      const int i = sel[(size_t)k];
-      dtw[k] = stw[i];
-      dwf[k] = swf[i];
-      dfc[k] = sfc[i];
-      u.S1 += (double)dtw[k].y;
-      u.SF += (double)dtw[k].y * (double)dfc[k];
-      u.SFF += (double)dtw[k].y * (double)dfc[k] * (double)dfc[k];
+    size_t k = 0;
+    for (int r : sel) {
+      const int64_t i0 = (int64_t)r * run, c = std::min(n - i0, (int64_t)run);
+      std::copy(stw + i0, stw + i0 + c, dtw + k);
+      std::copy(swf + i0, swf + i0 + c, dwf + k);
+      std::copy(sfc + i0, sfc + i0 + c, dfc + k);
+      k += (size_t)c;
+    }
+    for (k = 0; k < taken; ++k) {
+      const double w = dtw[k].y, f = dfc[k];
+      u.S1 += w;
+      u.SF += w * f;
+      u.SFF += w * f * f;
     }
     ev->n_sub = l + 1;
-    if (l == deciding) ev->weak = !(u.SFF - u.SF * u.SF / u.S1 > need);
+    if (l == deciding) {
+      ev->weak = !(u.SFF - u.SF * u.SF / u.S1 > need);
+      if (ev->weak) return;  // (in a batch with others: without the fourth)
+    }
   }
 }
 
@@ -2390,7 +2414,9 @@ morse_status morse_event_create(morse_ctx *ctx, const double *t,
   // of the stored FP32 values so that the device data is self-consistent
   // device layout: n float4 slots holding the arrays (t - t_ref, w)[n],
   // w Fc[n] and Fc[n] (structure of arrays, read as such by the sweeps)
-  std::vector<float4> h((size_t)n);
+  std::vector<float4> h;
+  h.reserve((size_t)n + (size_t)n / 3 + 2048);  // (room for the subsets)
+  h.resize((size_t)n);
   float2 *h_tw = reinterpret_cast<float2 *>(h.data());
   float *h_wf = reinterpret_cast<float *>(h_tw + n);
   float *h_fc = h_wf + n;

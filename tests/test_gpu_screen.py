@@ -247,11 +247,13 @@ def test_batch_of_weak_and_strong_light_curves(m, setup):
 
 
 def test_no_list_where_a_sample_says_it_would_be_long(m, setup):
-    """307 200 trajectories that all miss the light curve: the screen must end
+    """300 000 trajectories that all miss the light curve: the screen must end
     before the second and third subsets of the whole grid (half as much again
     as the search of a flat light curve, which is not screened)."""
-    ctx, mp = setup
-    g = m.Grid.make(40, 40, 16, 12, 1e-3, 0.5, -2.0, 2.0, 5.0, 80.0, True,
+    ctx = setup[0]
+    mp = ctx.build_map(1.0, 1e-3, 2.0, 1024, 4000, image_halfwidth=3.0,
+                       deflect="fp32")
+    g = m.Grid.make(30, 40, 25, 10, 1e-3, 0.5, -2.0, 2.0, 5.0, 80.0, True,
                     True, 16)
     ms = {}
     for kind in ("flat", "wave"):
@@ -266,4 +268,26 @@ def test_no_list_where_a_sample_says_it_would_be_long(m, setup):
         idx, val = _best(chi2, 16)
         assert np.array_equal(got["idx"], idx)
         assert np.array_equal(got["chi2"], val)
+    mp.free()
+    print(f"wave {ms['wave']:.3f} ms, flat {ms['flat']:.3f} ms")
     assert ms["wave"] < 1.35 * ms["flat"]
+
+
+def test_subsets_cost_little_of_an_event(m, setup):
+    """Light curves of 2^20 epochs have subsets, longer ones none: what they
+    add to making the event."""
+    import time
+    ctx = setup[0]
+    t = synth.epoch_times((1 << 20) + 1, 9)
+    f = 0.4 + 1.0 / np.sqrt(2e-4 + (t / 15.0) ** 2)
+    F, sig = synth.photometry(f, 9)
+    best = []
+    for n in (1 << 20, (1 << 20) + 1):
+        w = []
+        for _ in range(9):
+            t0 = time.perf_counter()
+            ctx.event(t[:n], F[:n], sig[:n]).free()
+            w.append(time.perf_counter() - t0)
+        best.append(min(w))
+    print(f"with subsets {best[0]:.4f} s, without {best[1]:.4f} s")
+    assert best[0] < 1.45 * best[1]
