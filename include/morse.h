@@ -633,11 +633,15 @@ morse_status morse_launch_count(const morse_ctx *ctx, uint64_t *n);
  *  MORSE_FAULT_ALLOC: the arg-th device allocation from now (arg >= 1)
  *    fails as cudaMalloc would when out of memory, without allocating; the
  *    call that makes it returns MORSE_ENOMEM.  One shot.
+ *  MORSE_FAULT_BUILD: the arg-th map build from now (arg >= 1) is not
+ *    launched; the call that makes it (a build, or a sweep with other maps'
+ *    builds and searches in flight) returns MORSE_ECUDA.  One shot.
  * Errors: EINVAL (unknown fault, arg out of range). */
 enum {
   MORSE_FAULT_NONE = 0,
   MORSE_FAULT_LOCK_HELD = 1,
-  MORSE_FAULT_ALLOC = 2
+  MORSE_FAULT_ALLOC = 2,
+  MORSE_FAULT_BUILD = 3
 };
 morse_status morse_inject_fault(morse_ctx *ctx, int fault, int64_t arg);
 

@@ -39,7 +39,7 @@ _lib = ctypes.CDLL(LIB_PATH)
 
 OK, EINVAL, ENOMEM, ECUDA, ETIMEOUT, EDEGENERATE, EUNSUPPORTED = range(7)
 # morse_inject_fault kinds (tests of the error paths)
-FAULT_NONE, FAULT_LOCK_HELD, FAULT_ALLOC = range(3)
+FAULT_NONE, FAULT_LOCK_HELD, FAULT_ALLOC, FAULT_BUILD = range(4)
 DEFLECT_FP64, DEFLECT_FP32 = 0, 1
 STORE_FP32, STORE_FP16LOG = 1, 2
 GEN_RAYS, GEN_POLY = 0, 1
@@ -592,7 +592,8 @@ class Context:
         """Make a bounded failure happen on purpose (morse_inject_fault):
         FAULT_LOCK_HELD (arg: spin limit) makes top-K searches give up their
         lock waits (ETIMEOUT); FAULT_ALLOC (arg: n) fails the n-th device
-        allocation from now (ENOMEM); FAULT_NONE clears."""
+        allocation from now (ENOMEM); FAULT_BUILD (arg: n) the n-th map
+        build (ECUDA); FAULT_NONE clears."""
         self._check(_lib.morse_inject_fault(self._h, int(kind), int(arg)),
                     "morse_inject_fault")
 

@@ -285,6 +285,8 @@ void map_release(morse_map *m) {
 // Queue the ray shooting and the texel conversion into existing storage
 // (no host synchronisation).
 morse_status enqueue_build(morse_ctx *ctx, morse_map *m, const BuildSpec &b) {
+  if (ctx->fault_build > 0 && --ctx->fault_build == 0)
+    return fail(ctx, MORSE_ECUDA, "injected failure of a map build");
   m->L = b.L;
   m->s = b.s;
   m->q = b.q;
@@ -1066,6 +1068,15 @@ morse_status sweep_impl(morse_ctx *ctx, const morse_event *ev,
       MORSE_CUDA(ctx, cudaEventCreateWithFlags(&ctx->sweep_ev[k],
                                                cudaEventDisableTiming));
   }
+  // The builds end before the call does, also where it fails half way: the
+  // buffers go back to the pool, and from it to the next map, in the order of
+  // the context's own stream alone.
+  struct BuildsEnd {
+    cudaStream_t st;
+    ~BuildsEnd() {
+      if (st) cudaStreamSynchronize(st);
+    }
+  } builds_end = {two ? ctx->build_stream : nullptr};
   morse_map *m = ctx->sweep_map;
   Plan pl;
   MORSE_TRY(plan_search(ctx, ev, grid, 0, grid_size(grid), false, h16, n_maps,
@@ -1869,6 +1880,7 @@ morse_status morse_create(morse_ctx **out, int device, void *cuda_stream) {
   c->spin_limit = kDefaultSpinLimit;
   c->fault_lock_held = 0;
   c->fault_alloc = 0;
+  c->fault_build = 0;
   c->batch_exec = nullptr;
   c->smem_optin = prop.sharedMemPerBlockOptin;
   if (cuda_stream) {
@@ -1962,6 +1974,7 @@ morse_status morse_inject_fault(morse_ctx *ctx, int fault, int64_t arg) {
       ctx->spin_limit = kDefaultSpinLimit;
       ctx->fault_lock_held = 0;
       ctx->fault_alloc = 0;
+      ctx->fault_build = 0;
       return MORSE_OK;
     case MORSE_FAULT_LOCK_HELD:
       if (arg < 1 || arg > (int64_t)kDefaultSpinLimit)
@@ -1975,6 +1988,12 @@ morse_status morse_inject_fault(morse_ctx *ctx, int fault, int64_t arg) {
         return fail(ctx, MORSE_EINVAL, "allocation index %lld < 1",
                     (long long)arg);
       ctx->fault_alloc = arg;
+      return MORSE_OK;
+    case MORSE_FAULT_BUILD:
+      if (arg < 1)
+        return fail(ctx, MORSE_EINVAL, "build index %lld < 1",
+                    (long long)arg);
+      ctx->fault_build = arg;
       return MORSE_OK;
     default:
       return fail(ctx, MORSE_EINVAL, "unknown fault %d", fault);

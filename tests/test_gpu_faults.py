@@ -119,3 +119,33 @@ def test_inject_fault_rejects_bad_arguments(m, setup):
             ctx.inject_fault(kind, arg)
         assert e.value.status == m.EINVAL
     ctx.inject_fault(m.FAULT_NONE, 0)
+
+
+def test_failed_build_of_a_sweep_leaves_no_build_running(m, setup):
+    """A sweep that fails at its third map, with the second one's build on
+    its own stream behind it: the next sweeps, of other sizes (the buffers are
+    given back and made anew) and of the same, give their own results."""
+    ctx, ev, mp, grid = setup
+    S, Q = np.array([0.9, 1.0, 1.1, 1.2]), np.array([1e-3, 3e-3, 1e-2, 0.1])
+
+    def sweep(npix, rays):
+        return ctx.sweep(ev, S, Q, 2.0, npix, rays, grid,
+                         image_halfwidth=3.0)
+
+    ref = {n: sweep(n, 8 * n) for n in (1024, 128, 256)}
+    for again in (128, 1024, 256):
+        sweep(1024, 8192)
+        ctx.inject_fault(m.FAULT_BUILD, 3)
+        with pytest.raises(m.MorseError) as e:
+            sweep(1024, 8192)
+        assert e.value.status == m.ECUDA
+        got = sweep(again, 8 * again)
+        for f in ("idx", "chi2", "Fs", "Fb"):
+            assert np.array_equal(got[f], ref[again][f]), f
+    ctx.inject_fault(m.FAULT_BUILD, 1)
+    with pytest.raises(m.MorseError):
+        ctx.build_map(1.0, 1e-2, 2.0, 64, 200)
+    ctx.build_map(1.0, 1e-2, 2.0, 64, 200).free()
+    with pytest.raises(m.MorseError) as e:
+        ctx.inject_fault(m.FAULT_BUILD, 0)
+    assert e.value.status == m.EINVAL
