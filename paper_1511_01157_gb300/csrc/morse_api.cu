@@ -210,7 +210,20 @@ morse_status check_build(morse_ctx *ctx, double s, double q, double extent,
 }
 
 // ---------------------------------------------------------------- maps
-// to the context's pool, after the stream's work so far
+// Waits for the whole device, as cudaFree does.  A user's handle may have
+// been read elsewhere than on the context's stream (morse_chi2_grad_dev
+// captured in a graph that is replayed on another one), and its memory goes to
+// the next handle in the order of that stream alone.
+void device_done(const morse_ctx *ctx) {
+  int dev = -1;
+  cudaGetDevice(&dev);
+  if (dev != ctx->device) cudaSetDevice(ctx->device);
+  cudaDeviceSynchronize();
+  if (dev >= 0 && dev != ctx->device) cudaSetDevice(dev);
+}
+
+// to the context's pool, after the stream's work so far (memory that nothing
+// else has read)
 void pool_free(morse_ctx *ctx, void *p) { cudaFreeAsync(p, ctx->stream); }
 
 morse_map *map_alloc(morse_ctx *ctx, int npix, bool counts) {
@@ -2231,7 +2244,10 @@ morse_status morse_map_half(const morse_map *map, uint16_t *host_codes,
 
 void morse_map_free(morse_map *map) {
   if (!map) return;
+  morse_ctx *ctx = map->ctx;
+  device_done(ctx);
   map_release(map);
+  cudaStreamSynchronize(ctx->stream);  // the pool gives back what is too much
 }
 
 // ------------------------------------------------------------------ events
@@ -2505,8 +2521,11 @@ morse_status morse_event_create(morse_ctx *ctx, const double *t,
 
 void morse_event_free(morse_event *ev) {
   if (!ev) return;
-  if (ev->ep) pool_free(ev->ctx, ev->ep);
+  morse_ctx *ctx = ev->ctx;
+  device_done(ctx);
+  if (ev->ep) pool_free(ctx, ev->ep);
   free(ev);
+  cudaStreamSynchronize(ctx->stream);
 }
 
 morse_status morse_event_info(const morse_event *ev, int64_t *n,

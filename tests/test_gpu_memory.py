@@ -1,0 +1,87 @@
+"""Device memory of the handles and the workspace.
+
+* Freed maps and events: the memory is the next handle's only when the whole
+  device has finished with it, and what the context keeps of it is bounded at
+  once, not at some later call.
+"""
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+MB = 1 << 20
+
+
+@pytest.fixture(scope="module")
+def m():
+    import paper_1511_01157_gb300 as lib
+    return lib
+
+
+def _event(ctx, n, seed=3):
+    t = synth.epoch_times(n, seed)
+    F, sig = synth.photometry(0.3 + 1.0 / np.sqrt(0.03 + (t / 18.0) ** 2),
+                              seed)
+    return ctx.event(t, F, sig)
+
+
+def test_freed_memory_is_given_back(m):
+    import torch
+    ctx = m.Context(0)
+
+    def maps():
+        return [ctx.build_map(s, 1e-3, 2.0, 4096, 4096, deflect="fp32")
+                for s in (0.9, 1.0, 1.1)]
+
+    for x in maps():
+        x.free()
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info(0)[0]
+    held = maps()
+    assert before - torch.cuda.mem_get_info(0)[0] > 900 * MB
+    for x in held:
+        x.free()
+    # (256 MB may stay with the context, some of it from the first maps)
+    assert before - torch.cuda.mem_get_info(0)[0] <= 288 * MB
+    ctx.close()
+
+
+def test_a_map_is_freed_after_every_streams_work(m):
+    """A captured gradient replayed on a stream of its own: freeing the map
+    and the event waits for the replays, and the next maps do not get their
+    memory before."""
+    import torch
+    lib_stream, other = torch.cuda.Stream(), torch.cuda.Stream()
+    ctx = m.Context(0, stream=lib_stream)
+    rng = np.random.default_rng(5)
+    n = 20000
+    th = np.stack([rng.uniform(-1, 1, n), 20 * np.exp(rng.uniform(-.3, .3, n)),
+                   .3 * np.exp(rng.uniform(-.5, .5, n)),
+                   rng.uniform(-.2, .2, n)], axis=1)
+    ev = _event(ctx, 3000)
+    mp = ctx.build_map(1.0, 1e-3, 2.0, 512, 4000, image_halfwidth=3.0,
+                       deflect="fp32")
+    ref, gref, *_ = ctx.chi2_grad(ev, mp, th)
+    theta = torch.tensor(th, device="cuda")
+    chi2 = torch.zeros(n, dtype=torch.float64, device="cuda")
+    grad = torch.zeros((n, 4), dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=lib_stream):
+        ctx.chi2_grad_dev(ev, mp, theta, chi2, grad)
+    with torch.cuda.stream(other):
+        for _ in range(100):
+            graph.replay()
+    mp.free()
+    ev.free()
+    more = [ctx.build_map(0.3, 0.5, 2.0, 512, 4000, image_halfwidth=3.0,
+                          deflect="fp32") for _ in range(3)]
+    evs = [_event(ctx, 3000, 8 + k) for k in range(3)]
+    torch.cuda.synchronize()
+    assert np.array_equal(chi2.cpu().numpy(), ref)
+    assert np.array_equal(grad.cpu().numpy(), gref)
+    for x in more + evs:
+        x.free()
+    ctx.close()
