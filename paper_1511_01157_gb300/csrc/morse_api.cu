@@ -512,7 +512,8 @@ cudaError_t pool_alloc(morse_ctx *ctx, void **p, size_t bytes) {
 
 cudaError_t dev_alloc(morse_ctx *ctx, void **p, size_t bytes) {
   *p = nullptr;
-  if (ctx && ctx->fault_alloc > 0 && --ctx->fault_alloc == 0)
+  ctx->alloc_injected = ctx->fault_alloc > 0 && --ctx->fault_alloc == 0;
+  if (ctx->alloc_injected)
     return cudaErrorMemoryAllocation;  // injected: nothing allocated
   return cudaMalloc(p, bytes);
 }
@@ -850,7 +851,20 @@ morse_status plan_search(morse_ctx *ctx, const morse_event *ev,
   pl->bytes = pl->off_out + out_bytes;
   pl->want = 0;
   pl->small = false;
-  if (!dense) pl->bytes = plan_screen(ev, g, count, true, pl->bytes, pl);
+  if (dense) return MORSE_OK;
+  const size_t plain = pl->bytes;
+  pl->bytes = plan_screen(ev, g, count, true, plain, pl);
+  if (pl->want > 0) {
+    // the screen's codes and lists (some ten bytes per trajectory) may be
+    // more than the device has left: then the unscreened search, whose
+    // workspace they came on top of
+    void *ws = nullptr;
+    const morse_status st = ws_reserve(ctx, pl->bytes, &ws);
+    if (st != MORSE_ENOMEM || ctx->alloc_injected) return st;
+    pl->want = 0;
+    pl->small = false;
+    pl->bytes = plain;
+  }
   return MORSE_OK;
 }
 
@@ -3016,9 +3030,17 @@ morse_status morse_grid_chi2_batch(morse_ctx *ctx,
   BatchHost H;
   MORSE_TRY(batch_prepare(ctx, evs, n_ev, maps, n_maps, grid, shape_ev, true,
                           H));
-  const BatchLayout L = batch_layout(H, pairs, K);
+  BatchLayout L = batch_layout(H, pairs, K);
   void *ws = nullptr;
-  MORSE_TRY(ws_reserve(ctx, L.bytes, &ws));
+  morse_status ws_st = ws_reserve(ctx, L.bytes, &ws);
+  if (ws_st == MORSE_ENOMEM && !ctx->alloc_injected && !H.tasks.empty()) {
+    // without the screen's scratch (as plan_search)
+    MORSE_TRY(batch_prepare(ctx, evs, n_ev, maps, n_maps, grid, shape_ev,
+                            false, H));
+    L = batch_layout(H, pairs, K);
+    ws_st = ws_reserve(ctx, L.bytes, &ws);
+  }
+  MORSE_TRY(ws_st);
   char *base = (char *)ws;
   morse::BatchParams Bp, Bm;
   double *t0abs, *tEv;

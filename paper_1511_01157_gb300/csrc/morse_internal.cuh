@@ -48,6 +48,7 @@ struct morse_ctx {
   int fault_lock_held;      // searches start with every block lock taken
   long long fault_alloc;    // > 0: the fault_alloc-th device allocation
                             // from now fails (then the count is spent)
+  bool alloc_injected;      // the last failed allocation was one of these
   long long fault_build;    // the same of the fault_build-th map build
   unsigned pub_tag;         // tag of the last top-K search launch
 };

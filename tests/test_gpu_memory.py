@@ -3,6 +3,8 @@
 * Freed maps and events: the memory is the next handle's only when the whole
   device has finished with it, and what the context keeps of it is bounded at
   once, not at some later call.
+* On a GPU that others have filled a search whose screen does not fit is the
+  unscreened one.
 """
 import numpy as np
 import pytest
@@ -84,4 +86,54 @@ def test_a_map_is_freed_after_every_streams_work(m):
     assert np.array_equal(grad.cpu().numpy(), gref)
     for x in more + evs:
         x.free()
+    ctx.close()
+
+
+def _fill(left):
+    """Takes the GPU's free memory but for `left` bytes."""
+    import torch
+    torch.cuda.empty_cache()
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info(0)[0]
+    x = torch.empty(free - left, dtype=torch.uint8, device="cuda")
+    assert torch.cuda.mem_get_info(0)[0] <= left + 8 * MB
+    return x
+
+
+@pytest.fixture
+def empty_torch():
+    import torch
+    yield
+    torch.cuda.empty_cache()
+
+
+def test_searches_whose_screen_does_not_fit(m, empty_torch):
+    kw = dict(image_halfwidth=3.0, deflect="fp32")
+    g = m.Grid.make(64, 128, 64, 32, 1e-3, 0.5, -2.0, 2.0, 5.0, 80.0, True,
+                    True, 16)                       # 116 MB with the screen
+    gb = m.Grid.make(40, 72, 25, 40, 1e-3, 0.5, -2.0, 2.0, 5.0, 80.0, True,
+                     True, 16)                      # 8 pairs, 20 MB of scratch each
+    small = m.Grid.make(10, 20, 10, 10, 1e-3, 0.5, -2.0, 2.0, 5.0, 80.0, True,
+                        True, 16)
+
+    def calls(ctx, grids):
+        ev = [_event(ctx, 200, s) for s in range(4)]
+        mp = [ctx.build_map(s, 1e-3, 2.0, 256, 1500, **kw) for s in (1., 1.2)]
+        return lambda: (ctx.grid_chi2(ev[0], mp[0], grids[0]),
+                        ctx.grid_chi2_batch(ev, mp, grids[1]))
+
+    with m.Context(0) as other:
+        f = calls(other, (g, gb))
+        ref = f()
+        del f
+    ctx = m.Context(0)
+    ctx.batch_tuning(False)
+    calls(ctx, (small, small))()  # (the kernels are loaded)
+    f = calls(ctx, (g, gb))
+    held = _fill(100 * MB)
+    got = f()
+    del held
+    for a, b in zip(got, ref):
+        for k in ("idx", "chi2", "Fs", "Fb"):
+            assert np.array_equal(a[k], b[k]), k
     ctx.close()
