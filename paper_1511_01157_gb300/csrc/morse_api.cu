@@ -210,15 +210,24 @@ morse_status check_build(morse_ctx *ctx, double s, double q, double extent,
 }
 
 // ---------------------------------------------------------------- maps
-// Waits for the whole device, as cudaFree does.  A user's handle may have
-// been read elsewhere than on the context's stream (morse_chi2_grad_dev
-// captured in a graph that is replayed on another one), and its memory goes to
-// the next handle in the order of that stream alone.
+// Waits for the whole device.  A user's handle may have been read elsewhere
+// than on the context's stream (morse_chi2_grad_dev captured in a graph that
+// is replayed on another one), and its memory goes to the next handle in the
+// order of that stream alone.  By cudaFree, which does it beside captures of
+// other threads too (cudaDeviceSynchronize breaks those), of a few bytes
+// beside the context's token (alone they would be a mapping of their own, 150
+// us to make and undo instead of 8).
 void device_done(const morse_ctx *ctx) {
   int dev = -1;
   cudaGetDevice(&dev);
   if (dev != ctx->device) cudaSetDevice(ctx->device);
-  cudaDeviceSynchronize();
+  void *p = nullptr;
+  if (cudaMalloc(&p, 256) == cudaSuccess) {
+    cudaFree(p);
+  } else {
+    cudaGetLastError();
+    cudaDeviceSynchronize();
+  }
   if (dev >= 0 && dev != ctx->device) cudaSetDevice(dev);
 }
 
@@ -1939,11 +1948,15 @@ morse_status morse_create(morse_ctx **out, int device, void *cuda_stream) {
                                   &keep);
       if (e != cudaSuccess) cudaMemPoolDestroy(c->pool);
     }
+    if (e == cudaSuccess) {
+      e = cudaMalloc(&c->token, 256);
+      if (e != cudaSuccess) cudaMemPoolDestroy(c->pool);
+    }
     if (e != cudaSuccess) {
       cudaGetLastError();
       if (c->own_stream) cudaStreamDestroy(c->stream);
       delete c;
-      return MORSE_ECUDA;
+      return e == cudaErrorMemoryAllocation ? MORSE_ENOMEM : MORSE_ECUDA;
     }
   }
   *out = c;
@@ -1963,6 +1976,7 @@ void morse_destroy(morse_ctx *ctx) {
   if (ctx->sweep_map2) map_release(ctx->sweep_map2);
   if (ctx->batch_exec) cudaGraphExecDestroy(ctx->batch_exec);
   if (ctx->ws) cudaFree(ctx->ws);
+  cudaFree(ctx->token);
   for (cudaEvent_t e : ctx->evpool) cudaEventDestroy(e);
   cudaStreamSynchronize(ctx->stream);
   cudaMemPoolDestroy(ctx->pool);  // (its memory once every handle is freed)

@@ -24,6 +24,7 @@ struct morse_ctx {
   char err[512];
   cudaMemPool_t pool;       // memory of maps and events, in the stream's
                             // order
+  void *token;              // 256 bytes (device_done)
   void *ws;                 // device workspace (grow-only)
   size_t ws_bytes;
   // per-call kernel timing: event pairs recorded around each launch, summed

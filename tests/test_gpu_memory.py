@@ -76,7 +76,11 @@ def test_a_map_is_freed_after_every_streams_work(m):
     with torch.cuda.stream(other):
         for _ in range(100):
             graph.replay()
+        done = torch.cuda.Event()
+        done.record()
+    assert not done.query()
     mp.free()
+    assert done.query()
     ev.free()
     more = [ctx.build_map(0.3, 0.5, 2.0, 512, 4000, image_halfwidth=3.0,
                           deflect="fp32") for _ in range(3)]
