@@ -273,8 +273,10 @@ size_t batch_smem_bytes(int ep_cap, int top_k) {
 
 template <bool H, int V>
 static int batch_occupancy(size_t smem) {
-  cudaFuncSetAttribute(k_batch<H, V>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (raise_smem(k_batch<H, V>) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
   // smallest shared-memory carveout that holds the block: the rest of the
   // SM's 256 KB serves as L1 for the map gathers
   int dev = 0, per_sm = 0;

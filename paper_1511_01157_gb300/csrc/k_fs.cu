@@ -421,9 +421,7 @@ static cudaError_t launch_fold(const float *A, int npix, double L, int R,
                                const float *W, const int *rowhw, float *out,
                                cudaStream_t st) {
   const size_t smem = fold_smem_bytes(R);
-  cudaError_t e = cudaFuncSetAttribute(
-      k_fs_fold<G, NL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-      (int)smem);
+  const cudaError_t e = raise_smem(k_fs_fold<G, NL>);
   if (e != cudaSuccess) return e;
   const dim3 grid((npix + kFoldTX - 1) / kFoldTX,
                   (npix + kFoldTY - 1) / kFoldTY);
@@ -451,8 +449,7 @@ cudaError_t launch_fs_conv(const float *A, int npix, double L, int R,
       return launch_fold<4, 8>(A, npix, L, R, W, rowhw, out, st);
   }
   const size_t smem = fs_smem_bytes(R);
-  cudaError_t e = cudaFuncSetAttribute(
-      k_fs_conv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = raise_smem(k_fs_conv);
   if (e != cudaSuccess) return e;
   dim3 grid((npix + kFsTX - 1) / kFsTX, (npix + kFsTY - 1) / kFsTY);
   k_fs_conv<<<grid, kFsThreads, smem, st>>>(A, npix, L, R, W, rowhw, out);

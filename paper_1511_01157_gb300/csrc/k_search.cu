@@ -712,8 +712,10 @@ size_t search_smem_bytes(int n_ep_smem, int top_k) {
 
 template <bool D, bool E, bool H>
 static int occupancy(size_t smem) {
-  cudaFuncSetAttribute(k_search<D, E, H>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (raise_smem(k_search<D, E, H>) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
 #if MORSE_SMEM_CARVEOUT
   // ask for the smallest shared-memory carveout that holds the block, so
   // the rest of the SM's 256 KB serves as L1 for the map gathers
@@ -784,9 +786,7 @@ size_t list_smem_bytes(const SearchParams &P, bool staged) {
 
 template <bool E, bool H>
 static int list_occupancy(size_t smem) {
-  if (cudaFuncSetAttribute(k_search_list<E, H>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem) != cudaSuccess) {
+  if (raise_smem(k_search_list<E, H>) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -880,41 +880,29 @@ cudaError_t launch_topk_merge(Entry *a, Entry *b, int lists, int k,
   return cudaSuccess;
 }
 
-static size_t finish_smem() {
-  const size_t sm = (size_t)kCandMax * 12;
-  static int set_of[64];
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev >= 64 || !set_of[dev]) {
-    cudaFuncSetAttribute(k_finish, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)sm);
-    cudaFuncSetAttribute(k_finish_batch,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (dev < 64) set_of[dev] = 1;
-  }
-  return sm;
-}
+constexpr size_t kFinishSmem = (size_t)kCandMax * 12;
 
 cudaError_t launch_finish(const FillParams &F, cudaStream_t st) {
-  k_finish<<<kCandMax / kFinishPer, kFinishThreads, finish_smem(), st>>>(F);
+  const cudaError_t e = raise_smem(k_finish);
+  if (e != cudaSuccess) return e;
+  k_finish<<<kCandMax / kFinishPer, kFinishThreads, kFinishSmem, st>>>(F);
   return cudaGetLastError();
 }
 
 cudaError_t launch_list_batch(const ScreenTask *t, int n,
                               const SearchParams &P0, cudaStream_t st) {
   const size_t sm = search_smem_bytes(0, P0.top_k);
-  cudaError_t e = cudaFuncSetAttribute(
-      P0.quadh ? (const void *)k_search_list_batch<true>
-               : (const void *)k_search_list_batch<false>,
-      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  cudaError_t e = raise_smem(P0.quadh ? k_search_list_batch<true>
+                                      : k_search_list_batch<false>);
+  if (e == cudaSuccess) e = raise_smem(k_finish_batch);
   if (e != cudaSuccess) return e;
   const dim3 grid(kListBatchBlocks, (unsigned)n);
   if (P0.quadh)
     k_search_list_batch<true><<<grid, kSearchWarps * 32, sm, st>>>(t);
   else
     k_search_list_batch<false><<<grid, kSearchWarps * 32, sm, st>>>(t);
-  const size_t fs = finish_smem();
-  k_finish_batch<<<dim3(2, (unsigned)n), kFinishThreads, fs, st>>>(t);
+  k_finish_batch<<<dim3(2, (unsigned)n), kFinishThreads, kFinishSmem, st>>>(
+      t);
   return cudaGetLastError();
 }
 

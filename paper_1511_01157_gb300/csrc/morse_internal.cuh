@@ -458,6 +458,27 @@ struct FillParams {
                             // (nullptr: none were)
 };
 
+// Lets a kernel have all the dynamic shared memory that the device allows it
+// (its static part taken off), whatever a launch then asks for: the limit
+// belongs to the process, and one set to a launch's own size is too small for
+// that launch when another thread's context sets it in between.
+template <typename K>
+inline cudaError_t raise_smem(K kernel) {
+  cudaFuncAttributes a;
+  cudaError_t e = cudaFuncGetAttributes(&a, (const void *)kernel);
+  if (e != cudaSuccess) return e;
+  int dev = 0, optin = 0;
+  cudaGetDevice(&dev);
+  e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin,
+                             dev);
+  if (e != cudaSuccess) return e;
+  const int most = optin - (int)a.sharedSizeBytes;
+  if (a.maxDynamicSharedSizeBytes >= most) return cudaSuccess;
+  return cudaFuncSetAttribute((const void *)kernel,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              most);
+}
+
 // ---------------------------------------------------------------- screen
 // One screened search of a batch: the kernels of a batch take an array of
 // them in device memory, one per blockIdx.y.
