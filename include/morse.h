@@ -29,10 +29,12 @@
  *  - Errors: every call returns a morse_status; morse_last_error() gives a
  *    message for the context's most recent failure.  No call aborts, traps
  *    or throws.  Invalid arguments return MORSE_EINVAL before any GPU work.
- *  - Memory: handles own their device memory (freed map and event memory
- *    stays with the context, at most 256 MB of it, for its next handles,
- *    until morse_destroy); input arrays are copied and
- *    stay owned by the caller; output arrays are caller-allocated HOST
+ *  - Memory: handles own their device memory.  Freed map and event memory
+ *    stays with the context for its next handles: at most 2 GB of it until
+ *    the context's next synchronous call, 256 MB until morse_destroy.  The
+ *    context's workspace grows with its calls: up to some 10 bytes per
+ *    trajectory of a search, 512 MB for a batch's, less where the device has
+ *    not as much.  Input arrays are copied and stay owned by the caller; output arrays are caller-allocated HOST
  *    memory unless the name ends in _dev.  Calls are synchronous on the
  *    context's stream unless noted.
  *  - Threads: a context may be used by one host thread at a time.

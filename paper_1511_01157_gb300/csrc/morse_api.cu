@@ -210,14 +210,13 @@ morse_status check_build(morse_ctx *ctx, double s, double q, double extent,
 }
 
 // ---------------------------------------------------------------- maps
-// Waits for the whole device.  A user's handle may have been read elsewhere
-// than on the context's stream (morse_chi2_grad_dev captured in a graph that
-// is replayed on another one), and its memory goes to the next handle in the
-// order of that stream alone.  By cudaFree, which does it beside captures of
-// other threads too (cudaDeviceSynchronize breaks those), of a few bytes
-// beside the context's token (alone they would be a mapping of their own, 150
-// us to make and undo instead of 8).
-void device_done(const morse_ctx *ctx) {
+// Before the memory of a user's handle goes back to the pool, and from it to
+// the next handle in the order of the context's stream.  All work on handles
+// is on that stream, but for morse_chi2_grad_dev captured in a graph, which may
+// run on any: then the whole device is waited for, by cudaFree, which does it
+// beside captures of other threads too (cudaDeviceSynchronize breaks those).
+void handle_done(const morse_ctx *ctx, bool captured) {
+  if (!captured) return;
   int dev = -1;
   cudaGetDevice(&dev);
   if (dev != ctx->device) cudaSetDevice(ctx->device);
@@ -229,6 +228,18 @@ void device_done(const morse_ctx *ctx) {
     cudaDeviceSynchronize();
   }
   if (dev >= 0 && dev != ctx->device) cudaSetDevice(dev);
+}
+
+// After it: the pool gives back what is above its threshold when the stream
+// synchronises, so that happens at least once per kPoolLoose bytes freed.
+// (At every free it would have the next large map mapped anew: 8192^2 texels
+// 4.2 ms against 1.0 to build.)
+const size_t kPoolLoose = (size_t)2 << 30;
+void handle_freed(morse_ctx *ctx, size_t bytes) {
+  ctx->pool_loose += bytes;
+  if (ctx->pool_loose <= kPoolLoose) return;
+  cudaStreamSynchronize(ctx->stream);
+  ctx->pool_loose = 0;
 }
 
 // to the context's pool, after the stream's work so far (memory that nothing
@@ -1948,15 +1959,11 @@ morse_status morse_create(morse_ctx **out, int device, void *cuda_stream) {
                                   &keep);
       if (e != cudaSuccess) cudaMemPoolDestroy(c->pool);
     }
-    if (e == cudaSuccess) {
-      e = cudaMalloc(&c->token, 256);
-      if (e != cudaSuccess) cudaMemPoolDestroy(c->pool);
-    }
     if (e != cudaSuccess) {
       cudaGetLastError();
       if (c->own_stream) cudaStreamDestroy(c->stream);
       delete c;
-      return e == cudaErrorMemoryAllocation ? MORSE_ENOMEM : MORSE_ECUDA;
+      return MORSE_ECUDA;
     }
   }
   *out = c;
@@ -1976,7 +1983,6 @@ void morse_destroy(morse_ctx *ctx) {
   if (ctx->sweep_map2) map_release(ctx->sweep_map2);
   if (ctx->batch_exec) cudaGraphExecDestroy(ctx->batch_exec);
   if (ctx->ws) cudaFree(ctx->ws);
-  cudaFree(ctx->token);
   for (cudaEvent_t e : ctx->evpool) cudaEventDestroy(e);
   cudaStreamSynchronize(ctx->stream);
   cudaMemPoolDestroy(ctx->pool);  // (its memory once every handle is freed)
@@ -2273,9 +2279,13 @@ morse_status morse_map_half(const morse_map *map, uint16_t *host_codes,
 void morse_map_free(morse_map *map) {
   if (!map) return;
   morse_ctx *ctx = map->ctx;
-  device_done(ctx);
+  handle_done(ctx, map->captured);
+  const size_t n = (size_t)map->npix * map->npix;
+  const size_t cell = sizeof(float4) + (map->quadh ? sizeof(uint2) : 0);
+  const size_t bytes = n * (sizeof(float) + sizeof(uint32_t)) +
+                       morse::quad_count(map->npix) * cell;
   map_release(map);
-  cudaStreamSynchronize(ctx->stream);  // the pool gives back what is too much
+  handle_freed(ctx, bytes);
 }
 
 // ------------------------------------------------------------------ events
@@ -2550,10 +2560,11 @@ morse_status morse_event_create(morse_ctx *ctx, const double *t,
 void morse_event_free(morse_event *ev) {
   if (!ev) return;
   morse_ctx *ctx = ev->ctx;
-  device_done(ctx);
+  handle_done(ctx, ev->captured);
+  const size_t bytes = sizeof(float4) * (size_t)ev->n;
   if (ev->ep) pool_free(ctx, ev->ep);
   free(ev);
-  cudaStreamSynchronize(ctx->stream);
+  handle_freed(ctx, bytes);
 }
 
 morse_status morse_event_info(const morse_event *ev, int64_t *n,
@@ -2805,6 +2816,10 @@ morse_status morse_chi2_grad_dev(morse_ctx *ctx, const morse_event *ev,
   memset(&P, 0, sizeof(P));
   map_params(map, &P);
   event_params(ev, &P);
+  // (a graph of the launch may run on any stream: handle_done)
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  MORSE_CUDA(ctx, cudaStreamIsCapturing(ctx->stream, &cap));
+  if (cap != cudaStreamCaptureStatusNone) map->captured = ev->captured = true;
   MORSE_CUDA(ctx, morse::launch_theta(P, theta, (int)n, ev->t_ref, chi2,
                                       grad, nullptr, nullptr, nullptr,
                                       ctx->sm_count, ctx->stream));

@@ -24,7 +24,7 @@ struct morse_ctx {
   char err[512];
   cudaMemPool_t pool;       // memory of maps and events, in the stream's
                             // order
-  void *token;              // 256 bytes (device_done)
+  size_t pool_loose;        // bytes freed to it since handle_freed waited
   void *ws;                 // device workspace (grow-only)
   size_t ws_bytes;
   // per-call kernel timing: event pairs recorded around each launch, summed
@@ -77,6 +77,7 @@ struct morse_map {
   double a_floor;           // half a ray (ray-shot maps), else 1e-6
   bool half_valid;          // the FP16 table holds the current values
   int lookup;               // MORSE_STORE_FP32 or MORSE_STORE_FP16LOG
+  mutable bool captured;    // a graph reads it (handle_done)
 };
 
 // Screening subsets of a light curve: at most this many, smallest first.
@@ -102,6 +103,7 @@ struct morse_event {
   double S1, SF, SFF, Fref; // FP64 sums of the stored FP32 values
   double invS1, CFF;        // 1/S_1, S_FF - S_F^2/S_1
   double t_span;            // max |t - t_ref| over the epochs
+  mutable bool captured;    // a graph reads it (handle_done)
 };
 
 namespace morse {
