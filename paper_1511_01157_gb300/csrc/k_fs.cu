@@ -126,7 +126,8 @@ __global__ void __launch_bounds__(kFsThreads)
 
 // The same convolution folded about the source's axis: W(dx, -dy) = W(dx,
 // dy), so the input rows y + dy and y - dy are added first, once for all dx,
-// and every weight is applied to the sum: half the multiply-adds, which
+// and every weight is applied to the sum (of halves, by twice the weight: the
+// sum stays in FP32's range with its texels): half the multiply-adds, which
 // bound k_fs_conv (with the FP64 additions of its row sums: two FP64-pipe
 // instructions per output and row, some 16 cycles each per warp).
 //
@@ -201,11 +202,11 @@ __global__ void __launch_bounds__(kFoldGroup *G, G == 2 ? 3 : 1)
   };
   for (int r = 0; r < kFoldTY; ++r)
     for (int c = threadIdx.x; c < width; c += (kFoldGroup * G)) {
-      const float v = texel(c, y0 + r);
+      const float v = 0.5f * texel(c, y0 + r);
       s_up[r * pitch + place(c)] = v;
       s_dn[r * pitch + place(c)] = v;
     }
-  for (int t = threadIdx.x; t < wn; t += (kFoldGroup * G)) s_w[t] = weight(t, 0);
+  for (int t = threadIdx.x; t < wn; t += (kFoldGroup * G)) s_w[t] = 2.f * weight(t, 0);
   float hi[kFoldOut], lo[kFoldOut];
 #pragma unroll
   for (int k = 0; k < kFoldOut; ++k) hi[k] = lo[k] = 0.f;
@@ -275,11 +276,11 @@ __global__ void __launch_bounds__(kFoldGroup *G, G == 2 ? 3 : 1)
     for (int i = 0; i < NL; ++i) {
       const int e = threadIdx.x + i * (kFoldGroup * G);
       if (e < width)
-        s_up[new_up * pitch + place(e)] = next[i];
+        s_up[new_up * pitch + place(e)] = 0.5f * next[i];
       else if (e < 2 * width)
-        s_dn[new_dn * pitch + place(e - width)] = next[i];
+        s_dn[new_dn * pitch + place(e - width)] = 0.5f * next[i];
       else if (e < 2 * width + wn)
-        s_w[((dy + 1) & 1) * wn + e - 2 * width] = next[i];
+        s_w[((dy + 1) & 1) * wn + e - 2 * width] = 2.f * next[i];
     }
     hw = hw_next;
     up = up + 1 == kFoldSlots ? 0 : up + 1;
@@ -310,8 +311,9 @@ __global__ void __launch_bounds__(kFoldGroup *G, G == 2 ? 3 : 1)
       lo[k] = __fadd_rn(lo[k], q[kFoldGroup]);
     }
     const int x = x0 + kFoldOut * tx + k;
-    if (x < npix && y < npix)
-      out[(size_t)y * npix + x] = __fadd_rn(hi[k], lo[k]);
+    if (x < npix && y < npix)  // (lo of an infinite sum: NaN)
+      out[(size_t)y * npix + x] =
+          isfinite(hi[k]) ? __fadd_rn(hi[k], lo[k]) : hi[k];
   }
 }
 

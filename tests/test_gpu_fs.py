@@ -100,3 +100,19 @@ def test_folded_convolution_matches_oracle(ctx, rho_px, npix):
     assert np.max(np.abs(got - ref) / ref) <= 2e-6
     fs.free()
     mp.free()
+
+
+@pytest.mark.parametrize("rho_px", [20.0, 62.4, 62.6, 90.0])
+def test_finite_source_of_values_near_the_largest_fp32(ctx, rho_px):
+    """Texels whose pairwise sums are beyond FP32, on both sides of R = 64,
+    and a map 2^40 times smaller: scaled, to the last bit."""
+    npix = 256
+    rng = np.random.default_rng(6)
+    A = rng.uniform(1.7e38, 3.2e38, (npix, npix)).astype(np.float32)
+    R = int(np.ceil(rho_px + 0.5))
+    got = [ctx.map_from_host(a, 2.0).finite_source(
+        rho_px * 4.0 / npix).values()[R:-R, R:-R]
+        for a in (A, A * np.float32(2.0 ** -40))]
+    assert np.isfinite(got[0]).all()
+    assert got[0].min() > 1.7e38
+    assert np.array_equal(got[0] * np.float32(2.0 ** -40), got[1])
