@@ -507,13 +507,15 @@ __global__ void __launch_bounds__(kAdjWarps * 32, MINB)
     SearchParams Q = P;  // the trajectory's map
     bool eval = false;
 #pragma unroll 1
-    for (int k = warp; k < warps * TPW; k += warps) {
+    for (int r = 0; r < TPW; ++r) {
+      const int k = warp + r * warps;
       eval = i0 + k < n && s_eval[k];
-      if (!eval) continue;
-      T = s_tr[k];
-      Q.quad = T.quad;
-      const Acc a = phase1<false, 0, UN>(Q, ep, T.c, lane);
-      if (lane == 0) s_acc[k] = a;
+      if (eval) {
+        T = s_tr[k];
+        Q.quad = T.quad;
+        const Acc a = phase1<false, 0, UN>(Q, ep, T.c, lane);
+        if (lane == 0) s_acc[k] = a;
+      }
     }
     __syncthreads();
     if (mine && s_eval[lane]) {
@@ -524,20 +526,22 @@ __global__ void __launch_bounds__(kAdjWarps * 32, MINB)
     }
     __syncthreads();
 #pragma unroll 1
-    for (int k = warp; k < warps * TPW; k += warps) {
+    for (int r = 0; r < TPW; ++r) {
+      const int k = warp + r * warps;
       if (TPW > 1) {
         eval = i0 + k < n && s_eval[k];
         if (eval) T = s_tr[k];
         Q.quad = T.quad;
       }
-      if (!eval) continue;
-      AdjSums a;
-      const double x =
-          adj_sweep<true, UN>(Q, ep, T, __double2float_rn(s_Fs[k]),
-                              __double2float_rn(s_Bc[k]), lane, a);
-      if (lane == 0) {
-        s_chi[k] = x;
-        s_sum[k] = a;
+      if (eval) {
+        AdjSums a;
+        const double x =
+            adj_sweep<true, UN>(Q, ep, T, __double2float_rn(s_Fs[k]),
+                                __double2float_rn(s_Bc[k]), lane, a);
+        if (lane == 0) {
+          s_chi[k] = x;
+          s_sum[k] = a;
+        }
       }
     }
     __syncthreads();
