@@ -344,6 +344,11 @@ __device__ __forceinline__ float rcpf(float x) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float r;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
 __device__ __forceinline__ cf divf(cf a, cf b) {
   const float r = rcpf(ab2(b));
   return {(a.re * b.re + a.im * b.im) * r, (a.im * b.re - a.re * b.im) * r};
@@ -425,20 +430,20 @@ __device__ __forceinline__ bool no_image(const cf (&b)[5], cf z, float f,
                                          float ra, float rb, float ma,
                                          float mb) {
   cf p = mk(1.f, 0.f), dp = mk(0.f, 0.f);
-  float s = 1.f, ds = 0.f;  // the same of the absolute values
-  const float az = sqrtf(ab2(z));
+  float s = 1.f, ds = 0.f;  // the same of the absolute values, or above
+  const float az = sqrt_approx(ab2(z));
 #pragma unroll
   for (int u = 4; u >= 0; --u) {
     dp = add(mul(dp, z), p);
     p = add(mul(p, z), b[u]);
     ds = ds * az + s;
-    s = s * az + sqrtf(ab2(b[u]));
+    s = s * az + (fabsf(b[u].re) + fabsf(b[u].im));
   }
   const float e = 40.f / 16777216.f;
-  const float rho = 5.f * (sqrtf(ab2(p)) + e * s) /
-                    (sqrtf(ab2(dp)) - e * ds);
-  return rho > 0.f && 4.f * rho * rho * fmaxf(ra, rb) < 1.f &&
-         2.f * rho * (1.f + 2.f * (ma * ra + mb * rb)) < f;
+  const float num = 5.f * (sqrt_approx(ab2(p)) + e * s);  // rho = num / den
+  const float den = sqrt_approx(ab2(dp)) - e * ds;
+  return den > 0.f && 4.f * num * num * fmaxf(ra, rb) < den * den &&
+         2.f * num * (1.f + 2.f * (ma * ra + mb * rb)) < f * den;
 }
 
 __global__ void __launch_bounds__(kPolyThreads)
@@ -519,7 +524,7 @@ __global__ void __launch_bounds__(kPolyThreads)
   cf w0[5], z0[5];  // their polished and their own places
   int ni = 0;
   cf zn = mk(0.f, 0.f);  // the other root that leaves Eq. 2 the furthest
-  float fn = 0.f, fn_sc = 0.f, ra_n = 0.f, rb_n = 0.f;
+  float fn = 0.f, sc_n = 1.f, ra_n = 0.f, rb_n = 0.f;
 #pragma unroll
   for (int t = 0; t < 5; ++t) w0[t] = z0[t] = mk(0.f, 0.f);
 #pragma unroll
@@ -539,10 +544,10 @@ __global__ void __launch_bounds__(kPolyThreads)
         // (a NaN is a candidate, which will not converge)
         const float af = sqrtf(ab2(f));
         cand = !(af >= 0.002f * sc);
-        if (!cand && af > fn_sc * sc) {
+        if (!cand && af * sc_n > fn * sc) {
           zn = w;
           fn = af;
-          fn_sc = af / sc;
+          sc_n = sc;
           ra_n = ra;
           rb_n = rb;
         }
@@ -562,6 +567,10 @@ __global__ void __launch_bounds__(kPolyThreads)
       ++ni;
     }
   }
+  // three images are all there are when one root is known not to be one: a
+  // candidate shown spurious, or another root (here, before the FP64 steps:
+  // after them the coefficients' registers cost a block per SM)
+  const bool three = ni == 3 && no_image(b, zn, fn, ra_n, rb_n, maf, mbf);
   double A_sum = 0.0;
   int parity = 0, images = 0;
   bool ok = ni >= 3;
@@ -612,11 +621,8 @@ __global__ void __launch_bounds__(kPolyThreads)
       ok = spurious(mb, ma, h, om, z0[t]);
     }
   }
-  // three images are all there are when one root is known not to be one: a
-  // candidate shown spurious, or another root
-  if (images == 3 && ni == 3)
-    ok = ok && (no_image(b, zn, fn, ra_n, rb_n, maf, mbf) ||
-                spurious(mb, ma, h, om, zn));
+  if (images == 3 && ni == 3 && !three)
+    ok = ok && spurious(mb, ma, h, om, zn);
   A[(size_t)j * npix + i] =
       ok && (images == 3 || images == 5) && parity == -1
           ? __double2float_rn(A_sum)
