@@ -595,10 +595,10 @@ __device__ __forceinline__ void pilot_bounds(const SearchParams &P,
 // (ranges of it), whose trajectories all miss the light curve by about as
 // much, and variables that none fits, 60 000 and 300 000 trajectories, 1100
 // to 8000 epochs: 1.10 to 1.55 times the unscreened search without the rule,
-// 0.91 to 1.06 with it (1.17 for the variable of 1100 epochs and 300 000);
-// one in 2 and one in 8 the same within 2 %, and searches that discard enough
-// within the runs' spread of what they were.
-constexpr int kSampleGive = 3;
+// 0.91 to 1.06 with it (1.18 for the variable of 1100 epochs and 300 000).
+// One in 2 and one in 3 did the same there, but a batch whose lists leave out
+// a quarter took up to 15 % more.  256 samples know the share to 2 %.
+constexpr int kSampleGive = 8;
 
 // The threshold: the top_k-th smallest of the pilot's bounds (K distinct
 // trajectories have chi^2 at or below it), by four passes of eight bits

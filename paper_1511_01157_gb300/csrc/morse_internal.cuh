@@ -359,7 +359,7 @@ struct ScreenBufs {
   unsigned pilot_cap, list0_cap, list_cap;
   unsigned want;            // pilot trajectories asked for
 };
-constexpr int kScreenBins = 1024, kScreenWords = 8, kScreenSample = 512;
+constexpr int kScreenBins = 1024, kScreenWords = 8, kScreenSample = 256;
 // bytes of hist, n and smp, which lie one after the other
 constexpr size_t kScreenHeadBytes =
     4 * (size_t)(kScreenBins + kScreenWords + kScreenSample);
