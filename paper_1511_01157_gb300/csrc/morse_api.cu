@@ -694,7 +694,8 @@ double pilot_want(int K, long long count) {
 // Whether a top-K search of `count` trajectories is screened, and the
 // workspace of it from offset `at` on (single: not one of a batch).  With a
 // weak light curve the screen only costs, but for grids of up to kWeakMax
-// trajectories with one subset, whose pilot makes up for it (screen_subsets).
+// trajectories with one subset, whose pilot makes up for it (screen_subsets),
+// and for large K (4096 of 200 000: 0.82 and 0.97 of the unscreened search).
 constexpr long long kWeakMax = 1 << 19;
 size_t plan_screen(const morse_event *ev, const morse_grid *g,
                    long long count, bool single, size_t at, Plan *pl) {
@@ -719,7 +720,9 @@ size_t plan_screen(const morse_event *ev, const morse_grid *g,
   if (ev->n_sub < 1 || count < 16384 || count > (1LL << 25) ||
       total >= 2147483648.0 || want * 4.0 > (double)count)
     return at;
-  if (single && ev->weak && (ev->n_sub > 1 || count > kWeakMax)) return at;
+  if (single && ev->weak && (ev->n_sub > 1 || count > kWeakMax) &&
+      64LL * pl->K < count)
+    return at;
   pl->want = (unsigned)want;
   pl->pilot_cap = 2 * pl->want;
   // (the rescreening's own rule: a list that leaves out less than one in
@@ -2398,7 +2401,7 @@ static void screen_subsets(morse_event *ev, std::vector<float4> &h, int64_t n,
       }
       if (rest <= 0.0 || capped >= m) break;
       const double f = (m - capped) / rest;
-      if (f < 1.0001 && f > 0.9999) break;
+      if (f < 1.001 && f > 0.999) break;
       scale *= f;
     }
     sel.clear();
