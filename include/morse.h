@@ -406,9 +406,10 @@ morse_status morse_peak_search(morse_ctx *ctx, const morse_event *ev,
  * scratch (grid tables, per-block top-K lists, fit records) in one static
  * device array of 4 MiB that every GPU loading the library holds until the
  * process exits, instead of the context's growable workspace.  Inputs,
- * output and results are exactly those of morse_grid_chi2 (same kernels,
- * same arithmetic, same parameter set-up); out is caller-allocated host
- * memory of top_k records.  Like morse_grid_chi2 the call is synchronous:
+ * output and results are exactly those of morse_grid_chi2 (the kernels of its
+ * unscreened search, same arithmetic, same parameter set-up; several times
+ * its time where that one is screened); out is caller-allocated host memory
+ * of top_k records.  Like morse_grid_chi2 the call is synchronous:
  * it returns once the records are on the host.
  *
  * The first call on each device looks up the array's device address

@@ -21,8 +21,8 @@
 //    first (k_screen.cu, all pairs of a chunk in each launch) and its listed
 //    trajectories searched; this kernel then only runs the pairs that ended
 //    without records (weak signal), from the screen's thresholds.  12 light
-//    curves x 4 maps x 200 000 trajectories, five seeds: 48, 69, 55, 48, 69
-//    -> 10, 22, 7.9, 8.0, 19 ms.
+//    curves x 4 maps x 200 000 trajectories, four seeds: 48, 69, 55, 69 ->
+//    9.6, 20.7, 7.2, 17.4 ms; light curves that are all weak are not screened.
 //  * Every trajectory's chi^2 is computed by the same device functions as
 //    the single-pair search (k_search), so the results of a batch are those
 //    of one morse_grid_chi2 call per pair, bit for bit.

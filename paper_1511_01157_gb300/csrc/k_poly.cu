@@ -333,10 +333,11 @@ __global__ void __launch_bounds__(kPolyThreads)
 // polished in FP64 (spurious).  (Without that proof, a root that the sweeps
 // had not brought to its place passed for no image: 51 of 1e8 texels about
 // the caustics of lenses of s = 2.5 to 28 lost a pair of images.)
-// Emulated on the CPU over 23 lenses (s 0.01 to 20, q 1e-8 to 5, maps about
-// the caustics among them): no texel kept differs from the oracle's value,
-// and less than 1 in 1000 is left to the general form (1 to 12 % in maps of a
-// few caustic sizes).  1024^2 map: 23.9 -> 1.09 ms.
+// Emulated on the CPU: of 1e8 texels about the caustics of lenses of s = 2.5 to
+// 28, and 1.8e7 over s 0.01 to 30, q 1e-8 to 10, L 0.02 to 100, none kept
+// differs from the general form's value by 1e-5, and fewer than 1 in 1000 is
+// left to that form where s is 0.3 to 3 (0.5 % of close lenses' maps, 17 %
+// over the whole range).  1024^2 map: 23.9 -> 1.10 ms.
 using cf = cx<float>;
 
 __device__ __forceinline__ float rcpf(float x) {

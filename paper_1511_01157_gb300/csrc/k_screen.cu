@@ -29,9 +29,13 @@
 // them about as well as the best).  The host screens from 16 384
 // trajectories and 128 epochs on; below that a search is bound by its
 // launches and its latency, and there are too few trajectories to rank.
-// Where the subsets discard too little (light curves of weak signal), the
-// whole range is searched as before (k_search), the screening costing a
-// share 64 / n_epochs.
+// Where the subsets discard too little the whole range is searched as before
+// (k_search).  Light curves whose signal is too weak for them are known on the
+// host and not screened (screen_subsets); the others cost the first subset's
+// walk (32 of up to 639 epochs, 64 of more: a share of 25 % at 128 epochs, 16
+// at 200, 2 at 3000, less what the pilot's threshold saves) and five launches
+// before a sample shows it: up to 5 % of a search of 300 000 trajectories,
+// 18 % in the worst case seen (k_list).
 //
 // Grids of up to kSmallGrid trajectories are too few to rank by subsets and
 // bound by latency: k_bounds takes upper and lower bounds of all of them over
@@ -794,26 +798,33 @@ __device__ __forceinline__ void load_task(const ScreenTask *t, ScreenTask &s) {
     dst[i] = __ldg(src + i);
   __syncthreads();
 }
-#define MORSE_SCREEN_KERNELS(NAME, BODY, THREADS, MIN)                       \
-  template <bool H>                                                          \
+#define MORSE_SCREEN_KERNELS(TEMPLATE, NAME, BODY, THREADS, MIN)             \
+  TEMPLATE                                                                   \
   __global__ void __launch_bounds__(THREADS, MIN)                            \
       NAME(const SearchParams P, const ScreenBufs B) {                       \
     BODY(P, B);                                                              \
   }                                                                          \
-  template <bool H>                                                          \
+  TEMPLATE                                                                   \
   __global__ void __launch_bounds__(THREADS, MIN)                            \
       NAME##_batch(const ScreenTask *t) {                                    \
     __shared__ ScreenTask s;                                                 \
     load_task(t + blockIdx.y, s);                                            \
     BODY(s.F.S, s.B);                                                        \
   }
-MORSE_SCREEN_KERNELS(k_screen, screen_all<H>, kScreenThreads, 4)
-MORSE_SCREEN_KERNELS(k_pilot_list, make_pilot_list, kListThreads, 1)
+#define MORSE_BY_TABLE template <bool H>
+#define MORSE_EITHER_TABLE
+MORSE_SCREEN_KERNELS(MORSE_BY_TABLE, k_screen, screen_all<H>, kScreenThreads,
+                     4)
+MORSE_SCREEN_KERNELS(MORSE_EITHER_TABLE, k_pilot_list, make_pilot_list,
+                     kListThreads, 1)
 #define MORSE_PILOT(P, B) pilot_bounds<H, false>(P, B)
-MORSE_SCREEN_KERNELS(k_pilot, MORSE_PILOT, kPilotWarps * 32, 4)
+MORSE_SCREEN_KERNELS(MORSE_BY_TABLE, k_pilot, MORSE_PILOT, kPilotWarps * 32, 4)
 #undef MORSE_PILOT
-MORSE_SCREEN_KERNELS(k_list, make_list, kListThreads, 1)
-MORSE_SCREEN_KERNELS(k_rescreen, rescreen_listed<H>, kScreenThreads, 4)
+MORSE_SCREEN_KERNELS(MORSE_EITHER_TABLE, k_list, make_list, kListThreads, 1)
+MORSE_SCREEN_KERNELS(MORSE_BY_TABLE, k_rescreen, rescreen_listed<H>,
+                     kScreenThreads, 4)
+#undef MORSE_BY_TABLE
+#undef MORSE_EITHER_TABLE
 #undef MORSE_SCREEN_KERNELS
 
 template <bool H>
@@ -844,7 +855,7 @@ static int append_grid(const SearchParams &P, int sm_count) {
 cudaError_t launch_screen_pilot_list(const SearchParams &P,
                                      const ScreenBufs &B, int sm_count,
                                      cudaStream_t st) {
-  k_pilot_list<false><<<append_grid(P, sm_count), kListThreads, 0, st>>>(P, B);
+  k_pilot_list<<<append_grid(P, sm_count), kListThreads, 0, st>>>(P, B);
   return cudaGetLastError();
 }
 
@@ -871,7 +882,7 @@ cudaError_t launch_bounds(const SearchParams &P, const ScreenBufs &B,
 
 cudaError_t launch_screen_list(const SearchParams &P, const ScreenBufs &B,
                                int sm_count, cudaStream_t st) {
-  k_list<false><<<append_grid(P, sm_count), kListThreads, 0, st>>>(P, B);
+  k_list<<<append_grid(P, sm_count), kListThreads, 0, st>>>(P, B);
   return cudaGetLastError();
 }
 
@@ -900,9 +911,9 @@ static cudaError_t screen_batch(const ScreenTask *t, int n,
       (B0.pilot_cap + kPilotTpg - 1) / kPilotTpg + kSampleBlocks;
   // a few tiles per block amortise the subset's staging and the histogram
   k_screen_batch<H><<<dim3((tiles + 3) / 4, y), kScreenThreads, 0, st>>>(t);
-  k_pilot_list_batch<false><<<dim3(chunks, y), kListThreads, 0, st>>>(t);
+  k_pilot_list_batch<<<dim3(chunks, y), kListThreads, 0, st>>>(t);
   k_pilot_batch<H><<<dim3(pilot, y), kPilotWarps * 32, 0, st>>>(t);
-  k_list_batch<false><<<dim3(chunks, y), kListThreads, 0, st>>>(t);
+  k_list_batch<<<dim3(chunks, y), kListThreads, 0, st>>>(t);
   if (rescreen)
     k_rescreen_batch<H><<<dim3((tiles + 7) / 8, y), kScreenThreads, 0, st>>>(
         t);

@@ -588,11 +588,6 @@ __global__ void k_fill(const FillParams F) {
 // sweep of the epochs.  With the threshold of a good pilot the candidates
 // are little more than the k records themselves (config 1: 267 for 256);
 // more than kCandMax go the general way.
-// Blocks per search of a batch's listed search: a long light curve of weak
-// signal can leave one search with most of the batch's work (12 blocks: 9.1
-// ms with half the SMs idle in its tail).
-constexpr int kListBatchBlocks = 76;
-
 constexpr int kFinishThreads = 1024, kFinishPer = kFinishThreads / 16;
 
 __device__ __forceinline__ void finish(const FillParams &F,
@@ -888,6 +883,12 @@ cudaError_t launch_finish(const FillParams &F, cudaStream_t st) {
   k_finish<<<kCandMax / kFinishPer, kFinishThreads, kFinishSmem, st>>>(F);
   return cudaGetLastError();
 }
+
+// Blocks per search of a batch's listed search, a quarter of what two per SM
+// hold: a long light curve of weak signal can leave one search with most of
+// the batch's work (12 blocks: 9.1 ms with half the SMs idle in its tail; one
+// per SM 10.2 -> 10.5 ms).
+constexpr int kListBatchBlocks = 76;
 
 cudaError_t launch_list_batch(const ScreenTask *t, int n,
                               const SearchParams &P0, cudaStream_t st) {

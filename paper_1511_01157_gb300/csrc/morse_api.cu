@@ -580,7 +580,6 @@ void event_params(const morse_event *ev, SearchParams *P) {
     ScreenLv &V = P->lv[l];
     V.ep = ev->ep + u.off;
     V.m = u.m;
-    V.S1 = (float)u.S1;
     V.iS1 = (float)(1.0 / u.S1);
     V.SF = (float)u.SF;
     V.sqSFF = nextafterf((float)sqrt(u.SFF), INFINITY);

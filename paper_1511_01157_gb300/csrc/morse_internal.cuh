@@ -244,7 +244,7 @@ constexpr int kPubLevels = 3;
 struct ScreenLv {
   const float4 *ep;
   int m;
-  float S1, iS1, SF, sqSFF, CFF;  // CFF rounded down, sqSFF up
+  float iS1, SF, sqSFF, CFF;  // CFF rounded down, sqSFF up
   float g;                  // relative error bound of the FP32 sums, doubled
 };
 
@@ -512,7 +512,8 @@ cudaError_t launch_screen_pilot(const SearchParams &P, const ScreenBufs &B,
 // code does not exceed it
 cudaError_t launch_screen_list(const SearchParams &P, const ScreenBufs &B,
                                int sm_count, cudaStream_t st);
-// the listed trajectories on the second subset (P.n_lv >= 2)
+// the listed trajectories on the second and third subsets (nothing is done
+// below three)
 cudaError_t launch_rescreen(const SearchParams &P, const ScreenBufs &B,
                             int sm_count, cudaStream_t st);
 // shared memory of the listed search with staged epochs (0: they do not
