@@ -428,15 +428,16 @@ morse_status morse_grid_chi2_noalloc(morse_ctx *ctx, const morse_event *ev,
                                      const morse_grid *grid, morse_fit *out);
 
 /* Batched search: n_ev light curves (any lengths) against n_maps maps,
- * every (event, map) pair searched over the same grid, in one persistent
- * kernel launch.  The pair (e, m) gets the top_k fits of
+ * every (event, map) pair searched over the same grid, in the same launches.
+ * The pair (e, m) gets the top_k fits of
  * morse_grid_chi2(ev[e], maps[m], grid), bit for bit, in
  * out[(e * n_maps + m) * top_k + r] (host, caller-allocated).  The maps
  * must share npix, extent and lookup table (FP32 or FP16); grid t0 values
  * are absolute times, each event's relative to its own t_ref.  The whole
- * sequence (a strided pilot pass per pair that seeds the pair's pruning
- * threshold, the main pass, the per-pair merges and the record fill) is
- * captured in a CUDA graph, which later calls of the same shape update and
+ * sequence (the pairs' screened searches, or where they are not screened a
+ * strided pilot pass per pair that seeds its pruning threshold, the
+ * persistent main pass over what is left, the per-pair merges and the record
+ * fill) is captured in a CUDA graph, which later calls of the same shape update and
  * replay.  Launch shapes per epoch-count bucket (trajectories per warp
  * group, groups per work unit, shared-memory staging of the epochs) come
  * from the autotuner (morse_batch_tuning) or from the default rule.
